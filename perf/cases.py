@@ -135,6 +135,11 @@ def _threshold(p, ratio):
     return float(((s[-k - 1] + s[-k]) / 2).float())
 
 
+def _ring(c):
+    """Slots of a ring cache that serves windows of W: allocated in blocks of 64."""
+    return -(-c["W"] // 64) * 64
+
+
 def _inputs(c, seed):
     """Everything of a case that is drawn; the same for prepare() and exact()."""
     g = _gen(seed)
@@ -149,7 +154,7 @@ def _inputs(c, seed):
         B, Hkv = c["B"], c["Hkv"]
         for n in ("qL", "qG"):
             x[n] = _bf(g, B, Hq, D)
-        for n, r in (("kR", c["W"]), ("vR", c["W"]), ("kG", c["L"]), ("vG", c["L"])):
+        for n, r in (("kR", _ring(c)), ("vR", _ring(c)), ("kG", c["L"]), ("vG", c["L"])):
             x[n] = _bf(g, B, r, Hkv, D)
         x["len"] = torch.randint(max(1, c["L"] // 2), c["L"] + 1, (B,), generator=g, device="cuda", dtype=torch.int32)
         x["p"] = torch.rand((B, 1), generator=g, device="cuda") * 0.98 + 0.01
@@ -216,7 +221,7 @@ def prepare(case, seed):
         return s
     Hq, D = c["Hq"], c["D"]
     if kind == "decode":
-        B, Hkv, W, Lc = c["B"], c["Hkv"], c["W"], c["L"]
+        B, Hkv, W, Lc = c["B"], c["Hkv"], _ring(c), c["L"]
         s["sel"] = _selection(B, 1)
         s["ws_s"] = _ws("logo_select_workspace_size", L.Dims(B, 1, 1, 1, 64))
         s["ws_l"] = _ws("logo_decode_workspace_size", L.Dims(B, W, Hq, Hkv, D))
@@ -426,7 +431,7 @@ def exact(case, seed):
         z = (x["p"] > x["b_th"]).double()
         ol, og = (torch.zeros((B, 1, Hq, D), dtype=torch.float64, device="cuda") for _ in range(2))
         for b, n in enumerate(x["len"].tolist()):
-            s = torch.arange(max(0, n - c["W"]), n, device="cuda") % c["W"]
+            s = torch.arange(max(0, n - c["W"]), n, device="cuda") % _ring(c)
             last = torch.tensor([len(s) - 1], device="cuda")
             ol[b] = _attn(x["qL"][b:b + 1], x["kR"][b, s], x["vR"][b, s], last, inf)[0]
             if z[b, 0] > 0:
