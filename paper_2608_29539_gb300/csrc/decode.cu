@@ -77,12 +77,13 @@ struct DecCfg {
 constexpr int kDecMaxChunks = 64;  // chunks per cache at most (the merge's weights: group x chunks <= 16 x 64)
 
 // Row j of the cache holds position pos_of(j) (or none: -1).  Dense cache:
-// j itself while j < len.  Ring of R slots: the latest position congruent to j
-// modulo R that is in the cache.
+// j itself while j < len (len <= R).  Ring of R slots: the latest position
+// congruent to j modulo R that is in the cache; a last sub-tile may reach past
+// the ring's R slots, and those rows hold nothing.
 template <bool RING>
 __device__ __forceinline__ int pos_of(int j, int len, int R)
 {
-    if (j >= len) return -1;
+    if (j >= len || (RING && j >= R)) return -1;
     return RING ? j + R * ((len - 1 - j) / R) : j;
 }
 

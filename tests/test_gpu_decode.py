@@ -73,6 +73,21 @@ def test_decode_local_ring(D, Hq, Hkv, R):
     check_close(np32(o), ref, f"decode local D{D} Hq{Hq} Hkv{Hkv} R{R}")
 
 
+@pytest.mark.parametrize("R,W", [(100, 100), (1000, 300), (1, 1), (65, 64)])
+def test_decode_local_ring_of_any_length(R, W):
+    """A ring whose last 64-row sub-tile reaches past its slots: the rows
+    beyond it hold nothing and weigh nothing in the softmax."""
+    from paper_2608_29539_gb300 import logo as L
+    Hq, Hkv, D = 4, 2, 128
+    B, Lmax = len(LENS), max(LENS)
+    kL, vL, _, _, qL, _ = _caches(B, Lmax, Hq, Hkv, D, seed=R + W)
+    dev = torch.device("cuda")
+    seq_len = torch.tensor(LENS, dtype=torch.int32, device=dev)
+    o = L.logo_decode_local_attn(qL.to(dev), _ring(kL, LENS, R, W).to(dev), _ring(vL, LENS, R, W).to(dev), seq_len, W)
+    torch.cuda.synchronize()
+    check_close(np32(o), _oracle_new_token(qL, kL, vL, LENS, W, list(range(B))), f"decode local ring R{R} W{W}")
+
+
 @pytest.mark.parametrize("D,Hq,Hkv", [(128, 8, 2), (64, 4, 4), (128, 16, 1)])
 def test_decode_global_selected_rows_only(D, Hq, Hkv):
     from paper_2608_29539_gb300 import logo as L
