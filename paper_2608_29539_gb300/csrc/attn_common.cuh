@@ -51,14 +51,7 @@ struct FwdItem {
     int slot;            // global split entry: partial-result slot; otherwise -1
 };
 
-// Does KV block n need the per-element visibility test for any row of the
-// item?  Rows see keys s with pos - W < s <= pos.
-__device__ __forceinline__ bool block_needs_mask(int n, int pos_min, int pos_max, int window)
-{
-    const int k0 = n * kBN, k1 = n * kBN + kBN - 1;
-    return !(k1 <= pos_min && k0 > pos_max - window);
-}
-
+// Rows see keys s with pos - W < s <= pos.
 __device__ __forceinline__ bool key_visible(int key, int pos, int window)
 {
     return key <= pos && key > pos - window;

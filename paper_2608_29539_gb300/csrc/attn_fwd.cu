@@ -3,27 +3,36 @@
 //   logo_local_attn_fwd          O^L = SoftmaxAttn_W(Q^L, K^L, V^L)   (Eq. 6)
 //   logo_global_sparse_attn_fwd  O^G_I = SoftmaxAttn_inf(Q^G_I, K^G, V^G) (Eq. 8)
 //
-// One persistent kernel template serves both.  A CTA (12 warps) loops over
+// One persistent kernel template serves both.  A CTA (16 warps) loops over
 // work items = (128-row query tile, query head):
-//   warp 8      TMA producer: Q tile once per item, then K blocks (local: K
-//               and V blocks) through a ring of shared-memory stages
-//               (128-byte swizzle)
-//   warp 11     global branch: V blocks through a ring of their own
-//   warp 9      S issuer (one thread): S = Q K^T into one of two TMEM S buffers
-//   warp 10     P.V issuer (one thread): O += P V into the TMEM O accumulator
+//   warp 12     TMA producer: Q tile once per item, then K blocks through a
+//               ring of shared-memory stages (128-byte swizzle)
+//   warp 15     V blocks through a ring of their own
+//   warp 13     S issuer (one thread): S = Q K^T into one of two TMEM S buffers
+//   warp 14     P.V issuer (one thread): O += P V into the TMEM O accumulator
 //               with P read straight from TMEM.  Two issuing threads keep the
 //               tensor pipe fed while either waits for its inputs: the issue
 //               queue is short, so a single thread that stops to wait starves
 //               the pipe (measured: 1728 vs 2427 TFLOP/s on the same MMA stream).
-//   warps 0..3  softmax: one thread per query row (its TMEM lane).  Online
-//               softmax in the log2 domain with conditional rescaling of O
-//               (only when the running max grows by more than 2^8); P goes
-//               back to TMEM as bf16 pairs, into one of two P buffers, so the
-//               softmax of block n never waits for the P.V of block n-1
-//               unless it has to rescale O.
-//   warps 4..7  epilogue: O out of TMEM once an item's last P.V is done,
-//               normalised and stored while the softmax warps start the next
-//               item.
+//   warps 0..3  softmax of the even KV blocks (S and P buffer 0), warps 4..7 of
+//               the odd ones (buffer 1); one thread per query row (its TMEM
+//               lane).  Online softmax in the log2 domain with conditional
+//               rescaling of O (only when the running max grows by more than
+//               2^8); P goes back to TMEM as bf16 pairs.  The running max is
+//               the one thing the blocks of a row share: the thread of block n
+//               reads the one block n-1 left in shared memory, right after its
+//               own row max, and leaves its own there before the exponentials,
+//               so the two warpgroups run half a block apart.  Each keeps the
+//               row sum of its own blocks.  One warpgroup for every block made
+//               its own latencies (barriers, TMEM round trips, ~2700 clocks a
+//               block with masks) the period; with two, measured at 16K (32
+//               heads, d 128) local 275 -> 236 us and global 242 -> 223 us, at
+//               8K (2 x 16 heads, d 64) local 140 -> 105 us.  What is left is
+//               ~1600 clocks a block against ~1350 of the same kernel without
+//               any softmax arithmetic.
+//   warps 8..11 epilogue: the two row sums combined, O out of TMEM once an
+//               item's last P.V is done, normalised and stored while the
+//               softmax warps are on the next item.
 // The KV blocks of an item are only those some row can see; blocks where
 // every row sees every key skip the per-element predicate (App. B's
 // three-region traversal; for the local branch the window edge is a second
@@ -46,32 +55,58 @@ template <int D>
 struct FwdCfg {
     static constexpr int kSub = D / 64;             // 64-column (128-byte) sub-tiles per row
     static constexpr int kTileBytes = kBM * D * 2;  // one Q / K / V tile
-    // K/V ring of three stages.  The global branch runs K and V as two rings
-    // with a producer each: a K stage is free once S of its block is done, a
-    // V stage once P.V is, so K loads run further ahead (global fwd -7% at
-    // 16K).  The local branch keeps one producer loading K and V of a block
-    // together into one stage that P.V frees (its short items ran 6% slower
-    // with the split).
-    static constexpr int kStages = 3;
+    // K and V are two rings with a producer each: a K stage is free once S of
+    // its block is done, a V stage once P.V is.  (One ring whose stage holds K
+    // and V of a block made S of block n + 3 wait for P.V of block n: with two
+    // softmax warpgroups that chain, not the tensor pipe, set the local
+    // branch's period.)  Three stages each at d = 128.
+    // d = 64 has the shared memory for six stages, and for a second Q buffer,
+    // so that an item's Q lands while the item before is computed.
+    static constexpr int kStages = D == 64 ? 6 : 3;
+    static constexpr int kQBufs = D == 64 ? 2 : 1;
     static constexpr int kOffQ = 0;
-    static constexpr int kOffK = kOffQ + kTileBytes;
+    static constexpr int kOffK = kOffQ + kQBufs * kTileBytes;
     static constexpr int kOffV = kOffK + kStages * kTileBytes;
-    static constexpr int kSmemBytes = kOffV + kStages * kTileBytes + 1024;  // + alignment slack
-    static constexpr uint32_t kColO = 0;     // O accumulator (D columns, fp32)
+    // the dynamic array is declared with the tiles' 1024-byte alignment, so it
+    // starts at the kernel's (at most 3 KB of) static shared memory rounded up
+    static constexpr int kSmemBytes = kOffV + kStages * kTileBytes;
+    // O accumulator (D columns, fp32); d = 64 has room for two, used in turn by
+    // the items, so that an item's first P.V never waits for the epilogue
+    static constexpr int kOBufs = D == 64 ? 2 : 1;
+    static constexpr uint32_t kColO = 0;
     static constexpr uint32_t kColS0 = 128;  // S buffers (128 columns, fp32)
     static constexpr uint32_t kColS1 = 256;
     static constexpr uint32_t kColP0 = 384;  // P buffers (128 keys as bf16 pairs: 64 columns)
     static constexpr uint32_t kColP1 = 448;
     static constexpr uint32_t kTmemCols = 512;
-    // 12 warps: softmax (0..3), epilogue (4..7), Q/K(/V) producer, S issuer,
-    // P.V issuer, global branch: V producer (8..11).  Launched at 168 registers a thread (384 x 168 =
-    // 64,512); the softmax warpgroup takes 224 (its row of S lives in
-    // registers), the epilogue 168 (a row of O), the control warps 88:
-    // 128 x (224 + 168 + 88) = 61,440.
-    static constexpr int kThreads = 384;
-    static constexpr uint32_t kRegsSoftmax = 224;
-    static constexpr uint32_t kRegsEpilogue = 168;
-    static constexpr uint32_t kRegsControl = 88;
+    // 16 warps: softmax of even and of odd blocks (0..3, 4..7), epilogue
+    // (8..11), Q/K producer, S issuer, P.V issuer, V producer (12..15).  Launched at 128 registers a thread (512 x 128 =
+    // 65,536); the softmax warpgroups take 184 (a row of S lives in
+    // registers; spills cost more than anything else here, as they miss the
+    // few KB of L1 that the tiles leave), the epilogue 96, the control warps 48:
+    // 128 x (184 + 184 + 96 + 48) = 65,536.
+    static constexpr int kThreads = 512;
+    static constexpr uint32_t kRegsSoftmax = 184;
+    static constexpr uint32_t kRegsEpilogue = 96;
+    static constexpr uint32_t kRegsControl = 48;
+};
+
+// Division of 0 <= n < 2^31 by a fixed d: n / d = (n m) >> (31 + l) with
+// l = ceil(log2 d), m = ceil(2^(31+l) / d) < 2^32 (Granlund and Montgomery,
+// "Division by invariant integers using multiplication").
+struct FastDiv {
+    uint32_t m, l;
+    int d;
+    FastDiv(int div = 1) : d(div)
+    {
+        l = 0;
+        while ((1ll << l) < div) ++l;
+        m = static_cast<uint32_t>(((1ull << (31 + l)) + div - 1) / div);
+    }
+    __device__ __forceinline__ int div(int n) const
+    {
+        return static_cast<int>(__umulhi(static_cast<uint32_t>(n) << 1, m) >> l);
+    }
 };
 
 struct FwdParams {
@@ -89,6 +124,7 @@ struct FwdParams {
     float* l_part;                 // ... and their row sums
     int B, T, Hq, Hkv, window, cap;
     int q_tiles;                   // local: query tiles per sequence
+    FastDiv by_hq, by_group, by_q_tiles;  // Hq, Hq / Hkv, q_tiles: every role decodes every item
     float scale_log2;              // softmax scale * log2(e)
 };
 
@@ -96,12 +132,12 @@ template <bool GLOBAL>
 __device__ __forceinline__ FwdItem decode_item(const FwdParams& p, int k)
 {
     FwdItem it;
-    it.h = k % p.Hq;
-    it.kvh = it.h / (p.Hq / p.Hkv);
-    const int tile = k / p.Hq;
+    const int tile = p.by_hq.div(k);
+    it.h = k - tile * p.Hq;
+    it.kvh = p.by_group.div(it.h);
     if (!GLOBAL) {
-        it.b = tile / p.q_tiles;
-        const int qt = tile % p.q_tiles;
+        it.b = p.by_q_tiles.div(tile);
+        const int qt = tile - it.b * p.q_tiles;
         it.row0 = qt * kBM;
         it.nrows = min(kBM, p.T - it.row0);
         it.pos_min = it.row0;
@@ -124,64 +160,49 @@ __device__ __forceinline__ FwdItem decode_item(const FwdParams& p, int k)
 }
 
 // Visibility inside one 128-key block: the row sees keys c with lo <= c <= hi;
-// every other s[c] becomes -inf.  Called by all 32 lanes of a warp, whose rows
-// are consecutive, so most 32-key groups are seen whole by every row of the
-// warp or by none of them; one warp reduction classifies the groups.  Selects
-// and moves cost two issue cycles per warp on this pipe, so only the groups
-// in between get the per-key select, and only against the bound that cuts
-// them; unseen groups get plain moves.
+// every other s[c] becomes -inf.  One 32-bit mask per 32 keys, whose bits
+// become the predicates of the selects: straight-line code, a select per key
+// and nothing per key to compare.  (Sorting the groups of 32 into seen whole,
+// unseen and cut, with a loop for each, was fewer instructions and took
+// 1100-2300 clocks a masked block against 300-500 of an unmasked one: its
+// branches ran from cold instruction cache.)
 __device__ __forceinline__ void mask_row_block(float (&s)[kBN], int lo, int hi)
 {
-    uint32_t cls = 0;  // per group g: bit g seen whole, 4+g unseen, 8+g lo does not cut, 12+g hi does not cut
 #pragma unroll
     for (int g = 0; g < kBN / 32; ++g) {
-        const bool lo_cuts = lo > 32 * g, hi_cuts = hi < 32 * g + 31;
-        cls |= (!lo_cuts && !hi_cuts) ? (1u << g) : 0u;
-        cls |= (hi < 32 * g || lo > 32 * g + 31) ? (16u << g) : 0u;
-        cls |= lo_cuts ? 0u : (256u << g);
-        cls |= hi_cuts ? 0u : (4096u << g);
-    }
-    cls = __reduce_and_sync(0xffffffffu, cls);
+        uint32_t up, down;  // (PTX shifts by 32 and more give 0)
+        asm("shr.u32 %0, 0xffffffff, %1;" : "=r"(up) : "r"(max(31 - (hi - 32 * g), 0)));
+        asm("shl.b32 %0, 0xffffffff, %1;" : "=r"(down) : "r"(max(lo - 32 * g, 0)));
+        const uint32_t m = up & down;
 #pragma unroll
-    for (int g = 0; g < kBN / 32; ++g) {
-        if (cls & (1u << g)) continue;
-        if (cls & (16u << g)) {
-            // (an opaque move: a constant assigned in this branch made the
-            // compiler spill the row)
-#pragma unroll
-            for (int i = 0; i < 32; ++i) asm volatile("mov.b32 %0, 0xff800000;" : "=f"(s[32 * g + i]));
-        } else if (cls & (256u << g)) {
-#pragma unroll
-            for (int i = 0; i < 32; ++i) s[32 * g + i] = 32 * g + i <= hi ? s[32 * g + i] : -INFINITY;
-        } else if (cls & (4096u << g)) {
-#pragma unroll
-            for (int i = 0; i < 32; ++i) s[32 * g + i] = 32 * g + i >= lo ? s[32 * g + i] : -INFINITY;
-        } else {
-#pragma unroll
-            for (int i = 0; i < 32; ++i)
-                s[32 * g + i] = (32 * g + i >= lo && 32 * g + i <= hi) ? s[32 * g + i] : -INFINITY;
-        }
+        for (int i = 0; i < 32; ++i) s[32 * g + i] = (m & (1u << i)) ? s[32 * g + i] : -INFINITY;
     }
 }
 
 template <int D, bool GLOBAL>
-__global__ void __launch_bounds__(384, 1) attn_fwd_kernel(const __grid_constant__ FwdParams p)
+__global__ void __launch_bounds__(512, 1) attn_fwd_kernel(const __grid_constant__ FwdParams p)
 {
     using C = FwdCfg<D>;
-    static_assert(128 * (C::kRegsSoftmax + C::kRegsEpilogue + C::kRegsControl) <= 384 * 168,
+    static_assert(128 * (2 * C::kRegsSoftmax + C::kRegsEpilogue + C::kRegsControl) <= 512 * 128,
                   "register split exceeds the launch allocation");
-    extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    __shared__ __align__(8) uint64_t bar_q_full, bar_q_empty, bar_drain, bar_drain_pv;
-    // bar_k_empty frees a K stage (global) or a K/V stage (local); bar_v_empty
-    // a V stage (global only)
+    extern __shared__ __align__(1024) uint8_t smem[];
+    __shared__ __align__(8) uint64_t bar_q_full[C::kQBufs], bar_q_empty[C::kQBufs], bar_drain, bar_drain_pv;
     __shared__ __align__(8) uint64_t bar_k_full[C::kStages], bar_k_empty[C::kStages];
     __shared__ __align__(8) uint64_t bar_v_full[C::kStages], bar_v_empty[C::kStages];
-    __shared__ __align__(8) uint64_t bar_s_full[2], bar_s_empty[2], bar_p_full[2], bar_p_free[2];
-    // softmax -> epilogue: 1/l of every row of an item (two slots), and O's
-    // columns free again once the epilogue has copied them out
-    __shared__ __align__(8) uint64_t bar_l_full[2], bar_l_empty[2], bar_o_free;
-    __shared__ float sh_inv_l[2][kBM];
+    __shared__ __align__(8) uint64_t bar_s_full[2], bar_s_empty[2], bar_p_full[2];
+    // P.V of block n done: barrier n % 4, so that a wait for block n - 1 or
+    // n - 2 can never be confused with the barrier's phase before
+    __shared__ __align__(8) uint64_t bar_pv_done[4];
+    // running max of every row after the newest block, handed from one softmax
+    // warpgroup's thread of the row to the other's (so one copy is enough): a
+    // barrier per warp and block parity
+    __shared__ __align__(8) uint64_t bar_m[2][4];
+    __shared__ float sh_m[kBM];
+    // softmax -> epilogue: max and sum of every row of an item over the even
+    // and over the odd blocks, and O's columns free again once the epilogue
+    // has copied them out
+    __shared__ __align__(8) uint64_t bar_l_full, bar_l_empty, bar_o_free[C::kOBufs];
+    __shared__ float2 sh_ml[2][kBM];
     __shared__ uint32_t tmem_base_sh;
     __shared__ volatile int abort_flag;
     // global branch: items are taken dynamically (longest first, whichever CTA
@@ -195,10 +216,16 @@ __global__ void __launch_bounds__(384, 1) attn_fwd_kernel(const __grid_constant_
     const uint32_t sK = smem_u32(smem + C::kOffK);
     const uint32_t sV = smem_u32(smem + C::kOffV);
 
+    if (smem_u32(smem) & 1023u) {  // (uniform) the swizzled tiles need the alignment asked for
+        record_status(LOGO_ERR_CUDA);
+        return;
+    }
     if (threadIdx.x == 0) {
         abort_flag = 0;
-        mbar_init(smem_u32(&bar_q_full), 1);
-        mbar_init(smem_u32(&bar_q_empty), 1);
+        for (int s = 0; s < C::kQBufs; ++s) {
+            mbar_init(smem_u32(&bar_q_full[s]), 1);
+            mbar_init(smem_u32(&bar_q_empty[s]), 1);
+        }
         mbar_init(smem_u32(&bar_drain), 1);
         mbar_init(smem_u32(&bar_drain_pv), 1);
         for (int s = 0; s < C::kStages; ++s) {
@@ -210,20 +237,22 @@ __global__ void __launch_bounds__(384, 1) attn_fwd_kernel(const __grid_constant_
         for (int s = 0; s < 4; ++s) {
             mbar_init(smem_u32(&bar_item_full[s]), 1);
             // the V producer, the two MMA threads, one lane per softmax / epilogue warp
-            mbar_init(smem_u32(&bar_item_empty[s]), 11);
+            mbar_init(smem_u32(&bar_item_empty[s]), 15);
+            mbar_init(smem_u32(&bar_pv_done[s]), 1);
+            mbar_init(smem_u32(&bar_m[0][s]), 1);
+            mbar_init(smem_u32(&bar_m[1][s]), 1);
         }
         for (int s = 0; s < 2; ++s) {
             mbar_init(smem_u32(&bar_s_full[s]), 1);
             mbar_init(smem_u32(&bar_s_empty[s]), 128);
             mbar_init(smem_u32(&bar_p_full[s]), 128);
-            mbar_init(smem_u32(&bar_p_free[s]), 1);
-            mbar_init(smem_u32(&bar_l_full[s]), 128);
-            mbar_init(smem_u32(&bar_l_empty[s]), 128);
         }
-        mbar_init(smem_u32(&bar_o_free), 128);
+        mbar_init(smem_u32(&bar_l_full), 256);
+        mbar_init(smem_u32(&bar_l_empty), 128);
+        for (int s = 0; s < C::kOBufs; ++s) mbar_init(smem_u32(&bar_o_free[s]), 128);
         fence_mbar_init();
     }
-    if (warp == 9) {
+    if (warp == 13) {
         tmem_alloc(smem_u32(&tmem_base_sh), C::kTmemCols);
         tmem_relinquish();
     }
@@ -253,10 +282,10 @@ __global__ void __launch_bounds__(384, 1) attn_fwd_kernel(const __grid_constant_
         return k;
     };
 
-    if (warp >= 8) {
+    if (warp >= 12) {
         // ------------------------------------------------------------ control warps
         setmaxnreg_dec<C::kRegsControl>();
-    if (warp == 8) {
+    if (warp == 12) {
         // ------------------------------------------------------------ producer
         if (lane == 0) {
             tma_prefetch_desc(&p.tm_q);
@@ -284,12 +313,19 @@ __global__ void __launch_bounds__(384, 1) attn_fwd_kernel(const __grid_constant_
                 }
                 if (k < 0) break;
                 const FwdItem it = decode_item<GLOBAL>(p, k);
-                if (!(ok = mbar_wait(smem_u32(&bar_q_empty), (item_i & 1) ^ 1, &abort_flag))) break;
-                const uint32_t qb = smem_u32(&bar_q_full);
+                const int qs = item_i % C::kQBufs, qf = item_i / C::kQBufs;
+                if (!(ok = mbar_wait(smem_u32(&bar_q_empty[qs]), (qf & 1) ^ 1, &abort_flag))) break;
+                const uint32_t qb = smem_u32(&bar_q_full[qs]);
                 mbar_arrive_expect_tx(qb, C::kTileBytes);
                 for (int s = 0; s < C::kSub; ++s)
-                    tma_load_4d(sQ + s * 16384, &p.tm_q, qb, 64 * s, it.h, it.row0, GLOBAL ? 0 : it.b, pol_q);
+                    tma_load_4d(sQ + qs * C::kTileBytes + s * 16384, &p.tm_q, qb, 64 * s, it.h, it.row0, GLOBAL ? 0 : it.b, pol_q);
                 ++q_fills;
+                if (!GLOBAL && C::kQBufs == 1 && k + gridDim.x < n_items) {
+                    // one Q buffer: the next item's Q can only be copied once S of
+                    // this item's last block is done, so bring it as far as L2 now
+                    const FwdItem nx = decode_item<GLOBAL>(p, k + gridDim.x);
+                    for (int s = 0; s < C::kSub; ++s) tma_prefetch_4d(&p.tm_q, 64 * s, nx.h, nx.row0, nx.b);
+                }
                 for (int n = it.blk_lo; n <= it.blk_hi; ++n, ++kv_it) {
                     const int st = kv_it % C::kStages, f = kv_it / C::kStages;
                     if (!(ok = mbar_wait(smem_u32(&bar_k_empty[st]), (f & 1) ^ 1, &abort_flag))) break;
@@ -298,29 +334,20 @@ __global__ void __launch_bounds__(384, 1) attn_fwd_kernel(const __grid_constant_
                     for (int s = 0; s < C::kSub; ++s)
                         tma_load_4d(sK + st * C::kTileBytes + s * 16384, &p.tm_k, kb, 64 * s, it.kvh, n * kBN, it.b,
                                     pol_kv);
-                    if (!GLOBAL) {  // V of the same block into the same stage
-                        const uint32_t vb = smem_u32(&bar_v_full[st]);
-                        mbar_arrive_expect_tx(vb, C::kTileBytes);
-                        for (int s = 0; s < C::kSub; ++s)
-                            tma_load_4d(sV + st * C::kTileBytes + s * 16384, &p.tm_v, vb, 64 * s, it.kvh, n * kBN,
-                                        it.b, pol_kv);
-                    }
                     last_fill[st] = f;
                 }
                 if (!ok) break;
             }
             if (!ok) {  // let copies already issued land before the CTA exits
-                if (q_fills > 0) mbar_wait_drain(smem_u32(&bar_q_full), (q_fills - 1) & 1);
+                for (int i = max(0, q_fills - C::kQBufs); i < q_fills; ++i)
+                    mbar_wait_drain(smem_u32(&bar_q_full[i % C::kQBufs]), (i / C::kQBufs) & 1);
                 for (int s = 0; s < C::kStages; ++s)
-                    if (last_fill[s] >= 0) {
-                        mbar_wait_drain(smem_u32(&bar_k_full[s]), last_fill[s] & 1);
-                        if (!GLOBAL) mbar_wait_drain(smem_u32(&bar_v_full[s]), last_fill[s] & 1);
-                    }
+                    if (last_fill[s] >= 0) mbar_wait_drain(smem_u32(&bar_k_full[s]), last_fill[s] & 1);
             }
         }
-    } else if (warp == 9) {
+    } else if (warp == 13) {
         // ------------------------------------------------------------ S issuer
-        // S = Q K^T of every block; the P.V products come from warp 6, so that
+        // S = Q K^T of every block; the P.V products come from warp 14, so that
         // neither stream's waits leave the tensor pipe without queued work
         // (the issue queue is short: an issuing thread runs only a few
         // instructions ahead of execution)
@@ -333,7 +360,9 @@ __global__ void __launch_bounds__(384, 1) attn_fwd_kernel(const __grid_constant_
                 if (k < 0) break;
                 const FwdItem it = decode_item<GLOBAL>(p, k);
                 const int nblk = it.blk_hi - it.blk_lo + 1;
-                if (!(ok = mbar_wait(smem_u32(&bar_q_full), item_i & 1, &abort_flag))) break;
+                const int qs = item_i % C::kQBufs;
+                const uint32_t qbase = sQ + qs * C::kTileBytes;
+                if (!(ok = mbar_wait(smem_u32(&bar_q_full[qs]), (item_i / C::kQBufs) & 1, &abort_flag))) break;
                 for (int j = 0; j < nblk && ok; ++j) {
                     const int itg = s_it + j;
                     const int st = (kv_it + j) % C::kStages, f = (kv_it + j) / C::kStages;
@@ -346,14 +375,14 @@ __global__ void __launch_bounds__(384, 1) attn_fwd_kernel(const __grid_constant_
 #pragma unroll
                     for (int ks = 0; ks < D / 16; ++ks) {
                         const uint32_t off = (ks >> 2) * 16384 + (ks & 3) * 32;
-                        umma_bf16_ss(dcol, sdesc_sw128(sQ + off, 16, 1024), sdesc_sw128(kbase + off, 16, 1024), idS,
+                        umma_bf16_ss(dcol, sdesc_sw128(qbase + off, 16, 1024), sdesc_sw128(kbase + off, 16, 1024), idS,
                                      ks > 0 ? 1u : 0u);
                     }
                     umma_commit(smem_u32(&bar_s_full[buf]));
-                    if (GLOBAL) umma_commit(smem_u32(&bar_k_empty[st]));  // K of this block is read
+                    umma_commit(smem_u32(&bar_k_empty[st]));  // K of this block is read
                 }
                 if (!ok) break;
-                umma_commit(smem_u32(&bar_q_empty));
+                umma_commit(smem_u32(&bar_q_empty[qs]));
                 kv_it += nblk;
                 s_it += nblk;
             }
@@ -362,7 +391,7 @@ __global__ void __launch_bounds__(384, 1) attn_fwd_kernel(const __grid_constant_
                 mbar_wait_drain(smem_u32(&bar_drain), 0);
             }
         }
-    } else if (warp == 10) {
+    } else if (warp == 14) {
         // ------------------------------------------------------------ P.V issuer
         if (lane == 0) {
             constexpr uint32_t idPV = idesc_bf16_f32(kBM, D, false, true);
@@ -373,6 +402,8 @@ __global__ void __launch_bounds__(384, 1) attn_fwd_kernel(const __grid_constant_
                 if (k < 0) break;
                 const FwdItem it = decode_item<GLOBAL>(p, k);
                 const int nblk = it.blk_hi - it.blk_lo + 1;
+                const int ob = item_i % C::kOBufs;
+                const uint32_t ocol = tmem + C::kColO + ob * D;
                 for (int j = 0; j < nblk && ok; ++j) {
                     const int itg = s_it + j;
                     const int st = (kv_it + j) % C::kStages, f = (kv_it + j) / C::kStages;
@@ -380,18 +411,18 @@ __global__ void __launch_bounds__(384, 1) attn_fwd_kernel(const __grid_constant_
                     if (!(ok = mbar_wait(smem_u32(&bar_v_full[st]), f & 1, &abort_flag))) break;
                     // the item's first P.V overwrites O: the epilogue warps have
                     // copied the previous item's O out of TMEM
-                    if (j == 0 && !(ok = mbar_wait(smem_u32(&bar_o_free), (item_i & 1) ^ 1, &abort_flag))) break;
+                    if (j == 0 && !(ok = mbar_wait(smem_u32(&bar_o_free[ob]), ((item_i / C::kOBufs) & 1) ^ 1, &abort_flag)))
+                        break;
                     tc_fence_after();
                     const uint32_t vbase = sV + st * C::kTileBytes;
                     const uint32_t pcol = tmem + ((itg & 1) ? C::kColP1 : C::kColP0);
 #pragma unroll
                     for (int ks = 0; ks < kBN / 16; ++ks) {
                         const uint64_t bdesc = sdesc_sw128(vbase + ks * 2048, 16384, 1024);
-                        umma_bf16_ts(tmem + C::kColO, pcol + ks * 8, bdesc, idPV, (j > 0 || ks > 0) ? 1u : 0u);
+                        umma_bf16_ts(ocol, pcol + ks * 8, bdesc, idPV, (j > 0 || ks > 0) ? 1u : 0u);
                     }
-                    umma_commit(smem_u32(&bar_p_free[itg & 1]));
-                    // V of this block is read (local: K and V, whose S was done before P)
-                    umma_commit(smem_u32(GLOBAL ? &bar_v_empty[st] : &bar_k_empty[st]));
+                    umma_commit(smem_u32(&bar_pv_done[itg & 3]));
+                    umma_commit(smem_u32(&bar_v_empty[st]));  // V of this block is read
                 }
                 if (!ok) break;
                 kv_it += nblk;
@@ -402,10 +433,10 @@ __global__ void __launch_bounds__(384, 1) attn_fwd_kernel(const __grid_constant_
                 mbar_wait_drain(smem_u32(&bar_drain_pv), 0);
             }
         }
-    } else if (GLOBAL && warp == 11) {
+    } else {
         // ------------------------------------------------------------ V producer
-        // global branch: V blocks through their own ring (a stage is freed by
-        // the P.V that read it), so a V load never holds up the next K load
+        // V blocks through their own ring (a stage is freed by the P.V that
+        // read it), so a V load never holds up the next K load
         if (lane == 0) {
             const uint64_t pol_kv = policy_evict_last();
             int kv_it = 0;
@@ -434,40 +465,50 @@ __global__ void __launch_bounds__(384, 1) attn_fwd_kernel(const __grid_constant_
             }
         }
     }
-    } else if (warp < 4) {
+    } else if (warp < 8) {
         // ------------------------------------------------------------ softmax
         setmaxnreg_inc<C::kRegsSoftmax>();
+        const int par = warp >> 2;  // this warpgroup takes the blocks with itg % 2 == par
         const int quad = warp & 3;  // TMEM lane quadrant this warp may access
         const int r = quad * 32 + lane;
         const uint32_t lane_off = static_cast<uint32_t>(quad * 32) << 16;
-        const int window = GLOBAL ? kNoWindow : p.window;
-        int itg = 0;
+        const uint32_t scol = tmem + lane_off + (par ? C::kColS1 : C::kColS0);
+        const uint32_t pcol = tmem + lane_off + (par ? C::kColP1 : C::kColP0);
+        const uint32_t bar_m_mine = smem_u32(&bar_m[par][quad]), bar_m_other = smem_u32(&bar_m[par ^ 1][quad]);
+        int itg0 = 0;  // KV blocks of the items before this one
         bool ok = true;
         for (int item_i = 0;; ++item_i) {
             const int k = consume_item(item_i, &ok, true);
             if (k < 0) break;
-            const FwdItem it = decode_item<GLOBAL>(p, k);
-            const bool row_valid = r < it.nrows;
-            int mypos;
-            if (GLOBAL) mypos = row_valid ? p.pos[it.row0 + r] : it.pos_max;
-            else mypos = row_valid ? it.row0 + r : it.pos_max;
-            float m_ref = -INFINITY;  // running max, log2 domain
+            // all that the loop below keeps of the item: its blocks, the ones that
+            // every row sees whole (open_lo .. open_hi), and this row's position
+            int nblk, blk_lo, open_lo, open_hi, mypos;
+            {
+                const FwdItem it = decode_item<GLOBAL>(p, k);
+                blk_lo = it.blk_lo;
+                nblk = it.blk_hi - it.blk_lo + 1;
+                open_hi = (it.pos_min + 1) / kBN - 1;
+                open_lo = GLOBAL || it.pos_max < p.window ? 0 : (it.pos_max - p.window) / kBN + 1;
+                const bool row_valid = r < it.nrows;
+                if (GLOBAL) mypos = row_valid ? p.pos[it.row0 + r] : it.pos_max;
+                else mypos = row_valid ? it.row0 + r : it.pos_max;
+            }
+            // The barriers a block waits on are nearly always complete by then; each
+            // is tested (non-blocking) well before, so that the test's latency
+            // overlaps other work, and only a warp that found one open waits.
+            bool s_seen = false;  // S of the next block
+            float m_own = -INFINITY;  // running max (log2 domain) this warpgroup's row sum is relative to
             float l = 0.f;
-            // The S-ready and P-buffer-free barriers are nearly always complete
-            // by the time they are needed; each is tested (non-blocking) well
-            // before that point, so the test's latency overlaps other work, and
-            // only a warp that found one incomplete waits on it.
-            bool s_ready = false;  // S of this block seen complete while the previous block ended
-            for (int n = it.blk_lo; n <= it.blk_hi; ++n, ++itg) {
-                const int buf = itg & 1, use = itg >> 1;
-                if (!s_ready) {
-                    ok = mbar_wait(smem_u32(&bar_s_full[buf]), use & 1, &abort_flag);
+#pragma unroll 1
+            for (int j = (itg0 ^ par) & 1; j < nblk; j += 2) {
+                const int itg = itg0 + j, n = blk_lo + j;
+                if (!__all_sync(0xffffffffu, s_seen)) {
+                    ok = mbar_wait(smem_u32(&bar_s_full[par]), (itg >> 1) & 1, &abort_flag);
                     __syncwarp();
                     if (!ok) break;
                 }
                 tc_fence_after();
                 float s[kBN];
-                const uint32_t scol = tmem + lane_off + (buf ? C::kColS1 : C::kColS0);
                 {
                     uint32_t v[kBN / 32][32];
 #pragma unroll
@@ -479,11 +520,11 @@ __global__ void __launch_bounds__(384, 1) attn_fwd_kernel(const __grid_constant_
                         for (int i = 0; i < 32; ++i) s[c * 32 + i] = __uint_as_float(v[c][i]);
                 }
                 tc_fence_before();
-                mbar_arrive(smem_u32(&bar_s_empty[buf]));
-                // P buffer itg%2 is free once the P.V two blocks back is done
-                const bool p_free_seen = mbar_test(smem_u32(&bar_p_free[itg & 1]), ((itg >> 1) & 1) ^ 1);
-                if (block_needs_mask(n, it.pos_min, it.pos_max, window))
-                    mask_row_block(s, mypos - window + 1 - n * kBN, mypos - n * kBN);
+                mbar_arrive(smem_u32(&bar_s_empty[par]));
+                const bool m_seen = itg == 0 || mbar_test(bar_m_other, ((itg - 1) >> 1) & 1);
+                float m_ref = sh_m[r];  // (of no use unless m_seen)
+                if (n < open_lo || n > open_hi)
+                    mask_row_block(s, GLOBAL ? -1 : mypos - p.window + 1 - n * kBN, mypos - n * kBN);
                 // 4 independent 3-input max chains and 4 packed-pair sums keep
                 // dependency chains short; exp arguments are formed two at a
                 // time with f32x2 FMAs
@@ -498,25 +539,46 @@ __global__ void __launch_bounds__(384, 1) attn_fwd_kernel(const __grid_constant_
                     }
                 }
                 const float mx = max3f(mx4[0], mx4[1], fmaxf(mx4[2], mx4[3]));
+                // the running max after the block before.  Waited for across an
+                // item's edge too (its value does not count there), so that the
+                // two warpgroups' phases on these barriers never drift apart
+                if (!__all_sync(0xffffffffu, m_seen)) {
+                    ok = mbar_wait(bar_m_other, ((itg - 1) >> 1) & 1, &abort_flag);
+                    __syncwarp();
+                    if (!ok) break;
+                    m_ref = sh_m[r];
+                }
+                if (j == 0) m_ref = -INFINITY;
                 const float m_new = fmaxf(m_ref, mx * p.scale_log2);
                 float alpha = 1.f;
                 bool rescale = false;
                 if (m_new > m_ref + 8.0f) {  // also taken when m_ref is still -inf
-                    alpha = ex2_approx(m_ref - m_new);
+                    // a row that has seen no key yet has P = 0 behind it: its O
+                    // needs no scaling (the window's last rows at an item's second
+                    // block, where the wait for P.V would stop their warp each time)
+                    rescale = m_ref != -INFINITY;
+                    if (rescale) alpha = ex2_approx(m_ref - m_new);
                     m_ref = m_new;
-                    rescale = true;
                 }
+                sh_m[r] = m_ref;
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar_m_mine);
+                // (global branch only: the local one has no register left for it)
+                const bool pv_seen =
+                    itg < 2 || (GLOBAL && mbar_test(smem_u32(&bar_pv_done[(itg - 2) & 3]), ((itg - 2) >> 2) & 1));
                 const float m_use = (m_ref == -INFINITY) ? 0.f : m_ref;
                 const uint64_t scale2 = f2_pack(p.scale_log2, p.scale_log2);
                 const uint64_t negm2 = f2_pack(-m_use, -m_use);
                 uint64_t acc2[4] = {0ull, 0ull, 0ull, 0ull};
+                uint32_t pk[2][32];  // P as bf16 pairs
 #pragma unroll
                 for (int c = 0; c < kBN; c += 2) {
                     float x0, x1;
                     f2_unpack(f2_fma(f2_pack(s[c], s[c + 1]), scale2, negm2), x0, x1);
-                    s[c] = ex2_approx(x0);
-                    s[c + 1] = ex2_approx(x1);
-                    acc2[(c >> 1) & 3] = f2_add(acc2[(c >> 1) & 3], f2_pack(s[c], s[c + 1]));
+                    x0 = ex2_approx(x0);
+                    x1 = ex2_approx(x1);
+                    acc2[(c >> 1) & 3] = f2_add(acc2[(c >> 1) & 3], f2_pack(x0, x1));
+                    pk[c >> 6][(c >> 1) & 31] = cvt_bf16x2(x0, x1);
                 }
                 float rs;
                 {
@@ -527,20 +589,31 @@ __global__ void __launch_bounds__(384, 1) attn_fwd_kernel(const __grid_constant_
                     f2_unpack(acc2[3], d0, d1);
                     rs = ((a0 + a1) + (b0 + b1)) + ((c0 + c1) + (d0 + d1));
                 }
-                l = l * alpha + rs;
-                // O may only be rescaled once the P.V of the previous block is done
-                const bool warp_rescale = __any_sync(0xffffffffu, rescale && n > it.blk_lo);
-                if (warp_rescale) {
-                    // P.V of block itg-1 done: the completion on its P buffer
-                    // (unambiguous: the one before it was awaited a block ago)
-                    ok = mbar_wait(smem_u32(&bar_p_free[(itg - 1) & 1]), ((itg - 1) >> 1) & 1, &abort_flag);
+                if (m_ref > m_own) {  // by this block or by one of the other warpgroup's
+                    l *= ex2_approx(m_own - m_ref);
+                    m_own = m_ref;
+                }
+                l += rs;
+                // the P buffer is free once the P.V two blocks back is done
+                if (!__all_sync(0xffffffffu, pv_seen)) {
+                    ok = mbar_wait(smem_u32(&bar_pv_done[(itg - 2) & 3]), ((itg - 2) >> 2) & 1, &abort_flag);
+                    __syncwarp();
+                    if (!ok) break;
+                }
+                tc_fence_after();
+#pragma unroll
+                for (int h = 0; h < 2; ++h) tmem_st32(pcol + 32 * h, pk[h]);
+                // O may only be rescaled once the P.V of the previous block is done.
+                // Done here, where the row of S no longer takes registers
+                if (__any_sync(0xffffffffu, rescale)) {
+                    ok = mbar_wait(smem_u32(&bar_pv_done[(itg - 1) & 3]), ((itg - 1) >> 2) & 1, &abort_flag);
                     __syncwarp();
                     if (!ok) break;
                     tc_fence_after();
                     // tcgen05.ld/st are warp-collective: rows that keep their max
                     // multiply by alpha = 1
-                    const uint32_t ocol = tmem + lane_off + C::kColO;
-#pragma unroll
+                    const uint32_t ocol = tmem + lane_off + C::kColO + (item_i % C::kOBufs) * D;
+#pragma unroll 1
                     for (int c = 0; c < D / 32; ++c) {
                         uint32_t v[32];
                         tmem_ld32(ocol + c * 32, v);
@@ -550,50 +623,27 @@ __global__ void __launch_bounds__(384, 1) attn_fwd_kernel(const __grid_constant_
                         tmem_st32(ocol + c * 32, v);
                     }
                 }
-                if (!__all_sync(0xffffffffu, p_free_seen)) {
-                    ok = mbar_wait(smem_u32(&bar_p_free[itg & 1]), ((itg >> 1) & 1) ^ 1, &abort_flag);
-                    __syncwarp();
-                    if (!ok) break;
-                }
-                tc_fence_after();
-                const uint32_t pcol = tmem + lane_off + ((itg & 1) ? C::kColP1 : C::kColP0);
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    uint32_t pk[32];
-#pragma unroll
-                    for (int i = 0; i < 32; ++i) pk[i] = cvt_bf16x2(s[64 * h + 2 * i], s[64 * h + 2 * i + 1]);
-                    tmem_st32(pcol + 32 * h, pk);
-                }
-                const bool s_seen = n < it.blk_hi && mbar_test(smem_u32(&bar_s_full[(itg + 1) & 1]), ((itg + 1) >> 1) & 1);
+                s_seen = j + 2 < nblk && mbar_test(smem_u32(&bar_s_full[par]), ((itg + 2) >> 1) & 1);
                 tmem_wait_st();
                 tc_fence_before();
-                mbar_arrive(smem_u32(&bar_p_full[itg & 1]));
-                s_ready = __all_sync(0xffffffffu, s_seen);
+                mbar_arrive(smem_u32(&bar_p_full[par]));
             }
             if (!ok) break;
-            // ---- end of the item: lse = (m + log2 l) ln 2, and 1/l to the
-            //      epilogue warps, which normalise O while this warp moves on
-            if (row_valid) {
-                const float lse = (m_ref + log2f(l)) * kLn2;
-                if (GLOBAL && it.slot < 0) p.lse[static_cast<int64_t>(it.h) * p.cap + it.row0 + r] = lse;
-                else if (!GLOBAL) p.lse[(static_cast<int64_t>(it.b) * p.Hq + it.h) * p.T + it.row0 + r] = lse;
-            }
-            const int ls = item_i & 1;
-            ok = mbar_wait(smem_u32(&bar_l_empty[ls]), ((item_i >> 1) & 1) ^ 1, &abort_flag);
+            itg0 += nblk;
+            // ---- end of the item: this warpgroup's max and row sum to the epilogue warps
+            ok = mbar_wait(smem_u32(&bar_l_empty), (item_i & 1) ^ 1, &abort_flag);
             __syncwarp();
             if (!ok) break;
-            // a share of a split KV range hands over its row sum (the merge
-            // normalises); everything else 1/l
-            sh_inv_l[ls][r] = (GLOBAL && it.slot >= 0) ? l : 1.0f / l;
-            if (GLOBAL && it.slot >= 0 && row_valid)
-                p.m_part[(static_cast<int64_t>(it.slot) * p.Hq + it.h) * kBM + r] = m_ref;
-            mbar_arrive(smem_u32(&bar_l_full[ls]));
+            sh_ml[par][r] = make_float2(m_own, l);
+            mbar_arrive(smem_u32(&bar_l_full));
         }
     } else {
         // ------------------------------------------------------------ epilogue
-        // warps 4..7: once an item's last P.V is done, copy O out of TMEM (then
-        // the next item's first P.V may overwrite it), and write O / l (or, for
-        // one share of a split KV range, the unnormalised O and the row sum)
+        // warps 8..11: the row's max and sum from the two softmax warpgroups;
+        // once an item's last P.V is done, O out of TMEM (then the next item's
+        // first P.V may overwrite it), and O / l and lse = (m + log2 l) ln 2 to
+        // memory (or, for one share of a split KV range, the unnormalised O, the
+        // max and the row sum)
         setmaxnreg_dec<C::kRegsEpilogue>();
         const int quad = warp & 3;
         const int r = quad * 32 + lane;
@@ -606,59 +656,116 @@ __global__ void __launch_bounds__(384, 1) attn_fwd_kernel(const __grid_constant_
             const FwdItem it = decode_item<GLOBAL>(p, k);
             const bool row_valid = r < it.nrows;
             itg += it.blk_hi - it.blk_lo + 1;
-            const int ls = item_i & 1;
-            ok = mbar_wait(smem_u32(&bar_l_full[ls]), (item_i >> 1) & 1, &abort_flag);
+            ok = mbar_wait(smem_u32(&bar_l_full), item_i & 1, &abort_flag);
             __syncwarp();
             if (!ok) break;
-            const float lv = sh_inv_l[ls][r];
-            mbar_arrive(smem_u32(&bar_l_empty[ls]));
+            const float2 ml0 = sh_ml[0][r], ml1 = sh_ml[1][r];
+            mbar_arrive(smem_u32(&bar_l_empty));
+            const float m = fmaxf(ml0.x, ml1.x);
+            const float l = (ml0.x == -INFINITY ? 0.f : ml0.y * ex2_approx(ml0.x - m)) +
+                            (ml1.x == -INFINITY ? 0.f : ml1.y * ex2_approx(ml1.x - m));
+            const bool whole = !GLOBAL || it.slot < 0;
+            const int64_t unit = static_cast<int64_t>(it.slot) * p.Hq + it.h;  // split entries only
+            if (row_valid) {
+                if (whole) {
+                    const float lse = (m + log2f(l)) * kLn2;
+                    if (GLOBAL) p.lse[static_cast<int64_t>(it.h) * p.cap + it.row0 + r] = lse;
+                    else p.lse[(static_cast<int64_t>(it.b) * p.Hq + it.h) * p.T + it.row0 + r] = lse;
+                } else {
+                    p.m_part[unit * kBM + r] = m;
+                    p.l_part[unit * kBM + r] = l;
+                }
+            }
+            const float inv_l = 1.0f / l;
+            float inv[2][2];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) inv[i >> 1][i & 1] = __shfl_sync(0xffffffffu, inv_l, i * 8 + (lane >> 2));
             // the item's last P.V (block itg - 1) is done
-            ok = mbar_wait(smem_u32(&bar_p_free[(itg - 1) & 1]), ((itg - 1) >> 1) & 1, &abort_flag);
+            ok = mbar_wait(smem_u32(&bar_pv_done[(itg - 1) & 3]), ((itg - 1) >> 2) & 1, &abort_flag);
             __syncwarp();
             if (!ok) break;
             tc_fence_after();
-            uint32_t ov[D / 32][32];
-            const uint32_t ocol = tmem + lane_off + C::kColO;
-#pragma unroll
-            for (int c = 0; c < D / 32; ++c) tmem_ld32(ocol + c * 32, ov[c]);
-            tmem_wait_ld();
-            tc_fence_before();
-            mbar_arrive(smem_u32(&bar_o_free));
-            if (GLOBAL && it.slot >= 0) {
+            const int ob = item_i % C::kOBufs;
+            const uint32_t ocol = tmem + lane_off + C::kColO + ob * D;
+            // this lane's 16-byte column slice of the warp's first row
+            logo_bf16* o0 = p.o + ((GLOBAL ? 0 : static_cast<int64_t>(it.b) * p.T) + it.row0 + quad * 32) * p.Hq * D +
+                            it.h * D + (lane & 3) * 8;
+            if (!whole) {
                 // one share of a split KV range: unnormalised O, stored transposed
                 // ([d][row]) so that the warp's 32 rows of a column are one line
-                const int64_t unit = static_cast<int64_t>(it.slot) * p.Hq + it.h;
                 float* pcol = p.o_part + unit * kBM * D + r;
+#pragma unroll 1
+                for (int c = 0; c < D / 32; ++c) {
+                    uint32_t v[32];
+                    tmem_ld32(ocol + c * 32, v);
+                    tmem_wait_ld();
 #pragma unroll
-                for (int c = 0; c < D / 32; ++c)
-#pragma unroll
-                    for (int i = 0; i < 32; ++i) pcol[(c * 32 + i) * kBM] = __uint_as_float(ov[c][i]);
-                if (row_valid) p.l_part[unit * kBM + r] = lv;
+                    for (int i = 0; i < 32; ++i) pcol[(c * 32 + i) * kBM] = __uint_as_float(v[i]);
+                }
+                tc_fence_before();
+                mbar_arrive(smem_u32(&bar_o_free[ob]));
                 continue;
             }
-            if (!row_valid) continue;
-            const float inv_l = lv;
-            logo_bf16* orow;
-            if (GLOBAL) orow = p.o + (static_cast<int64_t>(it.row0 + r) * p.Hq + it.h) * D;
-            else orow = p.o + ((static_cast<int64_t>(it.b) * p.T + it.row0 + r) * p.Hq + it.h) * D;
+            // O in 16 x 256-bit pieces (lane t: rows t / 4 and t / 4 + 8, two columns
+            // of every 8), as bf16 pairs; four lanes then trade pairs so that each
+            // has 8 adjacent columns, and a warp store is 8 rows of 64 contiguous
+            // bytes.  With a row per lane (32 rows, 32 lines a store) the item's
+            // stores held the load/store pipe for ~2000 clocks, and with it the
+            // softmax warps' barriers and TMEM stores.  O's columns are given back
+            // as soon as the last of them is read: the first 32 go out at once,
+            // the others wait as pairs until then.
+            constexpr int kEarly = 1;
+            uint32_t w[D / 32][2][8];  // [32 columns][rows 0..15 or 16..31][row t / 4: 4 pairs, row t / 4 + 8: 4 pairs]
+            auto load32 = [&](int c) {
+                uint32_t v[2][16];
+#pragma unroll
+                for (int hf = 0; hf < 2; ++hf) tmem_ld_16x256b_x4(ocol + (static_cast<uint32_t>(hf * 16) << 16) + c * 32, v[hf]);
+                tmem_wait_ld();
+#pragma unroll
+                for (int hf = 0; hf < 2; ++hf) {
+                    const float ia = inv[hf][0], ib = inv[hf][1];
+#pragma unroll
+                    for (int k4 = 0; k4 < 4; ++k4) {
+                        const uint32_t* x = v[hf] + 4 * k4;
+                        w[c][hf][k4] = cvt_bf16x2(__uint_as_float(x[0]) * ia, __uint_as_float(x[1]) * ia);
+                        w[c][hf][4 + k4] = cvt_bf16x2(__uint_as_float(x[2]) * ib, __uint_as_float(x[3]) * ib);
+                    }
+                }
+            };
+            auto store32 = [&](int c) {
+#pragma unroll
+                for (int hf = 0; hf < 2; ++hf)
+#pragma unroll
+                    for (int ab = 0; ab < 2; ++ab) {
+                        const uint32_t* x = w[c][hf] + 4 * ab;
+                        const bool b0 = lane & 1, b1 = lane & 2;
+                        const uint32_t r0 = __shfl_xor_sync(0xffffffffu, b0 ? x[0] : x[1], 1);
+                        const uint32_t r1 = __shfl_xor_sync(0xffffffffu, b0 ? x[2] : x[3], 1);
+                        const uint32_t y0 = b0 ? r0 : x[0], y1 = b0 ? x[1] : r0, y2 = b0 ? r1 : x[2], y3 = b0 ? x[3] : r1;
+                        const uint32_t q0 = __shfl_xor_sync(0xffffffffu, b1 ? y0 : y2, 2);
+                        const uint32_t q1 = __shfl_xor_sync(0xffffffffu, b1 ? y1 : y3, 2);
+                        const int row = hf * 16 + ab * 8 + (lane >> 2);
+                        if (quad * 32 + row < it.nrows)
+                            *reinterpret_cast<uint4*>(o0 + static_cast<int64_t>(row) * p.Hq * D + c * 32) =
+                                b1 ? make_uint4(q0, q1, y2, y3) : make_uint4(y0, y1, q0, q1);
+                    }
+            };
 #pragma unroll
             for (int c = 0; c < D / 32; ++c) {
-#pragma unroll
-                for (int q4 = 0; q4 < 4; ++q4) {
-                    const uint32_t* v = ov[c] + 8 * q4;
-                    uint4 w;
-                    w.x = pack_bf16x2(__uint_as_float(v[0]) * inv_l, __uint_as_float(v[1]) * inv_l);
-                    w.y = pack_bf16x2(__uint_as_float(v[2]) * inv_l, __uint_as_float(v[3]) * inv_l);
-                    w.z = pack_bf16x2(__uint_as_float(v[4]) * inv_l, __uint_as_float(v[5]) * inv_l);
-                    w.w = pack_bf16x2(__uint_as_float(v[6]) * inv_l, __uint_as_float(v[7]) * inv_l);
-                    *reinterpret_cast<uint4*>(orow + c * 32 + q4 * 8) = w;
+                load32(c);
+                if (c == D / 32 - 1) {
+                    tc_fence_before();
+                    mbar_arrive(smem_u32(&bar_o_free[ob]));
                 }
+                if (c < kEarly) store32(c);
             }
+#pragma unroll
+            for (int c = kEarly; c < D / 32; ++c) store32(c);
         }
     }
     tc_fence_before();
     __syncthreads();
-    if (warp == 9) {
+    if (warp == 13) {
         tc_fence_after();
         tmem_dealloc(tmem, C::kTmemCols);
     }
@@ -1003,6 +1110,9 @@ extern "C" int logo_local_attn_fwd(const logo_bf16* q, const logo_bf16* k, const
     prm.window = w;
     prm.cap = dims.B * dims.T;
     prm.q_tiles = (dims.T + kBM - 1) / kBM;
+    prm.by_hq = FastDiv(dims.Hq);
+    prm.by_group = FastDiv(dims.Hq / dims.Hkv);
+    prm.by_q_tiles = FastDiv(prm.q_tiles);
     prm.scale_log2 = scale * kLog2e;
     const int n_items = dims.B * prm.q_tiles * dims.Hq;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
@@ -1061,6 +1171,8 @@ extern "C" int logo_global_sparse_attn_fwd(const logo_bf16* q, const logo_bf16* 
     prm.window = kNoWindow;
     prm.cap = cap;
     prm.q_tiles = 0;
+    prm.by_hq = FastDiv(dims.Hq);
+    prm.by_group = FastDiv(dims.Hq / dims.Hkv);
     prm.scale_log2 = scale * kLog2e;
     const int n_items_upper =
         static_cast<int>((static_cast<int64_t>(cap) / kBM + dims.B) * dims.Hq + kMaxPartialUnits);
