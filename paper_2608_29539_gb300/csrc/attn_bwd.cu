@@ -35,11 +35,9 @@
 // the pre-pass builds once per call (App. B's precomputed search); the same
 // pre-pass gathers the selected Q rows and computes Dsum.
 //
-// d = 64, attn_bwd_kernel (6 warps, query tiles of 128 rows): one MMA warp
-// issues S^T, dP^T, then dV, dK and dQ into the S^T columns once the softmax
-// warps have written P^T and dS^T to shared memory; the first visible query
-// tile of a global item comes from a binary search over the packed positions;
-// dQ goes through fp32 atomics and a conversion pass.
+// d = 64, attn_bwd64_kernel (16 warps, query tiles of 128 rows): the same
+// split of the work over two MMA issuers, two softmax-backward warpgroups and
+// a drain warpgroup, laid out for 64-wide rows (below).
 #include <cuda_bf16.h>
 
 #include <cstdint>
@@ -52,29 +50,12 @@
 namespace logo {
 namespace {
 
-template <int D>
-struct BwdCfg {
-    static constexpr int kSub = D / 64;
-    static constexpr int kTileBytes = kBM * D * 2;
-    static constexpr int kOffK = 0;
-    static constexpr int kOffV = kOffK + kTileBytes;
-    static constexpr int kOffQ = kOffV + kTileBytes;
-    static constexpr int kOffDO = kOffQ + kTileBytes;
-    static constexpr int kOffP = kOffDO + kTileBytes;     // P^T  [128 keys][128 queries] bf16
-    static constexpr int kOffDS = kOffP + kBM * kBN * 2;  // dS^T [128 keys][128 queries] bf16
-    static constexpr int kSmemBytes = kOffDS + kBM * kBN * 2 + 1024;
-    static constexpr uint32_t kColDK = 0;
-    static constexpr uint32_t kColDV = 128;
-    static constexpr uint32_t kColST = 256;  // S^T, later dQ
-    static constexpr uint32_t kColDP = 384;  // dP^T
-    static constexpr uint32_t kTmemCols = 512;
-};
-
 struct BwdParams {
     CUtensorMap tm_q;   // local: Q [B,T,Hq,D]; global: packed [1,cap+128,Hq,D]
     CUtensorMap tm_do;  // same layout as tm_q
     CUtensorMap tm_k;   // [B,T,Hkv,D]
     CUtensorMap tm_v;
+    CUtensorMap tm_dq;  // d = 64: dq_acc, for the bulk reductions
     const float* lse;   // local [B,Hq,T]; global [Hq,cap]
     const float* dsum;  // same layout as lse
     float* dq_acc;      // local [B,T,Hq,D]; global [cap+128,Hq,D]
@@ -83,7 +64,7 @@ struct BwdParams {
     const int32_t* pos;
     const int32_t* cu_q;
     const int32_t* first_row;  // global: [B, nblk] first packed row of sequence b whose position reaches block j
-    logo_bf16* dq_fill;        // global, d = 128: dense dQ [B, T, Hq, D] whose unselected rows this kernel zeroes
+    logo_bf16* dq_fill;        // global: dense dQ [B, T, Hq, D] whose unselected rows this kernel zeroes
     int B, T, Hq, Hkv, window, cap, nblk, q_tiles;
     float scale, scale_log2;
 };
@@ -94,8 +75,9 @@ struct BwdItem {
     int row_lo, row_hi; // global: packed rows of sequence b
 };
 
-template <bool GLOBAL>
-__device__ __forceinline__ BwdItem decode_bwd(const BwdParams& p, int k)
+// BQ: query rows per tile
+template <int BQ, bool GLOBAL>
+__device__ __forceinline__ BwdItem decode_bwd2(const BwdParams& p, int k)
 {
     BwdItem it;
     it.kvh = k % p.Hkv;
@@ -104,342 +86,56 @@ __device__ __forceinline__ BwdItem decode_bwd(const BwdParams& p, int k)
     it.j = t / p.B;
     const int k0 = it.j * kBN;
     if (!GLOBAL) {
-        it.i_lo = it.j;
-        const int i_hi = min(p.q_tiles - 1, (k0 + kBN - 1 + p.window - 1) / kBM);
+        it.i_lo = k0 / BQ;
+        const int i_hi = min((p.T + BQ - 1) / BQ - 1, (k0 + kBN - 1 + p.window - 1) / BQ);
         it.ntiles = i_hi - it.i_lo + 1;
         it.row_lo = it.row_hi = 0;
     } else {
         it.row_lo = p.cu_q[it.b];
         it.row_hi = p.cu_q[it.b + 1];
-        // first packed row of the sequence whose position can see key k0
-        int lo = it.row_lo, hi = it.row_hi;
-        while (lo < hi) {
-            const int mid = (lo + hi) >> 1;
-            if (p.pos[mid] < k0) lo = mid + 1;
-            else hi = mid;
-        }
+        const int lo = p.first_row[it.b * p.nblk + it.j];  // precomputed search (App. B)
         if (lo >= it.row_hi) {
             it.i_lo = 0;
             it.ntiles = 0;
         } else {
-            it.i_lo = lo / kBM;
-            it.ntiles = (it.row_hi - 1) / kBM - it.i_lo + 1;
+            it.i_lo = lo / BQ;
+            it.ntiles = (it.row_hi - 1) / BQ - it.i_lo + 1;
         }
     }
     return it;
 }
 
-template <int D, bool GLOBAL>
-__global__ void __launch_bounds__(192, 1) attn_bwd_kernel(const __grid_constant__ BwdParams p)
+// One warp of each CTA: zero the dense dQ rows of the tokens that were not
+// selected (the conversion after the kernel writes only the selected rows).
+// The backward kernels leave nearly all of HBM's bandwidth idle; a separate
+// pass writing the whole dense tensor would not.
+__device__ __forceinline__ void zero_unselected_dq(const BwdParams& p, int D, int lane)
 {
-    using C = BwdCfg<D>;
-    extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    __shared__ __align__(8) uint64_t bar_kv_full, bar_kv_empty, bar_qdo_full, bar_qdo_empty, bar_st_full,
-        bar_ds_full, bar_dq_full, bar_dq_empty, bar_dkv_full, bar_dkv_empty, bar_drain, bar_stage;
-    __shared__ uint32_t tmem_base_sh;
-    __shared__ volatile int abort_flag;
-    __shared__ int sh_pos[2][kBM];
-    __shared__ float sh_lse[2][kBM];
-    __shared__ float sh_dsum[2][kBM];
-
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t sK = smem_u32(smem + C::kOffK), sV = smem_u32(smem + C::kOffV);
-    const uint32_t sQ = smem_u32(smem + C::kOffQ), sDO = smem_u32(smem + C::kOffDO);
-    const uint32_t sP = smem_u32(smem + C::kOffP), sDS = smem_u32(smem + C::kOffDS);
-    const int group = p.Hq / p.Hkv;
-    const int n_items = p.B * p.nblk * p.Hkv;
-
-    if (threadIdx.x == 0) {
-        abort_flag = 0;
-        mbar_init(smem_u32(&bar_kv_full), 1);
-        mbar_init(smem_u32(&bar_kv_empty), 1);
-        mbar_init(smem_u32(&bar_qdo_full), 1);
-        mbar_init(smem_u32(&bar_qdo_empty), 1);
-        mbar_init(smem_u32(&bar_st_full), 1);
-        mbar_init(smem_u32(&bar_ds_full), 128);
-        mbar_init(smem_u32(&bar_dq_full), 1);
-        mbar_init(smem_u32(&bar_dq_empty), 128);
-        mbar_init(smem_u32(&bar_dkv_full), 1);
-        mbar_init(smem_u32(&bar_dkv_empty), 128);
-        mbar_init(smem_u32(&bar_drain), 1);
-        mbar_init(smem_u32(&bar_stage), 128);
-        fence_mbar_init();
-    }
-    if (warp == 1) {
-        tmem_alloc(smem_u32(&tmem_base_sh), C::kTmemCols);
-        tmem_relinquish();
-    }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem = tmem_base_sh;
-
-    if (warp == 0) {
-        // ------------------------------------------------------------ producer
-        if (lane == 0) {
-            tma_prefetch_desc(&p.tm_q);
-            tma_prefetch_desc(&p.tm_do);
-            tma_prefetch_desc(&p.tm_k);
-            tma_prefetch_desc(&p.tm_v);
-            const uint64_t pol_q = policy_evict_last();
-            const uint64_t pol_kv = policy_evict_first();
-            int u = 0, kv_items = 0;
-            bool ok = true;
-            for (int k = blockIdx.x; k < n_items && ok; k += gridDim.x) {
-                const BwdItem it = decode_bwd<GLOBAL>(p, k);
-                if (it.ntiles == 0) continue;
-                if (!(ok = mbar_wait(smem_u32(&bar_kv_empty), (kv_items & 1) ^ 1, &abort_flag))) break;
-                const uint32_t kvb = smem_u32(&bar_kv_full);
-                mbar_arrive_expect_tx(kvb, 2 * C::kTileBytes);
-                for (int s = 0; s < C::kSub; ++s) {
-                    tma_load_4d(sK + s * 16384, &p.tm_k, kvb, 64 * s, it.kvh, it.j * kBN, it.b, pol_kv);
-                    tma_load_4d(sV + s * 16384, &p.tm_v, kvb, 64 * s, it.kvh, it.j * kBN, it.b, pol_kv);
-                }
-                ++kv_items;
-                const int n_it = group * it.ntiles;
-                for (int x = 0; x < n_it; ++x, ++u) {
-                    const int h = it.kvh * group + x / it.ntiles;
-                    const int i = it.i_lo + x % it.ntiles;
-                    if (!(ok = mbar_wait(smem_u32(&bar_qdo_empty), (u & 1) ^ 1, &abort_flag))) break;
-                    const uint32_t qb = smem_u32(&bar_qdo_full);
-                    mbar_arrive_expect_tx(qb, 2 * C::kTileBytes);
-                    const int cb = GLOBAL ? 0 : it.b;
-                    for (int s = 0; s < C::kSub; ++s) {
-                        tma_load_4d(sQ + s * 16384, &p.tm_q, qb, 64 * s, h, i * kBM, cb, pol_q);
-                        tma_load_4d(sDO + s * 16384, &p.tm_do, qb, 64 * s, h, i * kBM, cb, pol_q);
-                    }
-                }
+    const int64_t ntok = static_cast<int64_t>(p.B) * p.T;
+    const int64_t per = (ntok + gridDim.x - 1) / gridDim.x;
+    const int64_t t_begin = static_cast<int64_t>(blockIdx.x) * per;
+    const int64_t t_end = t_begin + per < ntok ? t_begin + per : ntok;
+    const int row_vecs = p.Hq * D / 8;  // 16-byte vectors per token row
+    int cur_b = -1, r = 0, r_hi = 0;
+    for (int64_t bt = t_begin; bt < t_end; ++bt) {
+        const int b = static_cast<int>(bt / p.T), t = static_cast<int>(bt % p.T);
+        if (b != cur_b) {  // first packed row of sequence b at or after position t
+            cur_b = b;
+            int lo = p.cu_q[b], hi = p.cu_q[b + 1];
+            r_hi = hi;
+            while (lo < hi) {
+                const int mid = (lo + hi) >> 1;
+                if (p.pos[mid] < t) lo = mid + 1;
+                else hi = mid;
             }
-            if (!ok) {
-                if (kv_items > 0) mbar_wait_drain(smem_u32(&bar_kv_full), (kv_items - 1) & 1);
-                if (u > 0) mbar_wait_drain(smem_u32(&bar_qdo_full), (u - 1) & 1);
-            }
+            r = lo;
         }
-    } else if (warp == 1) {
-        // ------------------------------------------------------------ MMA issuer
-        if (lane == 0) {
-            constexpr uint32_t idS = idesc_bf16_f32(kBM, kBN, false, false);  // S^T, dP^T
-            constexpr uint32_t idKM = idesc_bf16_f32(kBM, D, false, true);    // dV, dK
-            constexpr uint32_t idMM = idesc_bf16_f32(kBM, D, true, true);     // dQ
-            int u = 0, kv_items = 0;
-            bool ok = true;
-            for (int k = blockIdx.x; k < n_items && ok; k += gridDim.x) {
-                const BwdItem it = decode_bwd<GLOBAL>(p, k);
-                if (it.ntiles == 0) continue;
-                if (!(ok = mbar_wait(smem_u32(&bar_kv_full), kv_items & 1, &abort_flag))) break;
-                if (!(ok = mbar_wait(smem_u32(&bar_dkv_empty), (kv_items & 1) ^ 1, &abort_flag))) break;
-                const int n_it = group * it.ntiles;
-                for (int x = 0; x < n_it; ++x, ++u) {
-                    if (!(ok = mbar_wait(smem_u32(&bar_qdo_full), u & 1, &abort_flag))) break;
-                    if (!(ok = mbar_wait(smem_u32(&bar_dq_empty), (u & 1) ^ 1, &abort_flag))) break;
-                    tc_fence_after();
-#pragma unroll
-                    for (int ks = 0; ks < D / 16; ++ks) {
-                        const uint32_t off = (ks >> 2) * 16384 + (ks & 3) * 32;
-                        umma_bf16_ss(tmem + C::kColST, sdesc_sw128(sK + off, 16, 1024), sdesc_sw128(sQ + off, 16, 1024),
-                                     idS, ks > 0 ? 1u : 0u);
-                    }
-#pragma unroll
-                    for (int ks = 0; ks < D / 16; ++ks) {
-                        const uint32_t off = (ks >> 2) * 16384 + (ks & 3) * 32;
-                        umma_bf16_ss(tmem + C::kColDP, sdesc_sw128(sV + off, 16, 1024),
-                                     sdesc_sw128(sDO + off, 16, 1024), idS, ks > 0 ? 1u : 0u);
-                    }
-                    umma_commit(smem_u32(&bar_st_full));
-                    if (!(ok = mbar_wait(smem_u32(&bar_ds_full), u & 1, &abort_flag))) break;
-                    tc_fence_after();
-#pragma unroll
-                    for (int ks = 0; ks < kBM / 16; ++ks) {
-                        const uint32_t koff = (ks >> 2) * 16384 + (ks & 3) * 32;  // K-major step over queries
-                        const uint32_t moff = ks * 2048;                           // MN-major step over 16 rows
-                        const uint32_t acc = (x > 0 || ks > 0) ? 1u : 0u;
-                        umma_bf16_ss(tmem + C::kColDV, sdesc_sw128(sP + koff, 16, 1024),
-                                     sdesc_sw128(sDO + moff, 16384, 1024), idKM, acc);
-                        umma_bf16_ss(tmem + C::kColDK, sdesc_sw128(sDS + koff, 16, 1024),
-                                     sdesc_sw128(sQ + moff, 16384, 1024), idKM, acc);
-                    }
-#pragma unroll
-                    for (int ks = 0; ks < kBN / 16; ++ks) {
-                        const uint32_t moff = ks * 2048;  // 16 keys per step
-                        umma_bf16_ss(tmem + C::kColST, sdesc_sw128(sDS + moff, 16384, 1024),
-                                     sdesc_sw128(sK + moff, 16384, 1024), idMM, ks > 0 ? 1u : 0u);
-                    }
-                    umma_commit(smem_u32(&bar_dq_full));
-                    umma_commit(smem_u32(&bar_qdo_empty));
-                }
-                if (!ok) break;
-                umma_commit(smem_u32(&bar_kv_empty));
-                umma_commit(smem_u32(&bar_dkv_full));
-                ++kv_items;
-            }
-            if (!ok) {
-                umma_commit(smem_u32(&bar_drain));
-                mbar_wait_drain(smem_u32(&bar_drain), 0);
-            }
+        if (r < r_hi && p.pos[r] == t) {  // selected: converted later
+            ++r;
+            continue;
         }
-    } else {
-        // ------------------------------------------------------------ softmax-bwd / epilogues
-        const int quad = warp & 3;
-        const int t = quad * 32 + lane;  // key row for P^T/dS^T; query row for dQ
-        const uint32_t lane_off = static_cast<uint32_t>(quad * 32) << 16;
-        const int window = GLOBAL ? kNoWindow : p.window;
-        int u = 0, kv_items = 0;
-        bool ok = true;
-        for (int k = blockIdx.x; k < n_items && ok; k += gridDim.x) {
-            const BwdItem it = decode_bwd<GLOBAL>(p, k);
-            const int key = it.j * kBN + t;
-            const int64_t kv_off = ((static_cast<int64_t>(it.b) * p.T + key) * p.Hkv + it.kvh) * D;
-            if (it.ntiles == 0) {  // no selected row sees this block: dK = dV = 0
-                if (key < p.T) {
-                    for (int c = 0; c < D; c += 8) {
-                        *reinterpret_cast<uint4*>(p.dk + kv_off + c) = make_uint4(0, 0, 0, 0);
-                        *reinterpret_cast<uint4*>(p.dv + kv_off + c) = make_uint4(0, 0, 0, 0);
-                    }
-                }
-                continue;
-            }
-            const int n_it = group * it.ntiles;
-            for (int x = 0; x < n_it; ++x, ++u) {
-                const int h = it.kvh * group + x / it.ntiles;
-                const int i = it.i_lo + x % it.ntiles;
-                const int sb = u & 1;
-                // stage this query tile's positions, lse (log2 units) and Dsum
-                {
-                    int pc = -1;
-                    float l2 = 0.f, ds = 0.f;
-                    if (!GLOBAL) {
-                        const int q = i * kBM + t;
-                        if (q < p.T) {
-                            const int64_t idx = (static_cast<int64_t>(it.b) * p.Hq + h) * p.T + q;
-                            pc = q;
-                            l2 = p.lse[idx] * kLog2e;
-                            ds = p.dsum[idx];
-                        }
-                    } else {
-                        const int row = i * kBM + t;
-                        if (row >= it.row_lo && row < it.row_hi) {
-                            const int64_t idx = static_cast<int64_t>(h) * p.cap + row;
-                            pc = p.pos[row];
-                            l2 = p.lse[idx] * kLog2e;
-                            ds = p.dsum[idx];
-                        }
-                    }
-                    sh_pos[sb][t] = pc;
-                    sh_lse[sb][t] = l2;
-                    sh_dsum[sb][t] = ds;
-                }
-                // the four compute warps sync on a bounded barrier (never an
-                // unbounded bar.sync: an aborting warp must not strand others)
-                mbar_arrive(smem_u32(&bar_stage));
-                ok = mbar_wait(smem_u32(&bar_stage), u & 1, &abort_flag);
-                if (!ok) break;
-                ok = mbar_wait(smem_u32(&bar_st_full), u & 1, &abort_flag);
-                __syncwarp();
-                if (!ok) break;
-                tc_fence_after();
-#pragma unroll 1
-                for (int cc = 0; cc < kBM / 32; ++cc) {
-                    uint32_t sv[32], dpv[32];
-                    tmem_ld32(tmem + lane_off + C::kColST + cc * 32, sv);
-                    tmem_ld32(tmem + lane_off + C::kColDP + cc * 32, dpv);
-                    tmem_wait_ld();
-                    uint32_t pk[16], dk2[16];
-#pragma unroll
-                    for (int e = 0; e < 32; e += 2) {
-                        float pe[2], de[2];
-#pragma unroll
-                        for (int z = 0; z < 2; ++z) {
-                            const int c = cc * 32 + e + z;
-                            const int pc = sh_pos[sb][c];
-                            const bool vis = key_visible(key, pc, window);
-                            const float pr =
-                                vis ? ex2_approx(fmaf(__uint_as_float(sv[e + z]), p.scale_log2, -sh_lse[sb][c])) : 0.f;
-                            pe[z] = pr;
-                            de[z] = pr * (__uint_as_float(dpv[e + z]) - sh_dsum[sb][c]);
-                        }
-                        pk[e / 2] = pack_bf16x2(pe[0], pe[1]);
-                        dk2[e / 2] = pack_bf16x2(de[0], de[1]);
-                    }
-#pragma unroll
-                    for (int q4 = 0; q4 < 4; ++q4) {
-                        const int chunk = cc * 4 + q4;  // 16-byte chunk index along the query axis
-                        const uint32_t off = (chunk >> 3) * 16384 + sw128_offset(t, chunk & 7);
-                        st_shared_v4(sP + off, pk[4 * q4], pk[4 * q4 + 1], pk[4 * q4 + 2], pk[4 * q4 + 3]);
-                        st_shared_v4(sDS + off, dk2[4 * q4], dk2[4 * q4 + 1], dk2[4 * q4 + 2], dk2[4 * q4 + 3]);
-                    }
-                }
-                fence_proxy_async_smem();
-                tc_fence_before();
-                mbar_arrive(smem_u32(&bar_ds_full));
-                // dQ of query row t for this (tile, block): fp32 atomics
-                ok = mbar_wait(smem_u32(&bar_dq_full), u & 1, &abort_flag);
-                __syncwarp();
-                if (!ok) break;
-                tc_fence_after();
-                uint32_t dq[D];
-#pragma unroll
-                for (int cc = 0; cc < D / 32; ++cc) {
-                    uint32_t v[32];
-                    tmem_ld32(tmem + lane_off + C::kColST + cc * 32, v);
-                    tmem_wait_ld();
-#pragma unroll
-                    for (int e = 0; e < 32; ++e) dq[cc * 32 + e] = v[e];
-                }
-                tc_fence_before();
-                mbar_arrive(smem_u32(&bar_dq_empty));
-                if (sh_pos[sb][t] >= 0) {
-                    float* dst;
-                    if (GLOBAL) dst = p.dq_acc + (static_cast<int64_t>(i * kBM + t) * p.Hq + h) * D;
-                    else dst = p.dq_acc + ((static_cast<int64_t>(it.b) * p.T + i * kBM + t) * p.Hq + h) * D;
-#pragma unroll
-                    for (int c = 0; c < D; c += 4) {
-                        atomicAdd(reinterpret_cast<float4*>(dst + c),
-                                  make_float4(__uint_as_float(dq[c]) * p.scale, __uint_as_float(dq[c + 1]) * p.scale,
-                                              __uint_as_float(dq[c + 2]) * p.scale,
-                                              __uint_as_float(dq[c + 3]) * p.scale));
-                    }
-                }
-            }
-            if (!ok) break;
-            // ---- epilogue: dK (scaled) and dV of this KV block
-            ok = mbar_wait(smem_u32(&bar_dkv_full), kv_items & 1, &abort_flag);
-            __syncwarp();
-            if (!ok) break;
-            tc_fence_after();
-#pragma unroll
-            for (int which = 0; which < 2; ++which) {
-                const uint32_t col = which == 0 ? C::kColDK : C::kColDV;
-                const float mul = which == 0 ? p.scale : 1.0f;
-                logo_bf16* dst = (which == 0 ? p.dk : p.dv) + kv_off;
-#pragma unroll
-                for (int cc = 0; cc < D / 32; ++cc) {
-                    uint32_t v[32];
-                    tmem_ld32(tmem + lane_off + col + cc * 32, v);
-                    tmem_wait_ld();
-                    if (key < p.T) {
-#pragma unroll
-                        for (int q4 = 0; q4 < 4; ++q4) {
-                            uint4 w;
-                            w.x = pack_bf16x2(__uint_as_float(v[8 * q4 + 0]) * mul, __uint_as_float(v[8 * q4 + 1]) * mul);
-                            w.y = pack_bf16x2(__uint_as_float(v[8 * q4 + 2]) * mul, __uint_as_float(v[8 * q4 + 3]) * mul);
-                            w.z = pack_bf16x2(__uint_as_float(v[8 * q4 + 4]) * mul, __uint_as_float(v[8 * q4 + 5]) * mul);
-                            w.w = pack_bf16x2(__uint_as_float(v[8 * q4 + 6]) * mul, __uint_as_float(v[8 * q4 + 7]) * mul);
-                            *reinterpret_cast<uint4*>(dst + cc * 32 + q4 * 8) = w;
-                        }
-                    }
-                }
-            }
-            tc_fence_before();
-            mbar_arrive(smem_u32(&bar_dkv_empty));
-            ++kv_items;
-        }
-    }
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 1) {
-        tc_fence_after();
-        tmem_dealloc(tmem, C::kTmemCols);
+        uint4* dst = reinterpret_cast<uint4*>(p.dq_fill + bt * p.Hq * D);
+        for (int v = lane; v < row_vecs; v += 32) dst[v] = make_uint4(0u, 0u, 0u, 0u);
     }
 }
 
@@ -481,36 +177,6 @@ struct Bwd2Cfg {
     static constexpr uint32_t kTmemCols = 512;
     static constexpr int kThreads = 512;
 };
-
-template <bool GLOBAL>
-__device__ __forceinline__ BwdItem decode_bwd2(const BwdParams& p, int k)
-{
-    BwdItem it;
-    it.kvh = k % p.Hkv;
-    const int t = k / p.Hkv;
-    it.b = t % p.B;
-    it.j = t / p.B;
-    const int k0 = it.j * kBN;
-    constexpr int BQ = Bwd2Cfg::kBQ;
-    if (!GLOBAL) {
-        it.i_lo = k0 / BQ;
-        const int i_hi = min((p.T + BQ - 1) / BQ - 1, (k0 + kBN - 1 + p.window - 1) / BQ);
-        it.ntiles = i_hi - it.i_lo + 1;
-        it.row_lo = it.row_hi = 0;
-    } else {
-        it.row_lo = p.cu_q[it.b];
-        it.row_hi = p.cu_q[it.b + 1];
-        const int lo = p.first_row[it.b * p.nblk + it.j];  // precomputed search (App. B)
-        if (lo >= it.row_hi) {
-            it.i_lo = 0;
-            it.ntiles = 0;
-        } else {
-            it.i_lo = lo / BQ;
-            it.ntiles = (it.row_hi - 1) / BQ - it.i_lo + 1;
-        }
-    }
-    return it;
-}
 
 template <bool GLOBAL>
 __global__ void __launch_bounds__(Bwd2Cfg::kThreads, 1) attn_bwd2_kernel(const __grid_constant__ BwdParams p)
@@ -581,7 +247,7 @@ __global__ void __launch_bounds__(Bwd2Cfg::kThreads, 1) attn_bwd2_kernel(const _
             int u = 0, kv_items = 0;
             bool ok = true;
             for (int k = blockIdx.x; k < n_items && ok; k += gridDim.x) {
-                const BwdItem it = decode_bwd2<GLOBAL>(p, k);
+                const BwdItem it = decode_bwd2<BQ, GLOBAL>(p, k);
                 if (it.ntiles == 0) continue;
                 if (!(ok = mbar_wait(smem_u32(&bar_kv_empty), (kv_items & 1) ^ 1, &abort_flag))) break;
                 const uint32_t kvb = smem_u32(&bar_kv_full);
@@ -622,7 +288,7 @@ __global__ void __launch_bounds__(Bwd2Cfg::kThreads, 1) attn_bwd2_kernel(const _
             int u = 0, kv_items = 0;
             bool ok = true;
             for (int k = blockIdx.x; k < n_items && ok; k += gridDim.x) {
-                const BwdItem it = decode_bwd2<GLOBAL>(p, k);
+                const BwdItem it = decode_bwd2<BQ, GLOBAL>(p, k);
                 if (it.ntiles == 0) continue;
                 if (!(ok = mbar_wait(smem_u32(&bar_kv_full), kv_items & 1, &abort_flag))) break;
                 const int n_it = group * it.ntiles;
@@ -663,7 +329,7 @@ __global__ void __launch_bounds__(Bwd2Cfg::kThreads, 1) attn_bwd2_kernel(const _
             int u = 0, kv_items = 0;
             bool ok = true;
             for (int k = blockIdx.x; k < n_items && ok; k += gridDim.x) {
-                const BwdItem it = decode_bwd2<GLOBAL>(p, k);
+                const BwdItem it = decode_bwd2<BQ, GLOBAL>(p, k);
                 if (it.ntiles == 0) continue;
                 const int n_it = group * it.ntiles;
                 for (int x = 0; x < n_it; ++x, ++u) {
@@ -718,7 +384,7 @@ __global__ void __launch_bounds__(Bwd2Cfg::kThreads, 1) attn_bwd2_kernel(const _
         int u = 0;
         bool ok = true;
         for (int k = blockIdx.x; k < n_items && ok; k += gridDim.x) {
-            const BwdItem it = decode_bwd2<GLOBAL>(p, k);
+            const BwdItem it = decode_bwd2<BQ, GLOBAL>(p, k);
             if (it.ntiles == 0) continue;
             const int k0 = it.j * kBN;
             const int key = k0 + t;
@@ -841,7 +507,7 @@ __global__ void __launch_bounds__(Bwd2Cfg::kThreads, 1) attn_bwd2_kernel(const _
         int u = 0, kv_items = 0;
         bool ok = true;
         for (int k = blockIdx.x; k < n_items && ok; k += gridDim.x) {
-            const BwdItem it = decode_bwd2<GLOBAL>(p, k);
+            const BwdItem it = decode_bwd2<BQ, GLOBAL>(p, k);
             const int key = it.j * kBN + t;
             const int64_t kv_off = ((static_cast<int64_t>(it.b) * p.T + key) * p.Hkv + it.kvh) * D;
             if (it.ntiles == 0) {
@@ -918,38 +584,493 @@ __global__ void __launch_bounds__(Bwd2Cfg::kThreads, 1) attn_bwd2_kernel(const _
             mbar_arrive(smem_u32(&bar_dkv_empty));
             ++kv_items;
         }
-    } else if (GLOBAL && p.dq_fill) {
+    } else if (GLOBAL) {
         // ------------------------------------------------------------ dQ zero fill
-        // warp 14: zero the dense dQ rows of the tokens that were not selected
-        // (the conversion after this kernel writes only the selected rows).  This
-        // kernel leaves nearly all of HBM's bandwidth idle; a separate pass
-        // writing the whole dense tensor would not.
-        const int64_t ntok = static_cast<int64_t>(p.B) * p.T;
-        const int64_t per = (ntok + gridDim.x - 1) / gridDim.x;
-        const int64_t t_begin = static_cast<int64_t>(blockIdx.x) * per;
-        const int64_t t_end = t_begin + per < ntok ? t_begin + per : ntok;
-        const int row_vecs = p.Hq * D / 8;  // 16-byte vectors per token row
-        int cur_b = -1, r = 0, r_hi = 0;
-        for (int64_t bt = t_begin; bt < t_end; ++bt) {
-            const int b = static_cast<int>(bt / p.T), t = static_cast<int>(bt % p.T);
-            if (b != cur_b) {  // first packed row of sequence b at or after position t
-                cur_b = b;
-                int lo = p.cu_q[b], hi = p.cu_q[b + 1];
-                r_hi = hi;
-                while (lo < hi) {
-                    const int mid = (lo + hi) >> 1;
-                    if (p.pos[mid] < t) lo = mid + 1;
-                    else hi = mid;
+        zero_unselected_dq(p, D, lane);
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        tc_fence_after();
+        tmem_dealloc(tmem, C::kTmemCols);
+    }
+}
+
+// ---------------------------------------------------------------- d = 64
+// Query tiles of 128 rows: S^T and dP^T are 128 x 128, so a tile has twice the
+// elements per MMA instruction, per barrier and per reduced byte that 64-row
+// tiles would have (dQ has to be computed as queries x d: d x queries would be
+// an M = 64 product).  Per tile 4 + 4 MMAs of N = 128 (S^T, dP^T) and 8 + 8 + 8
+// of N = 64 (dV with P^T as the TMEM operand, dK, dQ).  Roles:
+//   warp 0       TMA: K/V of an item into one of two buffers (the next item's
+//                land during this one: an item has only a few tiles), Q/dO
+//                tiles through a 3-deep ring
+//   warp 1       MMA issuer A: S^T, dP^T
+//   warp 2       MMA issuer B: dV, dK, dQ
+//   warp 3       global branch: zero rows of the dense dQ for unselected tokens
+//   warps 4..11  two warpgroups, one per 64-query half of the tile; thread =
+//                key row: P^T (to TMEM as bf16 pairs) and dS^T (to shared
+//                memory) from S^T and dP^T, which it loads whole so that the
+//                MMAs of tile u+1 can overwrite them while it computes
+//   warps 12..15 dQ out of TMEM (thread = query row), staged 32 columns at a
+//                time and added to the fp32 accumulator by bulk tensor
+//                reductions, a warp's 32 rows by itself; dK/dV epilogue
+// P^T and dS^T are single buffers: TMEM is full (dK, dV, dQ 64 columns each,
+// S^T, dP^T 128 each, P^T 64), and the next tile's are only written once its
+// arithmetic is done, when the MMAs that read this tile's have ended.
+// The kernel before it ran the stages of a tile one after the other (one MMA
+// thread, one warpgroup for softmax and dQ atomics, no second tile in flight):
+// 2 x 8K, 16 heads, 1/8 selected 299 -> 139 us, 3 x 2987, 12/4 heads, window
+// 300 111 -> 53 us.
+struct Bwd64Cfg {
+    static constexpr int D = 64;
+    static constexpr int kBQ = 128;
+    static constexpr int kStages = 3;              // Q/dO ring depth
+    static constexpr int kTileBytes = 128 * D * 2; // K, V, Q or dO: 16 KB
+    static constexpr int kWarpStage = 32 * 128;    // dQ staging of one warp: 32 rows x 32 fp32
+    static constexpr int kOffKV = 0;               // 2 buffers of K, V
+    static constexpr int kOffQ = kOffKV + 4 * kTileBytes;              // stages of Q, dO
+    static constexpr int kOffDS = kOffQ + kStages * 2 * kTileBytes;    // [2 query halves][128 keys][64] bf16
+    static constexpr int kOffDQ = kOffDS + 128 * 128 * 2;
+    static constexpr int kSmemBytes = kOffDQ + 4 * kWarpStage + 1024;
+    static constexpr uint32_t kColDK = 0;
+    static constexpr uint32_t kColDV = 64;
+    static constexpr uint32_t kColDQ = 128;
+    static constexpr uint32_t kColP = 192;   // P^T, bf16 pairs
+    static constexpr uint32_t kColS = 256;   // S^T
+    static constexpr uint32_t kColDP = 384;  // dP^T
+    static constexpr uint32_t kTmemCols = 512;
+    static constexpr int kThreads = 512;
+    // launched at 128 registers a thread (512 x 128 = 65,536); the softmax
+    // warpgroups hold 64 columns of S^T and dP^T a thread (this split compiles
+    // without spills): 128 x (64 + 176 + 176 + 96) = 65,536
+    static constexpr uint32_t kRegsControl = 64;
+    static constexpr uint32_t kRegsSoftmax = 176;
+    static constexpr uint32_t kRegsDrain = 96;
+};
+
+template <bool GLOBAL>
+__global__ void __launch_bounds__(Bwd64Cfg::kThreads, 1) attn_bwd64_kernel(const __grid_constant__ BwdParams p)
+{
+    using C = Bwd64Cfg;
+    constexpr int D = C::D, BQ = C::kBQ, NS = C::kStages;
+    static_assert(128 * (2 * C::kRegsSoftmax + C::kRegsDrain + C::kRegsControl) <= 512 * 128,
+                  "register split exceeds the launch allocation");
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    __shared__ __align__(8) uint64_t bar_kv_full[2], bar_kv_empty[2], bar_dkv_full, bar_dkv_empty, bar_drain, bar_drain_b;
+    __shared__ __align__(8) uint64_t bar_qdo_full[NS], bar_qdo_empty[NS];
+    __shared__ __align__(8) uint64_t bar_st_full, bar_st_empty, bar_stage, bar_ds_full, bar_dq_full, bar_dq_empty;
+    __shared__ uint32_t tmem_base_sh;
+    __shared__ volatile int abort_flag;
+    __shared__ int sh_pos[2][BQ];
+    // per pair of query columns (2c, 2c+1): (-lse_2c, -lse_2c+1, -Dsum_2c, -Dsum_2c+1), lse in log2 units
+    __shared__ float4 sh_pair[2][BQ / 2];
+    __shared__ int sh_open[2][BQ / 32];  // per staging warp: every column sees every key of the block
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t sKV = smem_u32(smem + C::kOffKV), sQ = smem_u32(smem + C::kOffQ), sDS = smem_u32(smem + C::kOffDS);
+    const int group = p.Hq / p.Hkv;
+    const int n_items = p.B * p.nblk * p.Hkv;
+
+    if (threadIdx.x == 0) {
+        abort_flag = 0;
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(smem_u32(&bar_kv_full[b]), 1);
+            mbar_init(smem_u32(&bar_kv_empty[b]), 1);
+        }
+        for (int s = 0; s < NS; ++s) {
+            mbar_init(smem_u32(&bar_qdo_full[s]), 1);
+            mbar_init(smem_u32(&bar_qdo_empty[s]), 1);
+        }
+        mbar_init(smem_u32(&bar_dkv_full), 1);
+        mbar_init(smem_u32(&bar_dkv_empty), 128);
+        mbar_init(smem_u32(&bar_drain), 1);
+        mbar_init(smem_u32(&bar_drain_b), 1);
+        mbar_init(smem_u32(&bar_st_full), 1);
+        mbar_init(smem_u32(&bar_st_empty), 256);
+        mbar_init(smem_u32(&bar_stage), 256);
+        mbar_init(smem_u32(&bar_ds_full), 256);
+        mbar_init(smem_u32(&bar_dq_full), 1);
+        mbar_init(smem_u32(&bar_dq_empty), 128);
+        fence_mbar_init();
+    }
+    if (warp == 1) {
+        tmem_alloc(smem_u32(&tmem_base_sh), C::kTmemCols);
+        tmem_relinquish();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = tmem_base_sh;
+
+    if (warp < 4) {
+        setmaxnreg_dec<C::kRegsControl>();
+        if (warp == 0) {
+            // -------------------------------------------------------- producer
+            if (lane == 0) {
+                tma_prefetch_desc(&p.tm_q);
+                tma_prefetch_desc(&p.tm_do);
+                tma_prefetch_desc(&p.tm_k);
+                tma_prefetch_desc(&p.tm_v);
+                const uint64_t pol_q = policy_evict_last();
+                const uint64_t pol_kv = policy_evict_first();
+                int u = 0, kv_items = 0;
+                bool ok = true;
+                for (int k = blockIdx.x; k < n_items && ok; k += gridDim.x) {
+                    const BwdItem it = decode_bwd2<BQ, GLOBAL>(p, k);
+                    if (it.ntiles == 0) continue;
+                    const int kb = kv_items & 1;
+                    if (!(ok = mbar_wait(smem_u32(&bar_kv_empty[kb]), ((kv_items >> 1) & 1) ^ 1, &abort_flag))) break;
+                    const uint32_t kvb = smem_u32(&bar_kv_full[kb]);
+                    mbar_arrive_expect_tx(kvb, 2 * C::kTileBytes);
+                    tma_load_4d(sKV + kb * 2 * C::kTileBytes, &p.tm_k, kvb, 0, it.kvh, it.j * kBN, it.b, pol_kv);
+                    tma_load_4d(sKV + (kb * 2 + 1) * C::kTileBytes, &p.tm_v, kvb, 0, it.kvh, it.j * kBN, it.b, pol_kv);
+                    ++kv_items;
+                    const int n_it = group * it.ntiles;
+                    for (int x = 0; x < n_it; ++x, ++u) {
+                        const int h = it.kvh * group + x / it.ntiles;
+                        const int i = it.i_lo + x % it.ntiles;
+                        const int st = u % NS, f = u / NS;
+                        if (!(ok = mbar_wait(smem_u32(&bar_qdo_empty[st]), (f & 1) ^ 1, &abort_flag))) break;
+                        const uint32_t qb = smem_u32(&bar_qdo_full[st]);
+                        mbar_arrive_expect_tx(qb, 2 * C::kTileBytes);
+                        const int cb = GLOBAL ? 0 : it.b;
+                        tma_load_4d(sQ + st * 2 * C::kTileBytes, &p.tm_q, qb, 0, h, i * BQ, cb, pol_q);
+                        tma_load_4d(sQ + (st * 2 + 1) * C::kTileBytes, &p.tm_do, qb, 0, h, i * BQ, cb, pol_q);
+                    }
                 }
-                r = lo;
+                if (!ok) {  // let copies already issued land before the CTA exits
+                    for (int v = max(0, kv_items - 2); v < kv_items; ++v)
+                        mbar_wait_drain(smem_u32(&bar_kv_full[v & 1]), (v >> 1) & 1);
+                    for (int v = max(0, u - NS); v < u; ++v)
+                        mbar_wait_drain(smem_u32(&bar_qdo_full[v % NS]), (v / NS) & 1);
+                }
             }
-            if (r < r_hi && p.pos[r] == t) {  // selected: converted later
-                ++r;
+        } else if (warp == 1) {
+            // -------------------------------------------------------- MMA issuer A: S^T, dP^T
+            if (lane == 0) {
+                constexpr uint32_t idS = idesc_bf16_f32(kBN, BQ, false, false);
+                int u = 0, kv_items = 0;
+                bool ok = true;
+                for (int k = blockIdx.x; k < n_items && ok; k += gridDim.x) {
+                    const BwdItem it = decode_bwd2<BQ, GLOBAL>(p, k);
+                    if (it.ntiles == 0) continue;
+                    const uint32_t sK = sKV + (kv_items & 1) * 2 * C::kTileBytes, sV = sK + C::kTileBytes;
+                    if (!(ok = mbar_wait(smem_u32(&bar_kv_full[kv_items & 1]), (kv_items >> 1) & 1, &abort_flag))) break;
+                    const int n_it = group * it.ntiles;
+                    for (int x = 0; x < n_it; ++x, ++u) {
+                        const int st = u % NS;
+                        if (!(ok = mbar_wait(smem_u32(&bar_qdo_full[st]), (u / NS) & 1, &abort_flag))) break;
+                        // the softmax warps have loaded S^T, dP^T of tile u-1
+                        if (!(ok = mbar_wait(smem_u32(&bar_st_empty), (u & 1) ^ 1, &abort_flag))) break;
+                        tc_fence_after();
+                        const uint32_t qb = sQ + st * 2 * C::kTileBytes, ob = qb + C::kTileBytes;
+#pragma unroll
+                        for (int ks = 0; ks < D / 16; ++ks) {
+                            umma_bf16_ss(tmem + C::kColS, sdesc_sw128(sK + ks * 32, 16, 1024),
+                                         sdesc_sw128(qb + ks * 32, 16, 1024), idS, ks > 0 ? 1u : 0u);
+                            umma_bf16_ss(tmem + C::kColDP, sdesc_sw128(sV + ks * 32, 16, 1024),
+                                         sdesc_sw128(ob + ks * 32, 16, 1024), idS, ks > 0 ? 1u : 0u);
+                        }
+                        umma_commit(smem_u32(&bar_st_full));
+                    }
+                    if (!ok) break;
+                    ++kv_items;
+                }
+                if (!ok) {
+                    umma_commit(smem_u32(&bar_drain));
+                    mbar_wait_drain(smem_u32(&bar_drain), 0);
+                }
+            }
+        } else if (warp == 2) {
+            // -------------------------------------------------------- MMA issuer B: dV, dK, dQ
+            if (lane == 0) {
+                constexpr uint32_t idKV = idesc_bf16_f32(kBN, D, false, true);  // dV, dK: keys x d
+                constexpr uint32_t idQ = idesc_bf16_f32(BQ, D, true, true);     // dQ: queries x d
+                int u = 0, kv_items = 0;
+                bool ok = true;
+                for (int k = blockIdx.x; k < n_items && ok; k += gridDim.x) {
+                    const BwdItem it = decode_bwd2<BQ, GLOBAL>(p, k);
+                    if (it.ntiles == 0) continue;
+                    const uint32_t sK = sKV + (kv_items & 1) * 2 * C::kTileBytes;
+                    const int n_it = group * it.ntiles;
+                    for (int x = 0; x < n_it; ++x, ++u) {
+                        const int st = u % NS;
+                        if (!(ok = mbar_wait(smem_u32(&bar_ds_full), u & 1, &abort_flag))) break;
+                        if (x == 0 && !(ok = mbar_wait(smem_u32(&bar_dkv_empty), (kv_items & 1) ^ 1, &abort_flag))) break;
+                        tc_fence_after();
+                        const uint32_t qb = sQ + st * 2 * C::kTileBytes, ob = qb + C::kTileBytes;
+#pragma unroll
+                        for (int ks = 0; ks < BQ / 16; ++ks) {
+                            const uint32_t acc = (x > 0 || ks > 0) ? 1u : 0u;
+                            umma_bf16_ts(tmem + C::kColDV, tmem + C::kColP + 8 * ks,
+                                         sdesc_sw128(ob + ks * 2048, 16384, 1024), idKV, acc);
+                            umma_bf16_ss(tmem + C::kColDK, sdesc_sw128(sDS + (ks >> 2) * 16384 + (ks & 3) * 32, 16, 1024),
+                                         sdesc_sw128(qb + ks * 2048, 16384, 1024), idKV, acc);
+                        }
+                        // Q, dO of tile u are read: the ring stage is free before dQ
+                        umma_commit(smem_u32(&bar_qdo_empty[st]));
+                        // the drain warps have read tile u-1's dQ
+                        if (u > 0 && !(ok = mbar_wait(smem_u32(&bar_dq_empty), (u - 1) & 1, &abort_flag))) break;
+                        tc_fence_after();
+#pragma unroll
+                        for (int ks = 0; ks < kBN / 16; ++ks)
+                            umma_bf16_ss(tmem + C::kColDQ, sdesc_sw128(sDS + ks * 2048, 16384, 1024),
+                                         sdesc_sw128(sK + ks * 2048, 16384, 1024), idQ, ks > 0 ? 1u : 0u);
+                        umma_commit(smem_u32(&bar_dq_full));
+                    }
+                    if (!ok) break;
+                    umma_commit(smem_u32(&bar_kv_empty[kv_items & 1]));
+                    umma_commit(smem_u32(&bar_dkv_full));
+                    ++kv_items;
+                }
+                if (!ok) {
+                    umma_commit(smem_u32(&bar_drain_b));
+                    mbar_wait_drain(smem_u32(&bar_drain_b), 0);
+                }
+            }
+        } else if (GLOBAL) {
+            zero_unselected_dq(p, D, lane);
+        }
+    } else if (warp < 12) {
+        // ------------------------------------------------------------ P^T, dS^T
+        setmaxnreg_inc<C::kRegsSoftmax>();
+        const int quad = warp & 3;
+        const int half = (warp - 4) >> 2;  // query columns half*64 .. half*64+63
+        const int t = quad * 32 + lane;    // key row of the block
+        const int tw = threadIdx.x - 128;  // 0..255 across both warpgroups
+        const uint32_t lane_off = static_cast<uint32_t>(quad * 32) << 16;
+        int u = 0;
+        bool ok = true;
+        for (int k = blockIdx.x; k < n_items && ok; k += gridDim.x) {
+            const BwdItem it = decode_bwd2<BQ, GLOBAL>(p, k);
+            if (it.ntiles == 0) continue;
+            const int k0 = it.j * kBN;
+            const int key = k0 + t;
+            const int n_it = group * it.ntiles;
+            // staging values of a tile's query columns (position, lse, Dsum; -1 / 0 /
+            // 0 outside its rows): loaded one tile ahead by the first warpgroup
+            int pf_pos = -1;
+            float pf_lse = 0.f, pf_dsum = 0.f;
+            auto load_stage = [&](int x) {
+                const int h = it.kvh * group + x / it.ntiles;
+                const int i = it.i_lo + x % it.ntiles;
+                pf_pos = -1;
+                pf_lse = pf_dsum = 0.f;
+                const int row = i * BQ + tw;
+                if (!GLOBAL ? row < p.T : (row >= it.row_lo && row < it.row_hi)) {
+                    const int64_t idx = GLOBAL ? static_cast<int64_t>(h) * p.cap + row
+                                               : (static_cast<int64_t>(it.b) * p.Hq + h) * p.T + row;
+                    pf_pos = GLOBAL ? p.pos[row] : row;
+                    pf_lse = p.lse[idx];
+                    pf_dsum = p.dsum[idx];
+                }
+            };
+            if (tw < BQ) load_stage(0);
+            for (int x = 0; x < n_it; ++x, ++u) {
+                const int b = u & 1;
+                if (tw < BQ) {
+                    const bool pf_open = pf_pos >= k0 + kBN - 1 && (GLOBAL || pf_pos - k0 < p.window);
+                    sh_pos[b][tw] = pf_pos;
+                    float* pr = reinterpret_cast<float*>(&sh_pair[b][tw >> 1]);
+                    pr[tw & 1] = -(pf_lse * kLog2e);
+                    pr[2 + (tw & 1)] = -pf_dsum;
+                    const bool all_open = __all_sync(0xffffffffu, pf_open);
+                    if (lane == 0) sh_open[b][tw >> 5] = all_open ? 1 : 0;
+                }
+                mbar_arrive(smem_u32(&bar_stage));
+                ok = mbar_wait(smem_u32(&bar_stage), u & 1, &abort_flag);
+                if (!ok) break;
+                if (tw < BQ && x + 1 < n_it) load_stage(x + 1);
+                const bool open = sh_open[b][2 * half] && sh_open[b][2 * half + 1];
+                // the columns that see this key are adjacent: [lo, hi] of this half
+                int lo = 0, hi = 63;
+                if (!open) {
+                    const int i = it.i_lo + x % it.ntiles;
+                    if (!GLOBAL) {
+                        lo = key - i * BQ;
+                        hi = min(lo + p.window - 1, p.T - 1 - i * BQ);
+                    } else {  // positions ascend over the sequence's rows of the tile
+                        int a = max(0, it.row_lo - i * BQ), e = min(BQ, it.row_hi - i * BQ);
+                        hi = e - 1;
+                        while (a < e) {
+                            const int mid = (a + e) >> 1;
+                            if (sh_pos[b][mid] < key) a = mid + 1;
+                            else e = mid;
+                        }
+                        lo = a;
+                    }
+                    lo -= half * 64;
+                    hi -= half * 64;
+                }
+                ok = mbar_wait(smem_u32(&bar_st_full), u & 1, &abort_flag);
+                __syncwarp();
+                if (!ok) break;
+                tc_fence_after();
+                uint32_t sv[2][32], dpv[2][32];
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {
+                    tmem_ld32(tmem + lane_off + C::kColS + half * 64 + c * 32, sv[c]);
+                    tmem_ld32(tmem + lane_off + C::kColDP + half * 64 + c * 32, dpv[c]);
+                }
+                tmem_wait_ld();
+                tc_fence_before();
+                mbar_arrive(smem_u32(&bar_st_empty));  // S^T, dP^T of tile u+1 may now be written
+                // P = 2^(S*scale*log2e - lse), dS = P (dP - Dsum), two columns per
+                // f32x2 instruction; two branch-free copies of the loop (open tiles
+                // skip the visibility selects)
+                uint32_t pk[32], dk2[32];
+                const uint64_t scale2 = f2_pack(p.scale_log2, p.scale_log2);
+                auto columns = [&](auto masked) {
+                    constexpr bool kMasked = decltype(masked)::value;
+#pragma unroll
+                    for (int c = 0; c < 2; ++c) {
+                        uint32_t m = 0xffffffffu;
+                        if constexpr (kMasked) m = column_mask(lo - 32 * c, hi - 32 * c);
+#pragma unroll
+                        for (int e = 0; e < 32; e += 2) {
+                            const float4 q = sh_pair[b][(half * 64 + c * 32 + e) >> 1];
+                            float x0, x1;
+                            f2_unpack(f2_fma(f2_pack(__uint_as_float(sv[c][e]), __uint_as_float(sv[c][e + 1])), scale2,
+                                             f2_pack(q.x, q.y)),
+                                      x0, x1);
+                            float p0 = ex2_approx(x0), p1 = ex2_approx(x1);
+                            if constexpr (kMasked) {
+                                p0 = (m & (1u << e)) ? p0 : 0.f;
+                                p1 = (m & (2u << e)) ? p1 : 0.f;
+                            }
+                            const uint64_t t2 = f2_add(
+                                f2_pack(__uint_as_float(dpv[c][e]), __uint_as_float(dpv[c][e + 1])), f2_pack(q.z, q.w));
+                            float d0, d1;
+                            f2_unpack(f2_mul(f2_pack(p0, p1), t2), d0, d1);
+                            pk[c * 16 + e / 2] = cvt_bf16x2(p0, p1);
+                            dk2[c * 16 + e / 2] = cvt_bf16x2(d0, d1);
+                        }
+                    }
+                };
+                if (open) columns(std::false_type{});
+                else columns(std::true_type{});
+                // P^T (TMEM) and dS^T (shared) are free once the MMAs of tile u-1 are done
+                if (u > 0) {
+                    ok = mbar_wait(smem_u32(&bar_dq_full), (u - 1) & 1, &abort_flag);
+                    __syncwarp();
+                    if (!ok) break;
+                }
+                tc_fence_after();
+                tmem_st32(tmem + lane_off + C::kColP + half * 32, pk);
+#pragma unroll
+                for (int q4 = 0; q4 < 8; ++q4)
+                    st_shared_v4(sDS + half * 16384 + sw128_offset(t, q4), dk2[4 * q4], dk2[4 * q4 + 1], dk2[4 * q4 + 2],
+                                 dk2[4 * q4 + 3]);
+                tmem_wait_st();
+                fence_proxy_async_smem();
+                tc_fence_before();
+                mbar_arrive(smem_u32(&bar_ds_full));
+            }
+        }
+    } else {
+        // ------------------------------------------------------------ dQ drain, dK/dV epilogue
+        setmaxnreg_dec<C::kRegsDrain>();
+        const int quad = warp & 3;
+        const uint32_t lane_off = static_cast<uint32_t>(quad * 32) << 16;
+        const uint32_t stage = smem_u32(smem + C::kOffDQ) + quad * C::kWarpStage;
+        int u = 0, kv_items = 0;
+        bool ok = true;
+        for (int k = blockIdx.x; k < n_items && ok; k += gridDim.x) {
+            const BwdItem it = decode_bwd2<BQ, GLOBAL>(p, k);
+            const int64_t kv_off =
+                ((static_cast<int64_t>(it.b) * p.T + it.j * kBN + quad * 32) * p.Hkv + it.kvh) * D;  // this warp's first key
+            const int keys = p.T - (it.j * kBN + quad * 32);  // keys of the warp that exist (may exceed 32, or be negative)
+            if (it.ntiles == 0) {
+                // no selected query sees the block: zero dK, dV rows, four whole
+                // rows (8 lanes x 16 bytes each) per warp store
+                for (int r = lane >> 3; r < 32; r += 4) {
+                    if (r < keys) {
+                        const int64_t off = kv_off + static_cast<int64_t>(r) * p.Hkv * D + (lane & 7) * 8;
+                        *reinterpret_cast<uint4*>(p.dk + off) = make_uint4(0, 0, 0, 0);
+                        *reinterpret_cast<uint4*>(p.dv + off) = make_uint4(0, 0, 0, 0);
+                    }
+                }
                 continue;
             }
-            uint4* dst = reinterpret_cast<uint4*>(p.dq_fill + bt * p.Hq * D);
-            for (int v = lane; v < row_vecs; v += 32) dst[v] = make_uint4(0u, 0u, 0u, 0u);
+            const int n_it = group * it.ntiles;
+            for (int x = 0; x < n_it; ++x, ++u) {
+                const int h = it.kvh * group + x / it.ntiles;
+                const int row0 = (it.i_lo + x % it.ntiles) * BQ + quad * 32;  // this warp's first query row
+                ok = mbar_wait(smem_u32(&bar_dq_full), u & 1, &abort_flag);
+                __syncwarp();
+                if (!ok) break;
+                tc_fence_after();
+                uint32_t v[2][32];
+                tmem_ld32(tmem + lane_off + C::kColDQ, v[0]);
+                tmem_ld32(tmem + lane_off + C::kColDQ + 32, v[1]);
+                tmem_wait_ld();
+                tc_fence_before();
+                mbar_arrive(smem_u32(&bar_dq_empty));
+                // rows of other sequences or past the end add zero
+                const int row = row0 + lane;
+                const float mul = (!GLOBAL || (row >= it.row_lo && row < it.row_hi)) ? p.scale : 0.f;
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {
+                    // the reduction before has read the staging rows
+                    if (lane == 0) bulk_wait_read();
+                    __syncwarp();
+#pragma unroll
+                    for (int q4 = 0; q4 < 8; ++q4) {
+                        uint32_t w[4];
+#pragma unroll
+                        for (int e = 0; e < 4; ++e)
+                            w[e] = mul != 0.f ? __float_as_uint(__uint_as_float(v[c][4 * q4 + e]) * mul) : 0u;
+                        st_shared_v4(stage + sw128_offset(lane, q4), w[0], w[1], w[2], w[3]);
+                    }
+                    fence_proxy_async_smem();
+                    __syncwarp();
+                    if (lane == 0 && (GLOBAL || row0 < p.T)) {
+                        tma_reduce_add_4d(&p.tm_dq, stage, 32 * c, h, row0, GLOBAL ? 0 : it.b);
+                        bulk_commit();
+                    }
+                }
+            }
+            if (!ok) break;
+            ok = mbar_wait(smem_u32(&bar_dkv_full), kv_items & 1, &abort_flag);
+            __syncwarp();
+            if (!ok) break;
+            tc_fence_after();
+#pragma unroll
+            for (int which = 0; which < 2; ++which) {
+                const uint32_t col = which == 0 ? C::kColDK : C::kColDV;
+                const float mul = which == 0 ? p.scale : 1.0f;
+                logo_bf16* dst = (which == 0 ? p.dk : p.dv) + kv_off + (lane & 3) * 8;
+#pragma unroll
+                for (int cc = 0; cc < D / 32; ++cc) {
+                    uint32_t v[2][16];
+#pragma unroll
+                    for (int hf = 0; hf < 2; ++hf)
+                        tmem_ld_16x256b_x4(tmem + lane_off + (static_cast<uint32_t>(hf * 16) << 16) + col + cc * 32, v[hf]);
+                    tmem_wait_ld();
+                    if (which == 1 && cc == D / 32 - 1) {
+                        tc_fence_before();
+                        mbar_arrive(smem_u32(&bar_dkv_empty));
+                    }
+#pragma unroll
+                    for (int hf = 0; hf < 2; ++hf)
+#pragma unroll
+                        for (int ab = 0; ab < 2; ++ab) {
+                            uint32_t w[4];
+#pragma unroll
+                            for (int k4 = 0; k4 < 4; ++k4)
+                                w[k4] = cvt_bf16x2(__uint_as_float(v[hf][4 * k4 + 2 * ab]) * mul,
+                                                   __uint_as_float(v[hf][4 * k4 + 2 * ab + 1]) * mul);
+                            const uint4 o = quad_gather8(w, lane);
+                            const int r = hf * 16 + ab * 8 + (lane >> 2);
+                            if (r < keys) *reinterpret_cast<uint4*>(dst + static_cast<int64_t>(r) * p.Hkv * D + cc * 32) = o;
+                        }
+                }
+            }
+            ++kv_items;
         }
+        if (lane == 0) bulk_wait_all();
     }
     tc_fence_before();
     __syncthreads();
@@ -1048,7 +1169,7 @@ __global__ void __launch_bounds__(128) bwd_pre_kernel(const logo_bf16* __restric
     }
 }
 
-// Global branch, d = 128: dQ accumulator rows of the selected tokens -> their
+// Global branch: dQ accumulator rows of the selected tokens -> their
 // rows of the dense dq (the backward kernel zeroed the others); blocks stride
 // over the packed rows below the selected count.
 __global__ void __launch_bounds__(128) bwd_post_selected_kernel(const float* __restrict__ dq_acc,
@@ -1075,36 +1196,19 @@ __global__ void __launch_bounds__(128) bwd_post_selected_kernel(const float* __r
     }
 }
 
-// dQ accumulator (fp32) -> dq (bf16).  Local: elementwise.  Global: every
-// dense token writes its packed row's gradient, or zeros if not selected.
-template <bool GLOBAL>
-__global__ void __launch_bounds__(128) bwd_post_kernel(const float* __restrict__ dq_acc, const int32_t* __restrict__ pos,
-                                                       const int32_t* __restrict__ cu_q, int T, int H, int D,
+// Local branch: dQ accumulator (fp32) -> dq (bf16).
+__global__ void __launch_bounds__(128) bwd_post_kernel(const float* __restrict__ dq_acc, int row_elems,
                                                        logo_bf16* __restrict__ dq)
 {
     const int64_t bt = blockIdx.x;
-    const int row_elems = H * D;
-    int64_t src_row = bt;
-    if (GLOBAL) {
-        const int b = static_cast<int>(bt / T), t = static_cast<int>(bt % T);
-        int lo = cu_q[b], hi = cu_q[b + 1];
-        while (lo < hi) {
-            const int mid = (lo + hi) >> 1;
-            if (pos[mid] < t) lo = mid + 1;
-            else hi = mid;
-        }
-        src_row = (lo < cu_q[b + 1] && pos[lo] == t) ? lo : -1;
-    }
     for (int v = threadIdx.x; v < row_elems / 8; v += blockDim.x) {
-        uint4 w = make_uint4(0, 0, 0, 0);
-        if (src_row >= 0) {
-            const float4* s = reinterpret_cast<const float4*>(dq_acc + src_row * row_elems + v * 8);
-            const float4 a = s[0], c = s[1];
-            w.x = pack_bf16x2(a.x, a.y);
-            w.y = pack_bf16x2(a.z, a.w);
-            w.z = pack_bf16x2(c.x, c.y);
-            w.w = pack_bf16x2(c.z, c.w);
-        }
+        const float4* s = reinterpret_cast<const float4*>(dq_acc + bt * row_elems + v * 8);
+        const float4 a = s[0], c = s[1];
+        uint4 w;
+        w.x = pack_bf16x2(a.x, a.y);
+        w.y = pack_bf16x2(a.z, a.w);
+        w.z = pack_bf16x2(c.x, c.y);
+        w.w = pack_bf16x2(c.z, c.w);
         *reinterpret_cast<uint4*>(dq + bt * row_elems + v * 8) = w;
     }
 }
@@ -1172,12 +1276,11 @@ int launch_bwd(const BwdParams& prm, cudaStream_t st)
         }
         attn_bwd2_kernel<GLOBAL><<<grid, Bwd2Cfg::kThreads, Bwd2Cfg::kSmemBytes, st>>>(prm);
     } else {
-        using C = BwdCfg<D>;
         if (!attr_done) {
-            if (set_smem_limit(attn_bwd_kernel<D, GLOBAL>, C::kSmemBytes) != cudaSuccess) return LOGO_ERR_CUDA;
+            if (set_smem_limit(attn_bwd64_kernel<GLOBAL>, Bwd64Cfg::kSmemBytes) != cudaSuccess) return LOGO_ERR_CUDA;
             attr_done = true;
         }
-        attn_bwd_kernel<D, GLOBAL><<<grid, 192, C::kSmemBytes, st>>>(prm);
+        attn_bwd64_kernel<GLOBAL><<<grid, Bwd64Cfg::kThreads, Bwd64Cfg::kSmemBytes, st>>>(prm);
     }
     return cudaGetLastError() == cudaSuccess ? LOGO_OK : LOGO_ERR_CUDA;
 }
@@ -1227,11 +1330,12 @@ extern "C" int logo_local_attn_bwd(const logo_bf16* q, const logo_bf16* k, const
     bwd_pre_kernel<false><<<pre_grid, 128, 0, st>>>(o, dO, nullptr, rows, dims.T, dims.Hq, dims.D, 0, ws.dsum,
                                                     nullptr, ws.dq_acc, GlobalPrep{});
     BwdParams prm{};
-    const uint32_t qrows = dims.D == 128 ? Bwd2Cfg::kBQ : kBM;
+    const uint32_t qrows = dims.D == 128 ? Bwd2Cfg::kBQ : Bwd64Cfg::kBQ;
     if (!encode_bf16_4d(&prm.tm_q, q, dims.D, dims.Hq, dims.T, dims.B, 64, qrows) ||
         !encode_bf16_4d(&prm.tm_do, dO, dims.D, dims.Hq, dims.T, dims.B, 64, qrows) ||
         !encode_bf16_4d(&prm.tm_k, k, dims.D, dims.Hkv, dims.T, dims.B, 64, kBN) ||
-        !encode_bf16_4d(&prm.tm_v, v, dims.D, dims.Hkv, dims.T, dims.B, 64, kBN))
+        !encode_bf16_4d(&prm.tm_v, v, dims.D, dims.Hkv, dims.T, dims.B, 64, kBN) ||
+        (dims.D == 64 && !encode_f32_4d(&prm.tm_dq, ws.dq_acc, dims.D, dims.Hq, dims.T, dims.B, 32, 32)))
         return LOGO_ERR_CUDA;
     prm.lse = lse;
     prm.dsum = ws.dsum;
@@ -1250,7 +1354,7 @@ extern "C" int logo_local_attn_bwd(const logo_bf16* q, const logo_bf16* k, const
     prm.scale_log2 = scale * kLog2e;
     rc = dims.D == 128 ? launch_bwd<128, false>(prm, st) : launch_bwd<64, false>(prm, st);
     if (rc != LOGO_OK) return rc;
-    bwd_post_kernel<false><<<rows, 128, 0, st>>>(ws.dq_acc, nullptr, nullptr, dims.T, dims.Hq, dims.D, dq);
+    bwd_post_kernel<<<rows, 128, 0, st>>>(ws.dq_acc, dims.Hq * dims.D, dq);
     return cudaGetLastError() == cudaSuccess ? LOGO_OK : LOGO_ERR_CUDA;
 }
 
@@ -1286,11 +1390,13 @@ extern "C" int logo_global_sparse_attn_bwd(const logo_bf16* q, const logo_bf16* 
                                                     ws.doc, ws.dq_acc, gp);
     if (cudaGetLastError() != cudaSuccess) return LOGO_ERR_CUDA;
     BwdParams prm{};
-    const uint32_t qrows = dims.D == 128 ? Bwd2Cfg::kBQ : kBM;
+    const uint32_t qrows = dims.D == 128 ? Bwd2Cfg::kBQ : Bwd64Cfg::kBQ;
     if (!encode_bf16_4d(&prm.tm_q, ws.qc, dims.D, dims.Hq, static_cast<uint64_t>(cap) + kBM, 1, 64, qrows) ||
         !encode_bf16_4d(&prm.tm_do, ws.doc, dims.D, dims.Hq, static_cast<uint64_t>(cap) + kBM, 1, 64, qrows) ||
         !encode_bf16_4d(&prm.tm_k, k, dims.D, dims.Hkv, dims.T, dims.B, 64, kBN) ||
-        !encode_bf16_4d(&prm.tm_v, v, dims.D, dims.Hkv, dims.T, dims.B, 64, kBN))
+        !encode_bf16_4d(&prm.tm_v, v, dims.D, dims.Hkv, dims.T, dims.B, 64, kBN) ||
+        (dims.D == 64 &&
+         !encode_f32_4d(&prm.tm_dq, ws.dq_acc, dims.D, dims.Hq, static_cast<uint64_t>(cap) + kBM, 1, 32, 32)))
         return LOGO_ERR_CUDA;
     prm.lse = lse_c;
     prm.dsum = ws.dsum;
@@ -1300,7 +1406,7 @@ extern "C" int logo_global_sparse_attn_bwd(const logo_bf16* q, const logo_bf16* 
     prm.pos = pos;
     prm.cu_q = cu_q;
     prm.first_row = ws.first_row;
-    prm.dq_fill = dims.D == 128 ? dq : nullptr;
+    prm.dq_fill = dq;
     prm.B = dims.B;
     prm.T = dims.T;
     prm.Hq = dims.Hq;
@@ -1313,10 +1419,7 @@ extern "C" int logo_global_sparse_attn_bwd(const logo_bf16* q, const logo_bf16* 
     prm.scale_log2 = scale * kLog2e;
     rc = dims.D == 128 ? launch_bwd<128, true>(prm, st) : launch_bwd<64, true>(prm, st);
     if (rc != LOGO_OK) return rc;
-    if (dims.D == 128)
-        bwd_post_selected_kernel<<<grid_rows, 128, 0, st>>>(ws.dq_acc, pos, cu_q, n_sel_total, dims.B, dims.T,
-                                                            dims.Hq, dims.D, dq);
-    else
-        bwd_post_kernel<true><<<cap, 128, 0, st>>>(ws.dq_acc, pos, cu_q, dims.T, dims.Hq, dims.D, dq);
+    bwd_post_selected_kernel<<<grid_rows, 128, 0, st>>>(ws.dq_acc, pos, cu_q, n_sel_total, dims.B, dims.T, dims.Hq,
+                                                        dims.D, dq);
     return cudaGetLastError() == cudaSuccess ? LOGO_OK : LOGO_ERR_CUDA;
 }

@@ -57,6 +57,30 @@ __device__ __forceinline__ bool key_visible(int key, int pos, int window)
     return key <= pos && key > pos - window;
 }
 
+// 32 columns as a bit mask: bit c set for lo <= c <= hi (either may lie
+// outside 0..31; PTX shifts by 32 and more give 0).
+__device__ __forceinline__ uint32_t column_mask(int lo, int hi)
+{
+    uint32_t up, down;
+    asm("shr.u32 %0, 0xffffffff, %1;" : "=r"(up) : "r"(max(31 - hi, 0)));
+    asm("shl.b32 %0, 0xffffffff, %1;" : "=r"(down) : "r"(max(lo, 0)));
+    return up & down;
+}
+
+// Four lanes (a quad) hold, each, the bf16 pair of columns 8k + 2j, 8k + 2j + 1
+// of a row for k = 0..3 (j the lane's place in the quad): afterwards lane j has
+// the 8 adjacent columns 8j .. 8j + 7.
+__device__ __forceinline__ uint4 quad_gather8(const uint32_t (&x)[4], int lane)
+{
+    const bool b0 = lane & 1, b1 = lane & 2;
+    const uint32_t r0 = __shfl_xor_sync(0xffffffffu, b0 ? x[0] : x[1], 1);
+    const uint32_t r1 = __shfl_xor_sync(0xffffffffu, b0 ? x[2] : x[3], 1);
+    const uint32_t y0 = b0 ? r0 : x[0], y1 = b0 ? x[1] : r0, y2 = b0 ? r1 : x[2], y3 = b0 ? x[3] : r1;
+    const uint32_t q0 = __shfl_xor_sync(0xffffffffu, b1 ? y0 : y2, 2);
+    const uint32_t q1 = __shfl_xor_sync(0xffffffffu, b1 ? y1 : y3, 2);
+    return b1 ? make_uint4(q0, q1, y2, y3) : make_uint4(y0, y1, q0, q1);
+}
+
 // Sequence of packed row `row`: the b with cu_q[b] <= row < cu_q[b+1].
 __device__ __forceinline__ int seq_of_row(const int32_t* cu_q, int B, int row)
 {

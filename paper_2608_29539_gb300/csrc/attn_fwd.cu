@@ -170,10 +170,7 @@ __device__ __forceinline__ void mask_row_block(float (&s)[kBN], int lo, int hi)
 {
 #pragma unroll
     for (int g = 0; g < kBN / 32; ++g) {
-        uint32_t up, down;  // (PTX shifts by 32 and more give 0)
-        asm("shr.u32 %0, 0xffffffff, %1;" : "=r"(up) : "r"(max(31 - (hi - 32 * g), 0)));
-        asm("shl.b32 %0, 0xffffffff, %1;" : "=r"(down) : "r"(max(lo - 32 * g, 0)));
-        const uint32_t m = up & down;
+        const uint32_t m = column_mask(lo - 32 * g, hi - 32 * g);
 #pragma unroll
         for (int i = 0; i < 32; ++i) s[32 * g + i] = (m & (1u << i)) ? s[32 * g + i] : -INFINITY;
     }
@@ -715,7 +712,7 @@ __global__ void __launch_bounds__(512, 1) attn_fwd_kernel(const __grid_constant_
             // as soon as the last of them is read: the first 32 go out at once,
             // the others wait as pairs until then.
             constexpr int kEarly = 1;
-            uint32_t w[D / 32][2][8];  // [32 columns][rows 0..15 or 16..31][row t / 4: 4 pairs, row t / 4 + 8: 4 pairs]
+            uint32_t w[D / 32][2][2][4];  // [32 columns][rows 0..15 or 16..31][row t / 4 or t / 4 + 8][pairs]
             auto load32 = [&](int c) {
                 uint32_t v[2][16];
 #pragma unroll
@@ -727,8 +724,8 @@ __global__ void __launch_bounds__(512, 1) attn_fwd_kernel(const __grid_constant_
 #pragma unroll
                     for (int k4 = 0; k4 < 4; ++k4) {
                         const uint32_t* x = v[hf] + 4 * k4;
-                        w[c][hf][k4] = cvt_bf16x2(__uint_as_float(x[0]) * ia, __uint_as_float(x[1]) * ia);
-                        w[c][hf][4 + k4] = cvt_bf16x2(__uint_as_float(x[2]) * ib, __uint_as_float(x[3]) * ib);
+                        w[c][hf][0][k4] = cvt_bf16x2(__uint_as_float(x[0]) * ia, __uint_as_float(x[1]) * ia);
+                        w[c][hf][1][k4] = cvt_bf16x2(__uint_as_float(x[2]) * ib, __uint_as_float(x[3]) * ib);
                     }
                 }
             };
@@ -737,17 +734,10 @@ __global__ void __launch_bounds__(512, 1) attn_fwd_kernel(const __grid_constant_
                 for (int hf = 0; hf < 2; ++hf)
 #pragma unroll
                     for (int ab = 0; ab < 2; ++ab) {
-                        const uint32_t* x = w[c][hf] + 4 * ab;
-                        const bool b0 = lane & 1, b1 = lane & 2;
-                        const uint32_t r0 = __shfl_xor_sync(0xffffffffu, b0 ? x[0] : x[1], 1);
-                        const uint32_t r1 = __shfl_xor_sync(0xffffffffu, b0 ? x[2] : x[3], 1);
-                        const uint32_t y0 = b0 ? r0 : x[0], y1 = b0 ? x[1] : r0, y2 = b0 ? r1 : x[2], y3 = b0 ? x[3] : r1;
-                        const uint32_t q0 = __shfl_xor_sync(0xffffffffu, b1 ? y0 : y2, 2);
-                        const uint32_t q1 = __shfl_xor_sync(0xffffffffu, b1 ? y1 : y3, 2);
+                        const uint4 o = quad_gather8(w[c][hf][ab], lane);
                         const int row = hf * 16 + ab * 8 + (lane >> 2);
                         if (quad * 32 + row < it.nrows)
-                            *reinterpret_cast<uint4*>(o0 + static_cast<int64_t>(row) * p.Hq * D + c * 32) =
-                                b1 ? make_uint4(q0, q1, y2, y3) : make_uint4(y0, y1, q0, q1);
+                            *reinterpret_cast<uint4*>(o0 + static_cast<int64_t>(row) * p.Hq * D + c * 32) = o;
                     }
             };
 #pragma unroll

@@ -51,19 +51,30 @@ static EncodeTiledFn encode_fn()
     return fn;
 }
 
-bool encode_bf16_4d(CUtensorMap* map, const void* base, uint64_t d0, uint64_t d1, uint64_t d2, uint64_t d3,
-                    uint32_t box0, uint32_t box2)
+static bool encode_4d(CUtensorMap* map, CUtensorMapDataType type, uint64_t size, const void* base, uint64_t d0,
+                      uint64_t d1, uint64_t d2, uint64_t d3, uint32_t box0, uint32_t box2)
 {
     EncodeTiledFn fn = encode_fn();
     if (!fn) return false;
     cuuint64_t dims[4] = {d0, d1, d2, d3};
-    cuuint64_t strides[3] = {d0 * 2, d0 * d1 * 2, d0 * d1 * d2 * 2};
+    cuuint64_t strides[3] = {d0 * size, d0 * d1 * size, d0 * d1 * d2 * size};
     cuuint32_t box[4] = {box0, 1, box2, 1};
     cuuint32_t estr[4] = {1, 1, 1, 1};
-    CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, estr,
-                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    CUresult r = fn(map, type, 4, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                    CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS;
+}
+
+bool encode_bf16_4d(CUtensorMap* map, const void* base, uint64_t d0, uint64_t d1, uint64_t d2, uint64_t d3,
+                    uint32_t box0, uint32_t box2)
+{
+    return encode_4d(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, base, d0, d1, d2, d3, box0, box2);
+}
+
+bool encode_f32_4d(CUtensorMap* map, const void* base, uint64_t d0, uint64_t d1, uint64_t d2, uint64_t d3,
+                   uint32_t box0, uint32_t box2)
+{
+    return encode_4d(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, base, d0, d1, d2, d3, box0, box2);
 }
 
 }  // namespace logo

@@ -24,6 +24,10 @@ int device_sm_count();
 bool encode_bf16_4d(CUtensorMap* map, const void* base, uint64_t d0, uint64_t d1, uint64_t d2, uint64_t d3,
                     uint32_t box0, uint32_t box2);
 
+// The same over fp32 values (the box's innermost extent at most 32).
+bool encode_f32_4d(CUtensorMap* map, const void* base, uint64_t d0, uint64_t d1, uint64_t d2, uint64_t d3,
+                   uint32_t box0, uint32_t box2);
+
 // Round up to a multiple of `a`.
 inline size_t round_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
