@@ -16,7 +16,9 @@
 // and outputs bf16.
 // The kernels are bound as much by instruction issue as by HBM: without gains
 // (both NULL, i.e. 1) a separate instantiation drops the gain loads and the
-// unit multiplies and does the elementwise work as f32x2 pairs.
+// unit multiplies and does the elementwise work as f32x2 pairs; with gains,
+// token rows of up to 8192 elements have kernels of their own ("gains read"
+// below), and these serve the wider ones only.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -107,6 +109,15 @@ __device__ __forceinline__ void acc_add8(float4* sh, int nvec, int branch, int s
     b.x += c.v[4]; b.y += c.v[5]; b.z += c.v[6]; b.w += c.v[7];
     *p0 = a;
     *p1 = b;
+}
+
+// Sum over W consecutive lanes.
+template <int W>
+__device__ __forceinline__ float lane_sum(float x)
+{
+#pragma unroll
+    for (int o = W / 2; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    return x;
 }
 
 // Sum over the `width` consecutive lanes (a power of two <= 32) of one head.
@@ -466,6 +477,391 @@ __global__ void __launch_bounds__(kThreads, bwd_min_blocks<GPT, G, DGAIN, UNIT>(
     }
 }
 
+// ------------------------------------------------------------- gains read
+// The kernels for trained gains (either gain pointer given), Hq*D <= 8192: one
+// 16-byte vector of the token row per thread, and as many rows of threads as
+// fill 256 threads when the token row is short.  Each thread copies its
+// vectors of the next tokens into shared-memory slots of its own (cp.async, a
+// ring of kRing tokens; nothing but the thread itself reads them, so there is
+// no barrier), which keeps (kRing - 1) x 16 to 48 bytes a thread in flight at
+// no cost in registers: those hold the thread's gains and its sums of the
+// gains' gradients for the whole kernel.  The routing (row_of, z, p) of a
+// warp's next 32 tokens is loaded at once, one token a lane, 32 steps ahead:
+// the tokens of a block lie a grid apart, so each of these loads is a DRAM
+// access of its own, and fetched one step ahead they set the pace (2460 clocks
+// a step at 16K).  D is a template parameter and addresses advance by adding:
+// the first version of this layout ran 200 and 280 instructions a vector and
+// was bound by issue.  Before, a thread had one token's loads in flight,
+// fetched the gains from L1 for every token and kept the sums in shared
+// memory.  16K, 32 heads, d 128, 1/8 selected: forward 68 -> 48 us (6.3 TB/s,
+// 93% of HBM), backward with gain gradients 128 -> 80 us (5.4 TB/s).
+template <int MAXT>
+struct GainCfg {
+    // The forward runs two blocks of 512 threads an SM at 64 registers, its
+    // gains in shared-memory slots of the thread (one block at 80 registers
+    // with the gains in them: 54.5 against 48.6 us at 16K).  The backward's
+    // gains and sums take 32 registers: one block of 512 threads at up to 128;
+    // a token row of more than 512 vectors (Hq*D > 4096) takes a block of 1024
+    // at 64, where gains and sums sit in shared memory beside a shorter ring.
+    static constexpr int kRingFwd = 3;
+    static constexpr bool kInRegs = MAXT <= 512;
+    static constexpr int kRingBwd = kInRegs ? 4 : 2;
+};
+
+__device__ __forceinline__ void copy16_async(uint32_t dst, const void* src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copies_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void copies_wait()  // all but the newest N groups have landed
+{
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+struct Routing {
+    int row;  // packed row, -1: not selected (or no such token)
+    float p;
+
+    __device__ __forceinline__ void load(const uint8_t* z, const int32_t* row_of, const float* gate_p, int64_t t,
+                                         int64_t ntok)
+    {
+        const bool have = t < ntok;
+        const int r = have ? row_of[t] : -1;
+        const bool sel = have && z[t] != 0;
+        p = have ? gate_p[t] : 0.f;
+        row = sel ? r : -1;
+    }
+};
+
+// Routing of the tokens t0, t0 + step, t0 + 2 step, .. of a warp, handed out in
+// order; called by all 32 lanes.
+struct RoutingAhead {
+    Routing cur, next;  // of this lane's token in the batch of 32, and in the one after
+    int k;
+
+    __device__ __forceinline__ RoutingAhead(const uint8_t* z, const int32_t* row_of, const float* gate_p, int64_t t0,
+                                            int64_t step, int64_t ntok)
+        : k(0)
+    {
+        const int lane = threadIdx.x & 31;
+        cur.load(z, row_of, gate_p, t0 + lane * step, ntok);
+        next.load(z, row_of, gate_p, t0 + (lane + 32) * step, ntok);
+    }
+    // t: the token asked for
+    __device__ __forceinline__ Routing get(const uint8_t* z, const int32_t* row_of, const float* gate_p, int64_t t,
+                                           int64_t step, int64_t ntok)
+    {
+        const Routing r{__shfl_sync(0xffffffffu, cur.row, k), __shfl_sync(0xffffffffu, cur.p, k)};
+        if (++k == 32) {
+            k = 0;
+            cur = next;
+            next.load(z, row_of, gate_p, t + (33 + (threadIdx.x & 31)) * step, ntok);
+        }
+        return r;
+    }
+};
+
+// 8 floats of the thread in shared memory: float4 slot (2 k + half) * n + s.
+__device__ __forceinline__ Vec8 slot_load(const float4* sh, int n, int k, int s)
+{
+    const float4 a = sh[k * 2 * n + s], b = sh[(k * 2 + 1) * n + s];
+    return Vec8{{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w}};
+}
+
+__device__ __forceinline__ void slot_store(float4* sh, int n, int k, int s, const Vec8& x)
+{
+    sh[k * 2 * n + s] = make_float4(x.v[0], x.v[1], x.v[2], x.v[3]);
+    sh[(k * 2 + 1) * n + s] = make_float4(x.v[4], x.v[5], x.v[6], x.v[7]);
+}
+
+__device__ __forceinline__ Vec8 mul8(const Vec8& x, const Vec8& y)
+{
+    Vec8 r;
+#pragma unroll
+    for (int i = 0; i < 8; i += 2)
+        f2_unpack(f2_mul(f2_pack(x.v[i], x.v[i + 1]), f2_pack(y.v[i], y.v[i + 1])), r.v[i], r.v[i + 1]);
+    return r;
+}
+
+// acc += x * y * a
+__device__ __forceinline__ void fma8(Vec8& acc, const Vec8& x, const Vec8& y, float a)
+{
+    const uint64_t a2 = f2_pack(a, a);
+#pragma unroll
+    for (int i = 0; i < 8; i += 2)
+        f2_unpack(f2_fma(f2_mul(f2_pack(x.v[i], x.v[i + 1]), a2), f2_pack(y.v[i], y.v[i + 1]),
+                         f2_pack(acc.v[i], acc.v[i + 1])),
+                  acc.v[i], acc.v[i + 1]);
+}
+
+__device__ __forceinline__ float sumsq8(const Vec8& x)
+{
+    const Vec8 a[1] = {x};
+    return sumsq_g<1>(a);
+}
+
+__device__ __forceinline__ float dot8(const Vec8& x, const Vec8& y)
+{
+    const Vec8 a[1] = {x}, b[1] = {y};
+    return dot_g<1>(a, b);
+}
+
+// Where thread threadIdx.x stands: its row of threads (tpr of them, a multiple
+// of 32) and its vector there.
+template <int D>
+struct GainPlace {
+    int row, v, h, j0;
+    bool active;
+
+    __device__ __forceinline__ GainPlace(int tpr, int nvec)
+    {
+        row = threadIdx.x / tpr;
+        v = threadIdx.x - row * tpr;
+        active = v < nvec;
+        h = active ? v / (D / 8) : 0;
+        j0 = active ? v % (D / 8) : 0;
+    }
+};
+
+template <int D, int MAXT>
+__global__ void __launch_bounds__(MAXT, MAXT == 512 ? 2 : 1) combine_gained_fwd_kernel(
+    const logo_bf16* __restrict__ o_l, const logo_bf16* __restrict__ o_c, const float* __restrict__ gate_p,
+    const uint8_t* __restrict__ z, const int32_t* __restrict__ row_of, const float* __restrict__ gain_l,
+    const float* __restrict__ gain_g, float eps, logo_bf16* __restrict__ o, float* __restrict__ rstd_l,
+    float* __restrict__ rstd_g, int64_t ntok, int H, int tpr, int rows)
+{
+    constexpr int S = GainCfg<MAXT>::kRingFwd, VPR = D / 8;
+    extern __shared__ float4 sh_dyn[];  // ring [S][o_l, o_c][thread] of 16 bytes, then the gains
+    __shared__ Routing sh_rt[S][32];    // per warp
+    const int nvec = H * VPR, nthr = blockDim.x, warp = threadIdx.x >> 5;
+    const GainPlace<D> me(tpr, nvec);
+    float4* sh_gain = sh_dyn + S * 2 * nthr;
+    slot_store(sh_gain, nthr, 0, threadIdx.x, load_gain(gain_l, me.h, D, me.j0));
+    slot_store(sh_gain, nthr, 1, threadIdx.x, load_gain(gain_g, me.h, D, me.j0));
+    const int64_t step = static_cast<int64_t>(gridDim.x) * rows;
+    int64_t t = static_cast<int64_t>(blockIdx.x) * rows + me.row, t_issue = t;
+    const int64_t step_el = step * nvec * 8;             // elements from one of this thread's tokens to the next
+    int64_t off = (t * nvec + me.v) * 8, off_issue = off;
+    const logo_bf16* oc_v = o_c + me.v * 8;
+    RoutingAhead ahead(z, row_of, gate_p, t, step, ntok);
+    const uint32_t ring = smem_u32(sh_dyn + threadIdx.x), stage_bytes = 2 * nthr * 16;
+    uint32_t dst = ring;
+    Routing* rt_issue = &sh_rt[0][warp];
+    int n_issue = 0;
+    auto issue = [&]() {
+        const Routing nx = ahead.get(z, row_of, gate_p, t_issue, step, ntok);
+        if (me.active && t_issue < ntok) {
+            copy16_async(dst, o_l + off_issue);
+            if (nx.row >= 0) copy16_async(dst + nthr * 16, oc_v + static_cast<int64_t>(nx.row) * (nvec * 8));
+        }
+        copies_commit();
+        if ((threadIdx.x & 31) == 0) *rt_issue = nx;
+        t_issue += step;
+        off_issue += step_el;
+        const bool wrap = ++n_issue == S;
+        n_issue = wrap ? 0 : n_issue;
+        dst = wrap ? ring : dst + stage_bytes;
+        rt_issue = wrap ? &sh_rt[0][warp] : rt_issue + 32;
+    };
+#pragma unroll 1
+    for (int i = 0; i < S - 1; ++i) issue();
+    int st = 0;
+    const float4* slot = sh_dyn + threadIdx.x;
+    for (; t < ntok; t += step, off += step_el) {
+        __syncwarp();  // every lane has read the routing slot that is written next
+        issue();
+        copies_wait<S - 1>();
+        __syncwarp();
+        const Routing rt = sh_rt[st][warp];
+        const Vec8 x = unpack8(*reinterpret_cast<const uint4*>(slot));
+        const float r_l = rsqrtf(lane_sum<VPR>(sumsq8(x)) * (1.0f / D) + eps);
+        const bool sel = rt.row >= 0;
+        Vec8 out = mul8(axpby8(x, sel ? (1.0f - rt.p) * r_l : r_l, nullptr, 0.f),
+                        slot_load(sh_gain, nthr, 0, threadIdx.x));
+        if (sel) {
+            const Vec8 xg = unpack8(*reinterpret_cast<const uint4*>(slot + nthr));
+            const float r_g = rsqrtf(lane_sum<VPR>(sumsq8(xg)) * (1.0f / D) + eps);
+            fma8(out, xg, slot_load(sh_gain, nthr, 1, threadIdx.x), rt.p * r_g);
+            if (me.active && me.j0 == 0 && rstd_g) rstd_g[static_cast<int64_t>(rt.row) * H + me.h] = r_g;
+        }
+        if (me.active) {
+            store_bf16x8(o + off, out);
+            if (me.j0 == 0 && rstd_l) rstd_l[t * H + me.h] = r_l;
+        }
+        const bool wrap = ++st == S;
+        st = wrap ? 0 : st;
+        slot = wrap ? sh_dyn + threadIdx.x : slot + 2 * nthr;
+    }
+    copies_wait<0>();
+}
+
+// part (DGAIN): [gridDim.x][2][H*D] float32 per-block sums of the local and
+// global gain gradients.
+template <int D, int MAXT, bool DGAIN>
+__global__ void __launch_bounds__(MAXT) combine_gained_bwd_kernel(
+    const logo_bf16* __restrict__ dO, const logo_bf16* __restrict__ o_l, const logo_bf16* __restrict__ o_c,
+    const float* __restrict__ gate_p, const uint8_t* __restrict__ z, const int32_t* __restrict__ row_of,
+    const float* __restrict__ gain_l, const float* __restrict__ gain_g, float eps, logo_bf16* __restrict__ dO_l,
+    logo_bf16* __restrict__ dO_c, float* __restrict__ dgate_p, float* __restrict__ part, int64_t ntok, int H, int tpr,
+    int rows)
+{
+    constexpr int S = GainCfg<MAXT>::kRingBwd, VPR = D / 8;
+    constexpr bool kInRegs = GainCfg<MAXT>::kInRegs;
+    constexpr int kGroup = 8;  // tokens whose dp sums share a barrier
+    extern __shared__ float4 sh_dyn[];  // ring [S][dO, o_l, o_c][thread], gains and (DGAIN) sums unless in registers
+    __shared__ Routing sh_rt[S][32];    // per warp
+    __shared__ float sh_dp[2][kGroup][32];
+    const int nvec = H * VPR, nthr = blockDim.x, warp = threadIdx.x >> 5;
+    const GainPlace<D> me(tpr, nvec);
+    float4* sh_gain = sh_dyn + S * 3 * nthr;
+    float4* sh_sum = sh_gain + (kInRegs ? 0 : 4 * nthr);
+    const Vec8 gl_r = load_gain(gain_l, me.h, D, me.j0), gg_r = load_gain(gain_g, me.h, D, me.j0);
+    Vec8 sum_l{}, sum_g{};
+    if (!kInRegs) {
+        slot_store(sh_gain, nthr, 0, threadIdx.x, gl_r);
+        slot_store(sh_gain, nthr, 1, threadIdx.x, gg_r);
+        if (DGAIN) {
+            slot_store(sh_sum, nthr, 0, threadIdx.x, sum_l);
+            slot_store(sh_sum, nthr, 1, threadIdx.x, sum_g);
+        }
+    }
+    // slots of vectors and tokens that do not exist are never copied to
+    for (int i = 0; i < S * 3; ++i) sh_dyn[i * nthr + threadIdx.x] = make_float4(0.f, 0.f, 0.f, 0.f);
+    const int64_t step = static_cast<int64_t>(gridDim.x) * rows;
+    int64_t t = static_cast<int64_t>(blockIdx.x) * rows + me.row, t_issue = t;
+    const int64_t step_el = step * nvec * 8;
+    int64_t off = (t * nvec + me.v) * 8, off_issue = off;
+    const logo_bf16* oc_v = o_c + me.v * 8;
+    logo_bf16* dc_v = dO_c + me.v * 8;
+    RoutingAhead ahead(z, row_of, gate_p, t, step, ntok);
+    const uint32_t ring = smem_u32(sh_dyn + threadIdx.x), stage_bytes = 3 * nthr * 16;
+    uint32_t dst = ring;
+    Routing* rt_issue = &sh_rt[0][warp];
+    int n_issue = 0;
+    auto issue = [&]() {
+        const Routing nx = ahead.get(z, row_of, gate_p, t_issue, step, ntok);
+        if (me.active && t_issue < ntok) {
+            copy16_async(dst, dO + off_issue);
+            copy16_async(dst + nthr * 16, o_l + off_issue);
+            if (nx.row >= 0) copy16_async(dst + nthr * 32, oc_v + static_cast<int64_t>(nx.row) * (nvec * 8));
+        }
+        copies_commit();
+        if ((threadIdx.x & 31) == 0) *rt_issue = nx;
+        t_issue += step;
+        off_issue += step_el;
+        const bool wrap = ++n_issue == S;
+        n_issue = wrap ? 0 : n_issue;
+        dst = wrap ? ring : dst + stage_bytes;
+        rt_issue = wrap ? &sh_rt[0][warp] : rt_issue + 32;
+    };
+#pragma unroll 1
+    for (int i = 0; i < S - 1; ++i) issue();
+    int st = 0, k = 0, buf = 0;
+    const float4* slot = sh_dyn + threadIdx.x;
+    // every row of threads makes the same number of steps (the barriers)
+    for (int64_t tb = static_cast<int64_t>(blockIdx.x) * rows; tb < ntok; tb += step, t += step, off += step_el) {
+        __syncwarp();  // every lane has read the routing slot that is written next
+        issue();
+        copies_wait<S - 1>();
+        __syncwarp();
+        const Routing rt = sh_rt[st][warp];
+        const bool live = me.active && t < ntok;
+        const bool sel = rt.row >= 0;
+        const float pt = rt.p, wl = sel ? 1.0f - pt : 1.0f;
+        const Vec8 g = unpack8(*reinterpret_cast<const uint4*>(slot));
+        float dp = 0.f;
+        {  // dy = dO wl; dx = r gain dy - x r^3 mean(x gain dy); d gain = dy x r
+            const Vec8 x = unpack8(*reinterpret_cast<const uint4*>(slot + nthr));
+            const Vec8 gy = mul8(g, kInRegs ? gl_r : slot_load(sh_gain, nthr, 0, threadIdx.x));
+            const float ss = lane_sum<VPR>(sumsq8(x));
+            const float xd = lane_sum<VPR>(dot8(x, gy));
+            const float r = rsqrtf(ss * (1.0f / D) + eps);
+            if (live) store_bf16x8(dO_l + off, axpby8(gy, r * wl, &x, -(r * r * r * (xd * wl) * (1.0f / D))));
+            if (DGAIN && kInRegs) fma8(sum_l, g, x, live ? wl * r : 0.f);
+            if (DGAIN && !kInRegs && live) {
+                Vec8 a = slot_load(sh_sum, nthr, 0, threadIdx.x);
+                fma8(a, g, x, wl * r);
+                slot_store(sh_sum, nthr, 0, threadIdx.x, a);
+            }
+            dp = -r * xd;  // sum over d of dO o~L: the head's sum
+        }
+        if (sel) {
+            const Vec8 x = unpack8(*reinterpret_cast<const uint4*>(slot + 2 * nthr));
+            const Vec8 gy = mul8(g, kInRegs ? gg_r : slot_load(sh_gain, nthr, 1, threadIdx.x));
+            const float ss = lane_sum<VPR>(sumsq8(x));
+            const float xd = lane_sum<VPR>(dot8(x, gy));
+            const float r = rsqrtf(ss * (1.0f / D) + eps);
+            if (live)
+                store_bf16x8(dc_v + static_cast<int64_t>(rt.row) * (nvec * 8),
+                             axpby8(gy, r * pt, &x, -(r * r * r * (xd * pt) * (1.0f / D))));
+            if (DGAIN && kInRegs) fma8(sum_g, g, x, live ? pt * r : 0.f);
+            if (DGAIN && !kInRegs && live) {
+                Vec8 a = slot_load(sh_sum, nthr, 1, threadIdx.x);
+                fma8(a, g, x, pt * r);
+                slot_store(sh_sum, nthr, 1, threadIdx.x, a);
+            }
+            // dp_t = z_t sum over heads and d of dO (o~G - o~L): one lane a head
+            dp = lane_sum<32>(me.active && me.j0 == 0 ? dp + r * xd : 0.f);
+        }
+        if ((threadIdx.x & 31) == 0) sh_dp[buf][k][warp] = sel ? dp : 0.f;
+        if (++k == kGroup || tb + step >= ntok) {  // (two buffers: one barrier a group is enough)
+            __syncthreads();
+            if (me.v < k) {
+                const int64_t tj = t - (k - 1 - me.v) * step;
+                if (tj < ntok) {
+                    float s = 0.f;
+                    for (int w = 0; w < tpr / 32; ++w) s += sh_dp[buf][me.v][me.row * (tpr / 32) + w];
+                    dgate_p[tj] = s;
+                }
+            }
+            k = 0;
+            buf ^= 1;
+        }
+        const bool wrap = ++st == S;
+        st = wrap ? 0 : st;
+        slot = wrap ? sh_dyn + threadIdx.x : slot + 3 * nthr;
+    }
+    copies_wait<0>();
+    if (DGAIN) {
+        // the block's rows of threads in order, then its partial row
+        if (kInRegs) {
+            __syncthreads();  // the ring is free
+            sh_sum = sh_dyn;
+            slot_store(sh_sum, nthr, 0, threadIdx.x, sum_l);
+            slot_store(sh_sum, nthr, 1, threadIdx.x, sum_g);
+        }
+        __syncthreads();
+        if (me.row == 0 && me.active) {
+            float* pl = part + static_cast<int64_t>(blockIdx.x) * 2 * nvec * 8;
+#pragma unroll
+            for (int br = 0; br < 2; ++br)
+#pragma unroll
+                for (int half = 0; half < 2; ++half) {
+                    float4 a = sh_sum[(br * 2 + half) * nthr + threadIdx.x];
+                    for (int r = 1; r < rows; ++r) {
+                        const float4 b = sh_sum[(br * 2 + half) * nthr + r * tpr + threadIdx.x];
+                        a.x += b.x; a.y += b.y; a.z += b.z; a.w += b.w;
+                    }
+                    *reinterpret_cast<float4*>(pl + static_cast<int64_t>(br) * nvec * 8 + me.v * 8 + half * 4) = a;
+                }
+        }
+    }
+}
+
+// Threads per token row and rows of threads per block of the kernels above.
+struct GainShape {
+    int tpr, rows, threads;
+};
+
+GainShape gain_shape(const logo_dims& d)
+{
+    const int nvec = d.Hq * (d.D / 8);
+    const int tpr = (nvec + 31) / 32 * 32;
+    const int rows = tpr >= kThreads ? 1 : kThreads / tpr;
+    return GainShape{tpr, rows, tpr * rows};
+}
+
 // Vectors per group: two with unit gains when that leaves no thread of the
 // block idle (at least 2 x kThreads vectors per token), else one.
 int group_vectors(const logo_dims& d, bool unit)
@@ -482,27 +878,58 @@ int groups_per_thread(const logo_dims& d, int g)
 }
 
 // One wave of resident blocks (the grid-stride loop gives every block the
-// same number of tokens), capped by the token count.
+// same number of tokens), capped by the steps there are.
 template <typename K>
-int64_t wave_blocks(K kernel, int64_t ntok, size_t smem = 0)
+int64_t wave_blocks(K kernel, int64_t steps, size_t smem = 0, int threads = kThreads)
 {
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kThreads, smem) != cudaSuccess || per_sm < 1)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem) != cudaSuccess || per_sm < 1)
         per_sm = 1;
     const int64_t cap = static_cast<int64_t>(device_sm_count()) * per_sm;
-    return ntok < cap ? ntok : cap;
+    return steps < cap ? steps : cap;
 }
 
-// Dynamic shared memory of the gain-gradient backward: its accumulators.
+// Dynamic shared memory of the unit-gain backward with gain sums: its accumulators.
 size_t gains_smem(const logo_dims& d) { return static_cast<size_t>(4) * (d.Hq * d.D / 8) * sizeof(float4); }
 
 // The gain variant may need more than the default 48 KB of dynamic shared
 // memory (64 KB at Hq*D = 8192); the attribute is set before any occupancy
 // query or launch of it.
 template <typename K>
-bool gains_smem_ok(K kernel)
+bool gains_smem_ok(K kernel, size_t bytes = 4 * kMaxVecGains * sizeof(float4))
 {
-    return set_smem_limit(kernel, 4 * kMaxVecGains * static_cast<int>(sizeof(float4))) == cudaSuccess;
+    return set_smem_limit(kernel, static_cast<int>(bytes)) == cudaSuccess;
+}
+
+// A launch of the gains-read kernels; `slots`: float4 of shared memory per thread.
+struct GainLaunch {
+    GainShape sh;
+    size_t smem;
+    int64_t grid;
+};
+
+template <typename K>
+GainLaunch gain_launch(K kernel, const logo_dims& d, int slots)
+{
+    GainLaunch g{gain_shape(d), 0, 0};
+    g.smem = static_cast<size_t>(slots) * g.sh.threads * sizeof(float4);
+    gains_smem_ok(kernel, g.smem);
+    const int64_t ntok = static_cast<int64_t>(d.B) * d.T;
+    g.grid = wave_blocks(kernel, (ntok + g.sh.rows - 1) / g.sh.rows, g.smem, g.sh.threads);
+    return g;
+}
+
+// Calls f(kernel, float4 slots per thread) with the backward kernel that runs for these sizes.
+template <bool DGAIN, typename F>
+auto with_gained_bwd(const logo_dims& d, F f)
+{
+    constexpr int kSlots = 3 * GainCfg<512>::kRingBwd;
+    constexpr int kSlotsBig = 3 * GainCfg<1024>::kRingBwd + (DGAIN ? 8 : 4);
+    const bool big = gain_shape(d).threads > 512;
+    if (d.D == 128) return big ? f(combine_gained_bwd_kernel<128, 1024, DGAIN>, kSlotsBig)
+                               : f(combine_gained_bwd_kernel<128, 512, DGAIN>, kSlots);
+    return big ? f(combine_gained_bwd_kernel<64, 1024, DGAIN>, kSlotsBig)
+               : f(combine_gained_bwd_kernel<64, 512, DGAIN>, kSlots);
 }
 
 // Blocks of the gain-gradient backward (one partial row each): the larger of
@@ -511,21 +938,9 @@ int64_t gains_blocks(const logo_dims& d)
 {
     const int64_t ntok = static_cast<int64_t>(d.B) * d.T;
     const size_t smem = gains_smem(d);
-    int64_t with_gains = 0, unit = 0;
-    switch (groups_per_thread(d, 1)) {
-        case 1:
-            gains_smem_ok(combine_bwd_kernel<1, 1, true, false>);
-            with_gains = wave_blocks(combine_bwd_kernel<1, 1, true, false>, ntok, smem);
-            break;
-        case 2:
-            gains_smem_ok(combine_bwd_kernel<2, 1, true, false>);
-            with_gains = wave_blocks(combine_bwd_kernel<2, 1, true, false>, ntok, smem);
-            break;
-        default:
-            gains_smem_ok(combine_bwd_kernel<4, 1, true, false>);
-            with_gains = wave_blocks(combine_bwd_kernel<4, 1, true, false>, ntok, smem);
-            break;
-    }
+    const int64_t with_gains =
+        with_gained_bwd<true>(d, [&](auto kernel, int slots) { return gain_launch(kernel, d, slots).grid; });
+    int64_t unit = 0;
     const int gu = group_vectors(d, true), gpt = groups_per_thread(d, gu);
     if (gu == 1) {
         gains_smem_ok(combine_bwd_kernel<1, 1, true, true>);
@@ -585,12 +1000,23 @@ extern "C" int logo_combine(const logo_bf16* o_l, const logo_bf16* o_c, const fl
     } else if (unit) {  // fewer than 2 x kThreads vectors a token
         if (gpt == 1) { LOGO_COMBINE_FWD(1, 1, true); }
         else { LOGO_COMBINE_FWD(2, 1, true); }
+    } else if (dims.Hq * (dims.D / 8) > kMaxVecGains) {  // Hq * D > 8192: more vectors a token than threads
+        LOGO_COMBINE_FWD(8, 1, false);
     } else {
-        switch (gpt) {
-            case 1: LOGO_COMBINE_FWD(1, 1, false); break;
-            case 2: LOGO_COMBINE_FWD(2, 1, false); break;
-            case 4: LOGO_COMBINE_FWD(4, 1, false); break;
-            default: LOGO_COMBINE_FWD(8, 1, false); break;
+        auto run = [&](auto kernel, int slots) {
+            const GainLaunch L = gain_launch(kernel, dims, slots);
+            kernel<<<static_cast<unsigned>(L.grid), L.sh.threads, L.smem, st>>>(o_l, o_c, gate_p, z, row_of, gain_l,
+                                                                               gain_g, eps, o, rstd_l, rstd_g, ntok,
+                                                                               dims.Hq, L.sh.tpr, L.sh.rows);
+        };
+        constexpr int kSlots = 2 * GainCfg<512>::kRingFwd + 4;
+        const bool big = gain_shape(dims).threads > 512;
+        if (dims.D == 128) {
+            if (big) run(combine_gained_fwd_kernel<128, 1024>, kSlots);
+            else run(combine_gained_fwd_kernel<128, 512>, kSlots);
+        } else {
+            if (big) run(combine_gained_fwd_kernel<64, 1024>, kSlots);
+            else run(combine_gained_fwd_kernel<64, 512>, kSlots);
         }
     }
 #undef LOGO_COMBINE_FWD
@@ -633,12 +1059,15 @@ int combine_bwd_common(const logo_bf16* dO, const logo_bf16* o_l, const logo_bf1
         if (g == 1) { LOGO_COMBINE_BWD(1, 1, true, true); }
         else if (gpt == 1) { LOGO_COMBINE_BWD(1, 2, true, true); }
         else { LOGO_COMBINE_BWD(2, 2, true, true); }
-    } else if (gains) {
-        switch (gpt) {
-            case 1: LOGO_COMBINE_BWD(1, 1, true, false); break;
-            case 2: LOGO_COMBINE_BWD(2, 1, true, false); break;
-            default: LOGO_COMBINE_BWD(4, 1, true, false); break;
-        }
+    } else if (!unit && dims.Hq * (dims.D / 8) <= kMaxVecGains) {
+        auto run = [&](auto kernel, int slots) {
+            const GainLaunch L = gain_launch(kernel, dims, slots);
+            kernel<<<static_cast<unsigned>(L.grid), L.sh.threads, L.smem, st>>>(
+                dO, o_l, o_c, gate_p, z, row_of, gain_l, gain_g, eps, dO_l, dO_c, dgate_p, part, ntok, dims.Hq,
+                L.sh.tpr, L.sh.rows);
+            return static_cast<unsigned>(L.grid);
+        };
+        grid = gains ? with_gained_bwd<true>(dims, run) : with_gained_bwd<false>(dims, run);
     } else if (unit && g == 2) {
         switch (gpt) {
             case 1: LOGO_COMBINE_BWD(1, 2, false, true); break;
@@ -648,13 +1077,8 @@ int combine_bwd_common(const logo_bf16* dO, const logo_bf16* o_l, const logo_bf1
     } else if (unit) {  // fewer than 2 x kThreads vectors a token
         if (gpt == 1) { LOGO_COMBINE_BWD(1, 1, false, true); }
         else { LOGO_COMBINE_BWD(2, 1, false, true); }
-    } else {
-        switch (gpt) {
-            case 1: LOGO_COMBINE_BWD(1, 1, false, false); break;
-            case 2: LOGO_COMBINE_BWD(2, 1, false, false); break;
-            case 4: LOGO_COMBINE_BWD(4, 1, false, false); break;
-            default: LOGO_COMBINE_BWD(8, 1, false, false); break;
-        }
+    } else {  // gains read, Hq * D > 8192
+        LOGO_COMBINE_BWD(8, 1, false, false);
     }
 #undef LOGO_COMBINE_BWD
     if (cudaGetLastError() != cudaSuccess) return LOGO_ERR_CUDA;
