@@ -12,7 +12,9 @@
 //                        cu_q[] and the total N.
 //   write_kernel         per chunk: block-wide prefix sums (warp ballots) turn
 //                        the decisions into z, pos and row_of, in ascending t.
-// Ratio mode with 4K < T <= 128K takes one launch instead:
+// Threshold mode on up to 128K tokens of the batch takes one launch instead:
+//   select_threshold_kernel  one block, or one 8-CTA cluster, over all of them.
+// Ratio mode with 4K < T <= 128K takes one launch too:
 //   select_ratio_cluster_kernel  one 8-CTA cluster per sequence; the CTAs share
 //                        their radix histograms and counts through distributed
 //                        shared memory.  Up to 4K, select_ratio_small_kernel
@@ -515,6 +517,95 @@ __global__ void __cluster_dims__(kClusterCTAs, 1, 1) __launch_bounds__(1024)
     cluster.sync();  // no CTA leaves while another may still read its counts
 }
 
+// Threshold mode, B*T <= CTAS * 1024 * KPT: the whole selection in one block
+// (CTAS = 1) or one cluster.  The packed rows are the selected tokens of the
+// flattened [B*T] gates in order, so one scan over all of them serves every
+// sequence: thread i of CTA r owns KPT consecutive tokens, a block scan gives
+// the selected ones before it in its CTA, and the CTAs' totals, exchanged
+// through distributed shared memory, those before its CTA.  cu_q[b] is what
+// the thread that owns sequence b's first token has counted before it.
+// Latency is all of it: the three launches of the chunked path took 29 us for
+// 32 sequences of one token (its scan goes sequence by sequence) and 13 us for
+// 4 x 4096; this kernel 2.7 and 5.4 us (cold).
+template <int CTAS, int KPT>
+__global__ void __launch_bounds__(1024)
+    select_threshold_kernel(const float* __restrict__ p, int B, int T, float b_th_host,
+                            const float* __restrict__ b_th_dev, uint8_t* __restrict__ z, int32_t* __restrict__ pos,
+                            int32_t* __restrict__ cu_q, int32_t* __restrict__ row_of, int32_t* __restrict__ n_total)
+{
+    namespace cg = cooperative_groups;
+    __shared__ int sh_warp[32];
+    __shared__ int sh_total;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int n = B * T;
+    const int rank = CTAS > 1 ? static_cast<int>(blockIdx.x) : 0;
+    const int i0 = (rank * 1024 + static_cast<int>(threadIdx.x)) * KPT;
+    float g[KPT];  // all of a thread's loads in flight at once
+#pragma unroll
+    for (int u = 0; u < KPT; ++u) g[u] = i0 + u < n ? p[i0 + u] : 0.f;
+    const float b_th = b_th_dev ? *b_th_dev : b_th_host;
+    uint32_t sel = 0;
+#pragma unroll
+    for (int u = 0; u < KPT; ++u) sel |= (i0 + u < n && g[u] > b_th) ? 1u << u : 0u;  // Eq. 7, strict
+    const int mine = __popc(sel);
+    int x = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) sh_warp[warp] = x;
+    __syncthreads();
+    if (warp == 0) {
+        const int w0 = sh_warp[lane];
+        int w = w0;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, w, o);
+            if (lane >= o) w += y;
+        }
+        sh_warp[lane] = w - w0;  // exclusive over warps
+        if (lane == 31) sh_total = w;
+    }
+    __syncthreads();
+    int row = sh_warp[warp] + x - mine, total = sh_total;
+    if constexpr (CTAS > 1) {
+        cg::cluster_group cluster = cg::this_cluster();
+        cluster.sync();  // every CTA's total is published
+        total = 0;
+        int before = 0;
+#pragma unroll
+        for (int r = 0; r < CTAS; ++r) {
+            const int v = *cluster.map_shared_rank(&sh_total, r);
+            before += r < rank ? v : 0;
+            total += v;
+        }
+        row += before;
+        cluster.sync();  // no CTA leaves while another may still read its total
+    }
+    if (i0 < n) {
+        int b = i0 / T, t = i0 - b * T;
+#pragma unroll
+        for (int u = 0; u < KPT; ++u) {
+            if (i0 + u < n) {
+                const bool s = sel >> u & 1u;
+                if (t == 0) cu_q[b] = row;
+                z[i0 + u] = s ? 1 : 0;
+                row_of[i0 + u] = s ? row : -1;
+                if (s) pos[row++] = t;
+                if (++t == T) {
+                    t = 0;
+                    ++b;
+                }
+            }
+        }
+    }
+    if (rank == 0 && threadIdx.x == 0) {
+        cu_q[B] = total;
+        *n_total = total;
+    }
+}
+
 struct ChunkCounts {
     int gt;   // tokens selected outright in the chunk
     int eq;   // tokens tied with the threshold key (ratio mode)
@@ -576,16 +667,35 @@ __global__ void __launch_bounds__(kThreads) scan_kernel(const ChunkCounts* __res
 {
     __shared__ int sh_warp[kThreads / 32];
     int carry = 0;
+    if (!ratio_mode) {  // no ties: one scan over the chunks of every sequence
+        const int64_t total = static_cast<int64_t>(B) * nchunk;
+        for (int64_t c0 = 0; c0 < total; c0 += kThreads) {
+            const int64_t c = c0 + threadIdx.x;
+            const int gt = c < total ? counts[c].gt : 0;
+            int sum;
+            const int base = carry + block_excl_scan(gt, &sum, sh_warp);
+            if (c < total) {
+                plan[c] = ChunkPlan{base, 0};
+                if (c % nchunk == 0) cu_q[c / nchunk] = base;
+            }
+            carry += sum;
+        }
+        if (threadIdx.x == 0) {
+            cu_q[B] = carry;
+            *n_total = carry;
+        }
+        return;
+    }
     for (int b = 0; b < B; ++b) {
         if (threadIdx.x == 0) cu_q[b] = carry;
-        const int need = ratio_mode ? th[b].need_eq : 0;
+        const int need = th[b].need_eq;
         int eq_carry = 0;
         for (int c0 = 0; c0 < nchunk; c0 += kThreads) {
             const int c = c0 + threadIdx.x;
             ChunkCounts cc = (c < nchunk) ? counts[static_cast<int64_t>(b) * nchunk + c] : ChunkCounts{0, 0};
             int eq_tot;
             int eq_before = eq_carry + block_excl_scan(cc.eq, &eq_tot, sh_warp);
-            int take_eq = ratio_mode ? max(0, min(cc.eq, need - eq_before)) : 0;
+            int take_eq = max(0, min(cc.eq, need - eq_before));
             int sel = cc.gt + take_eq;
             int sel_tot;
             int base = carry + block_excl_scan(sel, &sel_tot, sh_warp);
@@ -656,6 +766,48 @@ struct SelectWs {
     ChunkPlan* plan;
 };
 
+template <int CTAS, int KPT>
+cudaError_t launch_threshold(const float* p, const logo_dims& d, float b_th, const float* b_th_dev, uint8_t* z,
+                             int32_t* pos, int32_t* cu_q, int32_t* row_of, int32_t* n_sel, cudaStream_t st)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(CTAS);
+    cfg.blockDim = dim3(1024);
+    cfg.stream = st;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = CTAS;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = CTAS > 1 ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, select_threshold_kernel<CTAS, KPT>, p, d.B, d.T, b_th, b_th_dev, z, pos, cu_q,
+                              row_of, n_sel);
+}
+
+// Threshold mode: one launch up to 128K tokens, else counts, scan, write.  Up
+// to 4K tokens one block is enough (four loads a thread); above, the cluster's
+// eight SMs share the loads and stores.
+int select_threshold(const float* p, const logo_dims& d, float b_th, const float* b_th_dev, uint8_t* z, int32_t* pos,
+                     int32_t* cu_q, int32_t* row_of, int32_t* n_sel, const SelectWs& ws, cudaStream_t st)
+{
+    const int64_t n = static_cast<int64_t>(d.B) * d.T;
+    cudaError_t e = cudaSuccess;
+    if (n <= 1024) e = launch_threshold<1, 1>(p, d, b_th, b_th_dev, z, pos, cu_q, row_of, n_sel, st);
+    else if (n <= 4 * 1024) e = launch_threshold<1, 4>(p, d, b_th, b_th_dev, z, pos, cu_q, row_of, n_sel, st);
+    else if (n <= 16 * 1024) e = launch_threshold<8, 2>(p, d, b_th, b_th_dev, z, pos, cu_q, row_of, n_sel, st);
+    else if (n <= 32 * 1024) e = launch_threshold<8, 4>(p, d, b_th, b_th_dev, z, pos, cu_q, row_of, n_sel, st);
+    else if (n <= 128 * 1024) e = launch_threshold<8, 16>(p, d, b_th, b_th_dev, z, pos, cu_q, row_of, n_sel, st);
+    else {
+        const int nchunk = (d.T + kChunk - 1) / kChunk;
+        const dim3 grid(nchunk, d.B);
+        count_kernel<<<grid, kThreads, 0, st>>>(p, d.T, nchunk, 0, b_th, b_th_dev, ws.th, ws.counts);
+        scan_kernel<<<1, kThreads, 0, st>>>(ws.counts, d.B, nchunk, 0, ws.th, ws.plan, cu_q, n_sel);
+        write_kernel<<<grid, kThreads, 0, st>>>(p, d.T, nchunk, 0, b_th, b_th_dev, ws.th, ws.plan, z, pos, row_of);
+        e = cudaGetLastError();
+    }
+    return e == cudaSuccess ? LOGO_OK : LOGO_ERR_CUDA;
+}
+
 size_t select_ws_layout(const logo_dims& d, char* base, SelectWs* ws)
 {
     const size_t nchunk = (static_cast<size_t>(d.T) + kChunk - 1) / kChunk;
@@ -703,10 +855,11 @@ extern "C" int logo_select(const float* gate_p, logo_dims dims, int mode, float 
     SelectWs ws;
     select_ws_layout(dims, static_cast<char*>(workspace), &ws);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    if (!ratio_mode) return select_threshold(gate_p, dims, b_th, nullptr, z, pos, cu_q, row_of, n_sel_total, ws, st);
     const int nchunk = (dims.T + kChunk - 1) / kChunk;
     // k = floor(rho * T), with rho read as float32 and the product in double
-    const int k = ratio_mode ? static_cast<int>(static_cast<double>(ratio) * dims.T) : 0;
-    if (ratio_mode && dims.T <= 4 * 1024) {  // one launch: one block per sequence
+    const int k = static_cast<int>(static_cast<double>(ratio) * dims.T);
+    if (dims.T <= 4 * 1024) {  // one launch: one block per sequence
         const int smem =
             static_cast<int>(round_up((static_cast<size_t>(dims.T) + dims.T / 16 + 1 + dims.T) * 4 + dims.T, 16));
         if (set_smem_limit(select_ratio_small_kernel<4>, smem) != cudaSuccess) return LOGO_ERR_CUDA;
@@ -714,7 +867,7 @@ extern "C" int logo_select(const float* gate_p, logo_dims dims, int mode, float 
                                                                  n_sel_total);
         return cudaGetLastError() == cudaSuccess ? LOGO_OK : LOGO_ERR_CUDA;
     }
-    if (ratio_mode && dims.T <= kClusterCTAs * 1024 * 16) {  // one launch: one 8-CTA cluster per sequence
+    if (dims.T <= kClusterCTAs * 1024 * 16) {  // one launch: one 8-CTA cluster per sequence
         const dim3 grid(dims.B * kClusterCTAs);
         const int per_cta = (dims.T + kClusterCTAs - 1) / kClusterCTAs;
         if (per_cta <= 2 * 1024)
@@ -731,12 +884,11 @@ extern "C" int logo_select(const float* gate_p, logo_dims dims, int mode, float 
                                                                    n_sel_total);
         return cudaGetLastError() == cudaSuccess ? LOGO_OK : LOGO_ERR_CUDA;
     }
-    if (ratio_mode) radix_select_kernel<<<dims.B, 1024, 0, st>>>(gate_p, dims.T, k, ws.th);
+    radix_select_kernel<<<dims.B, 1024, 0, st>>>(gate_p, dims.T, k, ws.th);
     dim3 grid(nchunk, dims.B);
-    count_kernel<<<grid, kThreads, 0, st>>>(gate_p, dims.T, nchunk, ratio_mode, b_th, nullptr, ws.th, ws.counts);
-    scan_kernel<<<1, kThreads, 0, st>>>(ws.counts, dims.B, nchunk, ratio_mode, ws.th, ws.plan, cu_q, n_sel_total);
-    write_kernel<<<grid, kThreads, 0, st>>>(gate_p, dims.T, nchunk, ratio_mode, b_th, nullptr, ws.th, ws.plan, z, pos,
-                                            row_of);
+    count_kernel<<<grid, kThreads, 0, st>>>(gate_p, dims.T, nchunk, 1, b_th, nullptr, ws.th, ws.counts);
+    scan_kernel<<<1, kThreads, 0, st>>>(ws.counts, dims.B, nchunk, 1, ws.th, ws.plan, cu_q, n_sel_total);
+    write_kernel<<<grid, kThreads, 0, st>>>(gate_p, dims.T, nchunk, 1, b_th, nullptr, ws.th, ws.plan, z, pos, row_of);
     return cudaGetLastError() == cudaSuccess ? LOGO_OK : LOGO_ERR_CUDA;
 }
 
@@ -755,12 +907,7 @@ extern "C" int logo_select_device_threshold(const float* gate_p, logo_dims dims,
     SelectWs ws;
     select_ws_layout(dims, static_cast<char*>(workspace), &ws);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const int nchunk = (dims.T + kChunk - 1) / kChunk;
-    dim3 grid(nchunk, dims.B);
-    count_kernel<<<grid, kThreads, 0, st>>>(gate_p, dims.T, nchunk, 0, 0.0f, b_th, ws.th, ws.counts);
-    scan_kernel<<<1, kThreads, 0, st>>>(ws.counts, dims.B, nchunk, 0, ws.th, ws.plan, cu_q, n_sel_total);
-    write_kernel<<<grid, kThreads, 0, st>>>(gate_p, dims.T, nchunk, 0, 0.0f, b_th, ws.th, ws.plan, z, pos, row_of);
-    return cudaGetLastError() == cudaSuccess ? LOGO_OK : LOGO_ERR_CUDA;
+    return select_threshold(gate_p, dims, 0.0f, b_th, z, pos, cu_q, row_of, n_sel_total, ws, st);
 }
 
 // ---------------------------------------------------------------------------
@@ -848,13 +995,13 @@ extern "C" int logo_select_noalloc(const float* gate_p, logo_dims dims, int mode
     SelectWs ws;
     select_ws_layout(dims, scratch, &ws);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    if (!ratio_mode) return select_threshold(gate_p, dims, b_th, nullptr, z, pos, cu_q, row_of, n_sel_total, ws, st);
     const int nchunk = static_cast<int>(nchunk64);
-    const int k = ratio_mode ? static_cast<int>(static_cast<double>(ratio) * dims.T) : 0;
-    if (ratio_mode) radix_select_kernel<<<dims.B, 1024, 0, st>>>(gate_p, dims.T, k, ws.th);
+    const int k = static_cast<int>(static_cast<double>(ratio) * dims.T);
+    radix_select_kernel<<<dims.B, 1024, 0, st>>>(gate_p, dims.T, k, ws.th);
     dim3 grid(nchunk, dims.B);
-    count_kernel<<<grid, kThreads, 0, st>>>(gate_p, dims.T, nchunk, ratio_mode, b_th, nullptr, ws.th, ws.counts);
-    scan_kernel<<<1, kThreads, 0, st>>>(ws.counts, dims.B, nchunk, ratio_mode, ws.th, ws.plan, cu_q, n_sel_total);
-    write_kernel<<<grid, kThreads, 0, st>>>(gate_p, dims.T, nchunk, ratio_mode, b_th, nullptr, ws.th, ws.plan, z, pos,
-                                            row_of);
+    count_kernel<<<grid, kThreads, 0, st>>>(gate_p, dims.T, nchunk, 1, b_th, nullptr, ws.th, ws.counts);
+    scan_kernel<<<1, kThreads, 0, st>>>(ws.counts, dims.B, nchunk, 1, ws.th, ws.plan, cu_q, n_sel_total);
+    write_kernel<<<grid, kThreads, 0, st>>>(gate_p, dims.T, nchunk, 1, b_th, nullptr, ws.th, ws.plan, z, pos, row_of);
     return cudaGetLastError() == cudaSuccess ? LOGO_OK : LOGO_ERR_CUDA;
 }
