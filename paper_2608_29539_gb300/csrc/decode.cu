@@ -9,26 +9,30 @@
 //   logo_decode_global_sparse_attn  only the packed selected rows attend their
 //                                   sequence's whole dense cache (Eq. 8)
 //
-// Both run one persistent kernel per call.  An item is one chunk of cache
-// rows (up to kDecSubMax sub-tiles of 64 rows) of one (row, KV head); a CTA
-// (4 warps) walks its items' sub-tiles through a 3-stage TMA ring (128-byte
+// Both run one persistent kernel per call.  The work is the sub-tiles (64
+// cache rows) of every (sequence, KV head) pair of the call, in order, and
+// each CTA takes an equal run of them, wherever pairs begin and end: sequences
+// differ in length and pairs seldom divide by the CTAs (chunks of 1024 rows
+// handed out one by one: 4 of 32 sequences of 8K to 16K rows selected 58 us,
+// now 49; all 32 selected 360 us, now 252, 6.5 TB/s).  Where that saves little
+// (many pairs of equal length, as the rings are) a CTA takes whole pairs.
+// A CTA (4 warps) walks its run through a 3-stage TMA ring (128-byte
 // swizzle), a stage refilled once all four warps have released it, and
 // serves every query head of the KV head's group from each: S = q.K^T and
 // O = P.V as warp-level bf16 products (mma.sync m16n8k16: the group's heads
 // are the 16 rows, so a group of up to 16 heads fills one tile).  Each warp
 // takes 16 rows of every sub-tile and keeps its own online softmax (running
-// max and sum per head, in log2 units) across the item's sub-tiles, P going
+// max and sum per head, in log2 units) across the piece's sub-tiles, P going
 // from the S fragments straight into the A fragments of the P.V product, so
 // nothing inside the sub-tile loop waits for another warp; the four warps'
-// results are combined exactly at the end of the item.
-// A row whose cache fits one chunk gets its output written by that item.
-// Longer caches are split into chunks for parallelism: each chunk leaves its
-// unnormalised O, max and sum, and the last chunk of a (row, KV head) to
+// results are combined exactly at the end of the piece.
+// A pair that lies whole inside one CTA's run gets its output written by that
+// CTA.  The pieces of the others (at most two a CTA: one at either end of its
+// run) leave their unnormalised O, max and sum, and the last piece of a pair to
 // finish (a counter per pair, cleared by the call) combines them exactly.
 // Decoding is bound by HBM: every cache byte serves only the group's heads.
-// In the global call the items of rows past the device-side count of
-// selected rows are never visited, so unselected sequences cost no cache
-// traffic and no host synchronisation is needed.
+// In the global call unselected sequences have no sub-tiles, so they cost no
+// cache traffic and no host synchronisation is needed.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -46,7 +50,8 @@ constexpr int kDecThreads = 128;  // 4 warps
 constexpr int kDecRows = 64;      // cache rows per sub-tile, 16 per warp
 constexpr int kDecRowsPerWarp = kDecRows / 4;
 constexpr int kDecMaxGroup = 16;  // query heads per KV head (the mma tile's 16 rows)
-constexpr int kDecSubMax = 16;    // sub-tiles per chunk preferred at most (1024 cache rows): the merge walks a row's chunks serially
+constexpr int kDecMinSub = 2;     // sub-tiles of a CTA's run at least
+constexpr int kDecSplitCost = 4;  // what cutting pairs into pieces has to save, in sub-tiles
 constexpr int kDecStages = 3;     // TMA ring depth
 
 struct DecParams {
@@ -56,10 +61,11 @@ struct DecParams {
     const int32_t* seq_len;   // [B] tokens in the cache, the new one included
     const int32_t* cu_q;      // global: [B+1] packed rows of the (B, 1) selection
     const int32_t* n_sel;     // global: [1]
-    float* part;              // [rows, Hq, nchunk, D + 2]: unnormalised o, then m, l (nchunk > 1)
-    int32_t* done;            // [rows, Hkv] chunks finished (nchunk > 1; cleared by the call)
+    float* part;              // [2 CTAs, group, D]: unnormalised o of a CTA's pieces of shared pairs
+    float2* part_ml;          // [2 CTAs, group]: their running max (log2 units) and sum
+    int32_t* done;            // [B, Hkv] pieces finished (cleared by the call); NULL: whole pairs only
     logo_bf16* out;           // [B, Hq, D] (global: packed rows)
-    int B, R, Hq, Hkv, window, nchunk, sub_per_chunk;
+    int B, R, Hq, Hkv, window, min_sub;
     float scale_log2;
 };
 
@@ -68,48 +74,86 @@ struct DecCfg {
     static constexpr int kHalfBytes = kDecRows * 128;         // 64 head-dim columns of the sub-tile's rows
     static constexpr int kTileBytes = (D / 64) * kHalfBytes;  // K or V sub-tile
     static constexpr int kStageBytes = 2 * kTileBytes;        // K then V
-    static constexpr int kOffW = kDecStages * kStageBytes;    // chunk-merge weights [group][chunks] fp32
+    static constexpr int kOffW = kDecStages * kStageBytes;    // merge weights [group][pieces] fp32
     static constexpr int kOffM = kOffW + 16 * 64 * 4;         // the warps' partial results, sized per group:
     // [warp][group][D + 2] fp32: unnormalised o, then m, l
     static constexpr int merge_bytes(int group) { return 4 * group * (D + 2) * 4; }
     static constexpr int smem_bytes(int group) { return kOffM + merge_bytes(group) + 1024; }
 };
-constexpr int kDecMaxChunks = 64;  // chunks per cache at most (the merge's weights: group x chunks <= 16 x 64)
+constexpr int kDecMaxPieces = 64;  // pieces of a pair at most (the merge's weights: group x pieces <= 16 x 64)
 
-// Row j of the cache holds position pos_of(j) (or none: -1).  Dense cache:
-// j itself while j < len (len <= R).  Ring of R slots: the latest position
-// congruent to j modulo R that is in the cache; a last sub-tile may reach past
-// the ring's R slots, and those rows hold nothing.
+// Which rows of a cache the new token sees.  Dense cache: rows below its
+// length.  Ring of R slots: position s sits in slot s mod R, so slot j holds
+// the position `age` before the newest (slot `newest`), and is seen while age
+// is below the window; slots past the ring's end (a last sub-tile may reach
+// there) hold nothing.
 template <bool RING>
-__device__ __forceinline__ int pos_of(int j, int len, int R)
-{
-    if (j >= len || (RING && j >= R)) return -1;
-    return RING ? j + R * ((len - 1 - j) / R) : j;
-}
+struct DecVisible {
+    int used, newest, R, window;
 
-// One item's place in the call: row r (sequence b), KV head, chunk c; its
-// sub-tiles [s0, s1) of the cache (empty when the chunk lies past the rows used).
-struct DecItem {
-    int r, b, kvh, c, len, s0, s1, nused;  // nused: chunks of the row holding cache rows
+    __device__ __forceinline__ DecVisible(int len, int R_, int window_)
+        : used(max(0, min(len, R_))), newest(RING ? (len - 1) % R_ : 0), R(R_), window(window_)
+    {
+    }
+    __device__ __forceinline__ bool row(int j) const
+    {
+        return j < used && (!RING || newest - j + (j > newest ? R : 0) < window);
+    }
+    __device__ __forceinline__ bool all16(int j) const  // rows j .. j + 15
+    {
+        return j + 16 <= used && (!RING || window >= used);
+    }
 };
 
+// Sub-tiles of sequence b's cache that the call reads (per KV head): its rows
+// in use; none for a sequence the global call does not have.
 template <bool RING>
-__device__ __forceinline__ DecItem dec_item(const DecParams& p, long long w)
+__device__ __forceinline__ int dec_subs(const DecParams& p, int b, int* len)
 {
-    DecItem it;
-    it.c = static_cast<int>(w % p.nchunk);
-    const long long t = w / p.nchunk;
-    it.kvh = static_cast<int>(t % p.Hkv);
-    it.r = static_cast<int>(t / p.Hkv);
-    it.b = RING ? it.r : seq_of_row(p.cu_q, p.B, it.r);
-    it.len = RING ? p.seq_len[it.b] : min(p.seq_len[it.b], p.R);  // a dense cache holds at most R tokens
-    const int rows_used = max(0, min(it.len, p.R));
-    const int subs = (rows_used + kDecRows - 1) / kDecRows;
-    it.nused = (subs + p.sub_per_chunk - 1) / p.sub_per_chunk;
-    it.s0 = it.c * p.sub_per_chunk;
-    it.s1 = min(subs, it.s0 + p.sub_per_chunk);
-    if (it.len < 1 || it.s0 >= it.s1) it.s1 = it.s0;  // nothing to do
-    return it;
+    int n = p.seq_len[b];
+    if (!RING) {
+        n = min(n, p.R);  // a dense cache holds at most R tokens
+        if (p.cu_q[b + 1] == p.cu_q[b]) n = 0;
+    }
+    *len = n;
+    return (max(0, min(n, p.R)) + kDecRows - 1) / kDecRows;
+}
+
+// A piece of a CTA's run: sub-tiles s .. s1 - 1 (s = s1: none, the run is
+// over) of pair (b, kvh), which has `subs` of them, the first at index pair0 of
+// the call's sequence; `left`: the run's sub-tiles after the piece.
+struct DecPiece {
+    int b, kvh, s, s1, subs, len, left, pair;
+    long long pair0;
+};
+
+// The next piece: of the next pair in order, or (whole pairs) of the pair a
+// grid further on.
+template <bool RING>
+__device__ __forceinline__ void dec_next_piece(const DecParams& p, DecPiece& c)
+{
+    c.pair0 += c.subs;
+    c.s = c.s1 = 0;
+    if (!p.done) {
+        c.subs = 0;
+        while (c.subs == 0) {
+            c.pair += gridDim.x;
+            if (c.pair >= p.B * p.Hkv) return;
+            c.b = c.pair / p.Hkv;
+            c.kvh = c.pair - c.b * p.Hkv;
+            c.subs = dec_subs<RING>(p, c.b, &c.len);
+        }
+        c.s1 = c.subs;
+        return;
+    }
+    if (c.left == 0) return;
+    if (++c.kvh == p.Hkv) {
+        c.kvh = 0;
+        c.subs = 0;
+        while (c.subs == 0 && ++c.b < p.B) c.subs = dec_subs<RING>(p, c.b, &c.len);
+    }
+    c.s1 = min(c.subs, c.left);
+    c.left -= c.s1;
 }
 
 template <int D, bool RING>
@@ -131,9 +175,8 @@ __global__ void __launch_bounds__(kDecThreads, 2) decode_attn_kernel(const __gri
     float* sW = reinterpret_cast<float*>(smem + C::kOffW);
     float* sM = reinterpret_cast<float*>(smem + C::kOffM);
     const uint32_t sRing = smem_u32(smem);
-    // rows of the call: every sequence (local), the selected packed rows (global)
-    const int n_rows = RING ? p.B : *p.n_sel;
-    const long long n_items = static_cast<long long>(n_rows) * p.Hkv * p.nchunk;
+    __shared__ long long sh_scan[4];
+    __shared__ DecPiece sh_start;
     if (tid == 0) {
         abort_flag = 0;
         for (int s = 0; s < kDecStages; ++s) {
@@ -141,31 +184,82 @@ __global__ void __launch_bounds__(kDecThreads, 2) decode_attn_kernel(const __gri
             mbar_init(smem_u32(&bar_empty[s]), 4);
         }
         fence_mbar_init();
+        tma_prefetch_desc(&p.tm_k);
+        tma_prefetch_desc(&p.tm_v);
     }
-    __syncthreads();
-
-    // ---- the producer (thread 0) walks the same sequence of sub-tiles as the
-    //      consumers, up to kDecStages ahead: (item w, sub-tile s) in order; a
-    //      stage is refilled once every warp has released it
-    long long pw = blockIdx.x;
-    int ps = 0, ps1 = 0;
-    auto producer_next = [&](DecItem* it_out) -> bool {  // the next sub-tile to load, or false
-        while (ps >= ps1) {
-            if (pw >= n_items) return false;
-            const DecItem it = dec_item<RING>(p, pw);
-            pw += gridDim.x;
-            ps = it.s0;
-            ps1 = it.s1;
-            *it_out = it;
-        }
-        return true;
+    DecPiece cur{};
+    long long S = 0, G = 0;
+    // a b / c; in 32 bits (a tenth of the instructions) for up to 1M sub-tiles: G < 2^11
+    auto muldiv = [&](long long a, long long b, long long c) -> long long {
+        if (S < (1 << 20)) return static_cast<uint32_t>(a * b) / static_cast<uint32_t>(c);
+        return a * b / c;
     };
-    DecItem pit{};
+    if (!p.done) {  // whole pairs, a grid apart
+        __syncthreads();
+        cur.pair = static_cast<int>(blockIdx.x) - static_cast<int>(gridDim.x);
+        dec_next_piece<RING>(p, cur);
+    } else {
+        // this CTA's run [lo, hi) of the call's S sub-tiles: the total first,
+        // then the pair that holds sub-tile lo
+        int len0 = 0;
+        const int subs0 = tid < p.B ? dec_subs<RING>(p, tid, &len0) : 0;  // of sequence tid, for both passes
+        long long mine = subs0;
+        int len;
+        for (int b = tid + kDecThreads; b < p.B; b += kDecThreads) mine += dec_subs<RING>(p, b, &len);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) mine += __shfl_xor_sync(0xffffffffu, mine, o);
+        if (lane == 0) sh_scan[warp] = mine;
+        __syncthreads();
+        S = (sh_scan[0] + sh_scan[1] + sh_scan[2] + sh_scan[3]) * p.Hkv;
+        __syncthreads();
+        G = max(1ll, min(static_cast<long long>(gridDim.x), S / p.min_sub));
+        if (blockIdx.x >= G || S == 0) return;
+        const long long lo = muldiv(S, blockIdx.x, G), hi = muldiv(S, blockIdx.x + 1, G);
+        long long carry = 0;
+        for (int b0 = 0; b0 < p.B; b0 += kDecThreads) {  // (one round for up to 128 sequences)
+            const int b = b0 + tid;
+            int n = len0;
+            const int subs = b0 == 0 ? subs0 : (b < p.B ? dec_subs<RING>(p, b, &n) : 0);
+            long long x = static_cast<long long>(subs) * p.Hkv;
+            const long long v = x;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const long long y = __shfl_up_sync(0xffffffffu, x, o);
+                if (lane >= o) x += y;
+            }
+            if (lane == 31) sh_scan[warp] = x;
+            __syncthreads();
+            long long base = carry;
+            for (int w = 0; w < warp; ++w) base += sh_scan[w];
+            const long long first = base + x - v;  // b's first sub-tile
+            if (subs > 0 && lo >= first && lo < first + v) {
+                DecPiece c{};
+                c.b = b;
+                c.subs = subs;
+                c.len = n;
+                c.kvh = static_cast<int>(lo - first) / subs;
+                c.pair0 = first + static_cast<long long>(c.kvh) * subs;
+                c.s = static_cast<int>(lo - c.pair0);
+                c.s1 = static_cast<int>(min(static_cast<long long>(subs), c.s + hi - lo));
+                c.left = static_cast<int>(hi - lo) - (c.s1 - c.s);
+                sh_start = c;
+            }
+            carry += sh_scan[0] + sh_scan[1] + sh_scan[2] + sh_scan[3];
+            __syncthreads();
+            if (carry > lo) break;
+        }
+        cur = sh_start;
+    }
+    // the CTA whose run holds sub-tile x
+    auto cta_of = [&](long long x) { return static_cast<int>(muldiv((x + 1) * G - 1, 1, S)); };
+
+    // ---- the producer (thread 0) walks the same run as the consumers, up to
+    //      kDecStages ahead; a stage is refilled once every warp has released it
+    DecPiece pit = cur;
     int issued = 0;
     bool ok = true;
     auto issue = [&]() {
-        if (tid != 0 || !ok) return;
-        if (!producer_next(&pit)) return;
+        if (tid != 0 || !ok || pit.s == pit.s1) return;
         const int st = issued % kDecStages;
         if (!(ok = mbar_wait(smem_u32(&bar_empty[st]), ((issued / kDecStages) & 1) ^ 1, &abort_flag))) return;
         const uint32_t bar = smem_u32(&bar_full[st]);
@@ -173,27 +267,28 @@ __global__ void __launch_bounds__(kDecThreads, 2) decode_attn_kernel(const __gri
         const uint64_t pol = policy_evict_first();
         mbar_arrive_expect_tx(bar, C::kStageBytes);
         for (int h = 0; h < D / 64; ++h) {
-            tma_load_4d(base + h * C::kHalfBytes, &p.tm_k, bar, 64 * h, pit.kvh, ps * kDecRows, pit.b, pol);
-            tma_load_4d(base + C::kTileBytes + h * C::kHalfBytes, &p.tm_v, bar, 64 * h, pit.kvh, ps * kDecRows, pit.b,
-                        pol);
+            tma_load_4d(base + h * C::kHalfBytes, &p.tm_k, bar, 64 * h, pit.kvh, pit.s * kDecRows, pit.b, pol);
+            tma_load_4d(base + C::kTileBytes + h * C::kHalfBytes, &p.tm_v, bar, 64 * h, pit.kvh, pit.s * kDecRows,
+                        pit.b, pol);
         }
-        ++ps;
         ++issued;
+        if (++pit.s == pit.s1) dec_next_piece<RING>(p, pit);
     };
     for (int i = 0; i < kDecStages - 1; ++i) issue();
 
     // Each warp takes 16 rows of every sub-tile (rows 16w..16w+15) and keeps an
-    // online softmax of its own across the item's sub-tiles, so no instruction
+    // online softmax of its own across the piece's sub-tiles, so no instruction
     // inside the sub-tile loop waits for another warp: S = q.K^T lands in mma
     // fragments, P = 2^(S - m) goes from those straight into the A fragments
     // of O += P.V (a pair of 8-column S tiles is one 16-deep A fragment), and
     // the four warps' results are combined once per item.
     constexpr int NT = D / 8;
     int consumed = 0;
-    for (long long w = blockIdx.x; w < n_items && ok; w += gridDim.x) {
-        const DecItem it = dec_item<RING>(p, w);
-        if (it.s0 >= it.s1) continue;
+    for (; cur.s < cur.s1 && ok; dec_next_piece<RING>(p, cur)) {
+        const DecPiece it = cur;
         const int h0 = it.kvh * group;
+        const int out_row = RING ? it.b : p.cu_q[it.b];
+        const DecVisible<RING> sees(it.len, p.R, p.window);
         // the group's queries as mma A fragments (rows = heads, zero past the group)
         uint32_t qa[D / 16][4];
         {
@@ -217,19 +312,18 @@ __global__ void __launch_bounds__(kDecThreads, 2) decode_attn_kernel(const __gri
 #pragma unroll
             for (int i = 0; i < 4; ++i) oc[nt][i] = 0.f;
 
-        for (int s = it.s0; s < it.s1; ++s, ++consumed) {
+        for (int s = it.s; s < it.s1; ++s, ++consumed) {
             issue();
             const int st = consumed % kDecStages;
             const uint32_t sK = sRing + st * C::kStageBytes, sV = sK + C::kTileBytes;
             ok = mbar_wait(smem_u32(&bar_full[st]), (consumed / kDecStages) & 1, &abort_flag) && ok;
             if (!(ok = __all_sync(0xffffffffu, ok))) break;  // the warp leaves together (mma.sync needs all lanes)
             const int j0 = s * kDecRows + warp * kDecRowsPerWarp;  // this warp's first cache row
-            if (lane < kDecRowsPerWarp) {
-                // a cache row the token does not see may hold anything, NaN included:
-                // zero its V so that P = 0 keeps it out of the product
-                const int spos = pos_of<RING>(j0 + lane, it.len, p.R);
-                const bool vis = spos >= 0 && (!RING || spos > it.len - 1 - p.window);
-                if (!vis) {
+            const bool open = sees.all16(j0);
+            if (!open) {
+                if (lane < kDecRowsPerWarp && !sees.row(j0 + lane)) {
+                    // a cache row the token does not see may hold anything, NaN included:
+                    // zero its V so that P = 0 keeps it out of the product
                     const int row = warp * kDecRowsPerWarp + lane;
 #pragma unroll
                     for (int half = 0; half < D / 64; ++half)
@@ -237,8 +331,8 @@ __global__ void __launch_bounds__(kDecThreads, 2) decode_attn_kernel(const __gri
                         for (int ch = 0; ch < 8; ++ch)
                             st_shared_v4(sV + half * C::kHalfBytes + sw128_offset(row, ch), 0u, 0u, 0u, 0u);
                 }
+                __syncwarp();
             }
-            __syncwarp();
             // ---- S = q.K^T over the warp's 16 rows (two 8-row tiles)
             float sc[2][4];
 #pragma unroll
@@ -261,9 +355,8 @@ __global__ void __launch_bounds__(kDecThreads, 2) decode_attn_kernel(const __gri
             for (int nt = 0; nt < 2; ++nt) {
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
-                    const int spos = pos_of<RING>(j0 + nt * 8 + 2 * tig + (i & 1), it.len, p.R);
-                    const bool vis = spos >= 0 && (!RING || spos > it.len - 1 - p.window);
-                    sc[nt][i] = vis ? sc[nt][i] * p.scale_log2 : -INFINITY;
+                    sc[nt][i] *= p.scale_log2;
+                    if (!open && !sees.row(j0 + nt * 8 + 2 * tig + (i & 1))) sc[nt][i] = -INFINITY;
                     mx[i >> 1] = fmaxf(mx[i >> 1], sc[nt][i]);
                 }
             }
@@ -364,7 +457,7 @@ __global__ void __launch_bounds__(kDecThreads, 2) decode_attn_kernel(const __gri
             sh_L[tid] = L;
         }
         __syncthreads();
-        if (it.nused == 1) {  // the whole cache in this item: normalise and write the output
+        if (it.s == 0 && it.s1 == it.subs) {  // the whole pair: normalise and write the output
             for (int i = tid; i < group * D; i += kDecThreads) {
                 const int hh = i / D, d = i % D;
                 float acc = 0.f;
@@ -372,93 +465,104 @@ __global__ void __launch_bounds__(kDecThreads, 2) decode_attn_kernel(const __gri
                 for (int wv = 0; wv < 4; ++wv) acc += sh_wm[wv][hh] * sM[(wv * group + hh) * (D + 2) + d];
                 const float L = sh_L[hh];
                 const __nv_bfloat16 bv = __float2bfloat16_rn(L > 0.f ? acc / L : 0.f);
-                p.out[(static_cast<int64_t>(it.r) * p.Hq + h0 + hh) * D + d] = *reinterpret_cast<const logo_bf16*>(&bv);
+                p.out[(static_cast<int64_t>(out_row) * p.Hq + h0 + hh) * D + d] = *reinterpret_cast<const logo_bf16*>(&bv);
             }
-            __syncthreads();  // the merge buffer is reused by the next item
+            __syncthreads();  // the merge buffer is reused by the next piece
             continue;
         }
-        // ---- a chunk of a longer cache: partial result, then the last chunk merges
-        for (int i = tid; i < group * D; i += kDecThreads) {
-            const int hh = i / D, d = i % D;
-            float acc = 0.f;
+        // ---- a piece of a pair that other CTAs have pieces of: partial result in
+        //      slot 1 of the pair's first CTA and slot 0 of the others, then the
+        //      last piece merges
+        const int c_first = cta_of(it.pair0), npieces = cta_of(it.pair0 + it.subs - 1) - c_first + 1;
+        {
+            const int64_t slot = static_cast<int64_t>(2 * blockIdx.x + (static_cast<int>(blockIdx.x) == c_first ? 1 : 0)) * group;
+            for (int i = tid; i < group * D; i += kDecThreads) {
+                const int hh = i / D, d = i % D;
+                float acc = 0.f;
 #pragma unroll
-            for (int wv = 0; wv < 4; ++wv) acc += sh_wm[wv][hh] * sM[(wv * group + hh) * (D + 2) + d];
-            float* dst = p.part + ((static_cast<int64_t>(it.r) * p.Hq + h0 + hh) * p.nchunk + it.c) * (D + 2);
-            dst[d] = acc;
-            if (d == 0) {
-                dst[D] = sh_M[hh];
-                dst[D + 1] = sh_L[hh];
+                for (int wv = 0; wv < 4; ++wv) acc += sh_wm[wv][hh] * sM[(wv * group + hh) * (D + 2) + d];
+                p.part[slot * D + i] = acc;
             }
+            if (tid < group) p.part_ml[slot + tid] = make_float2(sh_M[tid], sh_L[tid]);
         }
-        __syncthreads();  // every partial of this chunk is written
+        __syncthreads();  // every partial of this piece is written
         if (tid == 0) {
             __threadfence();
-            const int prev = atomicAdd(p.done + static_cast<int64_t>(it.r) * p.Hkv + it.kvh, 1);
-            sh_last = prev == it.nused - 1;
+            const int prev = atomicAdd(p.done + static_cast<int64_t>(it.b) * p.Hkv + it.kvh, 1);
+            sh_last = prev == npieces - 1;
             if (sh_last) __threadfence();
         }
         __syncthreads();
         if (sh_last) {
-            // M = max_c m_c, L = sum_c 2^(m_c - M) l_c, o = sum_c 2^(m_c - M) o_c / L,
-            // per head: the weights first (into sW), then thread (head, d) adds the chunks
-            for (int i = tid; i < group * it.nused; i += kDecThreads) {
-                const int hh = i / it.nused;
-                const float* base = p.part + (static_cast<int64_t>(it.r) * p.Hq + h0 + hh) * p.nchunk * (D + 2);
-                float M = -INFINITY;
-                for (int c = 0; c < it.nused; ++c) M = fmaxf(M, __ldcg(base + c * (D + 2) + D));
-                const int c = i % it.nused;
-                const float m = __ldcg(base + c * (D + 2) + D);
-                sW[hh * it.nused + c] = m == -INFINITY ? 0.f : ex2_approx(m - M);
+            // M = max_c m_c, L = sum_c 2^(m_c - M) l_c, o = sum_c 2^(m_c - M) o_c / L.
+            // A warp per head for the weights (a lane per piece, two at most: every
+            // max and sum arrives in one round of loads), then four columns a
+            // thread, eight pieces' loads in flight
+            auto slot_of = [&](int c) { return static_cast<int64_t>(2 * (c_first + c) + (c == 0 ? 1 : 0)) * group; };
+            for (int hh = warp; hh < group; hh += 4) {
+                float2 ml[2];
+#pragma unroll
+                for (int k = 0; k < 2; ++k)
+                    ml[k] = lane + 32 * k < npieces ? __ldcg(p.part_ml + slot_of(lane + 32 * k) + hh)
+                                                    : make_float2(-INFINITY, 0.f);
+                float M = fmaxf(ml[0].x, ml[1].x);
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+                float w[2], L = 0.f;
+#pragma unroll
+                for (int k = 0; k < 2; ++k) {
+                    w[k] = ml[k].x == -INFINITY ? 0.f : ex2_approx(ml[k].x - M);
+                    L += w[k] * ml[k].y;
+                }
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) L += __shfl_xor_sync(0xffffffffu, L, o);
+                const float inv = L > 0.f ? 1.0f / L : 0.f;
+#pragma unroll
+                for (int k = 0; k < 2; ++k)
+                    if (lane + 32 * k < npieces) sW[hh * npieces + lane + 32 * k] = w[k] * inv;
             }
             __syncthreads();
-            for (int i = tid; i < group * D; i += kDecThreads) {
-                const int hh = i / D, d = i % D;
-                const float* base = p.part + (static_cast<int64_t>(it.r) * p.Hq + h0 + hh) * p.nchunk * (D + 2);
-                const float* wts = sW + hh * it.nused;
-                float o = 0.f, L = 0.f;
-                for (int c = 0; c < it.nused; ++c) {
-                    const float wc = wts[c];
-                    o += wc * __ldcg(base + c * (D + 2) + d);
-                    L += wc * __ldcg(base + c * (D + 2) + D + 1);
+            for (int i = tid; i < group * (D / 4); i += kDecThreads) {
+                const int hh = i / (D / 4);
+                const float* wts = sW + hh * npieces;
+                float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 8
+                for (int c = 0; c < npieces; ++c) {
+                    const float4 v = __ldcg(reinterpret_cast<const float4*>(p.part + slot_of(c) * D) + i);
+                    const float w = wts[c];
+                    o.x += w * v.x;
+                    o.y += w * v.y;
+                    o.z += w * v.z;
+                    o.w += w * v.w;
                 }
-                const __nv_bfloat16 bv = __float2bfloat16_rn(L > 0.f ? o / L : 0.f);
-                p.out[(static_cast<int64_t>(it.r) * p.Hq + h0 + hh) * D + d] = *reinterpret_cast<const logo_bf16*>(&bv);
+                *reinterpret_cast<uint2*>(p.out + (static_cast<int64_t>(out_row) * p.Hq + h0) * D + 4 * i) =
+                    make_uint2(pack_bf16x2(o.x, o.y), pack_bf16x2(o.z, o.w));
             }
         }
-        __syncthreads();  // sW and the merge buffer are reused by the next item
+        __syncthreads();  // sW and the merge buffer are reused by the next piece
     }
     if (!ok && tid == 0) {  // let copies already issued land before the CTA exits
         for (int k = consumed; k < issued; ++k) mbar_wait_drain(smem_u32(&bar_full[k % kDecStages]), (k / kDecStages) & 1);
     }
 }
 
-// Chunks per (row, KV head): at least enough that a chunk holds at most
-// kDecSubMax sub-tiles, more while B x Hkv items would leave SMs idle, at most
-// one per sub-tile and kDecMaxChunks.  (rows: B, the most the global call can
-// have selected.)
-struct DecSplit {
-    int nchunk, sub_per_chunk;
-};
+constexpr int kDecCtasPerSm = 8;  // at most (the workspace's slots)
 
-DecSplit dec_split(const logo_dims& d)
+// part: [2 x CTAs, group, D] fp32, part_ml: [2 x CTAs, group] fp32 pairs, done: [B, Hkv] int32
+size_t decode_ws_layout(const logo_dims& d, char* base, DecParams* p)
 {
-    const int n_sub = (d.T + kDecRows - 1) / kDecRows;
-    const long long pairs = static_cast<long long>(d.B) * d.Hkv;
-    const long long want = (device_sm_count() + pairs - 1) / pairs;
-    long long nc = std::max<long long>(want, (n_sub + kDecSubMax - 1) / kDecSubMax);
-    nc = std::min<long long>(nc, std::min(n_sub, kDecMaxChunks));
-    nc = std::max<long long>(nc, 1);
-    const int spc = static_cast<int>((n_sub + nc - 1) / nc);
-    return DecSplit{(n_sub + spc - 1) / spc, spc};
-}
-
-// part: [B, Hq, nchunk, D + 2] fp32, then done: [B, Hkv] int32
-size_t decode_ws_bytes(const logo_dims& d, size_t* done_off = nullptr)
-{
-    const DecSplit sp = dec_split(d);
-    const size_t part = round_up(static_cast<size_t>(d.B) * d.Hq * sp.nchunk * (d.D + 2) * sizeof(float), 256);
-    if (done_off) *done_off = part;
-    return round_up(part + static_cast<size_t>(d.B) * d.Hkv * sizeof(int32_t), 256);
+    const size_t rows = 2 * static_cast<size_t>(kDecCtasPerSm) * device_sm_count() * (d.Hq / d.Hkv);
+    size_t off = round_up(rows * d.D * sizeof(float), 256);
+    const size_t o_ml = off;
+    off = round_up(off + rows * sizeof(float2), 256);
+    const size_t o_done = off;
+    off = round_up(off + static_cast<size_t>(d.B) * d.Hkv * sizeof(int32_t), 256);
+    if (p) {
+        p->part = reinterpret_cast<float*>(base);
+        p->part_ml = reinterpret_cast<float2*>(base + o_ml);
+        p->done = reinterpret_cast<int32_t*>(base + o_done);
+    }
+    return off;
 }
 
 int check_decode(const logo_dims& d)
@@ -491,12 +595,25 @@ int launch_decode(DecParams& prm, cudaStream_t st)
             per_sm = 1;
         per_sm_of[group] = per_sm;
     }
-    const long long items = static_cast<long long>(prm.B) * prm.Hkv * prm.nchunk;
-    const int grid = static_cast<int>(std::max(1ll, std::min(items, static_cast<long long>(per_sm) * device_sm_count())));
-    if (prm.nchunk > 1 &&  // the chunk counters start at zero
-        cudaMemsetAsync(prm.done, 0, static_cast<size_t>(prm.B) * prm.Hkv * sizeof(int32_t), st) != cudaSuccess)
-        return LOGO_ERR_CUDA;
-    decode_attn_kernel<D, RING><<<grid, kDecThreads, smem, st>>>(prm);
+    const long long n_sub = (prm.R + kDecRows - 1) / kDecRows, pairs = static_cast<long long>(prm.B) * prm.Hkv;
+    const long long ctas = static_cast<long long>(std::min(per_sm, kDecCtasPerSm)) * device_sm_count();
+    // Whole pairs when cutting them saves less than kDecSplitCost sub-tiles of
+    // the longest run (with full caches; the merge and the counters' clearing
+    // cost that much), else equal runs: short enough to fill the GPU, at least
+    // kDecMinSub, and long enough for kDecMaxPieces pieces of a pair.
+    const long long whole_run = (pairs + ctas - 1) / ctas * n_sub;
+    const long long cut_run = std::max<long long>(kDecMinSub, (pairs * n_sub + ctas - 1) / ctas);
+    long long grid;
+    if (whole_run <= cut_run + kDecSplitCost) {
+        prm.done = nullptr;
+        grid = std::min(pairs, ctas);
+    } else {
+        prm.min_sub = static_cast<int>(std::max<long long>(kDecMinSub, (n_sub + kDecMaxPieces - 3) / (kDecMaxPieces - 2)));
+        grid = std::max(1ll, std::min(pairs * n_sub / prm.min_sub, ctas));
+        if (cudaMemsetAsync(prm.done, 0, static_cast<size_t>(pairs) * sizeof(int32_t), st) != cudaSuccess)
+            return LOGO_ERR_CUDA;
+    }
+    decode_attn_kernel<D, RING><<<static_cast<unsigned>(grid), kDecThreads, smem, st>>>(prm);
     return cudaGetLastError() == cudaSuccess ? LOGO_OK : LOGO_ERR_CUDA;
 }
 
@@ -512,10 +629,8 @@ int run_decode(bool ring, const logo_bf16* q, const logo_bf16* k, const logo_bf1
     if (!aligned16(q) || !aligned16(k) || !aligned16(v) || !aligned16(out)) return LOGO_ERR_UNSUPPORTED;
     if (!(scale >= 0.0f)) return LOGO_ERR_INVALID_ARG;
     if (scale == 0.0f) scale = 1.0f / sqrtf(static_cast<float>(dims.D));
-    size_t done_off = 0;
-    const size_t need = decode_ws_bytes(dims, &done_off);
+    const size_t need = decode_ws_layout(dims, nullptr, nullptr);
     if (!workspace || workspace_bytes < need || !aligned16(workspace)) return LOGO_ERR_WORKSPACE;
-    const DecSplit sp = dec_split(dims);
     DecParams prm{};
     if (!encode_bf16_4d(&prm.tm_k, k, dims.D, dims.Hkv, dims.T, dims.B, 64, kDecRows) ||
         !encode_bf16_4d(&prm.tm_v, v, dims.D, dims.Hkv, dims.T, dims.B, 64, kDecRows))
@@ -524,16 +639,13 @@ int run_decode(bool ring, const logo_bf16* q, const logo_bf16* k, const logo_bf1
     prm.seq_len = seq_len;
     prm.cu_q = cu_q;
     prm.n_sel = n_sel;
-    prm.part = static_cast<float*>(workspace);
-    prm.done = reinterpret_cast<int32_t*>(static_cast<char*>(workspace) + done_off);
+    decode_ws_layout(dims, static_cast<char*>(workspace), &prm);
     prm.out = out;
     prm.B = dims.B;
     prm.R = dims.T;
     prm.Hq = dims.Hq;
     prm.Hkv = dims.Hkv;
     prm.window = window;
-    prm.nchunk = sp.nchunk;
-    prm.sub_per_chunk = sp.sub_per_chunk;
     prm.scale_log2 = scale * kLog2e;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (dims.D == 128) return ring ? launch_decode<128, true>(prm, st) : launch_decode<128, false>(prm, st);
@@ -551,7 +663,7 @@ using namespace logo;
 extern "C" size_t logo_decode_workspace_size(logo_dims dims)
 {
     if (check_decode(dims) != LOGO_OK) return 0;
-    return decode_ws_bytes(dims);
+    return decode_ws_layout(dims, nullptr, nullptr);
 }
 
 extern "C" int logo_decode_local_attn(const logo_bf16* q, const logo_bf16* k_ring, const logo_bf16* v_ring,
