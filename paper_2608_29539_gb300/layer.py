@@ -54,6 +54,9 @@ class LogoAttention:
         dev = torch.device(device)
         self.overlap = overlap
         self.side = torch.cuda.Stream(device=dev) if overlap and dev.type == "cuda" else None
+        if self.side is not None:  # recorded anew on every fork and join
+            self._forked, self._joined = torch.cuda.Event(), torch.cuda.Event()
+            self._side_handle = self.side.cuda_stream
         self.dims = L.Dims(c.B, c.T, c.Hq, c.Hkv, c.D)
         cap = c.B * c.T
         bf, f32, i32 = torch.bfloat16, torch.float32, torch.int32
@@ -88,38 +91,31 @@ class LogoAttention:
         self.ws = e((nbytes,), torch.uint8)
         self.ws_l = e((L.workspace_bytes("local_bwd", self.dims),), torch.uint8)
 
-    def _fork(self):
-        """Side stream for the local branch (None: run it in order)."""
-        if self.side is None:
-            return None
-        self.side.wait_stream(torch.cuda.current_stream())
-        return torch.cuda.stream(self.side)
-
-    def _join(self):
-        if self.side is not None:
-            torch.cuda.current_stream().wait_stream(self.side)
-
-    def _local_fwd(self, qL, kL, vL):
+    def _local_fwd(self, qL, kL, vL, stream):
         c = self.cfg
-        L.logo_local_attn_fwd(qL, kL, vL, c.window, c.scale, self.o_l, self.lse_l)
+        L.logo_local_attn_fwd(qL, kL, vL, c.window, c.scale, self.o_l, self.lse_l, stream=stream)
 
-    def _local_bwd(self, qL, kL, vL):
+    def _local_bwd(self, qL, kL, vL, stream):
         c = self.cfg
         L.logo_local_attn_bwd(qL, kL, vL, self.o_l, self.lse_l, self.dO_l, c.window, c.scale, self.dqL, self.dkL,
-                              self.dvL, workspace=self.ws_l)
+                              self.dvL, workspace=self.ws_l, stream=stream)
 
     def _branches(self, local, other):
-        """local() on the side stream beside other() on the caller's stream,
-        joined before returning; both in order without a side stream."""
-        ctx = self._fork()
-        if ctx is None:
+        """local(stream) on the side stream beside other() on the caller's
+        stream, joined before returning; both in order without a side stream.
+        (The local calls are given the stream's handle: making it torch's
+        current stream and back took longer than launching them.)"""
+        if self.side is None:
             other()
-            local()
+            local(None)
             return
-        with ctx:
-            local()
+        main = torch.cuda.current_stream()
+        self._forked.record(main)
+        self.side.wait_event(self._forked)
+        local(self._side_handle)
         other()
-        self._join()
+        self._joined.record(self.side)
+        main.wait_event(self._joined)
 
     def forward(self, qL, kL, vL, qG, kG, vG, gate_p, gain_l=None, gain_g=None):
         c = self.cfg
@@ -129,7 +125,7 @@ class LogoAttention:
         # (measured at 16K: 2.39 ms a step against 2.23 with this order)
         L.logo_select(gate_p, c.mode, c.b_th, c.ratio, self.z, self.pos, self.cu_q, self.row_of, self.n_sel,
                       workspace=self.ws)
-        self._branches(lambda: self._local_fwd(qL, kL, vL),
+        self._branches(lambda stream: self._local_fwd(qL, kL, vL, stream),
                        lambda: L.logo_global_sparse_attn_fwd(qG, kG, vG, self.pos, self.cu_q, self.n_sel, c.scale,
                                                              self.o_c, self.lse_c, workspace=self.ws))
         L.logo_combine(self.o_l, self.o_c, gate_p, self.z, self.row_of, gain_l, gain_g, c.eps, self.o, self.rstd_l,
@@ -140,7 +136,7 @@ class LogoAttention:
         c = self.cfg
         L.logo_combine_bwd(dO, self.o_l, self.o_c, gate_p, self.z, self.row_of, gain_l, gain_g, c.eps, self.dO_l,
                            self.dO_c, self.dgate)
-        self._branches(lambda: self._local_bwd(qL, kL, vL),
+        self._branches(lambda stream: self._local_bwd(qL, kL, vL, stream),
                        lambda: L.logo_global_sparse_attn_bwd(qG, kG, vG, self.pos, self.cu_q, self.n_sel, self.o_c,
                                                              self.lse_c, self.dO_c, c.scale, self.dqG, self.dkG,
                                                              self.dvG, workspace=self.ws))
@@ -180,7 +176,7 @@ class LogoAttention:
             self.dw_g = torch.empty_like(w_g)
         L.logo_combine_bwd_gains(dO, self.o_l, self.o_c, self.gate_p, self.z, self.row_of, gain_l, gain_g, c.eps,
                                  self.dO_l, self.dO_c, self.dgate, self.dgain_l, self.dgain_g)
-        self._branches(lambda: self._local_bwd(qL, kL, vL),
+        self._branches(lambda stream: self._local_bwd(qL, kL, vL, stream),
                        lambda: L.logo_global_sparse_attn_bwd(self.qG, self.kG, self.vG, self.pos, self.cu_q,
                                                              self.n_sel, self.o_c, self.lse_c, self.dO_c, c.scale,
                                                              self.dqG, self.dkG, self.dvG, workspace=self.ws))

@@ -9,6 +9,7 @@ there is no CPU path.  If the library has not been built, every call raises.
 from __future__ import annotations
 
 import ctypes
+import functools
 import os
 
 import torch
@@ -112,16 +113,27 @@ def lib():
     return _lib
 
 
+# The calls below are a few microseconds of host time each, as much as their
+# kernels take at small sizes, so nothing here is made twice: pointers go to
+# ctypes as plain integers, the current stream comes straight from torch's C
+# module, and the dims structures and workspace sizes (functions of the sizes
+# alone) are remembered.
 def _p(t):
-    return None if t is None else _vp(t.data_ptr())
+    return None if t is None else t.data_ptr()
+
+
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_current_device = getattr(torch._C, "_cuda_getDevice", None)
 
 
 def _stream():
-    return _vp(torch.cuda.current_stream().cuda_stream)
+    if _raw_stream is None or _current_device is None or not torch.cuda.is_initialized():
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(_current_device())
 
 
 def _call(name, *args):
-    rc = getattr(lib(), name)(*args)
+    rc = getattr(_lib or lib(), name)(*args)
     if rc != LOGO_OK:
         raise LogoError(name, rc)
 
@@ -133,14 +145,25 @@ def _need(t, dtype, name, shape=None):
         raise ValueError(f"{name} must be {dtype}, got {t.dtype}")
     if not t.is_contiguous():
         raise ValueError(f"{name} must be contiguous")
-    if shape is not None and tuple(t.shape) != tuple(shape):
+    if shape is not None and t.shape != shape:
         raise ValueError(f"{name} has shape {tuple(t.shape)}, expected {tuple(shape)}")
     return t
+
+
+@functools.lru_cache(maxsize=1024)
+def _dims(B, T, Hq, Hkv, D) -> Dims:
+    """A Dims that nobody writes to."""
+    return Dims(B, T, Hq, Hkv, D)
 
 
 def dims_of(q: torch.Tensor, k: torch.Tensor) -> Dims:
     B, T, Hq, D = q.shape
     return Dims(B, T, Hq, k.shape[2], D)
+
+
+def _dims_of(q: torch.Tensor, k: torch.Tensor) -> Dims:
+    B, T, Hq, D = q.shape
+    return _dims(B, T, Hq, k.shape[2], D)
 
 
 def _workspace(nbytes: int, device, ws=None):
@@ -151,12 +174,24 @@ def _workspace(nbytes: int, device, ws=None):
     return torch.empty(max(int(nbytes), 16), dtype=torch.uint8, device=device)
 
 
+@functools.lru_cache(maxsize=1024)
+def _size(fn: str, device: int, B, T, Hq, Hkv, D, *more) -> int:
+    return int(getattr(_lib or lib(), fn)(_dims(B, T, Hq, Hkv, D), *more))
+
+
+def _ws_bytes(fn: str, d: Dims, *more) -> int:
+    """logo_*_workspace_size for the current device (its SM count enters some)."""
+    device = _current_device() if _current_device is not None and torch.cuda.is_initialized() else -1
+    return _size(fn, device, d.B, d.T, d.Hq, d.Hkv, d.D, *more)
+
+
+_WS_FN = {"select": "logo_select_workspace_size", "local_bwd": "logo_local_attn_bwd_workspace_size",
+          "global_fwd": "logo_global_attn_fwd_workspace_size", "global_bwd": "logo_global_attn_bwd_workspace_size",
+          "combine_bwd_gains": "logo_combine_bwd_workspace_size"}
+
+
 def workspace_bytes(kind: str, dims: Dims) -> int:
-    fn = {"select": "logo_select_workspace_size", "local_bwd": "logo_local_attn_bwd_workspace_size",
-          "global_fwd": "logo_global_attn_fwd_workspace_size",
-          "global_bwd": "logo_global_attn_bwd_workspace_size",
-          "combine_bwd_gains": "logo_combine_bwd_workspace_size"}[kind]
-    return int(getattr(lib(), fn)(dims))
+    return _ws_bytes(_WS_FN[kind], dims)
 
 
 # ----------------------------------------------------------------------- API
@@ -182,7 +217,7 @@ def logo_select(gate_p, mode: int, b_th: float = 0.5, ratio: float = 0.0, z=None
     _need(gate_p, torch.float32, "gate_p")
     B, T = gate_p.shape
     dev = gate_p.device
-    dims = Dims(B, T, 1, 1, 64)
+    dims = _dims(B, T, 1, 1, 64)
     z = z if z is not None else torch.empty((B, T), dtype=torch.uint8, device=dev)
     pos = pos if pos is not None else torch.empty((B * T,), dtype=torch.int32, device=dev)
     cu_q = cu_q if cu_q is not None else torch.empty((B + 1,), dtype=torch.int32, device=dev)
@@ -204,7 +239,7 @@ def logo_gate_select(x, w_g, mode: int, b_th: float = 0.5, ratio: float = 0.0, g
     _need(w_g, torch.float32, "w_g")
     B, T, dm = x.shape
     dev = x.device
-    dims = Dims(B, T, 1, 1, 64)
+    dims = _dims(B, T, 1, 1, 64)
     gate_p = gate_p if gate_p is not None else torch.empty((B, T), dtype=torch.float32, device=dev)
     z = z if z is not None else torch.empty((B, T), dtype=torch.uint8, device=dev)
     pos = pos if pos is not None else torch.empty((B * T,), dtype=torch.int32, device=dev)
@@ -226,7 +261,7 @@ def logo_gate_bwd(x, w_g, gate_p, dgate_p, dx=None, accumulate: bool = False, dw
     _need(x, torch.bfloat16, "x")
     B, T, dm = x.shape
     dev = x.device
-    dims = Dims(B, T, 1, 1, 64)
+    dims = _dims(B, T, 1, 1, 64)
     if want_dx and dx is None:
         if accumulate:
             raise ValueError("accumulate needs the dx to add to")
@@ -234,7 +269,7 @@ def logo_gate_bwd(x, w_g, gate_p, dgate_p, dx=None, accumulate: bool = False, dw
     if not want_dx:
         dx = None
     dw_g = (dw_g if dw_g is not None else torch.empty((dm,), dtype=torch.float32, device=dev)) if want_dw else None
-    nbytes = int(lib().logo_gate_bwd_workspace_size(dims, dm)) if want_dw else 0
+    nbytes = _ws_bytes("logo_gate_bwd_workspace_size", dims, dm) if want_dw else 0
     ws = _workspace(nbytes, dev, workspace) if want_dw else None
     _call("logo_gate_bwd", _p(x), _p(w_g), _p(gate_p), _p(dgate_p), int(dm), dims, _p(dx), int(bool(accumulate)),
           _p(dw_g), _p(ws), nbytes, _stream())
@@ -257,7 +292,7 @@ def logo_branch_transform(u_l, a=None, s=None, b=None, rows=None, u_g=None):
     u_g = u_g if u_g is not None else torch.empty_like(u_l)
     pos, cu_q, n_sel = _transform_rows(rows)
     _call("logo_branch_transform", _p(u_l), _p(a), _p(s), _p(b), _p(pos), _p(cu_q), _p(n_sel), _p(u_g),
-          Dims(B, T, H, H, D), _stream())
+          _dims(B, T, H, H, D), _stream())
     return u_g
 
 
@@ -268,7 +303,7 @@ def logo_branch_transform_bwd(u_l, du_g, a=None, s=None, rows=None, du_l=None, a
     _need(u_l, torch.bfloat16, "u_l")
     B, T, H, D = u_l.shape
     dev = u_l.device
-    dims = Dims(B, T, H, H, D)
+    dims = _dims(B, T, H, H, D)
     if du_l is None:
         if accumulate:
             raise ValueError("accumulate needs the du_l to add to")
@@ -276,7 +311,7 @@ def logo_branch_transform_bwd(u_l, du_g, a=None, s=None, rows=None, du_l=None, a
     da = torch.empty((H, D, D), dtype=torch.float32, device=dev) if a is not None else None
     ds = torch.empty((H, D), dtype=torch.float32, device=dev) if a is None else None
     db = torch.empty((H, D), dtype=torch.float32, device=dev) if a is None else None
-    nbytes = int(lib().logo_branch_transform_bwd_workspace_size(dims))
+    nbytes = _ws_bytes("logo_branch_transform_bwd_workspace_size", dims)
     ws = _workspace(nbytes, dev, workspace)
     pos, cu_q, n_sel = _transform_rows(rows)
     _call("logo_branch_transform_bwd", _p(u_l), _p(a), _p(s), _p(pos), _p(cu_q), _p(n_sel), _p(du_g), _p(du_l),
@@ -292,7 +327,7 @@ def logo_select_device_threshold(gate_p, b_th, z=None, pos=None, cu_q=None, row_
     _need(b_th, torch.float32, "b_th", (1,))
     B, T = gate_p.shape
     dev = gate_p.device
-    dims = Dims(B, T, 1, 1, 64)
+    dims = _dims(B, T, 1, 1, 64)
     z = z if z is not None else torch.empty((B, T), dtype=torch.uint8, device=dev)
     pos = pos if pos is not None else torch.empty((B * T,), dtype=torch.int32, device=dev)
     cu_q = cu_q if cu_q is not None else torch.empty((B + 1,), dtype=torch.int32, device=dev)
@@ -313,7 +348,7 @@ def logo_budget_update(n_sel_total, B: int, T: int, rho: float, gamma: float, b_
     _need(b_th, torch.float32, "b_th", (1,))
     if f_out is not None:
         _need(f_out, torch.float32, "f_out", (1,))
-    _call("logo_budget_update", _p(n_sel_total), Dims(int(B), int(T), 1, 1, 64), float(rho), float(gamma),
+    _call("logo_budget_update", _p(n_sel_total), _dims(int(B), int(T), 1, 1, 64), float(rho), float(gamma),
           _p(b_th), _p(f_out), _stream())
     return b_th
 
@@ -325,7 +360,7 @@ def logo_pmask_initial_threshold(gamma: float, pmask_steps: int) -> float:
 
 def _decode_dims(q, k):
     B, Hq, D = q.shape
-    return Dims(B, k.shape[1], Hq, k.shape[2], D)
+    return _dims(B, k.shape[1], Hq, k.shape[2], D)
 
 
 def logo_decode_local_attn(q, k_ring, v_ring, seq_len, window: int, scale: float = 0.0, o=None, workspace=None):
@@ -338,7 +373,7 @@ def logo_decode_local_attn(q, k_ring, v_ring, seq_len, window: int, scale: float
     _need(seq_len, torch.int32, "seq_len", (q.shape[0],))
     dims = _decode_dims(q, k_ring)
     o = o if o is not None else torch.empty_like(q)
-    nbytes = int(lib().logo_decode_workspace_size(dims))
+    nbytes = _ws_bytes("logo_decode_workspace_size", dims)
     ws = _workspace(nbytes, q.device, workspace)
     _call("logo_decode_local_attn", _p(q), _p(k_ring), _p(v_ring), _p(seq_len), _p(o), dims, int(window),
           float(scale), _p(ws), nbytes, _stream())
@@ -358,7 +393,7 @@ def logo_decode_global_sparse_attn(q, k_cache, v_cache, seq_len, cu_q, n_sel_tot
     _need(n_sel_total, torch.int32, "n_sel_total", (1,))
     dims = _decode_dims(q, k_cache)
     o_c = o_c if o_c is not None else torch.empty_like(q)
-    nbytes = int(lib().logo_decode_workspace_size(dims))
+    nbytes = _ws_bytes("logo_decode_workspace_size", dims)
     ws = _workspace(nbytes, q.device, workspace)
     _call("logo_decode_global_sparse_attn", _p(q), _p(k_cache), _p(v_cache), _p(seq_len), _p(cu_q),
           _p(n_sel_total), _p(o_c), dims, float(scale), _p(ws), nbytes, _stream())
@@ -374,7 +409,7 @@ def logo_select_noalloc(gate_p, mode: int, b_th: float = 0.5, ratio: float = 0.0
     _need(gate_p, torch.float32, "gate_p")
     B, T = gate_p.shape
     dev = gate_p.device
-    dims = Dims(B, T, 1, 1, 64)
+    dims = _dims(B, T, 1, 1, 64)
     z = z if z is not None else torch.empty((B, T), dtype=torch.uint8, device=dev)
     pos = pos if pos is not None else torch.empty((B * T,), dtype=torch.int32, device=dev)
     cu_q = cu_q if cu_q is not None else torch.empty((B + 1,), dtype=torch.int32, device=dev)
@@ -385,21 +420,24 @@ def logo_select_noalloc(gate_p, mode: int, b_th: float = 0.5, ratio: float = 0.0
     return z, pos, cu_q, row_of, n_sel_total
 
 
-def logo_local_attn_fwd(q, k, v, window: int, scale: float = 0.0, o=None, lse=None):
-    """Eq. 6 local branch.  Returns (o [B,T,Hq,D] bf16, lse [B,Hq,T] fp32)."""
+def logo_local_attn_fwd(q, k, v, window: int, scale: float = 0.0, o=None, lse=None, *, stream=None):
+    """Eq. 6 local branch.  Returns (o [B,T,Hq,D] bf16, lse [B,Hq,T] fp32).
+    stream: raw handle of the stream to launch on (default: the current one)."""
     for t, n in ((q, "q"), (k, "k"), (v, "v")):
         _need(t, torch.bfloat16, n)
-    d = dims_of(q, k)
+    d = _dims_of(q, k)
     o = o if o is not None else torch.empty_like(q)
     lse = lse if lse is not None else torch.empty((d.B, d.Hq, d.T), dtype=torch.float32, device=q.device)
-    _call("logo_local_attn_fwd", _p(q), _p(k), _p(v), _p(o), _p(lse), d, int(window), float(scale), _stream())
+    _call("logo_local_attn_fwd", _p(q), _p(k), _p(v), _p(o), _p(lse), d, int(window), float(scale),
+          _stream() if stream is None else stream)
     return o, lse
 
 
 def logo_local_attn_bwd(q, k, v, o, lse, dO, window: int, scale: float = 0.0, dq=None, dk=None, dv=None,
-                        workspace=None):
-    """Gradients of the local branch.  Returns (dq, dk, dv)."""
-    d = dims_of(q, k)
+                        workspace=None, *, stream=None):
+    """Gradients of the local branch.  Returns (dq, dk, dv).
+    stream: as in logo_local_attn_fwd (with every output and the workspace given)."""
+    d = _dims_of(q, k)
     for t, n in ((q, "q"), (k, "k"), (v, "v"), (o, "o"), (dO, "dO")):
         _need(t, torch.bfloat16, n)
     _need(lse, torch.float32, "lse", (d.B, d.Hq, d.T))
@@ -409,7 +447,7 @@ def logo_local_attn_bwd(q, k, v, o, lse, dO, window: int, scale: float = 0.0, dq
     nbytes = workspace_bytes("local_bwd", d)
     ws = _workspace(nbytes, q.device, workspace)
     _call("logo_local_attn_bwd", _p(q), _p(k), _p(v), _p(o), _p(lse), _p(dO), _p(dq), _p(dk), _p(dv), d,
-          int(window), float(scale), _p(ws), nbytes, _stream())
+          int(window), float(scale), _p(ws), nbytes, _stream() if stream is None else stream)
     return dq, dk, dv
 
 
@@ -420,7 +458,7 @@ def logo_global_sparse_attn_fwd(q, k, v, pos, cu_q, n_sel_total, scale: float = 
         _need(t, torch.bfloat16, n)
     for t, n in ((pos, "pos"), (cu_q, "cu_q"), (n_sel_total, "n_sel_total")):
         _need(t, torch.int32, n)
-    d = dims_of(q, k)
+    d = _dims_of(q, k)
     cap = d.B * d.T
     o_c = o_c if o_c is not None else torch.empty((cap, d.Hq, d.D), dtype=torch.bfloat16, device=q.device)
     lse_c = lse_c if lse_c is not None else torch.empty((d.Hq, cap), dtype=torch.float32, device=q.device)
@@ -434,7 +472,7 @@ def logo_global_sparse_attn_fwd(q, k, v, pos, cu_q, n_sel_total, scale: float = 
 def logo_global_sparse_attn_bwd(q, k, v, pos, cu_q, n_sel_total, o_c, lse_c, dO_c, scale: float = 0.0, dq=None,
                                 dk=None, dv=None, workspace=None):
     """Row-sparse gradients of the global branch.  Returns (dq dense, dk, dv)."""
-    d = dims_of(q, k)
+    d = _dims_of(q, k)
     for t, n in ((q, "q"), (k, "k"), (v, "v"), (o_c, "o_c"), (dO_c, "dO_c")):
         _need(t, torch.bfloat16, n)
     _need(lse_c, torch.float32, "lse_c")
@@ -454,7 +492,7 @@ def logo_combine(o_l, o_c, gate_p, z, row_of, gain_l=None, gain_g=None, eps: flo
     _need(o_l, torch.bfloat16, "o_l")
     _need(o_c, torch.bfloat16, "o_c")
     B, T, H, D = o_l.shape
-    d = Dims(B, T, H, H, D)
+    d = _dims(B, T, H, H, D)
     o = o if o is not None else torch.empty_like(o_l)
     rstd_l = rstd_l if rstd_l is not None else torch.empty((B, T, H), dtype=torch.float32, device=o_l.device)
     rstd_g = rstd_g if rstd_g is not None else torch.empty((B * T, H), dtype=torch.float32, device=o_l.device)
@@ -468,7 +506,7 @@ def logo_combine_bwd(dO, o_l, o_c, gate_p, z, row_of, gain_l=None, gain_g=None, 
     """Backward of logo_combine with z fixed.  Returns (dO_l, dO_c, dgate_p)."""
     _need(dO, torch.bfloat16, "dO")
     B, T, H, D = o_l.shape
-    d = Dims(B, T, H, H, D)
+    d = _dims(B, T, H, H, D)
     dO_l = dO_l if dO_l is not None else torch.empty_like(o_l)
     dO_c = dO_c if dO_c is not None else torch.empty((B * T, H, D), dtype=torch.bfloat16, device=o_l.device)
     dgate_p = dgate_p if dgate_p is not None else torch.empty((B, T), dtype=torch.float32, device=o_l.device)
@@ -484,14 +522,14 @@ def logo_combine_bwd_gains(dO, o_l, o_c, gate_p, z, row_of, gain_l=None, gain_g=
     [Hq, D] float32."""
     _need(dO, torch.bfloat16, "dO")
     B, T, H, D = o_l.shape
-    d = Dims(B, T, H, H, D)
+    d = _dims(B, T, H, H, D)
     dev = o_l.device
     dO_l = dO_l if dO_l is not None else torch.empty_like(o_l)
     dO_c = dO_c if dO_c is not None else torch.empty((B * T, H, D), dtype=torch.bfloat16, device=dev)
     dgate_p = dgate_p if dgate_p is not None else torch.empty((B, T), dtype=torch.float32, device=dev)
     dgain_l = dgain_l if dgain_l is not None else torch.empty((H, D), dtype=torch.float32, device=dev)
     dgain_g = dgain_g if dgain_g is not None else torch.empty((H, D), dtype=torch.float32, device=dev)
-    nbytes = int(lib().logo_combine_bwd_workspace_size(d))
+    nbytes = workspace_bytes("combine_bwd_gains", d)
     ws = _workspace(nbytes, dev, workspace)
     _call("logo_combine_bwd_gains", _p(dO), _p(o_l), _p(o_c), _p(gate_p), _p(z), _p(row_of), _p(gain_l),
           _p(gain_g), float(eps), _p(dO_l), _p(dO_c), _p(dgate_p), _p(dgain_l), _p(dgain_g), d, _p(ws),
