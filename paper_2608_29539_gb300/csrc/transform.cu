@@ -8,15 +8,13 @@
 //
 // LP is a contraction of 2 d^2 FLOP per row and head against 4 d bytes moved:
 // at d = 128 that is 64 FLOP/byte, more than the CUDA cores can keep up with
-// at HBM speed, so it runs on the tensor cores.  On every row (K, V) a tcgen05
-// pipeline: TMA brings 128-row tiles of one head into shared memory next to
-// that head's A_h, one thread issues the MMAs into two TMEM buffers, four warps
-// drain them.  On the packed selected rows (Q; rows gathered by position)
-// warp-level mma.sync over 64-row tiles.  A block keeps one head's A_h and
-// walks a strided share of its row tiles.  The backward computes
-// dU^L = dU^G A_h^T on the same tiles and accumulates dA_h = U^L^T dU^G; per-
-// block partial dA are reduced in block order by a second kernel
-// (deterministic).  SO is elementwise; its per-block ds, db are summed by the
+// at HBM speed, so it runs on the tensor cores: tcgen05 pipelines over 128-row
+// tiles of a head beside that head's A_h in shared memory, one thread issuing
+// the MMAs into two TMEM buffers, four warps draining them (the forward on the
+// packed selected rows alone uses warp-level mma.sync over gathered 64-row
+// tiles).  The backward computes dU^L = dU^G A_h^T on the same tiles and
+// accumulates dA_h = U^L^T dU^G; per-CTA partial dA are reduced in order by a
+// second kernel (deterministic).  SO is elementwise; its per-block ds, db are summed by the
 // fixed-order column sum of colsum.cuh (deterministic too).
 #include <cuda_bf16.h>
 
@@ -31,7 +29,6 @@ namespace logo {
 namespace {
 
 constexpr int kTileRows = 64;
-constexpr int kChunksPerHead = 16;  // blocks per head (row tiles strided among them)
 
 // Row r of the listed set -> token index b*T + t (all rows: r itself).
 struct RowSet {
@@ -194,117 +191,42 @@ __global__ void __launch_bounds__(128) lp_fwd_kernel(const logo_bf16* __restrict
     }
 }
 
-// LP backward: du_l[row] (+)= du_g[row] A_h^T, and dA_h += u_l^T du_g over the
-// block's rows.  D/16 warps: for dU, warp w takes rows 16 (w % 4).. and output
-// columns 64 (w / 4)..; for dA, rows 16w.. of the D x D result.
-// part: [H][gridDim.x][D][D] float32.
-template <int D>
-__global__ void __launch_bounds__(D * 2) lp_bwd_kernel(const logo_bf16* __restrict__ u_l,
-                                                       const logo_bf16* __restrict__ a,
-                                                       const logo_bf16* __restrict__ du_g, RowSet R, int H,
-                                                       logo_bf16* __restrict__ du_l, int accumulate,
-                                                       float* __restrict__ part)
-{
-    constexpr int kThreads = D * 2;
-    extern __shared__ __align__(128) uint8_t smem[];
-    __shared__ int64_t tok[kTileRows];
-    const uint32_t sA = smem_u32(smem), sU = sA + D * D * 2, sG = sU + kTileRows * D * 2;
-    const int h = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int mi = lane >> 3, rr = lane & 7, gid = lane >> 2, tig = lane & 3;
-    load_matrix_async<D>(sA, a + static_cast<int64_t>(h) * D * D, kThreads);  // lands with the first tile
-    float acc_a[D / 8][4];
-#pragma unroll
-    for (int nt = 0; nt < D / 8; ++nt)
-#pragma unroll
-        for (int i = 0; i < 4; ++i) acc_a[nt][i] = 0.f;
-    const int n = row_count(R);
-    const int ntiles = (n + kTileRows - 1) / kTileRows;
-    const int rg = warp & 3, cb = (warp >> 2) * 64;  // dU: row group and first output column
-    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        const int r0 = tile * kTileRows, nr = min(kTileRows, n - r0);
-        if (threadIdx.x < kTileRows) tok[threadIdx.x] = threadIdx.x < nr ? row_token(R, r0 + threadIdx.x) : 0;
-        __syncthreads();
-        load_tile_async<D>(sU, u_l, tok, nr, H, h, kThreads);
-        load_tile_async<D>(sG, du_g, tok, nr, H, h, kThreads);
-        cp_async_commit();
-        cp_async_wait_all();
-        __syncthreads();
-        // dU = dG A^T: rows 16 rg.., output columns cb .. cb + 63 (A_h rows i)
-        {
-            float acc[8][4];
-#pragma unroll
-            for (int nt = 0; nt < 8; ++nt)
-#pragma unroll
-                for (int i = 0; i < 4; ++i) acc[nt][i] = 0.f;
-#pragma unroll
-            for (int ks = 0; ks < D / 16; ++ks) {  // k: A_h columns j
-                uint32_t fa[4];
-                ldsm_x4(sG + toff<D>(rg * 16 + (mi & 1) * 8 + rr, 2 * ks + (mi >> 1)), fa[0], fa[1], fa[2], fa[3]);
-#pragma unroll
-                for (int np = 0; np < 4; ++np) {
-                    uint32_t b0, b1, b2, b3;  // B(k = j, n = i) = A_h[i][j]: rows n, k contiguous
-                    ldsm_x4(sA + toff<D>(cb + np * 16 + (mi >> 1) * 8 + rr, 2 * ks + (mi & 1)), b0, b1, b2, b3);
-                    mma_bf16_16816(acc[2 * np], fa, b0, b1);
-                    mma_bf16_16816(acc[2 * np + 1], fa, b2, b3);
-                }
-            }
-#pragma unroll
-            for (int half = 0; half < 2; ++half) {
-                const int r = rg * 16 + gid + half * 8;
-                if (r < nr) {
-                    logo_bf16* dst = du_l + (tok[r] * H + h) * D + cb + 2 * tig;
-#pragma unroll
-                    for (int nt = 0; nt < 8; ++nt) {
-                        float x0 = acc[nt][2 * half], x1 = acc[nt][2 * half + 1];
-                        uint32_t* p = reinterpret_cast<uint32_t*>(dst + nt * 8);
-                        if (accumulate) {
-                            const float2 old = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(p));
-                            x0 += old.x;
-                            x1 += old.y;
-                        }
-                        *p = pack_bf16x2(x0, x1);
-                    }
-                }
-            }
-        }
-        // dA += U^T dG: result rows i = 16 warp .., all columns j; k = the tile's rows
-#pragma unroll
-        for (int ks = 0; ks < kTileRows / 16; ++ks) {
-            uint32_t fa[4];  // A(m = i, k = r) = U[r][i]: stored rows k, m contiguous
-            ldsm_x4_trans(sU + toff<D>(16 * ks + (mi >> 1) * 8 + rr, 2 * warp + (mi & 1)), fa[0], fa[1], fa[2], fa[3]);
-#pragma unroll
-            for (int np = 0; np < D / 16; ++np) {
-                uint32_t b0, b1, b2, b3;  // B(k = r, n = j) = dG[r][j]
-                ldsm_x4_trans(sG + toff<D>(16 * ks + (mi & 1) * 8 + rr, 2 * np + (mi >> 1)), b0, b1, b2, b3);
-                mma_bf16_16816(acc_a[2 * np], fa, b0, b1);
-                mma_bf16_16816(acc_a[2 * np + 1], fa, b2, b3);
-            }
-        }
-        __syncthreads();
-    }
-    cp_async_wait_all();  // a block with no tile still has A_h's copies in flight
-    float* pp = part + (static_cast<int64_t>(h) * gridDim.x + blockIdx.x) * D * D;
-#pragma unroll
-    for (int half = 0; half < 2; ++half) {
-        const int i = warp * 16 + gid + half * 8;
-#pragma unroll
-        for (int nt = 0; nt < D / 8; ++nt) {
-            pp[i * D + nt * 8 + 2 * tig] = acc_a[nt][2 * half];
-            pp[i * D + nt * 8 + 2 * tig + 1] = acc_a[nt][2 * half + 1];
-        }
-    }
-}
-
-// out[h][e] = sum over c (in order) of part[h][c][e], e < per_head.
+// out[h][e] = sum over c of part[h][c][e], e < per_head (a multiple of 4).
+// Thread (x, g) of a block adds chunks g, g + 4, .. of four columns, then the
+// four sums are added in order: a fixed order, and every load in flight.
 __global__ void __launch_bounds__(256) reduce_parts_kernel(const float* __restrict__ part, int nchunk, int per_head,
                                                            int H, float* __restrict__ out)
 {
-    const int64_t e = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (e >= static_cast<int64_t>(H) * per_head) return;
-    const int h = static_cast<int>(e / per_head), x = static_cast<int>(e % per_head);
-    float s = 0.f;
-    for (int c = 0; c < nchunk; ++c) s += part[(static_cast<int64_t>(h) * nchunk + c) * per_head + x];
-    out[e] = s;
+    __shared__ float4 sh[4][64];
+    const int x = threadIdx.x & 63, g = threadIdx.x >> 6;
+    const int64_t e = (static_cast<int64_t>(blockIdx.x) * 64 + x) * 4;
+    const bool have = e < static_cast<int64_t>(H) * per_head;
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (have) {
+        const int64_t h = e / per_head;
+        const float* src = part + h * nchunk * per_head + e % per_head;
+#pragma unroll 4
+        for (int c = g; c < nchunk; c += 4) {
+            const float4 v = *reinterpret_cast<const float4*>(src + static_cast<int64_t>(c) * per_head);
+            s.x += v.x;
+            s.y += v.y;
+            s.z += v.z;
+            s.w += v.w;
+        }
+    }
+    sh[g][x] = s;
+    __syncthreads();
+    if (g == 0 && have) {
+#pragma unroll
+        for (int k = 1; k < 4; ++k) {
+            const float4 v = sh[k][x];
+            s.x += v.x;
+            s.y += v.y;
+            s.z += v.z;
+            s.w += v.w;
+        }
+        *reinterpret_cast<float4*>(out + e) = s;
+    }
 }
 
 // SO forward: u_g = u_l * s + b on the listed rows; a thread per 8-element vector.
@@ -509,7 +431,6 @@ __global__ void __launch_bounds__(192, 1) lp_tc_fwd_kernel(const __grid_constant
     } else {
         // epilogue: warp w reads TMEM lanes 32 (w % 4) .. (its rows of the tile)
         const int quad = warp & 3;
-        const int r = quad * 32 + lane;
         const uint32_t lane_off = static_cast<uint32_t>(quad * 32) << 16;
         int k = 0;
         for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++k) {
@@ -518,28 +439,34 @@ __global__ void __launch_bounds__(192, 1) lp_tc_fwd_kernel(const __grid_constant
             __syncwarp();
             if (!ok) break;
             tc_fence_after();
-            const int b = tile / tiles_per_seq, t = (tile % tiles_per_seq) * 128 + r;
-            logo_bf16* dst = p.u_g + ((static_cast<int64_t>(b) * p.T + t) * p.H + h) * D;
+            // 16 x 256-bit pieces, four lanes trading bf16 pairs (quad_gather8): a warp
+            // store is 8 rows of 64 contiguous bytes, not 32 rows of 16
+            const int b = tile / tiles_per_seq, t0 = (tile % tiles_per_seq) * 128 + quad * 32;
+            logo_bf16* dst = p.u_g + ((static_cast<int64_t>(b) * p.T + t0) * p.H + h) * D + (lane & 3) * 8;
 #pragma unroll
             for (int c = 0; c < D / 32; ++c) {
-                uint32_t v[32];
-                tmem_ld32(tmem + lane_off + st * D + c * 32, v);
+                uint32_t v[2][16];
+#pragma unroll
+                for (int hf = 0; hf < 2; ++hf)
+                    tmem_ld_16x256b_x4(tmem + lane_off + (static_cast<uint32_t>(hf * 16) << 16) + st * D + c * 32, v[hf]);
                 tmem_wait_ld();
                 if (c == D / 32 - 1) {
                     tc_fence_before();
                     mbar_arrive(smem_u32(&bar_t_empty[st]));
                 }
-                if (t < p.T) {
 #pragma unroll
-                    for (int q4 = 0; q4 < 4; ++q4) {
-                        uint4 w;
-                        w.x = pack_bf16x2(__uint_as_float(v[8 * q4 + 0]), __uint_as_float(v[8 * q4 + 1]));
-                        w.y = pack_bf16x2(__uint_as_float(v[8 * q4 + 2]), __uint_as_float(v[8 * q4 + 3]));
-                        w.z = pack_bf16x2(__uint_as_float(v[8 * q4 + 4]), __uint_as_float(v[8 * q4 + 5]));
-                        w.w = pack_bf16x2(__uint_as_float(v[8 * q4 + 6]), __uint_as_float(v[8 * q4 + 7]));
-                        *reinterpret_cast<uint4*>(dst + c * 32 + q4 * 8) = w;
+                for (int hf = 0; hf < 2; ++hf)
+#pragma unroll
+                    for (int ab = 0; ab < 2; ++ab) {
+                        uint32_t w[4];
+#pragma unroll
+                        for (int k4 = 0; k4 < 4; ++k4)
+                            w[k4] = cvt_bf16x2(__uint_as_float(v[hf][4 * k4 + 2 * ab]),
+                                               __uint_as_float(v[hf][4 * k4 + 2 * ab + 1]));
+                        const uint4 o = quad_gather8(w, lane);
+                        const int row = hf * 16 + ab * 8 + (lane >> 2);
+                        if (t0 + row < p.T) *reinterpret_cast<uint4*>(dst + static_cast<int64_t>(row) * p.H * D + c * 32) = o;
                     }
-                }
             }
         }
     }
@@ -570,44 +497,71 @@ int launch_lp_tc_fwd(const logo_bf16* u_l, const logo_bf16* a, const logo_dims& 
     return cudaGetLastError() == cudaSuccess ? LOGO_OK : LOGO_ERR_CUDA;
 }
 
-// LP backward on every row, d = 128, with tcgen05.  Per 128-row tile of one
-// head: dU = dG A_h^T (A_h read as the K-major B operand: its rows are the
-// output dimension i, its columns the contracted j) into one of two TMEM
-// buffers, drained to du_l by warps 2..5; and dA_h += U^T dG (both tiles read
-// as MN-major operands: rows are the contracted dimension) accumulated in TMEM
-// over all the CTA's tiles, written as the CTA's partial at the end.
-struct LpTcBwdParams {
-    CUtensorMap tm_u, tm_g, tm_a;
+// LP backward with tcgen05, on every row (K, V) or on the packed selected rows
+// (Q).  A tile is 128 rows of 128 columns: one head of d = 128, or two
+// adjacent heads of d = 64 (a CTA keeps its heads and walks a strided share of
+// the row tiles).  Per tile: dU = dG A_h^T (A_h read as the K-major B operand:
+// its rows are the output dimension i, its columns the contracted j), per head,
+// into one of two TMEM buffers, drained to du_l by the epilogue warps; and
+// dA += U^T dG (both tiles read as MN-major operands: rows are the contracted
+// dimension), accumulated in TMEM over all the CTA's tiles and written as its
+// partial at the end (d = 64: the two 64 x 64 blocks on the diagonal; the
+// cross products of the two heads cost nothing that is in short supply).
+// Every row: tiles come by TMA.  Selected rows: four producer warps copy the
+// rows, wherever their tokens are, into the same swizzled layout (cp.async, one
+// tile ahead).  What dU is added to (accumulate) comes in the same way, as a
+// third tile; an epilogue warp adds its rows in place (a row a lane), reads them
+// back two whole rows a step and stores those.  (Reading and storing global
+// memory from the accumulator's layout, even as 64-byte pieces, left the load
+// latency and the lane exchange on the tile's path.)  With 3 tiles a stage only
+// one CTA fits an SM; memory bounds it: B2 T2432 d128, dA's sum over the
+// partials included: every row of 8 heads, added to dU (40 MB), 24 + 5 us when
+// stored from the accumulator's layout, now 17.5 + 4.2; half the rows of 32
+// heads (119 MB), 34 + 8 us with mma.sync tiles, now 15 + 5.6.
+constexpr int kMaxChunks = 32;  // partial dA per head at most (the workspace)
+
+struct LpBwdParams {
+    CUtensorMap tm_u, tm_g, tm_a, tm_d;
+    const logo_bf16* u_l;
+    const logo_bf16* du_g;
     logo_bf16* du_l;
     float* part;  // [H][gridDim.x][D][D]
+    RowSet rows;  // selected rows (GATHER)
     int B, T, H, accumulate;
 };
 
-struct LpTcBwdCfg {
-    static constexpr int D = 128;
+template <int D>
+struct LpBwdCfg {
+    static constexpr int kHeads = 128 / D;           // heads per CTA
     static constexpr int kHalf = 128 * 128;          // [128 rows][64] bf16
-    static constexpr int kTile = 2 * kHalf;          // 128 rows x 128
+    static constexpr int kTile = 2 * kHalf;          // 128 rows x 128 columns
+    static constexpr int kHalfA = D * 128;           // [D rows][64] bf16
     static constexpr int kOffA = 0;
-    static constexpr int kOffU = kTile;              // 2 stages of (U, G)
-    static constexpr int kSmemBytes = kOffU + 4 * kTile + 1024;
+    static constexpr int kOffU = 2 * kHalfA;         // 2 stages of (U, G, dU)
+    static constexpr int kStage = 3 * kTile;
+    static constexpr int kSmemBytes = kOffU + 2 * kStage + 1024;
     static constexpr uint32_t kColDA = 256;          // dU buffers at 0 and 128
     static constexpr uint32_t kTmemCols = 512;
 };
+constexpr int kLpBwdThreads = 288;  // warps 0..3 producers (TMA: one thread), 4 MMA issuer, 5..8 epilogue
 
-__global__ void __launch_bounds__(192, 1) lp_tc_bwd_kernel(const __grid_constant__ LpTcBwdParams p)
+template <int D, bool GATHER>
+__global__ void __launch_bounds__(kLpBwdThreads, 1) lp_tc_bwd_kernel(const __grid_constant__ LpBwdParams p)
 {
-    using C = LpTcBwdCfg;
-    constexpr int D = C::D;
+    using C = LpBwdCfg<D>;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     __shared__ __align__(8) uint64_t bar_a, bar_in_full[2], bar_in_empty[2], bar_t_full[2], bar_t_empty[2];
-    __shared__ __align__(8) uint64_t bar_da, bar_drain;
+    __shared__ __align__(8) uint64_t bar_d_empty[2], bar_da, bar_drain;
     __shared__ uint32_t tmem_sh;
     __shared__ volatile int abort_flag;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int h = blockIdx.y;
+    const int h0 = blockIdx.y * C::kHeads, heads = min(C::kHeads, p.H - h0);
+    const int cols = heads * D;                      // columns that exist (64 at an odd last head of d = 64)
+    const int row_elems = p.H * D;
     const int tiles_per_seq = (p.T + 127) / 128;
-    const int ntiles = p.B * tiles_per_seq;
+    const int n = GATHER ? row_count(p.rows) : 0;    // packed rows
+    const int ntiles = GATHER ? (n + 127) / 128 : p.B * tiles_per_seq;
     const uint32_t sA = smem_u32(smem + C::kOffA), sIn = smem_u32(smem + C::kOffU);
     if (threadIdx.x == 0) {
         abort_flag = 0;
@@ -615,14 +569,15 @@ __global__ void __launch_bounds__(192, 1) lp_tc_bwd_kernel(const __grid_constant
         mbar_init(smem_u32(&bar_da), 1);
         mbar_init(smem_u32(&bar_drain), 1);
         for (int s = 0; s < 2; ++s) {
-            mbar_init(smem_u32(&bar_in_full[s]), 1);
+            mbar_init(smem_u32(&bar_in_full[s]), GATHER ? 128 : 1);
             mbar_init(smem_u32(&bar_in_empty[s]), 1);
             mbar_init(smem_u32(&bar_t_full[s]), 1);
             mbar_init(smem_u32(&bar_t_empty[s]), 128);
+            mbar_init(smem_u32(&bar_d_empty[s]), 128);
         }
         fence_mbar_init();
     }
-    if (warp == 1) {
+    if (warp == 4) {
         tmem_alloc(smem_u32(&tmem_sh), C::kTmemCols);
         tmem_relinquish();
     }
@@ -630,38 +585,100 @@ __global__ void __launch_bounds__(192, 1) lp_tc_bwd_kernel(const __grid_constant
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_sh;
-    if (warp == 0) {
-        if (lane == 0) {
-            tma_prefetch_desc(&p.tm_u);
-            tma_prefetch_desc(&p.tm_g);
+    if (warp < 4) {
+        if (warp == 0 && lane == 0) {  // A_h of the CTA's heads, once
             tma_prefetch_desc(&p.tm_a);
-            const uint64_t pol = policy_evict_first(), pol_a = policy_evict_last();
-            mbar_arrive_expect_tx(smem_u32(&bar_a), C::kTile);
-            for (int s = 0; s < 2; ++s) tma_load_4d(sA + s * C::kHalf, &p.tm_a, smem_u32(&bar_a), 64 * s, 0, h * D, 0, pol_a);
-            int k = 0;
-            bool ok = true;
-            for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++k) {
-                const int st = k & 1;
-                if (!(ok = mbar_wait(smem_u32(&bar_in_empty[st]), ((k >> 1) & 1) ^ 1, &abort_flag))) break;
-                const int b = tile / tiles_per_seq, t0 = (tile % tiles_per_seq) * 128;
-                const uint32_t bar = smem_u32(&bar_in_full[st]);
-                const uint32_t ub = sIn + st * 2 * C::kTile, gb = ub + C::kTile;
-                mbar_arrive_expect_tx(bar, 2 * C::kTile);
-                for (int s = 0; s < 2; ++s) {
-                    tma_load_4d(ub + s * C::kHalf, &p.tm_u, bar, 64 * s, h, t0, b, pol);
-                    tma_load_4d(gb + s * C::kHalf, &p.tm_g, bar, 64 * s, h, t0, b, pol);
-                }
-            }
-            if (!ok) {
-                mbar_wait_drain(smem_u32(&bar_a), 0);
-                for (int j = k - 2 > 0 ? k - 2 : 0; j < k; ++j)
-                    mbar_wait_drain(smem_u32(&bar_in_full[j & 1]), (j >> 1) & 1);
+            mbar_arrive_expect_tx(smem_u32(&bar_a), heads * D * D * 2);
+            if (D == 128) {
+                for (int s = 0; s < 2; ++s)
+                    tma_load_4d(sA + s * C::kHalfA, &p.tm_a, smem_u32(&bar_a), 64 * s, 0, h0 * D, 0, policy_evict_last());
+            } else {
+                for (int s = 0; s < heads; ++s)
+                    tma_load_4d(sA + s * C::kHalfA, &p.tm_a, smem_u32(&bar_a), 0, 0, (h0 + s) * D, 0, policy_evict_last());
             }
         }
-    } else if (warp == 1) {
+        bool ok = true;
+        if (!GATHER) {
+            // -------------------------------------------------------- producer (TMA)
+            if (warp == 0 && lane == 0) {
+                tma_prefetch_desc(&p.tm_u);
+                tma_prefetch_desc(&p.tm_g);
+                const uint64_t pol = policy_evict_first();
+                int k = 0;
+                for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++k) {
+                    const int st = k & 1;
+                    if (!(ok = mbar_wait(smem_u32(&bar_in_empty[st]), ((k >> 1) & 1) ^ 1, &abort_flag))) break;
+                    if (!(ok = mbar_wait(smem_u32(&bar_d_empty[st]), ((k >> 1) & 1) ^ 1, &abort_flag))) break;
+                    const int b = tile / tiles_per_seq, t0 = (tile % tiles_per_seq) * 128;
+                    const uint32_t bar = smem_u32(&bar_in_full[st]);
+                    const uint32_t ub = sIn + st * C::kStage, gb = ub + C::kTile, db = gb + C::kTile;
+                    // (a head past the last one of d = 64 reads as zeros)
+                    mbar_arrive_expect_tx(bar, (p.accumulate ? 3 : 2) * C::kTile);
+                    for (int s = 0; s < 2; ++s) {
+                        const int c0 = D == 128 ? 64 * s : 0, hh = D == 128 ? h0 : h0 + s;
+                        tma_load_4d(ub + s * C::kHalf, &p.tm_u, bar, c0, hh, t0, b, pol);
+                        tma_load_4d(gb + s * C::kHalf, &p.tm_g, bar, c0, hh, t0, b, pol);
+                        if (p.accumulate) tma_load_4d(db + s * C::kHalf, &p.tm_d, bar, c0, hh, t0, b, pol);
+                    }
+                }
+                if (!ok) {
+                    for (int j = k - 2 > 0 ? k - 2 : 0; j < k; ++j)
+                        mbar_wait_drain(smem_u32(&bar_in_full[j & 1]), (j >> 1) & 1);
+                }
+            }
+        } else {
+            // -------------------------------------------------------- producers (gathered rows)
+            // warp w copies rows 32w .. 32w + 31 of a tile: a row a step, lanes 0..15
+            // its U, lanes 16..31 its G; rows and columns that do not exist are zero
+            // (dU's rows, when added to, two a step)
+            const logo_bf16* src = (lane < 16 ? p.u_l : p.du_g) + h0 * D + (lane & 15) * 8;
+            const bool have = (lane & 15) * 8 < cols;
+            int k = 0;
+            for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++k) {
+                const int st = k & 1;
+                const int r = tile * 128 + warp * 32 + lane;
+                const int tok = r < n ? static_cast<int>(row_token(p.rows, r)) : -1;
+                ok = mbar_wait(smem_u32(&bar_in_empty[st]), ((k >> 1) & 1) ^ 1, &abort_flag) &&
+                     mbar_wait(smem_u32(&bar_d_empty[st]), ((k >> 1) & 1) ^ 1, &abort_flag);
+                __syncwarp();
+                if (!(ok = __all_sync(0xffffffffu, ok))) break;
+                const uint32_t half = sIn + st * C::kStage + ((lane & 15) >> 3) * C::kHalf;
+                const uint32_t base = half + (lane < 16 ? 0 : C::kTile);
+#pragma unroll 8
+                for (int i = 0; i < 32; ++i) {
+                    const int t = __shfl_sync(0xffffffffu, tok, i);
+                    const uint32_t dst = base + sw128_offset(warp * 32 + i, lane & 7);
+                    if (t >= 0 && have) cp_async16(dst, src + static_cast<int64_t>(t) * row_elems);
+                    else st_shared_v4(dst, 0u, 0u, 0u, 0u);
+                }
+                if (p.accumulate) {
+#pragma unroll 8
+                    for (int i = 0; i < 16; ++i) {
+                        const int row = 2 * i + (lane >> 4), t = __shfl_sync(0xffffffffu, tok, row);
+                        if (t >= 0 && have)
+                            cp_async16(half + 2 * C::kTile + sw128_offset(warp * 32 + row, lane & 7),
+                                       p.du_l + static_cast<int64_t>(t) * row_elems + h0 * D + (lane & 15) * 8);
+                    }
+                }
+                cp_async_commit();
+                if (k > 0) {  // tile k-1 has landed while tile k was issued
+                    cp_async_wait_one();
+                    fence_proxy_async_smem();
+                    mbar_arrive(smem_u32(&bar_in_full[st ^ 1]));
+                }
+            }
+            cp_async_wait_all();
+            if (ok && k > 0) {
+                fence_proxy_async_smem();
+                mbar_arrive(smem_u32(&bar_in_full[(k - 1) & 1]));
+            }
+        }
+        if (!ok && warp == 0 && lane == 0) mbar_wait_drain(smem_u32(&bar_a), 0);
+    } else if (warp == 4) {
+        // ------------------------------------------------------------ MMA issuer
         if (lane == 0) {
             constexpr uint32_t id_du = idesc_bf16_f32(128, D, false, false);  // G K-major x A_h K-major
-            constexpr uint32_t id_da = idesc_bf16_f32(D, D, true, true);      // U^T, G: both MN-major
+            constexpr uint32_t id_da = idesc_bf16_f32(128, 128, true, true);  // U^T, G: both MN-major
             bool ok = mbar_wait(smem_u32(&bar_a), 0, &abort_flag);
             int k = 0;
             for (int tile = blockIdx.x; ok && tile < ntiles; tile += gridDim.x, ++k) {
@@ -669,13 +686,15 @@ __global__ void __launch_bounds__(192, 1) lp_tc_bwd_kernel(const __grid_constant
                 if (!(ok = mbar_wait(smem_u32(&bar_in_full[st]), (k >> 1) & 1, &abort_flag))) break;
                 if (!(ok = mbar_wait(smem_u32(&bar_t_empty[st]), ((k >> 1) & 1) ^ 1, &abort_flag))) break;
                 tc_fence_after();
-                const uint32_t ub = sIn + st * 2 * C::kTile, gb = ub + C::kTile;
+                const uint32_t ub = sIn + st * C::kStage, gb = ub + C::kTile;
 #pragma unroll
-                for (int ks = 0; ks < D / 16; ++ks) {  // contracted: j
-                    const uint32_t off = (ks >> 2) * C::kHalf + (ks & 3) * 32;
-                    umma_bf16_ss(tmem + st * D, sdesc_sw128(gb + off, 16, 1024), sdesc_sw128(sA + off, 16, 1024), id_du,
-                                 ks > 0 ? 1u : 0u);
-                }
+                for (int s = 0; s < C::kHeads; ++s)
+#pragma unroll
+                    for (int ks = 0; ks < D / 16; ++ks) {  // contracted: j
+                        const uint32_t half = ks >> 2, in = (ks & 3) * 32;
+                        umma_bf16_ss(tmem + st * 128 + s * D, sdesc_sw128(gb + (s + half) * C::kHalf + in, 16, 1024),
+                                     sdesc_sw128(sA + (s + half) * C::kHalfA + in, 16, 1024), id_du, ks > 0 ? 1u : 0u);
+                    }
 #pragma unroll
                 for (int ks = 0; ks < 128 / 16; ++ks) {  // contracted: the tile's rows
                     umma_bf16_ss(tmem + C::kColDA, sdesc_sw128(ub + ks * 2048, C::kHalf, 1024),
@@ -693,106 +712,136 @@ __global__ void __launch_bounds__(192, 1) lp_tc_bwd_kernel(const __grid_constant
             }
         }
     } else {
+        // ------------------------------------------------------------ epilogue
         const int quad = warp & 3;
-        const int r = quad * 32 + lane;
         const uint32_t lane_off = static_cast<uint32_t>(quad * 32) << 16;
+        logo_bf16* out = p.du_l + h0 * D + (lane & 15) * 8;
         int k = 0;
         bool ok = true;
         for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++k) {
             const int st = k & 1;
-            ok = mbar_wait(smem_u32(&bar_t_full[st]), (k >> 1) & 1, &abort_flag);
+            const uint32_t db = sIn + st * C::kStage + 2 * C::kTile;
+            // token of this lane's row (-1: no such row)
+            int tok;
+            if (GATHER) {
+                const int r = tile * 128 + quad * 32 + lane;
+                tok = r < n ? static_cast<int>(row_token(p.rows, r)) : -1;
+            } else {
+                const int b = tile / tiles_per_seq, t = (tile % tiles_per_seq) * 128 + quad * 32 + lane;
+                tok = t < p.T ? b * p.T + t : -1;
+            }
+            // the tile's dU has landed (with U and G), and the product is there
+            ok = mbar_wait(smem_u32(&bar_in_full[st]), (k >> 1) & 1, &abort_flag) &&
+                 mbar_wait(smem_u32(&bar_t_full[st]), (k >> 1) & 1, &abort_flag);
             __syncwarp();
             if (!ok) break;
             tc_fence_after();
-            const int b = tile / tiles_per_seq, t = (tile % tiles_per_seq) * 128 + r;
-            logo_bf16* dst = p.du_l + ((static_cast<int64_t>(b) * p.T + t) * p.H + h) * D;
 #pragma unroll
-            for (int c = 0; c < D / 32; ++c) {
+            for (int c = 0; c < 4; ++c) {
                 uint32_t v[32];
-                tmem_ld32(tmem + lane_off + st * D + c * 32, v);
+                tmem_ld32(tmem + lane_off + st * 128 + c * 32, v);
                 tmem_wait_ld();
-                if (c == D / 32 - 1) {
+                if (c == 3) {
                     tc_fence_before();
                     mbar_arrive(smem_u32(&bar_t_empty[st]));
                 }
-                if (t < p.T) {
 #pragma unroll
-                    for (int q4 = 0; q4 < 4; ++q4) {
-                        float x[8];
+                for (int q4 = 0; q4 < 4; ++q4) {
+                    const int chunk = c * 4 + q4;
+                    const uint32_t at = db + (chunk >> 3) * C::kHalf + sw128_offset(quad * 32 + lane, chunk & 7);
+                    float x[8];
 #pragma unroll
-                        for (int e = 0; e < 8; ++e) x[e] = __uint_as_float(v[8 * q4 + e]);
-                        uint4* dp = reinterpret_cast<uint4*>(dst + c * 32 + q4 * 8);
-                        if (p.accumulate) {
-                            const uint4 old = *dp;
-                            const __nv_bfloat162* o2 = reinterpret_cast<const __nv_bfloat162*>(&old);
+                    for (int e = 0; e < 8; ++e) x[e] = __uint_as_float(v[8 * q4 + e]);
+                    if (p.accumulate) {
+                        const uint4 old = ld_shared_v4(at);
+                        const __nv_bfloat162* o2 = reinterpret_cast<const __nv_bfloat162*>(&old);
 #pragma unroll
-                            for (int e = 0; e < 4; ++e) {
-                                const float2 f = __bfloat1622float2(o2[e]);
-                                x[2 * e] += f.x;
-                                x[2 * e + 1] += f.y;
-                            }
+                        for (int e = 0; e < 4; ++e) {
+                            const float2 f = __bfloat1622float2(o2[e]);
+                            x[2 * e] += f.x;
+                            x[2 * e + 1] += f.y;
                         }
-                        uint4 w;
-                        w.x = pack_bf16x2(x[0], x[1]);
-                        w.y = pack_bf16x2(x[2], x[3]);
-                        w.z = pack_bf16x2(x[4], x[5]);
-                        w.w = pack_bf16x2(x[6], x[7]);
-                        *dp = w;
                     }
+                    st_shared_v4(at, cvt_bf16x2(x[0], x[1]), cvt_bf16x2(x[2], x[3]), cvt_bf16x2(x[4], x[5]),
+                                 cvt_bf16x2(x[6], x[7]));
                 }
             }
+            __syncwarp();
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {  // two whole rows (of this warp's) a store
+                const int row = 2 * i + (lane >> 4), t = __shfl_sync(0xffffffffu, tok, row);
+                const uint4 w = ld_shared_v4(db + ((lane & 15) >> 3) * C::kHalf + sw128_offset(quad * 32 + row, lane & 7));
+                if (t >= 0 && (lane & 15) * 8 < cols)
+                    *reinterpret_cast<uint4*>(out + static_cast<int64_t>(t) * row_elems) = w;
+            }
+            fence_proxy_async_smem();  // the stage's next copies come after these reads and writes
+            mbar_arrive(smem_u32(&bar_d_empty[st]));
         }
-        // the CTA's dA partial: lane r holds row i = r, columns j
-        float* pp = p.part + ((static_cast<int64_t>(h) * gridDim.x + blockIdx.x) * D + r) * D;
-        if (ok && k == 0) {  // no tile: a zero partial (the launch gives every CTA one)
-            for (int j = 0; j < D; j += 4) *reinterpret_cast<float4*>(pp + j) = make_float4(0.f, 0.f, 0.f, 0.f);
+        // the CTA's dA partial: lane r holds row i = r % D of head h0 + r / D
+        const int r = quad * 32 + lane, s = r / D, i = r % D;
+        float* pp = p.part + ((static_cast<int64_t>(h0 + s) * gridDim.x + blockIdx.x) * D + i) * D;
+        if (ok && k == 0) {  // no tile: a zero partial
+            if (s < heads)
+                for (int j = 0; j < D; j += 4) *reinterpret_cast<float4*>(pp + j) = make_float4(0.f, 0.f, 0.f, 0.f);
         } else if (ok && mbar_wait(smem_u32(&bar_da), 0, &abort_flag)) {
             tc_fence_after();
+            const int first = (quad * 32 / D) * D;  // the head's columns (the same for the warp)
 #pragma unroll
             for (int c = 0; c < D / 32; ++c) {
                 uint32_t v[32];
-                tmem_ld32(tmem + lane_off + C::kColDA + c * 32, v);
+                tmem_ld32(tmem + lane_off + C::kColDA + first + c * 32, v);
                 tmem_wait_ld();
+                if (s < heads) {
 #pragma unroll
-                for (int e = 0; e < 32; e += 4)
-                    *reinterpret_cast<float4*>(pp + c * 32 + e) =
-                        make_float4(__uint_as_float(v[e]), __uint_as_float(v[e + 1]), __uint_as_float(v[e + 2]),
-                                    __uint_as_float(v[e + 3]));
+                    for (int e = 0; e < 32; e += 4)
+                        *reinterpret_cast<float4*>(pp + c * 32 + e) =
+                            make_float4(__uint_as_float(v[e]), __uint_as_float(v[e + 1]), __uint_as_float(v[e + 2]),
+                                        __uint_as_float(v[e + 3]));
+                }
             }
         }
     }
     tc_fence_before();
     __syncthreads();
-    if (warp == 1) {
+    if (warp == 4) {
         tc_fence_after();
         tmem_dealloc(tmem, C::kTmemCols);
     }
 }
 
-int launch_lp_tc_bwd(const logo_bf16* u_l, const logo_bf16* a, const logo_bf16* du_g, const logo_dims& d,
-                     logo_bf16* du_l, int accumulate, float* da, float* part, cudaStream_t st)
+template <int D, bool GATHER>
+int launch_lp_tc_bwd(const logo_bf16* u_l, const logo_bf16* a, const logo_bf16* du_g, const RowSet& rows,
+                     const logo_dims& d, logo_bf16* du_l, int accumulate, float* da, float* part, cudaStream_t st)
 {
-    constexpr int D = 128;
-    LpTcBwdParams prm{};
+    using C = LpBwdCfg<D>;
+    LpBwdParams prm{};
     if (!encode_bf16_4d(&prm.tm_u, u_l, D, d.Hq, d.T, d.B, 64, 128) ||
         !encode_bf16_4d(&prm.tm_g, du_g, D, d.Hq, d.T, d.B, 64, 128) ||
+        !encode_bf16_4d(&prm.tm_d, du_l, D, d.Hq, d.T, d.B, 64, 128) ||
         !encode_bf16_4d(&prm.tm_a, a, D, 1, static_cast<uint64_t>(d.Hq) * D, 1, 64, D))
         return LOGO_ERR_CUDA;
+    prm.u_l = u_l;
+    prm.du_g = du_g;
     prm.du_l = du_l;
     prm.part = part;
+    prm.rows = rows;
     prm.B = d.B;
     prm.T = d.T;
     prm.H = d.Hq;
     prm.accumulate = accumulate;
-    if (set_smem_limit(lp_tc_bwd_kernel, LpTcBwdCfg::kSmemBytes) != cudaSuccess) return LOGO_ERR_CUDA;
-    const int ntiles = d.B * ((d.T + 127) / 128);
-    int per_head = device_sm_count() / d.Hq;
-    per_head = per_head < 1 ? 1 : (per_head > ntiles ? ntiles : per_head);
-    per_head = per_head > kChunksPerHead ? kChunksPerHead : per_head;  // the workspace holds that many partials
-    lp_tc_bwd_kernel<<<dim3(per_head, d.Hq), 192, LpTcBwdCfg::kSmemBytes, st>>>(prm);
+    if (set_smem_limit(lp_tc_bwd_kernel<D, GATHER>, C::kSmemBytes) != cudaSuccess) return LOGO_ERR_CUDA;
+    // one CTA an SM; selected rows: the tiles are not known here, every row is the most
+    const int groups = (d.Hq + C::kHeads - 1) / C::kHeads;
+    const int ntiles = GATHER ? (d.B * d.T + 127) / 128 : d.B * ((d.T + 127) / 128);
+    int per_group = device_sm_count() / groups;
+    per_group = per_group < 1 ? 1 : (per_group > ntiles ? ntiles : per_group);
+    per_group = per_group > kMaxChunks ? kMaxChunks : per_group;
+    const int rounds = (ntiles + per_group - 1) / per_group;
+    per_group = (ntiles + rounds - 1) / rounds;  // the fewest partial dA for as many rounds
+    lp_tc_bwd_kernel<D, GATHER><<<dim3(per_group, groups), kLpBwdThreads, C::kSmemBytes, st>>>(prm);
     if (cudaGetLastError() != cudaSuccess) return LOGO_ERR_CUDA;
-    const int64_t total = static_cast<int64_t>(d.Hq) * D * D;
-    reduce_parts_kernel<<<static_cast<unsigned>((total + 255) / 256), 256, 0, st>>>(part, per_head, D * D, d.Hq, da);
+    const int64_t vecs = static_cast<int64_t>(d.Hq) * D * D / 4;
+    reduce_parts_kernel<<<static_cast<unsigned>((vecs + 63) / 64), 256, 0, st>>>(part, per_group, D * D, d.Hq, da);
     return cudaGetLastError() == cudaSuccess ? LOGO_OK : LOGO_ERR_CUDA;
 }
 
@@ -832,20 +881,6 @@ int launch_lp_fwd(const logo_bf16* u_l, const logo_bf16* a, const RowSet& R, int
     int chunks = per_sm * device_sm_count() / H;
     chunks = chunks < 1 ? 1 : chunks > 64 ? 64 : chunks;
     lp_fwd_kernel<D><<<dim3(chunks, H), 128, smem, st>>>(u_l, a, R, H, u_g);
-    return cudaGetLastError() == cudaSuccess ? LOGO_OK : LOGO_ERR_CUDA;
-}
-
-template <int D>
-int launch_lp_bwd(const logo_bf16* u_l, const logo_bf16* a, const logo_bf16* du_g, const RowSet& R, int H,
-                  logo_bf16* du_l, int accumulate, float* da, float* part, cudaStream_t st)
-{
-    const int smem = D * D * 2 + 2 * kTileRows * D * 2;
-    if (set_smem_limit(lp_bwd_kernel<D>, smem) != cudaSuccess) return LOGO_ERR_CUDA;
-    lp_bwd_kernel<D><<<dim3(kChunksPerHead, H), D * 2, smem, st>>>(u_l, a, du_g, R, H, du_l, accumulate, part);
-    if (cudaGetLastError() != cudaSuccess) return LOGO_ERR_CUDA;
-    const int64_t total = static_cast<int64_t>(H) * D * D;
-    reduce_parts_kernel<<<static_cast<unsigned>((total + 255) / 256), 256, 0, st>>>(part, kChunksPerHead, D * D, H,
-                                                                                   da);
     return cudaGetLastError() == cudaSuccess ? LOGO_OK : LOGO_ERR_CUDA;
 }
 
@@ -889,7 +924,7 @@ extern "C" size_t logo_branch_transform_bwd_workspace_size(logo_dims dims)
 {
     if (dims.B < 1 || dims.T < 1 || dims.Hq < 1 || (dims.D != 64 && dims.D != 128) || dims.Hq * dims.D > 8192)
         return 0;
-    const size_t lp = static_cast<size_t>(dims.Hq) * kChunksPerHead * dims.D * dims.D * sizeof(float);
+    const size_t lp = static_cast<size_t>(dims.Hq) * kMaxChunks * dims.D * dims.D * sizeof(float);
     const size_t so = static_cast<size_t>(so_bwd_blocks(dims)) * 2 * dims.Hq * dims.D * sizeof(float);
     return lp > so ? lp : so;
 }
@@ -912,12 +947,12 @@ extern "C" int logo_branch_transform_bwd(const logo_bf16* u_l, const logo_bf16* 
     const RowSet R{pos, cu_q, n_sel_total, dims.B, dims.T};
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     float* part = static_cast<float*>(workspace);
-    if (a_lp && !pos && dims.D == 128)  // every row: the tcgen05 pipeline
-        return launch_lp_tc_bwd(u_l, a_lp, du_g, dims, du_l, accumulate, da_lp, part, st);
-    if (a_lp) {
-        return dims.D == 128 ? launch_lp_bwd<128>(u_l, a_lp, du_g, R, dims.Hq, du_l, accumulate, da_lp, part, st)
-                             : launch_lp_bwd<64>(u_l, a_lp, du_g, R, dims.Hq, du_l, accumulate, da_lp, part, st);
-    }
+    if (a_lp && dims.D == 128)
+        return pos ? launch_lp_tc_bwd<128, true>(u_l, a_lp, du_g, R, dims, du_l, accumulate, da_lp, part, st)
+                   : launch_lp_tc_bwd<128, false>(u_l, a_lp, du_g, R, dims, du_l, accumulate, da_lp, part, st);
+    if (a_lp)
+        return pos ? launch_lp_tc_bwd<64, true>(u_l, a_lp, du_g, R, dims, du_l, accumulate, da_lp, part, st)
+                   : launch_lp_tc_bwd<64, false>(u_l, a_lp, du_g, R, dims, du_l, accumulate, da_lp, part, st);
     const int grid = so_bwd_blocks(dims);
     switch (so_vpt(dims)) {
         case 1: so_bwd_kernel<1><<<grid, 256, 0, st>>>(u_l, s_so, du_g, R, dims.Hq, dims.D, du_l, accumulate, part); break;
