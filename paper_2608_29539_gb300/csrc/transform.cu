@@ -514,10 +514,10 @@ int launch_lp_tc_fwd(const logo_bf16* u_l, const logo_bf16* a, const logo_dims& 
 // back two whole rows a step and stores those.  (Reading and storing global
 // memory from the accumulator's layout, even as 64-byte pieces, left the load
 // latency and the lane exchange on the tile's path.)  With 3 tiles a stage only
-// one CTA fits an SM; memory bounds it: B2 T2432 d128, dA's sum over the
-// partials included: every row of 8 heads, added to dU (40 MB), 24 + 5 us when
-// stored from the accumulator's layout, now 17.5 + 4.2; half the rows of 32
-// heads (119 MB), 34 + 8 us with mma.sync tiles, now 15 + 5.6.
+// one CTA fits an SM; memory bounds it.  T8192 d128, dA's sum over the partials
+// included: every row of 8 heads, added to dU (67 MB), 24 + 5 us when stored
+// from the accumulator's layout, now 17.5 + 4.2; an eighth of the rows of 32
+// heads (34 MB), 34 + 8 us with mma.sync tiles, now 15 + 5.6.
 constexpr int kMaxChunks = 32;  // partial dA per head at most (the workspace)
 
 struct LpBwdParams {
