@@ -502,14 +502,15 @@ __global__ void __launch_bounds__(Bwd2Cfg::kThreads, 1) attn_bwd2_kernel(const _
     } else if (warp < 14) {
         // ------------------------------------------------------------ dQ drain, dK/dV epilogue
         const int quad = warp & 3;
-        const int t = quad * 32 + lane;  // head-dim row of dQ^T; key row of dK/dV
+        const int t = quad * 32 + lane;  // head-dim row of dQ^T
         const uint32_t lane_off = static_cast<uint32_t>(quad * 32) << 16;
         int u = 0, kv_items = 0;
         bool ok = true;
         for (int k = blockIdx.x; k < n_items && ok; k += gridDim.x) {
             const BwdItem it = decode_bwd2<BQ, GLOBAL>(p, k);
-            const int key = it.j * kBN + t;
-            const int64_t kv_off = ((static_cast<int64_t>(it.b) * p.T + key) * p.Hkv + it.kvh) * D;
+            const int64_t kv_off =
+                ((static_cast<int64_t>(it.b) * p.T + it.j * kBN + quad * 32) * p.Hkv + it.kvh) * D;  // this warp's first key
+            const int keys = p.T - (it.j * kBN + quad * 32);  // keys of the warp that exist (may exceed 32, or be negative)
             if (it.ntiles == 0) {
                 // no selected query sees the block: zero dK, dV rows, two whole
                 // rows (16 lanes x 16 bytes each) per warp store, this warp's 32 keys
@@ -557,31 +558,41 @@ __global__ void __launch_bounds__(Bwd2Cfg::kThreads, 1) attn_bwd2_kernel(const _
             __syncwarp();
             if (!ok) break;
             tc_fence_after();
+            // 16 x 256-bit pieces, four lanes trading bf16 pairs (quad_gather8): a warp
+            // store is 8 rows of 64 contiguous bytes, not 32 rows of 16, which took
+            // 5800 clocks an item behind the reductions, with every role waiting
+            // (2 x 4K, 16 heads, 1/8 selected: the kernel 78 -> 71 us)
 #pragma unroll
             for (int which = 0; which < 2; ++which) {
                 const uint32_t col = which == 0 ? C::kColDK : C::kColDV;
                 const float mul = which == 0 ? p.scale : 1.0f;
-                logo_bf16* dst = (which == 0 ? p.dk : p.dv) + kv_off;
+                logo_bf16* dst = (which == 0 ? p.dk : p.dv) + kv_off + (lane & 3) * 8;
 #pragma unroll
                 for (int cc = 0; cc < D / 32; ++cc) {
-                    uint32_t v[32];
-                    tmem_ld32(tmem + lane_off + col + cc * 32, v);
-                    tmem_wait_ld();
-                    if (key < p.T) {
+                    uint32_t v[2][16];
 #pragma unroll
-                        for (int q4 = 0; q4 < 4; ++q4) {
-                            uint4 w;
-                            w.x = pack_bf16x2(__uint_as_float(v[8 * q4 + 0]) * mul, __uint_as_float(v[8 * q4 + 1]) * mul);
-                            w.y = pack_bf16x2(__uint_as_float(v[8 * q4 + 2]) * mul, __uint_as_float(v[8 * q4 + 3]) * mul);
-                            w.z = pack_bf16x2(__uint_as_float(v[8 * q4 + 4]) * mul, __uint_as_float(v[8 * q4 + 5]) * mul);
-                            w.w = pack_bf16x2(__uint_as_float(v[8 * q4 + 6]) * mul, __uint_as_float(v[8 * q4 + 7]) * mul);
-                            *reinterpret_cast<uint4*>(dst + cc * 32 + q4 * 8) = w;
-                        }
+                    for (int hf = 0; hf < 2; ++hf)
+                        tmem_ld_16x256b_x4(tmem + lane_off + (static_cast<uint32_t>(hf * 16) << 16) + col + cc * 32, v[hf]);
+                    tmem_wait_ld();
+                    if (which == 1 && cc == D / 32 - 1) {
+                        tc_fence_before();
+                        mbar_arrive(smem_u32(&bar_dkv_empty));
                     }
+#pragma unroll
+                    for (int hf = 0; hf < 2; ++hf)
+#pragma unroll
+                        for (int ab = 0; ab < 2; ++ab) {
+                            uint32_t w[4];
+#pragma unroll
+                            for (int k4 = 0; k4 < 4; ++k4)
+                                w[k4] = cvt_bf16x2(__uint_as_float(v[hf][4 * k4 + 2 * ab]) * mul,
+                                                   __uint_as_float(v[hf][4 * k4 + 2 * ab + 1]) * mul);
+                            const uint4 o = quad_gather8(w, lane);
+                            const int r = hf * 16 + ab * 8 + (lane >> 2);
+                            if (r < keys) *reinterpret_cast<uint4*>(dst + static_cast<int64_t>(r) * p.Hkv * D + cc * 32) = o;
+                        }
                 }
             }
-            tc_fence_before();
-            mbar_arrive(smem_u32(&bar_dkv_empty));
             ++kv_items;
         }
     } else if (GLOBAL) {
