@@ -93,27 +93,4 @@ __device__ __forceinline__ int seq_of_row(const int32_t* cu_q, int B, int row)
     return lo;
 }
 
-// Gather the selected rows of the dense Q into the packed layout (App. B) and
-// zero the 128 rows after the last one, so that a partial final tile reads
-// finite values.
-static __global__ void __launch_bounds__(256)
-    gather_rows_kernel(const logo_bf16* __restrict__ q, const int32_t* __restrict__ pos,
-                       const int32_t* __restrict__ cu_q, const int32_t* __restrict__ n_sel, int B, int T,
-                       int row_elems, logo_bf16* __restrict__ qc)
-{
-    const int n = *n_sel;
-    const int vecs = row_elems / 8;
-    for (int row = blockIdx.x; row < n + kBM; row += gridDim.x) {
-        uint4* dst = reinterpret_cast<uint4*>(qc + static_cast<int64_t>(row) * row_elems);
-        if (row < n) {
-            const int b = seq_of_row(cu_q, B, row);
-            const uint4* src =
-                reinterpret_cast<const uint4*>(q + (static_cast<int64_t>(b) * T + pos[row]) * row_elems);
-            for (int v = threadIdx.x; v < vecs; v += blockDim.x) dst[v] = src[v];
-        } else {
-            for (int v = threadIdx.x; v < vecs; v += blockDim.x) dst[v] = make_uint4(0, 0, 0, 0);
-        }
-    }
-}
-
 }  // namespace logo

@@ -38,8 +38,8 @@
 // three-region traversal; for the local branch the window edge is a second
 // masked region), and inside a masked block only the 32-key groups a row
 // sees in part are tested key by key.  Global items come from a schedule
-// ordered by cost (longest first) that a one-block kernel builds on the
-// device, so nothing here needs the selected count on the host.
+// ordered by cost (longest first) that one block of the kernel before builds on
+// the device, so nothing here needs the selected count on the host.
 #include <cuda_bf16.h>
 
 #include <cstdint>
@@ -810,15 +810,11 @@ __device__ __forceinline__ int sched_block_scan(int v, int* total, int* sh)
     return r;
 }
 
-__global__ void __launch_bounds__(1024) global_schedule_kernel(const int32_t* __restrict__ pos,
-                                                               const int32_t* __restrict__ cu_q, int B, int Hq,
-                                                               int n_sm, int32_t* __restrict__ tile_off,
-                                                               GlobalTile* __restrict__ unsorted,
-                                                               GlobalTile* __restrict__ sorted,
-                                                               int32_t* __restrict__ n_tiles,
-                                                               int32_t* __restrict__ next_item,
-                                                               SplitTile* __restrict__ splits,
-                                                               int32_t* __restrict__ n_splits)
+__device__ __forceinline__ void global_schedule(const int32_t* __restrict__ pos, const int32_t* __restrict__ cu_q, int B,
+                                                int Hq, int n_sm, int32_t* __restrict__ tile_off,
+                                                GlobalTile* __restrict__ unsorted, GlobalTile* __restrict__ sorted,
+                                                int32_t* __restrict__ n_tiles, int32_t* __restrict__ next_item,
+                                                SplitTile* __restrict__ splits, int32_t* __restrict__ n_splits)
 {
     __shared__ int sh_nt, sh_chunk, sh_worth;
     __shared__ int sh_scan[33];
@@ -939,6 +935,50 @@ __global__ void __launch_bounds__(1024) global_schedule_kernel(const int32_t* __
     }
 }
 
+struct GlobalFwdWs {
+    logo_bf16* qc;
+    GlobalTile* unsorted;
+    GlobalTile* sorted;
+    int32_t* tile_off;
+    int32_t* n_tiles;
+    int32_t* next_item;
+    int32_t* n_splits;
+    SplitTile* splits;
+    float* o_part;
+    float* m_part;
+    float* l_part;
+};
+
+// Both preparations of a global call in one launch: block 0 makes the schedule,
+// the others gather the selected rows of the dense Q into the packed layout
+// (App. B), 256 threads a row, and zero the 128 rows after the last one, so that
+// a partial final tile reads finite values.  Each is a chain of a few dependent
+// loads in a launch of its own otherwise, one after the other (5-7.5 and 5-6 us
+// on the device at 2 x 4K to 16K tokens; together 6-8).
+__global__ void __launch_bounds__(1024) global_prep_kernel(const logo_bf16* __restrict__ q, const int32_t* __restrict__ pos,
+                                                           const int32_t* __restrict__ cu_q,
+                                                           const int32_t* __restrict__ n_sel, int B, int T, int Hq,
+                                                           int row_elems, int n_sm, GlobalFwdWs ws)
+{
+    if (blockIdx.x == 0) {
+        global_schedule(pos, cu_q, B, Hq, n_sm, ws.tile_off, ws.unsorted, ws.sorted, ws.n_tiles, ws.next_item, ws.splits,
+                        ws.n_splits);
+        return;
+    }
+    const int n = *n_sel;
+    const int vecs = row_elems / 8;
+    for (int row = (blockIdx.x - 1) * 4 + (threadIdx.x >> 8); row < n + kBM; row += (gridDim.x - 1) * 4) {
+        uint4* dst = reinterpret_cast<uint4*>(ws.qc + static_cast<int64_t>(row) * row_elems);
+        if (row < n) {
+            const int b = seq_of_row(cu_q, B, row);
+            const uint4* src = reinterpret_cast<const uint4*>(q + (static_cast<int64_t>(b) * T + pos[row]) * row_elems);
+            for (int v = threadIdx.x & 255; v < vecs; v += 256) dst[v] = src[v];
+        } else {
+            for (int v = threadIdx.x & 255; v < vecs; v += 256) dst[v] = make_uint4(0, 0, 0, 0);
+        }
+    }
+}
+
 // Combine the shares of every split tile: per (row, head), M = max_s m_s,
 // L = sum_s 2^(m_s - M) l_s, O = sum_s 2^(m_s - M) O_s / L, lse = (M + log2 L)
 // ln 2.  A share whose keys the row cannot see has m_s = -inf and weighs 0.
@@ -991,20 +1031,6 @@ __global__ void __launch_bounds__(128) merge_splits_kernel(const SplitTile* __re
         if (g == 0) lse[static_cast<int64_t>(h) * cap + st.row0 + r] = (M + log2f(L)) * kLn2;
     }
 }
-
-struct GlobalFwdWs {
-    logo_bf16* qc;
-    GlobalTile* unsorted;
-    GlobalTile* sorted;
-    int32_t* tile_off;
-    int32_t* n_tiles;
-    int32_t* next_item;
-    int32_t* n_splits;
-    SplitTile* splits;
-    float* o_part;
-    float* m_part;
-    float* l_part;
-};
 
 size_t global_fwd_ws_layout(const logo_dims& d, char* base, GlobalFwdWs* ws)
 {
@@ -1134,11 +1160,9 @@ extern "C" int logo_global_sparse_attn_fwd(const logo_bf16* q, const logo_bf16* 
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int cap = dims.B * dims.T;
     const int row_elems = dims.Hq * dims.D;
-    const int gather_grid = max(1, min(cap + kBM, device_sm_count() * 8));
-    gather_rows_kernel<<<gather_grid, 256, 0, st>>>(q, pos, cu_q, n_sel_total, dims.B, dims.T, row_elems, ws.qc);
     const int n_sm = device_sm_count();
-    global_schedule_kernel<<<1, 1024, 0, st>>>(pos, cu_q, dims.B, dims.Hq, n_sm, ws.tile_off, ws.unsorted, ws.sorted,
-                                               ws.n_tiles, ws.next_item, ws.splits, ws.n_splits);
+    const int grid = 1 + min((cap + kBM + 3) / 4, n_sm * 2 - 1);
+    global_prep_kernel<<<grid, 1024, 0, st>>>(q, pos, cu_q, n_sel_total, dims.B, dims.T, dims.Hq, row_elems, n_sm, ws);
     if (cudaGetLastError() != cudaSuccess) return LOGO_ERR_CUDA;
     FwdParams prm{};
     if (!encode_bf16_4d(&prm.tm_q, ws.qc, dims.D, dims.Hq, static_cast<uint64_t>(cap) + kBM, 1, 64, kBM) ||
