@@ -56,8 +56,11 @@ struct BwdParams {
     CUtensorMap tm_k;   // [B,T,Hkv,D]
     CUtensorMap tm_v;
     CUtensorMap tm_dq;  // d = 64: dq_acc, for the bulk reductions
-    const float* lse;   // local [B,Hq,T]; global [Hq,cap]
+    const float* lse;   // d = 128: local [B,Hq,T]; global [Hq,cap]
     const float* dsum;  // same layout as lse
+    const float4* stats;  // d = 64: local [B,Hq][stat_rows / 2], global [Hq][stat_rows / 2] (RowStats)
+    const int32_t* pos_c; // d = 64, global: pos, on a 16-byte boundary
+    int64_t stat_rows;
     float* dq_acc;      // local [B,T,Hq,D]; global [cap+128,Hq,D]
     logo_bf16* dk;      // [B,T,Hkv,D]
     logo_bf16* dv;
@@ -615,7 +618,7 @@ __global__ void __launch_bounds__(Bwd2Cfg::kThreads, 1) attn_bwd2_kernel(const _
 // of N = 64 (dV with P^T as the TMEM operand, dK, dQ).  Roles:
 //   warp 0       TMA: K/V of an item into one of two buffers (the next item's
 //                land during this one: an item has only a few tiles), Q/dO
-//                tiles through a 3-deep ring
+//                tiles and their rows' lse and Dsum through a 3-deep ring
 //   warp 1       MMA issuer A: S^T, dP^T
 //   warp 2       MMA issuer B: dV, dK, dQ
 //   warp 3       global branch: zero rows of the dense dQ for unselected tokens
@@ -653,8 +656,8 @@ struct Bwd64Cfg {
     static constexpr uint32_t kTmemCols = 512;
     static constexpr int kThreads = 512;
     // launched at 128 registers a thread (512 x 128 = 65,536); the softmax
-    // warpgroups hold 64 columns of S^T and dP^T a thread (this split compiles
-    // without spills): 128 x (64 + 176 + 176 + 96) = 65,536
+    // warpgroups hold 64 columns of S^T and dP^T a thread (of the splits this one
+    // spills least, four words): 128 x (64 + 176 + 176 + 96) = 65,536
     static constexpr uint32_t kRegsControl = 64;
     static constexpr uint32_t kRegsSoftmax = 176;
     static constexpr uint32_t kRegsDrain = 96;
@@ -671,18 +674,34 @@ __global__ void __launch_bounds__(Bwd64Cfg::kThreads, 1) attn_bwd64_kernel(const
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     __shared__ __align__(8) uint64_t bar_kv_full[2], bar_kv_empty[2], bar_dkv_full, bar_dkv_empty, bar_drain, bar_drain_b;
     __shared__ __align__(8) uint64_t bar_qdo_full[NS], bar_qdo_empty[NS];
-    __shared__ __align__(8) uint64_t bar_st_full, bar_st_empty, bar_stage, bar_ds_full, bar_dq_full, bar_dq_empty;
+    __shared__ __align__(8) uint64_t bar_st_full, bar_st_empty, bar_ds_full, bar_dq_full, bar_dq_empty;
     __shared__ uint32_t tmem_base_sh;
     __shared__ volatile int abort_flag;
-    __shared__ int sh_pos[2][BQ];
-    // per pair of query columns (2c, 2c+1): (-lse_2c, -lse_2c+1, -Dsum_2c, -Dsum_2c+1), lse in log2 units
-    __shared__ float4 sh_pair[2][BQ / 2];
-    __shared__ int sh_open[2][BQ / 32];  // per staging warp: every column sees every key of the block
+    // of a stage's query columns (2c, 2c+1): (-lse_2c, -lse_2c+1, -Dsum_2c, -Dsum_2c+1),
+    // lse in log2 units, and (global) their positions
+    __shared__ __align__(16) float4 sh_pair[NS][BQ / 2];
+    __shared__ __align__(16) int sh_pos[NS][BQ];
+    constexpr uint32_t kStageBytes = 2 * C::kTileBytes + sizeof(sh_pair[0]) + (GLOBAL ? sizeof(sh_pos[0]) : 0);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t sKV = smem_u32(smem + C::kOffKV), sQ = smem_u32(smem + C::kOffQ), sDS = smem_u32(smem + C::kOffDS);
     const int group = p.Hq / p.Hkv;
     const int n_items = p.B * p.nblk * p.Hkv;
+
+    // no divisions in the roles' loops: the next tile of an item (head by head),
+    // the next stage of the ring and the parity of its turn
+    auto next_tile = [](const BwdItem& it, int& h, int& i) {
+        if (++i == it.i_lo + it.ntiles) {
+            i = it.i_lo;
+            ++h;
+        }
+    };
+    auto next_stage = [](int& st, int& turn) {
+        if (++st == NS) {
+            st = 0;
+            turn ^= 1;
+        }
+    };
 
     if (threadIdx.x == 0) {
         abort_flag = 0;
@@ -700,7 +719,6 @@ __global__ void __launch_bounds__(Bwd64Cfg::kThreads, 1) attn_bwd64_kernel(const
         mbar_init(smem_u32(&bar_drain_b), 1);
         mbar_init(smem_u32(&bar_st_full), 1);
         mbar_init(smem_u32(&bar_st_empty), 256);
-        mbar_init(smem_u32(&bar_stage), 256);
         mbar_init(smem_u32(&bar_ds_full), 256);
         mbar_init(smem_u32(&bar_dq_full), 1);
         mbar_init(smem_u32(&bar_dq_empty), 128);
@@ -726,7 +744,7 @@ __global__ void __launch_bounds__(Bwd64Cfg::kThreads, 1) attn_bwd64_kernel(const
                 tma_prefetch_desc(&p.tm_v);
                 const uint64_t pol_q = policy_evict_last();
                 const uint64_t pol_kv = policy_evict_first();
-                int u = 0, kv_items = 0;
+                int u = 0, st = 0, turn = 0, kv_items = 0;
                 bool ok = true;
                 for (int k = blockIdx.x; k < n_items && ok; k += gridDim.x) {
                     const BwdItem it = decode_bwd2<BQ, GLOBAL>(p, k);
@@ -739,16 +757,18 @@ __global__ void __launch_bounds__(Bwd64Cfg::kThreads, 1) attn_bwd64_kernel(const
                     tma_load_4d(sKV + (kb * 2 + 1) * C::kTileBytes, &p.tm_v, kvb, 0, it.kvh, it.j * kBN, it.b, pol_kv);
                     ++kv_items;
                     const int n_it = group * it.ntiles;
-                    for (int x = 0; x < n_it; ++x, ++u) {
-                        const int h = it.kvh * group + x / it.ntiles;
-                        const int i = it.i_lo + x % it.ntiles;
-                        const int st = u % NS, f = u / NS;
-                        if (!(ok = mbar_wait(smem_u32(&bar_qdo_empty[st]), (f & 1) ^ 1, &abort_flag))) break;
+                    for (int x = 0, h = it.kvh * group, i = it.i_lo; x < n_it; ++x, ++u) {
+                        if (!(ok = mbar_wait(smem_u32(&bar_qdo_empty[st]), turn ^ 1, &abort_flag))) break;
                         const uint32_t qb = smem_u32(&bar_qdo_full[st]);
-                        mbar_arrive_expect_tx(qb, 2 * C::kTileBytes);
+                        mbar_arrive_expect_tx(qb, kStageBytes);
                         const int cb = GLOBAL ? 0 : it.b;
+                        const int64_t plane = GLOBAL ? h : static_cast<int64_t>(it.b) * p.Hq + h;
+                        bulk_load(smem_u32(sh_pair[st]), p.stats + (plane * p.stat_rows + i * BQ) / 2, sizeof(sh_pair[0]), qb);
+                        if (GLOBAL) bulk_load(smem_u32(sh_pos[st]), p.pos_c + i * BQ, sizeof(sh_pos[0]), qb);
                         tma_load_4d(sQ + st * 2 * C::kTileBytes, &p.tm_q, qb, 0, h, i * BQ, cb, pol_q);
                         tma_load_4d(sQ + (st * 2 + 1) * C::kTileBytes, &p.tm_do, qb, 0, h, i * BQ, cb, pol_q);
+                        next_tile(it, h, i);
+                        next_stage(st, turn);
                     }
                 }
                 if (!ok) {  // let copies already issued land before the CTA exits
@@ -762,7 +782,7 @@ __global__ void __launch_bounds__(Bwd64Cfg::kThreads, 1) attn_bwd64_kernel(const
             // -------------------------------------------------------- MMA issuer A: S^T, dP^T
             if (lane == 0) {
                 constexpr uint32_t idS = idesc_bf16_f32(kBN, BQ, false, false);
-                int u = 0, kv_items = 0;
+                int u = 0, st = 0, turn = 0, kv_items = 0;
                 bool ok = true;
                 for (int k = blockIdx.x; k < n_items && ok; k += gridDim.x) {
                     const BwdItem it = decode_bwd2<BQ, GLOBAL>(p, k);
@@ -771,8 +791,7 @@ __global__ void __launch_bounds__(Bwd64Cfg::kThreads, 1) attn_bwd64_kernel(const
                     if (!(ok = mbar_wait(smem_u32(&bar_kv_full[kv_items & 1]), (kv_items >> 1) & 1, &abort_flag))) break;
                     const int n_it = group * it.ntiles;
                     for (int x = 0; x < n_it; ++x, ++u) {
-                        const int st = u % NS;
-                        if (!(ok = mbar_wait(smem_u32(&bar_qdo_full[st]), (u / NS) & 1, &abort_flag))) break;
+                        if (!(ok = mbar_wait(smem_u32(&bar_qdo_full[st]), turn, &abort_flag))) break;
                         // the softmax warps have loaded S^T, dP^T of tile u-1
                         if (!(ok = mbar_wait(smem_u32(&bar_st_empty), (u & 1) ^ 1, &abort_flag))) break;
                         tc_fence_after();
@@ -785,6 +804,7 @@ __global__ void __launch_bounds__(Bwd64Cfg::kThreads, 1) attn_bwd64_kernel(const
                                          sdesc_sw128(ob + ks * 32, 16, 1024), idS, ks > 0 ? 1u : 0u);
                         }
                         umma_commit(smem_u32(&bar_st_full));
+                        next_stage(st, turn);
                     }
                     if (!ok) break;
                     ++kv_items;
@@ -799,7 +819,7 @@ __global__ void __launch_bounds__(Bwd64Cfg::kThreads, 1) attn_bwd64_kernel(const
             if (lane == 0) {
                 constexpr uint32_t idKV = idesc_bf16_f32(kBN, D, false, true);  // dV, dK: keys x d
                 constexpr uint32_t idQ = idesc_bf16_f32(BQ, D, true, true);     // dQ: queries x d
-                int u = 0, kv_items = 0;
+                int u = 0, st = 0, turn = 0, kv_items = 0;
                 bool ok = true;
                 for (int k = blockIdx.x; k < n_items && ok; k += gridDim.x) {
                     const BwdItem it = decode_bwd2<BQ, GLOBAL>(p, k);
@@ -807,7 +827,6 @@ __global__ void __launch_bounds__(Bwd64Cfg::kThreads, 1) attn_bwd64_kernel(const
                     const uint32_t sK = sKV + (kv_items & 1) * 2 * C::kTileBytes;
                     const int n_it = group * it.ntiles;
                     for (int x = 0; x < n_it; ++x, ++u) {
-                        const int st = u % NS;
                         if (!(ok = mbar_wait(smem_u32(&bar_ds_full), u & 1, &abort_flag))) break;
                         if (x == 0 && !(ok = mbar_wait(smem_u32(&bar_dkv_empty), (kv_items & 1) ^ 1, &abort_flag))) break;
                         tc_fence_after();
@@ -830,6 +849,7 @@ __global__ void __launch_bounds__(Bwd64Cfg::kThreads, 1) attn_bwd64_kernel(const
                             umma_bf16_ss(tmem + C::kColDQ, sdesc_sw128(sDS + ks * 2048, 16384, 1024),
                                          sdesc_sw128(sK + ks * 2048, 16384, 1024), idQ, ks > 0 ? 1u : 0u);
                         umma_commit(smem_u32(&bar_dq_full));
+                        next_stage(st, turn);
                     }
                     if (!ok) break;
                     umma_commit(smem_u32(&bar_kv_empty[kv_items & 1]));
@@ -850,64 +870,39 @@ __global__ void __launch_bounds__(Bwd64Cfg::kThreads, 1) attn_bwd64_kernel(const
         const int quad = warp & 3;
         const int half = (warp - 4) >> 2;  // query columns half*64 .. half*64+63
         const int t = quad * 32 + lane;    // key row of the block
-        const int tw = threadIdx.x - 128;  // 0..255 across both warpgroups
         const uint32_t lane_off = static_cast<uint32_t>(quad * 32) << 16;
-        int u = 0;
+        int u = 0, st = 0, turn = 0;
         bool ok = true;
         for (int k = blockIdx.x; k < n_items && ok; k += gridDim.x) {
             const BwdItem it = decode_bwd2<BQ, GLOBAL>(p, k);
             if (it.ntiles == 0) continue;
             const int k0 = it.j * kBN;
             const int key = k0 + t;
-            const int n_it = group * it.ntiles;
-            // staging values of a tile's query columns (position, lse, Dsum; -1 / 0 /
-            // 0 outside its rows): loaded one tile ahead by the first warpgroup
-            int pf_pos = -1;
-            float pf_lse = 0.f, pf_dsum = 0.f;
-            auto load_stage = [&](int x) {
-                const int h = it.kvh * group + x / it.ntiles;
-                const int i = it.i_lo + x % it.ntiles;
-                pf_pos = -1;
-                pf_lse = pf_dsum = 0.f;
-                const int row = i * BQ + tw;
-                if (!GLOBAL ? row < p.T : (row >= it.row_lo && row < it.row_hi)) {
-                    const int64_t idx = GLOBAL ? static_cast<int64_t>(h) * p.cap + row
-                                               : (static_cast<int64_t>(it.b) * p.Hq + h) * p.T + row;
-                    pf_pos = GLOBAL ? p.pos[row] : row;
-                    pf_lse = p.lse[idx];
-                    pf_dsum = p.dsum[idx];
-                }
-            };
-            if (tw < BQ) load_stage(0);
-            for (int x = 0; x < n_it; ++x, ++u) {
-                const int b = u & 1;
-                if (tw < BQ) {
-                    const bool pf_open = pf_pos >= k0 + kBN - 1 && (GLOBAL || pf_pos - k0 < p.window);
-                    sh_pos[b][tw] = pf_pos;
-                    float* pr = reinterpret_cast<float*>(&sh_pair[b][tw >> 1]);
-                    pr[tw & 1] = -(pf_lse * kLog2e);
-                    pr[2 + (tw & 1)] = -pf_dsum;
-                    const bool all_open = __all_sync(0xffffffffu, pf_open);
-                    if (lane == 0) sh_open[b][tw >> 5] = all_open ? 1 : 0;
-                }
-                mbar_arrive(smem_u32(&bar_stage));
-                ok = mbar_wait(smem_u32(&bar_stage), u & 1, &abort_flag);
+            const int row_first = it.i_lo * BQ, row_end = row_first + it.ntiles * BQ;
+            int row0 = row_first;
+            for (int left = group * it.ntiles; left > 0; --left, ++u) {
+                ok = mbar_wait(smem_u32(&bar_qdo_full[st]), turn, &abort_flag);
+                __syncwarp();
                 if (!ok) break;
-                if (tw < BQ && x + 1 < n_it) load_stage(x + 1);
-                const bool open = sh_open[b][2 * half] && sh_open[b][2 * half + 1];
+                // every column of the half sees every key of the block
+                bool open;
+                {
+                    const int r0 = row0 + half * 64, r1 = r0 + 63;
+                    if (!GLOBAL) open = r0 >= k0 + kBN - 1 && r1 < p.T && r1 - k0 < p.window;
+                    else open = r0 >= it.row_lo && r1 < it.row_hi && sh_pos[st][half * 64] >= k0 + kBN - 1;
+                }
                 // the columns that see this key are adjacent: [lo, hi] of this half
                 int lo = 0, hi = 63;
                 if (!open) {
-                    const int i = it.i_lo + x % it.ntiles;
                     if (!GLOBAL) {
-                        lo = key - i * BQ;
-                        hi = min(lo + p.window - 1, p.T - 1 - i * BQ);
+                        lo = key - row0;
+                        hi = min(lo + p.window - 1, p.T - 1 - row0);
                     } else {  // positions ascend over the sequence's rows of the tile
-                        int a = max(0, it.row_lo - i * BQ), e = min(BQ, it.row_hi - i * BQ);
+                        int a = max(0, it.row_lo - row0), e = min(BQ, it.row_hi - row0);
                         hi = e - 1;
                         while (a < e) {
                             const int mid = (a + e) >> 1;
-                            if (sh_pos[b][mid] < key) a = mid + 1;
+                            if (sh_pos[st][mid] < key) a = mid + 1;
                             else e = mid;
                         }
                         lo = a;
@@ -941,7 +936,7 @@ __global__ void __launch_bounds__(Bwd64Cfg::kThreads, 1) attn_bwd64_kernel(const
                         if constexpr (kMasked) m = column_mask(lo - 32 * c, hi - 32 * c);
 #pragma unroll
                         for (int e = 0; e < 32; e += 2) {
-                            const float4 q = sh_pair[b][(half * 64 + c * 32 + e) >> 1];
+                            const float4 q = sh_pair[st][(half * 64 + c * 32 + e) >> 1];
                             float x0, x1;
                             f2_unpack(f2_fma(f2_pack(__uint_as_float(sv[c][e]), __uint_as_float(sv[c][e + 1])), scale2,
                                              f2_pack(q.x, q.y)),
@@ -978,6 +973,8 @@ __global__ void __launch_bounds__(Bwd64Cfg::kThreads, 1) attn_bwd64_kernel(const
                 fence_proxy_async_smem();
                 tc_fence_before();
                 mbar_arrive(smem_u32(&bar_ds_full));
+                row0 = row0 + BQ == row_end ? row_first : row0 + BQ;
+                next_stage(st, turn);
             }
         }
     } else {
@@ -1006,9 +1003,8 @@ __global__ void __launch_bounds__(Bwd64Cfg::kThreads, 1) attn_bwd64_kernel(const
                 continue;
             }
             const int n_it = group * it.ntiles;
-            for (int x = 0; x < n_it; ++x, ++u) {
-                const int h = it.kvh * group + x / it.ntiles;
-                const int row0 = (it.i_lo + x % it.ntiles) * BQ + quad * 32;  // this warp's first query row
+            for (int x = 0, h = it.kvh * group, i = it.i_lo; x < n_it; ++x, ++u, next_tile(it, h, i)) {
+                const int row0 = i * BQ + quad * 32;  // this warp's first query row
                 ok = mbar_wait(smem_u32(&bar_dq_full), u & 1, &abort_flag);
                 __syncwarp();
                 if (!ok) break;
@@ -1099,6 +1095,22 @@ __global__ void __launch_bounds__(Bwd64Cfg::kThreads, 1) attn_bwd64_kernel(const
 // and build, for every sequence b and KV block j, the first packed row of b
 // whose position reaches the block's first key (App. B's precomputed search
 // that lets the backward skip every query tile before it).
+// For d = 64 the pass writes what the backward kernel needs of a row as the
+// kernel's shared memory holds it, (-lse, -lse, -Dsum, -Dsum) of two adjacent
+// rows with lse in log2 units, in planes of a multiple of 128 rows (rows that do
+// not exist are zero) and with the positions beside them: a tile's are then two
+// bulk copies that come with its Q and dO.  (Loaded, converted and stored by the
+// softmax warps with a barrier of all 256 threads, and divisions in the roles'
+// loops: 2 x 8K, 16 heads, 1/8 selected, all kernels of the call 158 -> 149 us.)
+struct RowStats {
+    const float* lse;  // local [B,H,T]; global [H,cap]
+    float* out;        // null: d = 128, dsum is written instead
+    int32_t* pos;      // global
+    int64_t rows;      // of a plane
+};
+
+__host__ __device__ constexpr int64_t stat_rows(int64_t rows) { return (rows + kBM - 1) / kBM * kBM; }
+
 struct GlobalPrep {
     const logo_bf16* q;   // dense [B, T, H, D]
     const int32_t* pos;
@@ -1113,7 +1125,7 @@ __global__ void __launch_bounds__(128) bwd_pre_kernel(const logo_bf16* __restric
                                                       const int32_t* __restrict__ n_sel, int rows_host, int T, int H,
                                                       int D, int cap, float* __restrict__ dsum,
                                                       logo_bf16* __restrict__ do_copy, float* __restrict__ dq_acc,
-                                                      GlobalPrep gp)
+                                                      GlobalPrep gp, RowStats rst)
 {
     const int n = GLOBAL ? *n_sel : rows_host;
     const int rows = GLOBAL ? n + kBM : rows_host;
@@ -1131,8 +1143,19 @@ __global__ void __launch_bounds__(128) bwd_pre_kernel(const logo_bf16* __restric
             gp.first_row[idx] = lo;
         }
     }
+    auto put_stats = [&](int64_t plane, int64_t r, float nlse, float ndsum) {
+        float* at = rst.out + (plane * rst.rows + (r & ~static_cast<int64_t>(1))) * 2 + (r & 1);
+        at[0] = nlse;
+        at[2] = ndsum;
+    };
+    if (!GLOBAL && rst.out) {  // the rows that fill a plane's last tile
+        const int pad = static_cast<int>(rst.rows) - T;
+        for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < rows / T * H * pad; idx += gridDim.x * blockDim.x)
+            put_stats(idx / pad, T + idx % pad, 0.f, 0.f);
+    }
     for (int row = blockIdx.x; row < rows; row += gridDim.x) {
         const bool live = row < n;
+        if (GLOBAL && rst.out && threadIdx.x == 0) rst.pos[row] = live ? gp.pos[row] : 0;
         const int64_t base = static_cast<int64_t>(row) * H * D;
         if (GLOBAL) {
             uint4* dst = reinterpret_cast<uint4*>(gp.qc + base);
@@ -1168,7 +1191,12 @@ __global__ void __launch_bounds__(128) bwd_pre_kernel(const logo_bf16* __restric
                 float4* z = reinterpret_cast<float4*>(dq_acc + base + h * D + jj * 8);
                 z[0] = make_float4(0.f, 0.f, 0.f, 0.f);
                 z[1] = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (live && jj == 0) {
+                if (jj == 0 && rst.out) {
+                    const int b = GLOBAL ? 0 : row / T, tt = GLOBAL ? row : row % T;
+                    const int64_t lse_row = GLOBAL ? static_cast<int64_t>(h) * cap + row
+                                                   : (static_cast<int64_t>(b) * H + h) * T + tt;
+                    put_stats(static_cast<int64_t>(b) * H + h, tt, live ? -(rst.lse[lse_row] * kLog2e) : 0.f, -acc);
+                } else if (live && jj == 0) {
                     if (GLOBAL) dsum[static_cast<int64_t>(h) * cap + row] = acc;
                     else {
                         const int b = row / T, tt = row % T;
@@ -1227,7 +1255,8 @@ __global__ void __launch_bounds__(128) bwd_post_kernel(const float* __restrict__
 struct BwdWs {
     logo_bf16* qc;
     logo_bf16* doc;
-    float* dsum;
+    float* dsum;  // d = 128; d = 64: the row stats
+    int32_t* pos_c;
     float* dq_acc;
     int32_t* first_row;
 };
@@ -1237,11 +1266,13 @@ size_t local_bwd_ws_layout(const logo_dims& d, char* base, BwdWs* ws)
     const size_t rows = static_cast<size_t>(d.B) * d.T;
     size_t off = 0;
     const size_t o_ds = off;
-    off = round_up(off + rows * d.Hq * sizeof(float), 256);
+    const size_t stats = d.D == 64 ? static_cast<size_t>(d.B) * stat_rows(d.T) * 2 : rows;
+    off = round_up(off + stats * d.Hq * sizeof(float), 256);
     const size_t o_dq = off;
     off = round_up(off + (rows + kBM) * d.Hq * d.D * sizeof(float), 256);
     if (ws) {
         ws->qc = ws->doc = nullptr;
+        ws->pos_c = nullptr;
         ws->dsum = reinterpret_cast<float*>(base + o_ds);
         ws->dq_acc = reinterpret_cast<float*>(base + o_dq);
         ws->first_row = nullptr;
@@ -1259,13 +1290,17 @@ size_t global_bwd_ws_layout(const logo_dims& d, char* base, BwdWs* ws)
     const size_t o_do = off;
     off = round_up(off + rows * d.Hq * d.D * 2, 256);
     const size_t o_ds = off;
-    off = round_up(off + cap * d.Hq * sizeof(float), 256);
+    const size_t stats = d.D == 64 ? static_cast<size_t>(stat_rows(rows)) * 2 : cap;
+    off = round_up(off + stats * d.Hq * sizeof(float), 256);
+    const size_t o_pc = off;
+    if (d.D == 64) off = round_up(off + stat_rows(rows) * sizeof(int32_t), 256);
     const size_t o_dq = off;
     off = round_up(off + rows * d.Hq * d.D * sizeof(float), 256);
     const size_t o_fr = off;
     off = round_up(off + static_cast<size_t>(d.B) * ((d.T + kBN - 1) / kBN) * sizeof(int32_t), 256);
     if (ws) {
         ws->first_row = reinterpret_cast<int32_t*>(base + o_fr);
+        ws->pos_c = reinterpret_cast<int32_t*>(base + o_pc);
         ws->qc = reinterpret_cast<logo_bf16*>(base + o_qc);
         ws->doc = reinterpret_cast<logo_bf16*>(base + o_do);
         ws->dsum = reinterpret_cast<float*>(base + o_ds);
@@ -1338,9 +1373,12 @@ extern "C" int logo_local_attn_bwd(const logo_bf16* q, const logo_bf16* k, const
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int rows = dims.B * dims.T;
     const int pre_grid = max(1, min(rows, device_sm_count() * 16));
+    const RowStats rst{lse, dims.D == 64 ? ws.dsum : nullptr, nullptr, stat_rows(dims.T)};
     bwd_pre_kernel<false><<<pre_grid, 128, 0, st>>>(o, dO, nullptr, rows, dims.T, dims.Hq, dims.D, 0, ws.dsum,
-                                                    nullptr, ws.dq_acc, GlobalPrep{});
+                                                    nullptr, ws.dq_acc, GlobalPrep{}, rst);
     BwdParams prm{};
+    prm.stats = reinterpret_cast<const float4*>(rst.out);
+    prm.stat_rows = rst.rows;
     const uint32_t qrows = dims.D == 128 ? Bwd2Cfg::kBQ : Bwd64Cfg::kBQ;
     if (!encode_bf16_4d(&prm.tm_q, q, dims.D, dims.Hq, dims.T, dims.B, 64, qrows) ||
         !encode_bf16_4d(&prm.tm_do, dO, dims.D, dims.Hq, dims.T, dims.B, 64, qrows) ||
@@ -1397,10 +1435,14 @@ extern "C" int logo_global_sparse_attn_bwd(const logo_bf16* q, const logo_bf16* 
     const int grid_rows = max(1, min(cap + kBM, device_sm_count() * 16));
     const int nblk = (dims.T + kBN - 1) / kBN;
     const GlobalPrep gp{q, pos, cu_q, ws.qc, ws.first_row, dims.B, nblk};
+    const RowStats rst{lse_c, dims.D == 64 ? ws.dsum : nullptr, ws.pos_c, stat_rows(static_cast<int64_t>(cap) + kBM)};
     bwd_pre_kernel<true><<<grid_rows, 128, 0, st>>>(o_c, dO_c, n_sel_total, 0, dims.T, dims.Hq, dims.D, cap, ws.dsum,
-                                                    ws.doc, ws.dq_acc, gp);
+                                                    ws.doc, ws.dq_acc, gp, rst);
     if (cudaGetLastError() != cudaSuccess) return LOGO_ERR_CUDA;
     BwdParams prm{};
+    prm.stats = reinterpret_cast<const float4*>(rst.out);
+    prm.pos_c = rst.pos;
+    prm.stat_rows = rst.rows;
     const uint32_t qrows = dims.D == 128 ? Bwd2Cfg::kBQ : Bwd64Cfg::kBQ;
     if (!encode_bf16_4d(&prm.tm_q, ws.qc, dims.D, dims.Hq, static_cast<uint64_t>(cap) + kBM, 1, 64, qrows) ||
         !encode_bf16_4d(&prm.tm_do, ws.doc, dims.D, dims.Hq, static_cast<uint64_t>(cap) + kBM, 1, 64, qrows) ||
