@@ -1192,7 +1192,13 @@ extern "C" int logo_global_sparse_attn_fwd(const logo_bf16* q, const logo_bf16* 
         static_cast<int>((static_cast<int64_t>(cap) / kBM + dims.B) * dims.Hq + kMaxPartialUnits);
     rc = dims.D == 128 ? launch_fwd<128, true>(prm, n_items_upper, st) : launch_fwd<64, true>(prm, n_items_upper, st);
     if (rc != LOGO_OK) return rc;
-    // always launched (a fixed launch sequence, capturable in a graph); exits at once without splits
+    // Splitting a tile takes kSplitMinGainBlocks of gain over shares of at least
+    // kMinSplitBlocks: with fewer blocks in a sequence nothing is ever split.
+    // Otherwise the merge is always launched (a fixed launch sequence, capturable
+    // in a graph); it exits at once without splits.  (Its launch was 3 of the 25 us
+    // of device time, and as much of the host's, in a 512-token layer.)
+    if ((dims.T + kBN - 1) / kBN < kMinSplitBlocks + kSplitMinGainBlocks)
+        return cudaGetLastError() == cudaSuccess ? LOGO_OK : LOGO_ERR_CUDA;
     const int merge_grid = n_sm * 4;
     if (dims.D == 128)
         merge_splits_kernel<128><<<merge_grid, 128, 0, st>>>(ws.splits, ws.n_splits, dims.Hq, cap, ws.o_part,
