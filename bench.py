@@ -176,6 +176,19 @@ def launches_per_step(w):
     return n
 
 
+def gpu_launches_per_step(w):
+    """The launches of a step as they are issued: the global forward's gather
+    and schedule share one, its merge has none in sequences too short to be
+    split (fewer than 32 blocks of 128 keys), and threshold selection takes
+    one for up to 128K tokens of the batch."""
+    n = launches_per_step(w) - 1
+    if -(-w.T // 128) < 32:
+        n -= 1
+    if w.mode != "ratio" and w.B * w.T <= 131072:
+        n -= LAUNCHES_PER_STEP["select"] - 1
+    return n
+
+
 def step_calls(layer, g):
     """The seven calls of one step, in order, as (name, thunk) pairs."""
     from paper_2608_29539_gb300 import logo as L
@@ -398,7 +411,7 @@ def routing_bench(layer, x, w, dev):
         L.logo_budget_update(rl_bufs[4], w.B, w.T, w.ratio, 2.0 ** -11, b_dev, f_out=f_dev)
 
     # each step reads the threshold the previous one wrote: 50 steps in one graph
-    return {"us_per_step": graph_ms(routing_step, 50) * 1e3, "launches_per_step": 4,
+    return {"us_per_step": graph_ms(routing_step, 50) * 1e3, "launches_per_step": 2 if w.B * w.T <= 131072 else 4,
             "note": "logo_select_device_threshold + logo_budget_update, no host sync; device time per step "
                     "(50 steps captured as one CUDA graph)"}
 
@@ -442,7 +455,7 @@ def fusions_bench(layer, x, w, dev, pk):
     ms = timed(gate)
     byts = ntok * dm * 2 + ntok * 4
     out["gate_select"] = {"ms": ms, "GB_per_s": byts / ms / 1e6, "frac_of_hbm_peak": byts / ms / 1e6 / pk["hbm"],
-                          "bytes": byts, "d_model": dm, "launches": 5}
+                          "bytes": byts, "d_model": dm, "launches": 2 if w.T <= 131072 else 5}
     ms = timed(gate_bwd)
     byts = 3 * ntok * dm * 2 + 2 * ntok * 4
     out["gate_bwd"] = {"ms": ms, "GB_per_s": byts / ms / 1e6, "frac_of_hbm_peak": byts / ms / 1e6 / pk["hbm"],
@@ -647,7 +660,7 @@ def native_arm(a, rank, world, local_rank, dist_on):
             "launch": ("one CUDA graph replay per step; the local calls on a second stream beside the "
                        "global calls" if graph is not None else "eager calls, one stream"),
             "eager_ms_per_step": eager_ms,
-            "gpu_launches": launches_per_step(w) * a.steps, "clocks": clk.summary()}
+            "gpu_launches": gpu_launches_per_step(w) * a.steps, "clocks": clk.summary()}
 
     # ---- dense comparison: the same global kernels with every token selected
     if not a.no_dense:
