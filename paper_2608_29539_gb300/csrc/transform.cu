@@ -518,7 +518,7 @@ int launch_lp_tc_fwd(const logo_bf16* u_l, const logo_bf16* a, const logo_dims& 
 // included: every row of 8 heads, added to dU (67 MB), 24 + 5 us when stored
 // from the accumulator's layout, now 17.5 + 4.2; an eighth of the rows of 32
 // heads (34 MB), 34 + 8 us with mma.sync tiles, now 15 + 5.6.
-constexpr int kMaxChunks = 32;  // partial dA per head at most (the workspace)
+constexpr int kMaxChunks = 32;  // partial dA per head at most
 
 struct LpBwdParams {
     CUtensorMap tm_u, tm_g, tm_a, tm_d;
@@ -809,6 +809,15 @@ __global__ void __launch_bounds__(kLpBwdThreads, 1) lp_tc_bwd_kernel(const __gri
     }
 }
 
+// CTAs a head (d = 64: a pair of heads) at most: one an SM.  As many partial dA
+// a head are in the workspace.
+int lp_bwd_chunks(const logo_dims& d)
+{
+    const int groups = d.D == 64 ? (d.Hq + 1) / 2 : d.Hq;
+    const int per_group = device_sm_count() / groups;
+    return per_group < 1 ? 1 : (per_group > kMaxChunks ? kMaxChunks : per_group);
+}
+
 template <int D, bool GATHER>
 int launch_lp_tc_bwd(const logo_bf16* u_l, const logo_bf16* a, const logo_bf16* du_g, const RowSet& rows,
                      const logo_dims& d, logo_bf16* du_l, int accumulate, float* da, float* part, cudaStream_t st)
@@ -830,12 +839,11 @@ int launch_lp_tc_bwd(const logo_bf16* u_l, const logo_bf16* a, const logo_bf16* 
     prm.H = d.Hq;
     prm.accumulate = accumulate;
     if (set_smem_limit(lp_tc_bwd_kernel<D, GATHER>, C::kSmemBytes) != cudaSuccess) return LOGO_ERR_CUDA;
-    // one CTA an SM; selected rows: the tiles are not known here, every row is the most
+    // selected rows: the tiles are not known here, every row is the most
     const int groups = (d.Hq + C::kHeads - 1) / C::kHeads;
     const int ntiles = GATHER ? (d.B * d.T + 127) / 128 : d.B * ((d.T + 127) / 128);
-    int per_group = device_sm_count() / groups;
-    per_group = per_group < 1 ? 1 : (per_group > ntiles ? ntiles : per_group);
-    per_group = per_group > kMaxChunks ? kMaxChunks : per_group;
+    int per_group = lp_bwd_chunks(d);
+    per_group = per_group > ntiles ? ntiles : per_group;
     const int rounds = (ntiles + per_group - 1) / per_group;
     per_group = (ntiles + rounds - 1) / rounds;  // the fewest partial dA for as many rounds
     lp_tc_bwd_kernel<D, GATHER><<<dim3(per_group, groups), kLpBwdThreads, C::kSmemBytes, st>>>(prm);
@@ -924,7 +932,7 @@ extern "C" size_t logo_branch_transform_bwd_workspace_size(logo_dims dims)
 {
     if (dims.B < 1 || dims.T < 1 || dims.Hq < 1 || (dims.D != 64 && dims.D != 128) || dims.Hq * dims.D > 8192)
         return 0;
-    const size_t lp = static_cast<size_t>(dims.Hq) * kMaxChunks * dims.D * dims.D * sizeof(float);
+    const size_t lp = static_cast<size_t>(dims.Hq) * lp_bwd_chunks(dims) * dims.D * dims.D * sizeof(float);
     const size_t so = static_cast<size_t>(so_bwd_blocks(dims)) * 2 * dims.Hq * dims.D * sizeof(float);
     return lp > so ? lp : so;
 }
