@@ -10,9 +10,9 @@
 // at d = 128 that is 64 FLOP/byte, more than the CUDA cores can keep up with
 // at HBM speed, so it runs on the tensor cores: tcgen05 pipelines over 128-row
 // tiles of a head beside that head's A_h in shared memory, one thread issuing
-// the MMAs into two TMEM buffers, four warps draining them (the forward on the
-// packed selected rows alone uses warp-level mma.sync over gathered 64-row
-// tiles).  The backward computes dU^L = dU^G A_h^T on the same tiles and
+// the MMAs into two TMEM buffers, four warps draining them; tiles of every row
+// come by TMA, tiles of the packed selected rows are gathered by four warps with
+// cp.async.  The backward computes dU^L = dU^G A_h^T on the same tiles and
 // accumulates dA_h = U^L^T dU^G; per-CTA partial dA are reduced in order by a
 // second kernel (deterministic).  SO is elementwise; its per-block ds, db are summed by the
 // fixed-order column sum of colsum.cuh (deterministic too).
@@ -27,8 +27,6 @@
 
 namespace logo {
 namespace {
-
-constexpr int kTileRows = 64;
 
 // Row r of the listed set -> token index b*T + t (all rows: r itself).
 struct RowSet {
@@ -50,14 +48,6 @@ __device__ __forceinline__ int64_t row_token(const RowSet& R, int r)
     return static_cast<int64_t>(b) * R.T + R.pos[r];
 }
 
-// [rows][D] bf16 tile in shared memory, 16-byte chunk c of row r stored at
-// chunk c ^ (r & 7): the 8 rows an ldmatrix reads hit 8 different bank groups.
-template <int D>
-__device__ __forceinline__ uint32_t toff(int row, int chunk)
-{
-    return static_cast<uint32_t>(row * (D * 2) + ((chunk ^ (row & 7)) << 4));
-}
-
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src)
 {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(src) : "memory");
@@ -65,131 +55,6 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src)
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_one() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
-
-__device__ __forceinline__ void st_shared_b32(uint32_t addr, uint32_t v)
-{
-    asm volatile("st.shared.b32 [%0], %1;\n" ::"r"(addr), "r"(v) : "memory");
-}
-
-// Start the copies of rows [0, nrows) of a tile (token indices in tok[]) of
-// head h into shared memory; rows past the end are zeroed with plain stores.
-// The copies complete at the caller's cp.async wait.
-template <int D>
-__device__ __forceinline__ void load_tile_async(uint32_t dst, const logo_bf16* src, const int64_t* tok, int nrows,
-                                                int H, int h, int nthreads)
-{
-    constexpr int kChunks = D / 8;
-    for (int idx = threadIdx.x; idx < kTileRows * kChunks; idx += nthreads) {
-        const int r = idx / kChunks, c = idx % kChunks;
-        if (r < nrows) cp_async16(dst + toff<D>(r, c), src + (tok[r] * H + h) * D + c * 8);
-        else st_shared_v4(dst + toff<D>(r, c), 0u, 0u, 0u, 0u);
-    }
-}
-
-template <int D>
-__device__ __forceinline__ void load_matrix_async(uint32_t dst, const logo_bf16* a, int nthreads)
-{
-    constexpr int kChunks = D / 8;
-    for (int idx = threadIdx.x; idx < D * kChunks; idx += nthreads) {
-        const int r = idx / kChunks, c = idx % kChunks;
-        cp_async16(dst + toff<D>(r, c), a + r * D + c * 8);
-    }
-}
-
-// token index of row r of the listed set, 0 past the end
-__device__ __forceinline__ int64_t tile_token(const RowSet& R, int n, int r) { return r < n ? row_token(R, r) : 0; }
-
-// LP forward: u_g[row] = u_l[row] A_h.  4 warps, 16 rows of the 64-row tile
-// each.  A block walks a strided share of its head's row tiles with two tile
-// buffers: the copies of A_h start before the row count is read, the token
-// lists of the first two tiles are looked up together, and tile k+2 is
-// fetched (cp.async) while tile k+1 is in flight and tile k is multiplied.
-// A warp writes its results back over its own 16 rows of the tile (the only
-// rows its MMAs read), so the stores to global memory leave as whole 2D-byte
-// row pieces, two rows per warp instruction, instead of 16-byte fragments.
-template <int D>
-__global__ void __launch_bounds__(128) lp_fwd_kernel(const logo_bf16* __restrict__ u_l,
-                                                     const logo_bf16* __restrict__ a, RowSet R, int H,
-                                                     logo_bf16* __restrict__ u_g)
-{
-    constexpr int kTileBytes = kTileRows * D * 2;
-    constexpr int kChunks = D / 8;
-    extern __shared__ __align__(128) uint8_t smem[];
-    __shared__ int64_t tok[2][kTileRows];
-    const uint32_t sA = smem_u32(smem), sU = sA + D * D * 2;
-    const int h = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int mi = lane >> 3, rr = lane & 7, gid = lane >> 2, tig = lane & 3;
-    load_matrix_async<D>(sA, a + static_cast<int64_t>(h) * D * D, 128);  // joins the first tile's group
-    const int n = row_count(R);
-    const int ntiles = (n + kTileRows - 1) / kTileRows;
-    const int step = gridDim.x;
-    int tile = blockIdx.x;
-    if (tile >= ntiles) {  // no tile: let A_h's copies land before the block exits
-        cp_async_wait_all();
-        return;
-    }
-    {  // threads 0..63: rows of the first tile, 64..127: rows of the second
-        const int which = threadIdx.x / kTileRows, r = threadIdx.x % kTileRows;
-        tok[which][r] = tile_token(R, n, (tile + which * step) * kTileRows + r);
-    }
-    __syncthreads();
-    load_tile_async<D>(sU, u_l, tok[0], min(kTileRows, n - tile * kTileRows), H, h, 128);
-    cp_async_commit();
-    if (tile + step < ntiles) {
-        load_tile_async<D>(sU + kTileBytes, u_l, tok[1], min(kTileRows, n - (tile + step) * kTileRows), H, h, 128);
-        cp_async_commit();
-    }
-    for (int k = 0; tile < ntiles; tile += step, ++k) {
-        const int buf = k & 1;
-        const int nr = min(kTileRows, n - tile * kTileRows);
-        if (tile + step < ntiles) cp_async_wait_one();  // tile k+1 may stay in flight
-        else cp_async_wait_all();
-        __syncthreads();
-        const uint32_t sT = sU + buf * kTileBytes;
-        float acc[D / 8][4];
-#pragma unroll
-        for (int nt = 0; nt < D / 8; ++nt)
-#pragma unroll
-            for (int i = 0; i < 4; ++i) acc[nt][i] = 0.f;
-#pragma unroll
-        for (int ks = 0; ks < D / 16; ++ks) {
-            uint32_t fa[4];
-            ldsm_x4(sT + toff<D>(warp * 16 + (mi & 1) * 8 + rr, 2 * ks + (mi >> 1)), fa[0], fa[1], fa[2], fa[3]);
-#pragma unroll
-            for (int np = 0; np < D / 16; ++np) {
-                uint32_t b0, b1, b2, b3;  // A_h rows k (input dim), columns n (output dim)
-                ldsm_x4_trans(sA + toff<D>(16 * ks + (mi & 1) * 8 + rr, 2 * np + (mi >> 1)), b0, b1, b2, b3);
-                mma_bf16_16816(acc[2 * np], fa, b0, b1);
-                mma_bf16_16816(acc[2 * np + 1], fa, b2, b3);
-            }
-        }
-        __syncwarp();
-#pragma unroll
-        for (int half = 0; half < 2; ++half) {
-            const int r = warp * 16 + gid + half * 8;
-#pragma unroll
-            for (int nt = 0; nt < D / 8; ++nt)
-                st_shared_b32(sT + toff<D>(r, nt) + 4 * tig, pack_bf16x2(acc[nt][2 * half], acc[nt][2 * half + 1]));
-        }
-        __syncwarp();
-#pragma unroll
-        for (int idx = lane; idx < 16 * kChunks; idx += 32) {
-            const int r = warp * 16 + idx / kChunks, c = idx % kChunks;
-            if (r < nr) {
-                const uint4 v = ld_shared_v4(sT + toff<D>(r, c));
-                *reinterpret_cast<uint4*>(u_g + (tok[buf][r] * H + h) * D + c * 8) = v;
-            }
-        }
-        __syncthreads();  // buffer buf and tok[buf] are free
-        const int after = tile + 2 * step;  // tile k+2 goes where tile k was
-        if (after < ntiles) {
-            if (threadIdx.x < kTileRows) tok[buf][threadIdx.x] = tile_token(R, n, after * kTileRows + threadIdx.x);
-            __syncthreads();
-            load_tile_async<D>(sT, u_l, tok[buf], min(kTileRows, n - after * kTileRows), H, h, 128);
-            cp_async_commit();
-        }
-    }
-}
 
 // out[h][e] = sum over c of part[h][c][e], e < per_head (a multiple of 4).
 // Thread (x, g) of a block adds chunks g, g + 4, .. of four columns, then the
@@ -318,17 +183,24 @@ __global__ void __launch_bounds__(256) so_bwd_kernel(const logo_bf16* __restrict
 }
 
 // ------------------------------------------------------------------------
-// LP on every row (K and V) with tcgen05: a tile is 128 rows of one head.
-// Roles: warp 0 TMA (A_h once, U tiles through a 2-deep ring), warp 1 MMA
-// issuer (D[128 x D] = U_tile A_h into one of two TMEM buffers), warps 2..5
-// epilogue (TMEM -> bf16 -> global).  A CTA keeps one head; the row tiles of
-// that head are strided over gridDim.x CTAs.  Shared memory: A_h as 64-column
-// halves of [D rows][64] (128-byte swizzle), read as the MN-major B operand;
-// U tiles as 64-column halves of [128 rows][64], the K-major A operand.
+// LP forward with tcgen05, on every row (K, V) or on the packed selected rows
+// (Q): a tile is 128 rows of one head.  Roles: one warp (every row: TMA) or four
+// (selected rows, gathered by cp.async one tile ahead) bring U tiles through a
+// 2-deep ring, after A_h once; the next warp issues the MMAs (D[128 x D] =
+// U_tile A_h into one of two TMEM buffers); four warps drain them (bf16).  A CTA
+// keeps one head; the row tiles of that head are strided over gridDim.x CTAs.
+// Shared memory: A_h as 64-column halves of [D rows][64] (128-byte swizzle), read
+// as the MN-major B operand; U tiles as 64-column halves of [128 rows][64], the
+// K-major A operand.  Memory bounds it on every row; on few selected rows the
+// chain of dependent loads at a CTA's start (count, positions, rows) does:
+// T 8192, an eighth of the rows of 32 heads of 128 (17 MB) 8.5 us (a kernel of
+// mma.sync tiles of 64 rows took 10.2).
 struct LpTcParams {
     CUtensorMap tm_u;   // u_l [B,T,H,D] as (d, h, t, b), box {64, 1, 128, 1}
     CUtensorMap tm_a;   // a [H*D rows][D] as (j, 1, row, 1), box {64, 1, D, 1}
+    const logo_bf16* u_l;
     logo_bf16* u_g;
+    RowSet rows;        // selected rows (GATHER)
     int B, T, H;
 };
 
@@ -344,8 +216,11 @@ struct LpTcCfg {
     static constexpr uint32_t kTmemCols = D == 128 ? 256 : 128;  // two D-column result buffers
 };
 
-template <int D>
-__global__ void __launch_bounds__(192, 1) lp_tc_fwd_kernel(const __grid_constant__ LpTcParams p)
+template <bool GATHER>
+constexpr int kLpProducers = GATHER ? 4 : 1;  // warps
+
+template <int D, bool GATHER>
+__global__ void __launch_bounds__(32 * (kLpProducers<GATHER> + 5), 1) lp_tc_fwd_kernel(const __grid_constant__ LpTcParams p)
 {
     using C = LpTcCfg<D>;
     extern __shared__ uint8_t smem_raw[];
@@ -354,23 +229,25 @@ __global__ void __launch_bounds__(192, 1) lp_tc_fwd_kernel(const __grid_constant
     __shared__ uint32_t tmem_sh;
     __shared__ volatile int abort_flag;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    constexpr int kMma = kLpProducers<GATHER>;  // the MMA issuer; the warps before it are producers
     const int h = blockIdx.y;
     const int tiles_per_seq = (p.T + 127) / 128;
-    const int ntiles = p.B * tiles_per_seq;
+    const int n = GATHER ? row_count(p.rows) : 0;  // packed rows
+    const int ntiles = GATHER ? (n + 127) / 128 : p.B * tiles_per_seq;
     const uint32_t sA = smem_u32(smem + C::kOffA), sU = smem_u32(smem + C::kOffU);
     if (threadIdx.x == 0) {
         abort_flag = 0;
         mbar_init(smem_u32(&bar_a), 1);
         mbar_init(smem_u32(&bar_drain), 1);
         for (int s = 0; s < 2; ++s) {
-            mbar_init(smem_u32(&bar_u_full[s]), 1);
+            mbar_init(smem_u32(&bar_u_full[s]), GATHER ? 128 : 1);
             mbar_init(smem_u32(&bar_u_empty[s]), 1);
             mbar_init(smem_u32(&bar_t_full[s]), 1);
             mbar_init(smem_u32(&bar_t_empty[s]), 128);
         }
         fence_mbar_init();
     }
-    if (warp == 1) {
+    if (warp == kMma) {
         tmem_alloc(smem_u32(&tmem_sh), C::kTmemCols);
         tmem_relinquish();
     }
@@ -378,32 +255,71 @@ __global__ void __launch_bounds__(192, 1) lp_tc_fwd_kernel(const __grid_constant
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_sh;
-    if (warp == 0) {
-        if (lane == 0) {
-            tma_prefetch_desc(&p.tm_u);
+    if (warp < kMma) {
+        if (warp == 0 && lane == 0) {
             tma_prefetch_desc(&p.tm_a);
-            const uint64_t pol_u = policy_evict_first(), pol_a = policy_evict_last();
             mbar_arrive_expect_tx(smem_u32(&bar_a), C::kABytes);
             for (int s = 0; s < D / 64; ++s)
-                tma_load_4d(sA + s * C::kHalfA, &p.tm_a, smem_u32(&bar_a), 64 * s, 0, h * D, 0, pol_a);
-            int k = 0;
-            bool ok = true;
+                tma_load_4d(sA + s * C::kHalfA, &p.tm_a, smem_u32(&bar_a), 64 * s, 0, h * D, 0, policy_evict_last());
+        }
+        bool ok = true;
+        int k = 0;
+        if (!GATHER) {
+            // -------------------------------------------------------- producer (TMA)
+            if (warp == 0 && lane == 0) {
+                tma_prefetch_desc(&p.tm_u);
+                const uint64_t pol_u = policy_evict_first();
+                for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++k) {
+                    const int st = k & 1;
+                    if (!(ok = mbar_wait(smem_u32(&bar_u_empty[st]), ((k >> 1) & 1) ^ 1, &abort_flag))) break;
+                    const int b = tile / tiles_per_seq, t0 = (tile % tiles_per_seq) * 128;
+                    mbar_arrive_expect_tx(smem_u32(&bar_u_full[st]), C::kUBytes);
+                    for (int s = 0; s < D / 64; ++s)
+                        tma_load_4d(sU + st * C::kUBytes + s * C::kHalfU, &p.tm_u, smem_u32(&bar_u_full[st]), 64 * s, h,
+                                    t0, b, pol_u);
+                }
+                if (!ok) {  // let the copies already issued land before the CTA exits
+                    for (int j = k - 2 > 0 ? k - 2 : 0; j < k; ++j)
+                        mbar_wait_drain(smem_u32(&bar_u_full[j & 1]), (j >> 1) & 1);
+                }
+            }
+        } else {
+            // -------------------------------------------------------- producers (gathered rows)
+            // warp w copies rows 32w .. 32w + 31 of a tile, whole rows side by side in
+            // a step; rows that do not exist are zero
+            constexpr int kChunks = D / 8, kStep = 32 / kChunks;  // lanes a row, rows a step
+            const int c = lane % kChunks;
+            const logo_bf16* src = p.u_l + h * D + c * 8;
             for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++k) {
                 const int st = k & 1;
-                if (!(ok = mbar_wait(smem_u32(&bar_u_empty[st]), ((k >> 1) & 1) ^ 1, &abort_flag))) break;
-                const int b = tile / tiles_per_seq, t0 = (tile % tiles_per_seq) * 128;
-                mbar_arrive_expect_tx(smem_u32(&bar_u_full[st]), C::kUBytes);
-                for (int s = 0; s < D / 64; ++s)
-                    tma_load_4d(sU + st * C::kUBytes + s * C::kHalfU, &p.tm_u, smem_u32(&bar_u_full[st]), 64 * s, h,
-                                t0, b, pol_u);
+                const int r = tile * 128 + warp * 32 + lane;
+                const int64_t tok = r < n ? row_token(p.rows, r) : -1;
+                ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bar_u_empty[st]), ((k >> 1) & 1) ^ 1, &abort_flag));
+                if (!ok) break;
+                const uint32_t base = sU + st * C::kUBytes + (c >> 3) * C::kHalfU;
+#pragma unroll 8
+                for (int i = 0; i < 32; i += kStep) {
+                    const int row = i + lane / kChunks;
+                    const int64_t t = __shfl_sync(0xffffffffu, tok, row);
+                    const uint32_t dst = base + sw128_offset(warp * 32 + row, c & 7);
+                    if (t >= 0) cp_async16(dst, src + t * p.H * D);
+                    else st_shared_v4(dst, 0u, 0u, 0u, 0u);
+                }
+                cp_async_commit();
+                if (k > 0) {  // tile k-1 has landed while tile k was issued
+                    cp_async_wait_one();
+                    fence_proxy_async_smem();
+                    mbar_arrive(smem_u32(&bar_u_full[st ^ 1]));
+                }
             }
-            if (!ok) {  // let the copies already issued land before the CTA exits
-                mbar_wait_drain(smem_u32(&bar_a), 0);
-                for (int j = k - 2 > 0 ? k - 2 : 0; j < k; ++j)
-                    mbar_wait_drain(smem_u32(&bar_u_full[j & 1]), (j >> 1) & 1);
+            cp_async_wait_all();
+            if (ok && k > 0) {
+                fence_proxy_async_smem();
+                mbar_arrive(smem_u32(&bar_u_full[(k - 1) & 1]));
             }
         }
-    } else if (warp == 1) {
+        if (!ok && warp == 0 && lane == 0) mbar_wait_drain(smem_u32(&bar_a), 0);
+    } else if (warp == kMma) {
         if (lane == 0) {
             constexpr uint32_t idesc = idesc_bf16_f32(128, D, false, true);
             bool ok = mbar_wait(smem_u32(&bar_a), 0, &abort_flag);
@@ -435,14 +351,25 @@ __global__ void __launch_bounds__(192, 1) lp_tc_fwd_kernel(const __grid_constant
         int k = 0;
         for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++k) {
             const int st = k & 1;
-            const bool ok = mbar_wait(smem_u32(&bar_t_full[st]), (k >> 1) & 1, &abort_flag);
-            __syncwarp();
+            const bool ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bar_t_full[st]), (k >> 1) & 1, &abort_flag));
             if (!ok) break;
             tc_fence_after();
             // 16 x 256-bit pieces, four lanes trading bf16 pairs (quad_gather8): a warp
             // store is 8 rows of 64 contiguous bytes, not 32 rows of 16
             const int b = tile / tiles_per_seq, t0 = (tile % tiles_per_seq) * 128 + quad * 32;
-            logo_bf16* dst = p.u_g + ((static_cast<int64_t>(b) * p.T + t0) * p.H + h) * D + (lane & 3) * 8;
+            logo_bf16* dst = p.u_g + h * D + (lane & 3) * 8;
+            logo_bf16* at[2][2];  // GATHER: this lane's rows t / 4, + 8, + 16, + 24 (null: no such row)
+            if constexpr (GATHER) {
+                const int r = tile * 128 + quad * 32 + lane;
+                const int64_t tok = r < n ? row_token(p.rows, r) : -1;
+#pragma unroll
+                for (int x = 0; x < 4; ++x) {
+                    const int64_t t = __shfl_sync(0xffffffffu, tok, x * 8 + (lane >> 2));
+                    at[x >> 1][x & 1] = t >= 0 ? dst + t * p.H * D : nullptr;
+                }
+            } else {
+                dst += (static_cast<int64_t>(b) * p.T + t0) * p.H * D;
+            }
 #pragma unroll
             for (int c = 0; c < D / 32; ++c) {
                 uint32_t v[2][16];
@@ -464,36 +391,43 @@ __global__ void __launch_bounds__(192, 1) lp_tc_fwd_kernel(const __grid_constant
                             w[k4] = cvt_bf16x2(__uint_as_float(v[hf][4 * k4 + 2 * ab]),
                                                __uint_as_float(v[hf][4 * k4 + 2 * ab + 1]));
                         const uint4 o = quad_gather8(w, lane);
-                        const int row = hf * 16 + ab * 8 + (lane >> 2);
-                        if (t0 + row < p.T) *reinterpret_cast<uint4*>(dst + static_cast<int64_t>(row) * p.H * D + c * 32) = o;
+                        if constexpr (GATHER) {
+                            if (at[hf][ab]) *reinterpret_cast<uint4*>(at[hf][ab] + c * 32) = o;
+                        } else {
+                            const int row = hf * 16 + ab * 8 + (lane >> 2);
+                            if (t0 + row < p.T) *reinterpret_cast<uint4*>(dst + static_cast<int64_t>(row) * p.H * D + c * 32) = o;
+                        }
                     }
             }
         }
     }
     tc_fence_before();
     __syncthreads();
-    if (warp == 1) {
+    if (warp == kMma) {
         tc_fence_after();
         tmem_dealloc(tmem, C::kTmemCols);
     }
 }
 
-template <int D>
-int launch_lp_tc_fwd(const logo_bf16* u_l, const logo_bf16* a, const logo_dims& d, logo_bf16* u_g, cudaStream_t st)
+template <int D, bool GATHER>
+int launch_lp_tc_fwd(const logo_bf16* u_l, const logo_bf16* a, const RowSet& rows, const logo_dims& d, logo_bf16* u_g,
+                     cudaStream_t st)
 {
     LpTcParams prm{};
     if (!encode_bf16_4d(&prm.tm_u, u_l, D, d.Hq, d.T, d.B, 64, 128) ||
         !encode_bf16_4d(&prm.tm_a, a, D, 1, static_cast<uint64_t>(d.Hq) * D, 1, 64, D))
         return LOGO_ERR_CUDA;
+    prm.u_l = u_l;
     prm.u_g = u_g;
+    prm.rows = rows;
     prm.B = d.B;
     prm.T = d.T;
     prm.H = d.Hq;
-    if (set_smem_limit(lp_tc_fwd_kernel<D>, LpTcCfg<D>::kSmemBytes) != cudaSuccess) return LOGO_ERR_CUDA;
-    const int ntiles = d.B * ((d.T + 127) / 128);
+    if (set_smem_limit(lp_tc_fwd_kernel<D, GATHER>, LpTcCfg<D>::kSmemBytes) != cudaSuccess) return LOGO_ERR_CUDA;
+    const int ntiles = GATHER ? (d.B * d.T + 127) / 128 : d.B * ((d.T + 127) / 128);  // at most
     int per_head = (2 * device_sm_count()) / d.Hq;
     per_head = per_head < 1 ? 1 : (per_head > ntiles ? ntiles : per_head);
-    lp_tc_fwd_kernel<D><<<dim3(per_head, d.Hq), 192, LpTcCfg<D>::kSmemBytes, st>>>(prm);
+    lp_tc_fwd_kernel<D, GATHER><<<dim3(per_head, d.Hq), 32 * (kLpProducers<GATHER> + 5), LpTcCfg<D>::kSmemBytes, st>>>(prm);
     return cudaGetLastError() == cudaSuccess ? LOGO_OK : LOGO_ERR_CUDA;
 }
 
@@ -877,21 +811,6 @@ int check_transform(const logo_dims& d, const void* u, const void* out)
     return LOGO_OK;
 }
 
-template <int D>
-int launch_lp_fwd(const logo_bf16* u_l, const logo_bf16* a, const RowSet& R, int H, logo_bf16* u_g,
-                  cudaStream_t st)
-{
-    const int smem = D * D * 2 + 2 * kTileRows * D * 2;  // A_h and two row tiles
-    if (set_smem_limit(lp_fwd_kernel<D>, smem) != cudaSuccess) return LOGO_ERR_CUDA;
-    // one wave: blocks per SM as shared memory allows (3 at d = 128, 64 KB each),
-    // split evenly over the heads; each block walks a strided share of its head's tiles
-    const int per_sm = D == 128 ? 3 : 6;
-    int chunks = per_sm * device_sm_count() / H;
-    chunks = chunks < 1 ? 1 : chunks > 64 ? 64 : chunks;
-    lp_fwd_kernel<D><<<dim3(chunks, H), 128, smem, st>>>(u_l, a, R, H, u_g);
-    return cudaGetLastError() == cudaSuccess ? LOGO_OK : LOGO_ERR_CUDA;
-}
-
 }  // namespace
 int transform_tu_status(int clear) { return read_tu_status(clear); }
 
@@ -912,13 +831,13 @@ extern "C" int logo_branch_transform(const logo_bf16* u_l, const logo_bf16* a_lp
     if (a_lp && !aligned16(a_lp)) return LOGO_ERR_UNSUPPORTED;
     const RowSet R{pos, cu_q, n_sel_total, dims.B, dims.T};
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (a_lp && !pos) {  // every row: the tcgen05 pipeline
-        return dims.D == 128 ? launch_lp_tc_fwd<128>(u_l, a_lp, dims, u_g, st)
-                             : launch_lp_tc_fwd<64>(u_l, a_lp, dims, u_g, st);
+    if (a_lp && !pos) {
+        return dims.D == 128 ? launch_lp_tc_fwd<128, false>(u_l, a_lp, R, dims, u_g, st)
+                             : launch_lp_tc_fwd<64, false>(u_l, a_lp, R, dims, u_g, st);
     }
-    if (a_lp) {  // the packed selected rows (Q): warp-level MMA over gathered rows
-        return dims.D == 128 ? launch_lp_fwd<128>(u_l, a_lp, R, dims.Hq, u_g, st)
-                             : launch_lp_fwd<64>(u_l, a_lp, R, dims.Hq, u_g, st);
+    if (a_lp) {  // the packed selected rows (Q)
+        return dims.D == 128 ? launch_lp_tc_fwd<128, true>(u_l, a_lp, R, dims, u_g, st)
+                             : launch_lp_tc_fwd<64, true>(u_l, a_lp, R, dims, u_g, st);
     }
     const int64_t work = static_cast<int64_t>(dims.B) * dims.T * dims.Hq * dims.D / 8;
     const int64_t cap = static_cast<int64_t>(device_sm_count()) * 8;
