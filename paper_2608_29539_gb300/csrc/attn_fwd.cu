@@ -187,9 +187,13 @@ __global__ void __launch_bounds__(512, 1) attn_fwd_kernel(const __grid_constant_
     __shared__ __align__(8) uint64_t bar_k_full[C::kStages], bar_k_empty[C::kStages];
     __shared__ __align__(8) uint64_t bar_v_full[C::kStages], bar_v_empty[C::kStages];
     __shared__ __align__(8) uint64_t bar_s_full[2], bar_s_empty[2], bar_p_full[2];
-    // P.V of block n done: barrier n % 4, so that a wait for block n - 1 or
-    // n - 2 can never be confused with the barrier's phase before
-    __shared__ __align__(8) uint64_t bar_pv_done[4];
+    // P.V of block n done, for the softmax: barrier n % 2.  Its waits, for n - 2
+    // and then perhaps n - 1, are made at block n: the phases before are known to
+    // have ended, the ones after need block n's P.  For the epilogue, P.V of an
+    // item's last block done: a barrier per O buffer, whose next phase needs that
+    // buffer's bar_o_free.  (It cannot wait on bar_pv_done: with two O buffers
+    // the next item's products go on beside it and end later phases.)
+    __shared__ __align__(8) uint64_t bar_pv_done[2], bar_o_full[C::kOBufs];
     // running max of every row after the newest block, handed from one softmax
     // warpgroup's thread of the row to the other's (so one copy is enough): a
     // barrier per warp and block parity
@@ -235,7 +239,6 @@ __global__ void __launch_bounds__(512, 1) attn_fwd_kernel(const __grid_constant_
             mbar_init(smem_u32(&bar_item_full[s]), 1);
             // the V producer, the two MMA threads, one lane per softmax / epilogue warp
             mbar_init(smem_u32(&bar_item_empty[s]), 15);
-            mbar_init(smem_u32(&bar_pv_done[s]), 1);
             mbar_init(smem_u32(&bar_m[0][s]), 1);
             mbar_init(smem_u32(&bar_m[1][s]), 1);
         }
@@ -243,10 +246,14 @@ __global__ void __launch_bounds__(512, 1) attn_fwd_kernel(const __grid_constant_
             mbar_init(smem_u32(&bar_s_full[s]), 1);
             mbar_init(smem_u32(&bar_s_empty[s]), 128);
             mbar_init(smem_u32(&bar_p_full[s]), 128);
+            mbar_init(smem_u32(&bar_pv_done[s]), 1);
         }
         mbar_init(smem_u32(&bar_l_full), 256);
         mbar_init(smem_u32(&bar_l_empty), 128);
-        for (int s = 0; s < C::kOBufs; ++s) mbar_init(smem_u32(&bar_o_free[s]), 128);
+        for (int s = 0; s < C::kOBufs; ++s) {
+            mbar_init(smem_u32(&bar_o_full[s]), 1);
+            mbar_init(smem_u32(&bar_o_free[s]), 128);
+        }
         fence_mbar_init();
     }
     if (warp == 13) {
@@ -418,10 +425,11 @@ __global__ void __launch_bounds__(512, 1) attn_fwd_kernel(const __grid_constant_
                         const uint64_t bdesc = sdesc_sw128(vbase + ks * 2048, 16384, 1024);
                         umma_bf16_ts(ocol, pcol + ks * 8, bdesc, idPV, (j > 0 || ks > 0) ? 1u : 0u);
                     }
-                    umma_commit(smem_u32(&bar_pv_done[itg & 3]));
+                    umma_commit(smem_u32(&bar_pv_done[itg & 1]));
                     umma_commit(smem_u32(&bar_v_empty[st]));  // V of this block is read
                 }
                 if (!ok) break;
+                umma_commit(smem_u32(&bar_o_full[ob]));
                 kv_it += nblk;
                 s_it += nblk;
             }
@@ -562,7 +570,7 @@ __global__ void __launch_bounds__(512, 1) attn_fwd_kernel(const __grid_constant_
                 if (lane == 0) mbar_arrive(bar_m_mine);
                 // (global branch only: the local one has no register left for it)
                 const bool pv_seen =
-                    itg < 2 || (GLOBAL && mbar_test(smem_u32(&bar_pv_done[(itg - 2) & 3]), ((itg - 2) >> 2) & 1));
+                    itg < 2 || (GLOBAL && mbar_test(smem_u32(&bar_pv_done[(itg - 2) & 1]), ((itg - 2) >> 1) & 1));
                 const float m_use = (m_ref == -INFINITY) ? 0.f : m_ref;
                 const uint64_t scale2 = f2_pack(p.scale_log2, p.scale_log2);
                 const uint64_t negm2 = f2_pack(-m_use, -m_use);
@@ -593,7 +601,7 @@ __global__ void __launch_bounds__(512, 1) attn_fwd_kernel(const __grid_constant_
                 l += rs;
                 // the P buffer is free once the P.V two blocks back is done
                 if (!__all_sync(0xffffffffu, pv_seen)) {
-                    ok = mbar_wait(smem_u32(&bar_pv_done[(itg - 2) & 3]), ((itg - 2) >> 2) & 1, &abort_flag);
+                    ok = mbar_wait(smem_u32(&bar_pv_done[(itg - 2) & 1]), ((itg - 2) >> 1) & 1, &abort_flag);
                     __syncwarp();
                     if (!ok) break;
                 }
@@ -603,7 +611,7 @@ __global__ void __launch_bounds__(512, 1) attn_fwd_kernel(const __grid_constant_
                 // O may only be rescaled once the P.V of the previous block is done.
                 // Done here, where the row of S no longer takes registers
                 if (__any_sync(0xffffffffu, rescale)) {
-                    ok = mbar_wait(smem_u32(&bar_pv_done[(itg - 1) & 3]), ((itg - 1) >> 2) & 1, &abort_flag);
+                    ok = mbar_wait(smem_u32(&bar_pv_done[(itg - 1) & 1]), ((itg - 1) >> 1) & 1, &abort_flag);
                     __syncwarp();
                     if (!ok) break;
                     tc_fence_after();
@@ -645,14 +653,12 @@ __global__ void __launch_bounds__(512, 1) attn_fwd_kernel(const __grid_constant_
         const int quad = warp & 3;
         const int r = quad * 32 + lane;
         const uint32_t lane_off = static_cast<uint32_t>(quad * 32) << 16;
-        int itg = 0;
         bool ok = true;
         for (int item_i = 0;; ++item_i) {
             const int k = consume_item(item_i, &ok, true);
             if (k < 0) break;
             const FwdItem it = decode_item<GLOBAL>(p, k);
             const bool row_valid = r < it.nrows;
-            itg += it.blk_hi - it.blk_lo + 1;
             ok = mbar_wait(smem_u32(&bar_l_full), item_i & 1, &abort_flag);
             __syncwarp();
             if (!ok) break;
@@ -677,12 +683,12 @@ __global__ void __launch_bounds__(512, 1) attn_fwd_kernel(const __grid_constant_
             float inv[2][2];
 #pragma unroll
             for (int i = 0; i < 4; ++i) inv[i >> 1][i & 1] = __shfl_sync(0xffffffffu, inv_l, i * 8 + (lane >> 2));
-            // the item's last P.V (block itg - 1) is done
-            ok = mbar_wait(smem_u32(&bar_pv_done[(itg - 1) & 3]), ((itg - 1) >> 2) & 1, &abort_flag);
+            // the item's last P.V is done
+            const int ob = item_i % C::kOBufs;
+            ok = mbar_wait(smem_u32(&bar_o_full[ob]), (item_i / C::kOBufs) & 1, &abort_flag);
             __syncwarp();
             if (!ok) break;
             tc_fence_after();
-            const int ob = item_i % C::kOBufs;
             const uint32_t ocol = tmem + lane_off + C::kColO + ob * D;
             // this lane's 16-byte column slice of the warp's first row
             logo_bf16* o0 = p.o + ((GLOBAL ? 0 : static_cast<int64_t>(it.b) * p.T) + it.row0 + quad * 32) * p.Hq * D +
