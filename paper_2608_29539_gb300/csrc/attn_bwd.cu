@@ -441,12 +441,12 @@ __global__ void __launch_bounds__(Bwd2Cfg::kThreads, 1) attn_bwd2_kernel(const _
                     if (lane == 0) sh_open[b][tw >> 5] = all_open ? 1 : 0;
                 }
                 mbar_arrive(smem_u32(&bar_stage));
-                ok = mbar_wait(smem_u32(&bar_stage), u & 1, &abort_flag);
-                if (!ok) break;
+                mbar_wait(smem_u32(&bar_stage), u & 1, &abort_flag);  // (if it gave up, so will the next wait)
                 if (tw < BQ && x + 1 < n_it) load_stage(x + 1);
                 const bool open = sh_open[b][0] && sh_open[b][1];
                 ok = mbar_wait(smem_u32(&bar_st_full), u & 1, &abort_flag);
                 __syncwarp();
+                ok = warp_all(ok);
                 if (!ok) break;
                 tc_fence_after();
                 uint32_t sv[32], dpv[32];
@@ -489,8 +489,7 @@ __global__ void __launch_bounds__(Bwd2Cfg::kThreads, 1) attn_bwd2_kernel(const _
                 // P^T (TMEM) / dS^T (shared) buffer b is free once the MMAs of tile
                 // u-2 are done.  Waiting here rather than before the loads lets
                 // S^T, dP^T of tile u+1 enter the MMA queue earlier.
-                ok = mbar_wait(smem_u32(&bar_dq_full[b]), ((u >> 1) & 1) ^ 1, &abort_flag);
-                __syncwarp();
+                ok = warp_all(mbar_wait(smem_u32(&bar_dq_full[b]), ((u >> 1) & 1) ^ 1, &abort_flag));
                 if (!ok) break;
                 tc_fence_after();
                 // P^T row t: query columns half*32.. as 16 bf16 pairs, the TMEM
@@ -540,8 +539,7 @@ __global__ void __launch_bounds__(Bwd2Cfg::kThreads, 1) attn_bwd2_kernel(const _
                 const int h = it.kvh * group + x / it.ntiles;
                 const int i = it.i_lo + x % it.ntiles;
                 const int b = u & 1;
-                ok = mbar_wait(smem_u32(&bar_dq_full[b]), (u >> 1) & 1, &abort_flag);
-                __syncwarp();
+                ok = warp_all(mbar_wait(smem_u32(&bar_dq_full[b]), (u >> 1) & 1, &abort_flag));
                 if (!ok) break;
                 tc_fence_after();
                 uint32_t v0[32], v1[32];
@@ -563,8 +561,7 @@ __global__ void __launch_bounds__(Bwd2Cfg::kThreads, 1) attn_bwd2_kernel(const _
                 for (int c = 0; c < 32; ++c) atomicAdd(base + (32 + c) * rs, __uint_as_float(v1[c]) * p.scale);
             }
             if (!ok) break;
-            ok = mbar_wait(smem_u32(&bar_dkv_full), kv_items & 1, &abort_flag);
-            __syncwarp();
+            ok = warp_all(mbar_wait(smem_u32(&bar_dkv_full), kv_items & 1, &abort_flag));
             if (!ok) break;
             tc_fence_after();
             // 16 x 256-bit pieces, four lanes trading bf16 pairs (quad_gather8): a warp
@@ -887,9 +884,7 @@ __global__ void __launch_bounds__(Bwd64Cfg::kThreads, 1) attn_bwd64_kernel(const
             const int row_first = it.i_lo * BQ, row_end = row_first + it.ntiles * BQ;
             int row0 = row_first;
             for (int left = group * it.ntiles; left > 0; --left, ++u) {
-                ok = mbar_wait(smem_u32(&bar_qdo_full[st]), turn, &abort_flag);
-                __syncwarp();
-                if (!ok) break;
+                mbar_wait(smem_u32(&bar_qdo_full[st]), turn, &abort_flag);  // (if it gave up, so will the next wait)
                 // every column of the half sees every key of the block
                 bool open;
                 {
@@ -916,7 +911,7 @@ __global__ void __launch_bounds__(Bwd64Cfg::kThreads, 1) attn_bwd64_kernel(const
                     lo -= half * 64;
                     hi -= half * 64;
                 }
-                ok = mbar_wait(smem_u32(&bar_st_full), u & 1, &abort_flag);
+                ok = mbar_wait_warp(smem_u32(&bar_st_full), u & 1, &abort_flag);
                 __syncwarp();
                 if (!ok) break;
                 tc_fence_after();
@@ -965,7 +960,7 @@ __global__ void __launch_bounds__(Bwd64Cfg::kThreads, 1) attn_bwd64_kernel(const
                 else columns(std::true_type{});
                 // P^T (TMEM) and dS^T (shared) are free once the MMAs of tile u-1 are done
                 if (u > 0) {
-                    ok = mbar_wait(smem_u32(&bar_dq_full), (u - 1) & 1, &abort_flag);
+                    ok = mbar_wait_warp(smem_u32(&bar_dq_full), (u - 1) & 1, &abort_flag);
                     __syncwarp();
                     if (!ok) break;
                 }
@@ -1011,7 +1006,7 @@ __global__ void __launch_bounds__(Bwd64Cfg::kThreads, 1) attn_bwd64_kernel(const
             const int n_it = group * it.ntiles;
             for (int x = 0, h = it.kvh * group, i = it.i_lo; x < n_it; ++x, ++u, next_tile(it, h, i)) {
                 const int row0 = i * BQ + quad * 32;  // this warp's first query row
-                ok = mbar_wait(smem_u32(&bar_dq_full), u & 1, &abort_flag);
+                ok = mbar_wait_warp(smem_u32(&bar_dq_full), u & 1, &abort_flag);
                 __syncwarp();
                 if (!ok) break;
                 tc_fence_after();
@@ -1046,7 +1041,7 @@ __global__ void __launch_bounds__(Bwd64Cfg::kThreads, 1) attn_bwd64_kernel(const
                 }
             }
             if (!ok) break;
-            ok = mbar_wait(smem_u32(&bar_dkv_full), kv_items & 1, &abort_flag);
+            ok = mbar_wait_warp(smem_u32(&bar_dkv_full), kv_items & 1, &abort_flag);
             __syncwarp();
             if (!ok) break;
             tc_fence_after();

@@ -275,7 +275,9 @@ __global__ void __launch_bounds__(512, 1) attn_fwd_kernel(const __grid_constant_
             return k < n_items ? k : -1;
         }
         const int slot = u & 3;
-        if (!(*ok = mbar_wait(smem_u32(&bar_item_full[slot]), (u >> 2) & 1, &abort_flag))) return -1;
+        const uint32_t full = smem_u32(&bar_item_full[slot]), turn = (u >> 2) & 1;
+        *ok = whole_warp ? mbar_wait_warp(full, turn, &abort_flag) : mbar_wait(full, turn, &abort_flag);
+        if (!*ok) return -1;
         const int k = item_ring[slot];
         if (whole_warp) {
             __syncwarp();
@@ -508,7 +510,9 @@ __global__ void __launch_bounds__(512, 1) attn_fwd_kernel(const __grid_constant_
             for (int j = (itg0 ^ par) & 1; j < nblk; j += 2) {
                 const int itg = itg0 + j, n = blk_lo + j;
                 if (!__all_sync(0xffffffffu, s_seen)) {
-                    ok = mbar_wait(smem_u32(&bar_s_full[par]), (itg >> 1) & 1, &abort_flag);
+                    // (the __syncwarp here and at the waits below: without any, the
+                    // allocator spills 40 bytes of the row of S)
+                    ok = mbar_wait_warp(smem_u32(&bar_s_full[par]), (itg >> 1) & 1, &abort_flag);
                     __syncwarp();
                     if (!ok) break;
                 }
@@ -548,7 +552,7 @@ __global__ void __launch_bounds__(512, 1) attn_fwd_kernel(const __grid_constant_
                 // item's edge too (its value does not count there), so that the
                 // two warpgroups' phases on these barriers never drift apart
                 if (!__all_sync(0xffffffffu, m_seen)) {
-                    ok = mbar_wait(bar_m_other, ((itg - 1) >> 1) & 1, &abort_flag);
+                    ok = mbar_wait_warp(bar_m_other, ((itg - 1) >> 1) & 1, &abort_flag);
                     __syncwarp();
                     if (!ok) break;
                     m_ref = sh_m[r];
@@ -601,7 +605,7 @@ __global__ void __launch_bounds__(512, 1) attn_fwd_kernel(const __grid_constant_
                 l += rs;
                 // the P buffer is free once the P.V two blocks back is done
                 if (!__all_sync(0xffffffffu, pv_seen)) {
-                    ok = mbar_wait(smem_u32(&bar_pv_done[(itg - 2) & 1]), ((itg - 2) >> 1) & 1, &abort_flag);
+                    ok = mbar_wait_warp(smem_u32(&bar_pv_done[(itg - 2) & 1]), ((itg - 2) >> 1) & 1, &abort_flag);
                     __syncwarp();
                     if (!ok) break;
                 }
@@ -611,7 +615,7 @@ __global__ void __launch_bounds__(512, 1) attn_fwd_kernel(const __grid_constant_
                 // O may only be rescaled once the P.V of the previous block is done.
                 // Done here, where the row of S no longer takes registers
                 if (__any_sync(0xffffffffu, rescale)) {
-                    ok = mbar_wait(smem_u32(&bar_pv_done[(itg - 1) & 1]), ((itg - 1) >> 1) & 1, &abort_flag);
+                    ok = mbar_wait_warp(smem_u32(&bar_pv_done[(itg - 1) & 1]), ((itg - 1) >> 1) & 1, &abort_flag);
                     __syncwarp();
                     if (!ok) break;
                     tc_fence_after();
@@ -636,8 +640,7 @@ __global__ void __launch_bounds__(512, 1) attn_fwd_kernel(const __grid_constant_
             if (!ok) break;
             itg0 += nblk;
             // ---- end of the item: this warpgroup's max and row sum to the epilogue warps
-            ok = mbar_wait(smem_u32(&bar_l_empty), (item_i & 1) ^ 1, &abort_flag);
-            __syncwarp();
+            ok = mbar_wait_warp(smem_u32(&bar_l_empty), (item_i & 1) ^ 1, &abort_flag);
             if (!ok) break;
             sh_ml[par][r] = make_float2(m_own, l);
             mbar_arrive(smem_u32(&bar_l_full));
@@ -659,8 +662,7 @@ __global__ void __launch_bounds__(512, 1) attn_fwd_kernel(const __grid_constant_
             if (k < 0) break;
             const FwdItem it = decode_item<GLOBAL>(p, k);
             const bool row_valid = r < it.nrows;
-            ok = mbar_wait(smem_u32(&bar_l_full), item_i & 1, &abort_flag);
-            __syncwarp();
+            ok = mbar_wait_warp(smem_u32(&bar_l_full), item_i & 1, &abort_flag);
             if (!ok) break;
             const float2 ml0 = sh_ml[0][r], ml1 = sh_ml[1][r];
             mbar_arrive(smem_u32(&bar_l_empty));
@@ -685,8 +687,7 @@ __global__ void __launch_bounds__(512, 1) attn_fwd_kernel(const __grid_constant_
             for (int i = 0; i < 4; ++i) inv[i >> 1][i & 1] = __shfl_sync(0xffffffffu, inv_l, i * 8 + (lane >> 2));
             // the item's last P.V is done
             const int ob = item_i % C::kOBufs;
-            ok = mbar_wait(smem_u32(&bar_o_full[ob]), (item_i / C::kOBufs) & 1, &abort_flag);
-            __syncwarp();
+            ok = mbar_wait_warp(smem_u32(&bar_o_full[ob]), (item_i / C::kOBufs) & 1, &abort_flag);
             if (!ok) break;
             tc_fence_after();
             const uint32_t ocol = tmem + lane_off + C::kColO + ob * D;

@@ -317,8 +317,9 @@ __global__ void __launch_bounds__(kDecThreads, 2) decode_attn_kernel(const __gri
             issue();
             const int st = consumed % kDecStages;
             const uint32_t sK = sRing + st * C::kStageBytes, sV = sK + C::kTileBytes;
-            ok = mbar_wait(smem_u32(&bar_full[st]), (consumed / kDecStages) & 1, &abort_flag) && ok;
-            if (!(ok = __all_sync(0xffffffffu, ok))) break;  // the warp leaves together (mma.sync needs all lanes)
+            // the warp leaves together, lane 0's failed issue included (mma.sync needs all lanes)
+            ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bar_full[st]), (consumed / kDecStages) & 1, &abort_flag) && ok);
+            if (!ok) break;
             const int j0 = s * kDecRows + warp * kDecRowsPerWarp;  // this warp's first cache row
             const bool open = sees.all16(j0);
             if (!open) {

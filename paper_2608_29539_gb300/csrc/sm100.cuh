@@ -131,6 +131,33 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     }
 }
 
+// A wait by a whole warp that goes on to warp collectives needs one answer for
+// all 32 lanes: of lanes waiting each for itself, one may give up while another
+// still sees the phase complete, and those two would part before a collective.
+// Two ways to it, which differ in how the polls of several warps interleave:
+// the lanes poll together (mbar_wait_warp), or vote after each one's own wait.
+__device__ __forceinline__ bool warp_all(bool ok)
+{
+    if (__any_sync(0xffffffffu, !ok)) ok = false;
+    return ok;
+}
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag)
+{
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    const uint32_t t0 = globaltimer_lo();
+    for (uint32_t it = 1;; ++it) {
+        if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+        if ((it & 63u) == 0) {
+            const bool late = globaltimer_lo() - t0 > kWaitBudgetNs;
+            if (late) {
+                *abort_flag = 1;
+                record_status(LOGO_ERR_TIMEOUT);
+            }
+            if (__any_sync(0xffffffffu, late || *abort_flag)) return false;
+        }
+    }
+}
+
 // Bounded wait used only on the way out of an aborted kernel (to let copies
 // already in flight land); it ignores the abort flag.
 __device__ __forceinline__ bool mbar_wait_drain(uint32_t bar, uint32_t parity)

@@ -294,7 +294,7 @@ __global__ void __launch_bounds__(32 * (kLpProducers<GATHER> + 5), 1) lp_tc_fwd_
                 const int st = k & 1;
                 const int r = tile * 128 + warp * 32 + lane;
                 const int64_t tok = r < n ? row_token(p.rows, r) : -1;
-                ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bar_u_empty[st]), ((k >> 1) & 1) ^ 1, &abort_flag));
+                ok = mbar_wait_warp(smem_u32(&bar_u_empty[st]), ((k >> 1) & 1) ^ 1, &abort_flag);
                 if (!ok) break;
                 const uint32_t base = sU + st * C::kUBytes + (c >> 3) * C::kHalfU;
 #pragma unroll 8
@@ -351,7 +351,7 @@ __global__ void __launch_bounds__(32 * (kLpProducers<GATHER> + 5), 1) lp_tc_fwd_
         int k = 0;
         for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++k) {
             const int st = k & 1;
-            const bool ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bar_t_full[st]), (k >> 1) & 1, &abort_flag));
+            const bool ok = mbar_wait_warp(smem_u32(&bar_t_full[st]), (k >> 1) & 1, &abort_flag);
             if (!ok) break;
             tc_fence_after();
             // 16 x 256-bit pieces, four lanes trading bf16 pairs (quad_gather8): a warp
@@ -572,10 +572,9 @@ __global__ void __launch_bounds__(kLpBwdThreads, 1) lp_tc_bwd_kernel(const __gri
                 const int st = k & 1;
                 const int r = tile * 128 + warp * 32 + lane;
                 const int tok = r < n ? static_cast<int>(row_token(p.rows, r)) : -1;
-                ok = mbar_wait(smem_u32(&bar_in_empty[st]), ((k >> 1) & 1) ^ 1, &abort_flag) &&
-                     mbar_wait(smem_u32(&bar_d_empty[st]), ((k >> 1) & 1) ^ 1, &abort_flag);
-                __syncwarp();
-                if (!(ok = __all_sync(0xffffffffu, ok))) break;
+                ok = mbar_wait_warp(smem_u32(&bar_in_empty[st]), ((k >> 1) & 1) ^ 1, &abort_flag) &&
+                     mbar_wait_warp(smem_u32(&bar_d_empty[st]), ((k >> 1) & 1) ^ 1, &abort_flag);
+                if (!ok) break;
                 const uint32_t half = sIn + st * C::kStage + ((lane & 15) >> 3) * C::kHalf;
                 const uint32_t base = half + (lane < 16 ? 0 : C::kTile);
 #pragma unroll 8
@@ -665,9 +664,8 @@ __global__ void __launch_bounds__(kLpBwdThreads, 1) lp_tc_bwd_kernel(const __gri
                 tok = t < p.T ? b * p.T + t : -1;
             }
             // the tile's dU has landed (with U and G), and the product is there
-            ok = mbar_wait(smem_u32(&bar_in_full[st]), (k >> 1) & 1, &abort_flag) &&
-                 mbar_wait(smem_u32(&bar_t_full[st]), (k >> 1) & 1, &abort_flag);
-            __syncwarp();
+            ok = mbar_wait_warp(smem_u32(&bar_in_full[st]), (k >> 1) & 1, &abort_flag) &&
+                 mbar_wait_warp(smem_u32(&bar_t_full[st]), (k >> 1) & 1, &abort_flag);
             if (!ok) break;
             tc_fence_after();
 #pragma unroll
@@ -717,7 +715,7 @@ __global__ void __launch_bounds__(kLpBwdThreads, 1) lp_tc_bwd_kernel(const __gri
         if (ok && k == 0) {  // no tile: a zero partial
             if (s < heads)
                 for (int j = 0; j < D; j += 4) *reinterpret_cast<float4*>(pp + j) = make_float4(0.f, 0.f, 0.f, 0.f);
-        } else if (ok && mbar_wait(smem_u32(&bar_da), 0, &abort_flag)) {
+        } else if (ok && mbar_wait_warp(smem_u32(&bar_da), 0, &abort_flag)) {
             tc_fence_after();
             const int first = (quad * 32 / D) * D;  // the head's columns (the same for the warp)
 #pragma unroll
