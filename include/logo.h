@@ -338,11 +338,13 @@ LOGO_API int logo_branch_transform(const logo_bf16* u_l, const logo_bf16* a_lp, 
  *   rows, for du_g [B,T,H,D] bf16 (read on the listed rows):
  *   du_l = du_g A_h^T (LP) or du_g * s_h (SO), written, or added to du_l when
  *      accumulate = 1 (the caller's gradient of U^L from the local branch);
- *   LP: da_lp [H,D,D] float32 = sum over the rows of u_l^T du_g;
+ *   LP: da_lp [H,D,D] float32 = sum over the rows of u_l^T du_g (4-byte
+ *      alignment is enough for it, as for ds_so and db_so);
  *   SO: ds_so, db_so [H,D] float32 = sums of du_g * u_l and of du_g (either may
  *      be NULL).  Parameter gradients are summed per block, then over the blocks
  *      in a fixed order (deterministic).
- * Workspace: logo_branch_transform_bwd_workspace_size(dims) bytes. */
+ * Workspace: logo_branch_transform_bwd_workspace_size(dims) bytes;
+ *      LOGO_ERR_WORKSPACE if it is smaller or (LP) not 16-byte aligned. */
 LOGO_API size_t logo_branch_transform_bwd_workspace_size(logo_dims dims);
 LOGO_API int logo_branch_transform_bwd(const logo_bf16* u_l, const logo_bf16* a_lp, const float* s_so,
                                        const int32_t* pos, const int32_t* cu_q, const int32_t* n_sel_total,
@@ -384,7 +386,7 @@ LOGO_API int logo_combine_bwd(const logo_bf16* dO, const logo_bf16* o_l, const l
  *      blocks in a fixed order: the result is deterministic on a given GPU.
  * Workspace: logo_combine_bwd_workspace_size(dims) bytes of device memory.
  * Errors: LOGO_ERR_UNSUPPORTED if Hq*D > 8192; LOGO_ERR_WORKSPACE if the
- *      workspace is short; otherwise as logo_combine_bwd. */
+ *      workspace is short or not 16-byte aligned; otherwise as logo_combine_bwd. */
 LOGO_API size_t logo_combine_bwd_workspace_size(logo_dims dims);
 LOGO_API int logo_combine_bwd_gains(const logo_bf16* dO, const logo_bf16* o_l, const logo_bf16* o_c,
                                     const float* gate_p, const uint8_t* z, const int32_t* row_of,

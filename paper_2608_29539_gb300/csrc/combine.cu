@@ -1043,6 +1043,7 @@ int combine_bwd_common(const logo_bf16* dO, const logo_bf16* o_l, const logo_bf1
         if (dims.Hq * (dims.D / 8) > kMaxVecGains) return LOGO_ERR_UNSUPPORTED;  // Hq * D <= 8192
         if (!workspace) return LOGO_ERR_INVALID_ARG;
         if (workspace_bytes < logo_combine_bwd_workspace_size(dims)) return LOGO_ERR_WORKSPACE;
+        if (!aligned16(workspace)) return LOGO_ERR_WORKSPACE;  // the partial sums go there as float4
     }
     const int64_t ntok = static_cast<int64_t>(dims.B) * dims.T;
     const size_t smem = gains ? gains_smem(dims) : 0;

@@ -58,7 +58,8 @@ __device__ __forceinline__ void cp_async_wait_one() { asm volatile("cp.async.wai
 
 // out[h][e] = sum over c of part[h][c][e], e < per_head (a multiple of 4).
 // Thread (x, g) of a block adds chunks g, g + 4, .. of four columns, then the
-// four sums are added in order: a fixed order, and every load in flight.
+// four sums are added in order: a fixed order, and every load in flight.  `out`
+// is the caller's and may lie on any 4-byte boundary.
 __global__ void __launch_bounds__(256) reduce_parts_kernel(const float* __restrict__ part, int nchunk, int per_head,
                                                            int H, float* __restrict__ out)
 {
@@ -90,7 +91,14 @@ __global__ void __launch_bounds__(256) reduce_parts_kernel(const float* __restri
             s.z += v.z;
             s.w += v.w;
         }
-        *reinterpret_cast<float4*>(out + e) = s;
+        if ((reinterpret_cast<uintptr_t>(out) & 15u) == 0) {
+            *reinterpret_cast<float4*>(out + e) = s;
+        } else {
+            out[e] = s.x;
+            out[e + 1] = s.y;
+            out[e + 2] = s.z;
+            out[e + 3] = s.w;
+        }
     }
 }
 
@@ -869,6 +877,7 @@ extern "C" int logo_branch_transform_bwd(const logo_bf16* u_l, const logo_bf16* 
     if (pos && (!cu_q || !n_sel_total)) return LOGO_ERR_INVALID_ARG;
     if (!aligned16(du_g) || (a_lp && !aligned16(a_lp))) return LOGO_ERR_UNSUPPORTED;
     if (!workspace || workspace_bytes < logo_branch_transform_bwd_workspace_size(dims)) return LOGO_ERR_WORKSPACE;
+    if (a_lp && !aligned16(workspace)) return LOGO_ERR_WORKSPACE;  // the partial dA go there as float4
     const RowSet R{pos, cu_q, n_sel_total, dims.B, dims.T};
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     float* part = static_cast<float*>(workspace);
