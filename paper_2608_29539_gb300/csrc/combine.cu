@@ -902,18 +902,22 @@ bool gains_smem_ok(K kernel, size_t bytes = 4 * kMaxVecGains * sizeof(float4))
 }
 
 // A launch of the gains-read kernels; `slots`: float4 of shared memory per thread.
+// A kernel's limit is set to what its largest block takes, whatever this call's
+// size: calls of other sizes may be under way on other threads.
 struct GainLaunch {
     GainShape sh;
     size_t smem;
     int64_t grid;
+    bool ok;
 };
 
 template <typename K>
 GainLaunch gain_launch(K kernel, const logo_dims& d, int slots)
 {
-    GainLaunch g{gain_shape(d), 0, 0};
+    GainLaunch g{gain_shape(d), 0, 0, false};
     g.smem = static_cast<size_t>(slots) * g.sh.threads * sizeof(float4);
-    gains_smem_ok(kernel, g.smem);
+    const int max_threads = g.sh.threads > 512 ? 1024 : 512;
+    g.ok = gains_smem_ok(kernel, static_cast<size_t>(slots) * max_threads * sizeof(float4));
     const int64_t ntok = static_cast<int64_t>(d.B) * d.T;
     g.grid = wave_blocks(kernel, (ntok + g.sh.rows - 1) / g.sh.rows, g.smem, g.sh.threads);
     return g;
@@ -1005,19 +1009,21 @@ extern "C" int logo_combine(const logo_bf16* o_l, const logo_bf16* o_c, const fl
     } else {
         auto run = [&](auto kernel, int slots) {
             const GainLaunch L = gain_launch(kernel, dims, slots);
-            kernel<<<static_cast<unsigned>(L.grid), L.sh.threads, L.smem, st>>>(o_l, o_c, gate_p, z, row_of, gain_l,
-                                                                               gain_g, eps, o, rstd_l, rstd_g, ntok,
-                                                                               dims.Hq, L.sh.tpr, L.sh.rows);
+            if (L.ok)
+                kernel<<<static_cast<unsigned>(L.grid), L.sh.threads, L.smem, st>>>(
+                    o_l, o_c, gate_p, z, row_of, gain_l, gain_g, eps, o, rstd_l, rstd_g, ntok, dims.Hq, L.sh.tpr,
+                    L.sh.rows);
+            return L.ok;
         };
+        bool ok;
         constexpr int kSlots = 2 * GainCfg<512>::kRingFwd + 4;
         const bool big = gain_shape(dims).threads > 512;
         if (dims.D == 128) {
-            if (big) run(combine_gained_fwd_kernel<128, 1024>, kSlots);
-            else run(combine_gained_fwd_kernel<128, 512>, kSlots);
+            ok = big ? run(combine_gained_fwd_kernel<128, 1024>, kSlots) : run(combine_gained_fwd_kernel<128, 512>, kSlots);
         } else {
-            if (big) run(combine_gained_fwd_kernel<64, 1024>, kSlots);
-            else run(combine_gained_fwd_kernel<64, 512>, kSlots);
+            ok = big ? run(combine_gained_fwd_kernel<64, 1024>, kSlots) : run(combine_gained_fwd_kernel<64, 512>, kSlots);
         }
+        if (!ok) return LOGO_ERR_CUDA;
     }
 #undef LOGO_COMBINE_FWD
     return cudaGetLastError() == cudaSuccess ? LOGO_OK : LOGO_ERR_CUDA;
@@ -1063,12 +1069,14 @@ int combine_bwd_common(const logo_bf16* dO, const logo_bf16* o_l, const logo_bf1
     } else if (!unit && dims.Hq * (dims.D / 8) <= kMaxVecGains) {
         auto run = [&](auto kernel, int slots) {
             const GainLaunch L = gain_launch(kernel, dims, slots);
+            if (!L.ok) return 0u;
             kernel<<<static_cast<unsigned>(L.grid), L.sh.threads, L.smem, st>>>(
                 dO, o_l, o_c, gate_p, z, row_of, gain_l, gain_g, eps, dO_l, dO_c, dgate_p, part, ntok, dims.Hq,
                 L.sh.tpr, L.sh.rows);
             return static_cast<unsigned>(L.grid);
         };
         grid = gains ? with_gained_bwd<true>(dims, run) : with_gained_bwd<false>(dims, run);
+        if (grid == 0) return LOGO_ERR_CUDA;
     } else if (unit && g == 2) {
         switch (gpt) {
             case 1: LOGO_COMBINE_BWD(1, 2, false, true); break;
