@@ -59,6 +59,7 @@ struct BwdParams {
     const float* lse;   // d = 128: local [B,Hq,T]; global [Hq,cap]
     const float* dsum;  // same layout as lse
     const float4* stats;  // d = 64: local [B,Hq][stat_rows / 2], global [Hq][stat_rows / 2] (RowStats)
+    const float4* stats0; // d = 64, local: zeros, for the rows of a tile past the sequence's end
     const int32_t* pos_c; // d = 64, global: pos, on a 16-byte boundary
     int64_t stat_rows;
     float* dq_acc;      // local [B,T,Hq,D]; global [cap+128,Hq,D]
@@ -766,8 +767,16 @@ __global__ void __launch_bounds__(Bwd64Cfg::kThreads, 1) attn_bwd64_kernel(const
                         mbar_arrive_expect_tx(qb, kStageBytes);
                         const int cb = GLOBAL ? 0 : it.b;
                         const int64_t plane = GLOBAL ? h : static_cast<int64_t>(it.b) * p.Hq + h;
-                        bulk_load(smem_u32(sh_pair[st]), p.stats + (plane * p.stat_rows + i * BQ) / 2, sizeof(sh_pair[0]), qb);
-                        if (GLOBAL) bulk_load(smem_u32(sh_pos[st]), p.pos_c + i * BQ, sizeof(sh_pos[0]), qb);
+                        const float4* stats = p.stats + (plane * p.stat_rows + i * BQ) / 2;
+                        if (GLOBAL) {
+                            bulk_load(smem_u32(sh_pair[st]), stats, sizeof(sh_pair[0]), qb);
+                            bulk_load(smem_u32(sh_pos[st]), p.pos_c + i * BQ, sizeof(sh_pos[0]), qb);
+                        } else {
+                            const uint32_t have = min(BQ, static_cast<int>(p.stat_rows) - i * BQ) / 2 * sizeof(float4);
+                            bulk_load(smem_u32(sh_pair[st]), stats, have, qb);
+                            if (have < sizeof(sh_pair[0]))
+                                bulk_load(smem_u32(sh_pair[st]) + have, p.stats0, sizeof(sh_pair[0]) - have, qb);
+                        }
                         tma_load_4d(sQ + st * 2 * C::kTileBytes, &p.tm_q, qb, 0, h, i * BQ, cb, pol_q);
                         tma_load_4d(sQ + (st * 2 + 1) * C::kTileBytes, &p.tm_do, qb, 0, h, i * BQ, cb, pol_q);
                         next_tile(it, h, i);
@@ -1098,9 +1107,11 @@ __global__ void __launch_bounds__(Bwd64Cfg::kThreads, 1) attn_bwd64_kernel(const
 // that lets the backward skip every query tile before it).
 // For d = 64 the pass writes what the backward kernel needs of a row as the
 // kernel's shared memory holds it, (-lse, -lse, -Dsum, -Dsum) of two adjacent
-// rows with lse in log2 units, in planes of a multiple of 128 rows (rows that do
-// not exist are zero) and with the positions beside them: a tile's are then two
-// bulk copies that come with its Q and dO.  (Loaded, converted and stored by the
+// rows with lse in log2 units, and with the positions beside them: a tile's are
+// then two bulk copies that come with its Q and dO.  Rows of a tile that do not
+// exist are zero: the packed rows' plane is filled to a multiple of 128, the
+// local branch's planes (one a sequence and head, perhaps of a single row) to an
+// even length only, and the rest of a last tile comes from one block of zeros.  (Loaded, converted and stored by the
 // softmax warps with a barrier of all 256 threads, and divisions in the roles'
 // loops: 2 x 8K, 16 heads, 1/8 selected, all kernels of the call 158 -> 149 us.)
 struct RowStats {
@@ -1108,9 +1119,12 @@ struct RowStats {
     float* out;        // null: d = 128, dsum is written instead
     int32_t* pos;      // global
     int64_t rows;      // of a plane
+    float4* zeros;     // local: the statistics of kBM rows that do not exist
 };
 
-__host__ __device__ constexpr int64_t stat_rows(int64_t rows) { return (rows + kBM - 1) / kBM * kBM; }
+__host__ __device__ constexpr int64_t packed_stat_rows(int64_t rows) { return (rows + kBM - 1) / kBM * kBM; }
+__host__ __device__ constexpr int64_t local_stat_rows(int64_t T) { return (T + 1) / 2 * 2; }
+constexpr size_t kStatZeros = kBM / 2 * sizeof(float4);
 
 struct GlobalPrep {
     const logo_bf16* q;   // dense [B, T, H, D]
@@ -1149,11 +1163,8 @@ __global__ void __launch_bounds__(128) bwd_pre_kernel(const logo_bf16* __restric
         at[0] = nlse;
         at[2] = ndsum;
     };
-    if (!GLOBAL && rst.out) {  // the rows that fill a plane's last tile
-        const int pad = static_cast<int>(rst.rows) - T;
-        for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < rows / T * H * pad; idx += gridDim.x * blockDim.x)
-            put_stats(idx / pad, T + idx % pad, 0.f, 0.f);
-    }
+    if (!GLOBAL && rst.out && blockIdx.x == 0)
+        for (int i = threadIdx.x; i < kBM / 2; i += blockDim.x) rst.zeros[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     for (int row = blockIdx.x; row < rows; row += gridDim.x) {
         const bool live = row < n;
         if (GLOBAL && rst.out && threadIdx.x == 0) rst.pos[row] = live ? gp.pos[row] : 0;
@@ -1196,7 +1207,9 @@ __global__ void __launch_bounds__(128) bwd_pre_kernel(const logo_bf16* __restric
                     const int b = GLOBAL ? 0 : row / T, tt = GLOBAL ? row : row % T;
                     const int64_t lse_row = GLOBAL ? static_cast<int64_t>(h) * cap + row
                                                    : (static_cast<int64_t>(b) * H + h) * T + tt;
-                    put_stats(static_cast<int64_t>(b) * H + h, tt, live ? -(rst.lse[lse_row] * kLog2e) : 0.f, -acc);
+                    const int64_t plane = static_cast<int64_t>(b) * H + h;
+                    put_stats(plane, tt, live ? -(rst.lse[lse_row] * kLog2e) : 0.f, -acc);
+                    if (!GLOBAL && tt + 1 == T && tt + 1 < rst.rows) put_stats(plane, tt + 1, 0.f, 0.f);
                 } else if (live && jj == 0) {
                     if (GLOBAL) dsum[static_cast<int64_t>(h) * cap + row] = acc;
                     else {
@@ -1257,6 +1270,7 @@ struct BwdWs {
     logo_bf16* qc;
     logo_bf16* doc;
     float* dsum;  // d = 128; d = 64: the row stats
+    float4* zeros;
     int32_t* pos_c;
     float* dq_acc;
     int32_t* first_row;
@@ -1267,13 +1281,16 @@ size_t local_bwd_ws_layout(const logo_dims& d, char* base, BwdWs* ws)
     const size_t rows = static_cast<size_t>(d.B) * d.T;
     size_t off = 0;
     const size_t o_ds = off;
-    const size_t stats = d.D == 64 ? static_cast<size_t>(d.B) * stat_rows(d.T) * 2 : rows;
+    const size_t stats = d.D == 64 ? static_cast<size_t>(d.B) * local_stat_rows(d.T) * 2 : rows;
     off = round_up(off + stats * d.Hq * sizeof(float), 256);
+    const size_t o_zr = off;
+    if (d.D == 64) off = round_up(off + kStatZeros, 256);
     const size_t o_dq = off;
     off = round_up(off + (rows + kBM) * d.Hq * d.D * sizeof(float), 256);
     if (ws) {
         ws->qc = ws->doc = nullptr;
         ws->pos_c = nullptr;
+        ws->zeros = reinterpret_cast<float4*>(base + o_zr);
         ws->dsum = reinterpret_cast<float*>(base + o_ds);
         ws->dq_acc = reinterpret_cast<float*>(base + o_dq);
         ws->first_row = nullptr;
@@ -1291,16 +1308,17 @@ size_t global_bwd_ws_layout(const logo_dims& d, char* base, BwdWs* ws)
     const size_t o_do = off;
     off = round_up(off + rows * d.Hq * d.D * 2, 256);
     const size_t o_ds = off;
-    const size_t stats = d.D == 64 ? static_cast<size_t>(stat_rows(rows)) * 2 : cap;
+    const size_t stats = d.D == 64 ? static_cast<size_t>(packed_stat_rows(rows)) * 2 : cap;
     off = round_up(off + stats * d.Hq * sizeof(float), 256);
     const size_t o_pc = off;
-    if (d.D == 64) off = round_up(off + stat_rows(rows) * sizeof(int32_t), 256);
+    if (d.D == 64) off = round_up(off + packed_stat_rows(rows) * sizeof(int32_t), 256);
     const size_t o_dq = off;
     off = round_up(off + rows * d.Hq * d.D * sizeof(float), 256);
     const size_t o_fr = off;
     off = round_up(off + static_cast<size_t>(d.B) * ((d.T + kBN - 1) / kBN) * sizeof(int32_t), 256);
     if (ws) {
         ws->first_row = reinterpret_cast<int32_t*>(base + o_fr);
+        ws->zeros = nullptr;
         ws->pos_c = reinterpret_cast<int32_t*>(base + o_pc);
         ws->qc = reinterpret_cast<logo_bf16*>(base + o_qc);
         ws->doc = reinterpret_cast<logo_bf16*>(base + o_do);
@@ -1374,11 +1392,12 @@ extern "C" int logo_local_attn_bwd(const logo_bf16* q, const logo_bf16* k, const
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int rows = dims.B * dims.T;
     const int pre_grid = max(1, min(rows, device_sm_count() * 16));
-    const RowStats rst{lse, dims.D == 64 ? ws.dsum : nullptr, nullptr, stat_rows(dims.T)};
+    const RowStats rst{lse, dims.D == 64 ? ws.dsum : nullptr, nullptr, local_stat_rows(dims.T), ws.zeros};
     bwd_pre_kernel<false><<<pre_grid, 128, 0, st>>>(o, dO, nullptr, rows, dims.T, dims.Hq, dims.D, 0, ws.dsum,
                                                     nullptr, ws.dq_acc, GlobalPrep{}, rst);
     BwdParams prm{};
     prm.stats = reinterpret_cast<const float4*>(rst.out);
+    prm.stats0 = rst.zeros;
     prm.stat_rows = rst.rows;
     const uint32_t qrows = dims.D == 128 ? Bwd2Cfg::kBQ : Bwd64Cfg::kBQ;
     if (!encode_bf16_4d(&prm.tm_q, q, dims.D, dims.Hq, dims.T, dims.B, 64, qrows) ||
@@ -1436,7 +1455,8 @@ extern "C" int logo_global_sparse_attn_bwd(const logo_bf16* q, const logo_bf16* 
     const int grid_rows = max(1, min(cap + kBM, device_sm_count() * 16));
     const int nblk = (dims.T + kBN - 1) / kBN;
     const GlobalPrep gp{q, pos, cu_q, ws.qc, ws.first_row, dims.B, nblk};
-    const RowStats rst{lse_c, dims.D == 64 ? ws.dsum : nullptr, ws.pos_c, stat_rows(static_cast<int64_t>(cap) + kBM)};
+    const RowStats rst{lse_c, dims.D == 64 ? ws.dsum : nullptr, ws.pos_c, packed_stat_rows(static_cast<int64_t>(cap) + kBM),
+                       nullptr};
     bwd_pre_kernel<true><<<grid_rows, 128, 0, st>>>(o_c, dO_c, n_sel_total, 0, dims.T, dims.Hq, dims.D, cap, ws.dsum,
                                                     ws.doc, ws.dq_acc, gp, rst);
     if (cudaGetLastError() != cudaSuccess) return LOGO_ERR_CUDA;
