@@ -420,9 +420,19 @@ def logo_select_noalloc(gate_p, mode: int, b_th: float = 0.5, ratio: float = 0.0
     return z, pos, cu_q, row_of, n_sel_total
 
 
+def _own_buffers(stream, *buffers):
+    """A buffer made here belongs to the current stream, and goes back to its pool
+    while a kernel on another stream may still use it."""
+    if stream is not None and any(b is None for b in buffers):
+        raise ValueError("stream= needs every output and workspace given")
+
+
 def logo_local_attn_fwd(q, k, v, window: int, scale: float = 0.0, o=None, lse=None, *, stream=None):
     """Eq. 6 local branch.  Returns (o [B,T,Hq,D] bf16, lse [B,Hq,T] fp32).
-    stream: raw handle of the stream to launch on (default: the current one)."""
+    stream: raw handle of the stream to launch on (default: the current one);
+    every output must then be given, and the tensors' lifetimes on that stream are
+    the caller's."""
+    _own_buffers(stream, o, lse)
     for t, n in ((q, "q"), (k, "k"), (v, "v")):
         _need(t, torch.bfloat16, n)
     d = _dims_of(q, k)
@@ -436,7 +446,8 @@ def logo_local_attn_fwd(q, k, v, window: int, scale: float = 0.0, o=None, lse=No
 def logo_local_attn_bwd(q, k, v, o, lse, dO, window: int, scale: float = 0.0, dq=None, dk=None, dv=None,
                         workspace=None, *, stream=None):
     """Gradients of the local branch.  Returns (dq, dk, dv).
-    stream: as in logo_local_attn_fwd (with every output and the workspace given)."""
+    stream: as in logo_local_attn_fwd, with every output and the workspace given."""
+    _own_buffers(stream, dq, dk, dv, workspace)
     d = _dims_of(q, k)
     for t, n in ((q, "q"), (k, "k"), (v, "v"), (o, "o"), (dO, "dO")):
         _need(t, torch.bfloat16, n)
