@@ -54,9 +54,8 @@ class LogoAttention:
         dev = torch.device(device)
         self.overlap = overlap
         self.side = torch.cuda.Stream(device=dev) if overlap and dev.type == "cuda" else None
-        if self.side is not None:  # recorded anew on every fork and join
+        if dev.type == "cuda":  # recorded anew on every fork and join
             self._forked, self._joined = torch.cuda.Event(), torch.cuda.Event()
-            self._side_handle = self.side.cuda_stream
         self.dims = L.Dims(c.B, c.T, c.Hq, c.Hkv, c.D)
         cap = c.B * c.T
         bf, f32, i32 = torch.bfloat16, torch.float32, torch.int32
@@ -109,12 +108,12 @@ class LogoAttention:
             other()
             local(None)
             return
-        main = torch.cuda.current_stream()
+        main, side = torch.cuda.current_stream(), self.side
         self._forked.record(main)
-        self.side.wait_event(self._forked)
-        local(self._side_handle)
+        side.wait_event(self._forked)
+        local(side.cuda_stream)
         other()
-        self._joined.record(self.side)
+        self._joined.record(side)
         main.wait_event(self._joined)
 
     def forward(self, qL, kL, vL, qG, kG, vG, gate_p, gain_l=None, gain_g=None):
