@@ -106,14 +106,16 @@ struct DecVisible {
 };
 
 // Sub-tiles of sequence b's cache that the call reads (per KV head): its rows
-// in use; none for a sequence the global call does not have.
+// in use; none for a sequence the global call does not have (n_rows: its packed
+// rows, read once).
 template <bool RING>
-__device__ __forceinline__ int dec_subs(const DecParams& p, int b, int* len)
+__device__ __forceinline__ int dec_subs(const DecParams& p, int n_rows, int b, int* len)
 {
     int n = p.seq_len[b];
     if (!RING) {
         n = min(n, p.R);  // a dense cache holds at most R tokens
-        if (p.cu_q[b + 1] == p.cu_q[b]) n = 0;
+        const int row = p.cu_q[b];
+        if (p.cu_q[b + 1] == row || row >= n_rows) n = 0;
     }
     *len = n;
     return (max(0, min(n, p.R)) + kDecRows - 1) / kDecRows;
@@ -130,7 +132,7 @@ struct DecPiece {
 // The next piece: of the next pair in order, or (whole pairs) of the pair a
 // grid further on.
 template <bool RING>
-__device__ __forceinline__ void dec_next_piece(const DecParams& p, DecPiece& c)
+__device__ __forceinline__ void dec_next_piece(const DecParams& p, int n_rows, DecPiece& c)
 {
     c.pair0 += c.subs;
     c.s = c.s1 = 0;
@@ -141,7 +143,7 @@ __device__ __forceinline__ void dec_next_piece(const DecParams& p, DecPiece& c)
             if (c.pair >= p.B * p.Hkv) return;
             c.b = c.pair / p.Hkv;
             c.kvh = c.pair - c.b * p.Hkv;
-            c.subs = dec_subs<RING>(p, c.b, &c.len);
+            c.subs = dec_subs<RING>(p, n_rows, c.b, &c.len);
         }
         c.s1 = c.subs;
         return;
@@ -150,7 +152,7 @@ __device__ __forceinline__ void dec_next_piece(const DecParams& p, DecPiece& c)
     if (++c.kvh == p.Hkv) {
         c.kvh = 0;
         c.subs = 0;
-        while (c.subs == 0 && ++c.b < p.B) c.subs = dec_subs<RING>(p, c.b, &c.len);
+        while (c.subs == 0 && ++c.b < p.B) c.subs = dec_subs<RING>(p, n_rows, c.b, &c.len);
     }
     c.s1 = min(c.subs, c.left);
     c.left -= c.s1;
@@ -187,6 +189,7 @@ __global__ void __launch_bounds__(kDecThreads, 2) decode_attn_kernel(const __gri
         tma_prefetch_desc(&p.tm_k);
         tma_prefetch_desc(&p.tm_v);
     }
+    const int n_rows = RING ? 0 : *p.n_sel;
     DecPiece cur{};
     long long S = 0, G = 0;
     // a b / c; in 32 bits (a tenth of the instructions) for up to 1M sub-tiles: G < 2^11
@@ -197,15 +200,15 @@ __global__ void __launch_bounds__(kDecThreads, 2) decode_attn_kernel(const __gri
     if (!p.done) {  // whole pairs, a grid apart
         __syncthreads();
         cur.pair = static_cast<int>(blockIdx.x) - static_cast<int>(gridDim.x);
-        dec_next_piece<RING>(p, cur);
+        dec_next_piece<RING>(p, n_rows, cur);
     } else {
         // this CTA's run [lo, hi) of the call's S sub-tiles: the total first,
         // then the pair that holds sub-tile lo
         int len0 = 0;
-        const int subs0 = tid < p.B ? dec_subs<RING>(p, tid, &len0) : 0;  // of sequence tid, for both passes
+        const int subs0 = tid < p.B ? dec_subs<RING>(p, n_rows, tid, &len0) : 0;  // of sequence tid, for both passes
         long long mine = subs0;
         int len;
-        for (int b = tid + kDecThreads; b < p.B; b += kDecThreads) mine += dec_subs<RING>(p, b, &len);
+        for (int b = tid + kDecThreads; b < p.B; b += kDecThreads) mine += dec_subs<RING>(p, n_rows, b, &len);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) mine += __shfl_xor_sync(0xffffffffu, mine, o);
         if (lane == 0) sh_scan[warp] = mine;
@@ -219,7 +222,7 @@ __global__ void __launch_bounds__(kDecThreads, 2) decode_attn_kernel(const __gri
         for (int b0 = 0; b0 < p.B; b0 += kDecThreads) {  // (one round for up to 128 sequences)
             const int b = b0 + tid;
             int n = len0;
-            const int subs = b0 == 0 ? subs0 : (b < p.B ? dec_subs<RING>(p, b, &n) : 0);
+            const int subs = b0 == 0 ? subs0 : (b < p.B ? dec_subs<RING>(p, n_rows, b, &n) : 0);
             long long x = static_cast<long long>(subs) * p.Hkv;
             const long long v = x;
 #pragma unroll
@@ -272,7 +275,7 @@ __global__ void __launch_bounds__(kDecThreads, 2) decode_attn_kernel(const __gri
                         pit.b, pol);
         }
         ++issued;
-        if (++pit.s == pit.s1) dec_next_piece<RING>(p, pit);
+        if (++pit.s == pit.s1) dec_next_piece<RING>(p, n_rows, pit);
     };
     for (int i = 0; i < kDecStages - 1; ++i) issue();
 
@@ -284,7 +287,7 @@ __global__ void __launch_bounds__(kDecThreads, 2) decode_attn_kernel(const __gri
     // the four warps' results are combined once per item.
     constexpr int NT = D / 8;
     int consumed = 0;
-    for (; cur.s < cur.s1 && ok; dec_next_piece<RING>(p, cur)) {
+    for (; cur.s < cur.s1 && ok; dec_next_piece<RING>(p, n_rows, cur)) {
         const DecPiece it = cur;
         const int h0 = it.kvh * group;
         const int out_row = RING ? it.b : p.cu_q[it.b];
