@@ -560,12 +560,28 @@ __global__ void __launch_bounds__(kDecThreads, 2) decode_attn_kernel(const __gri
     }
 }
 
-constexpr int kDecCtasPerSm = 8;  // at most (the workspace's slots)
+constexpr int kDecCtasPerSm = 2;  // resident at most: what the registers of 128 threads allow
+
+// How a call's sub-tiles are cut into runs: at least min_sub each (short enough
+// to fill the GPU, at least kDecMinSub, and long enough for kDecMaxPieces pieces
+// of a pair), by at most `ctas` CTAs.
+struct DecCut {
+    int min_sub;
+    long long ctas;
+};
+
+DecCut dec_cut(const logo_dims& d, long long resident)
+{
+    const long long n_sub = (d.T + kDecRows - 1) / kDecRows, subs = static_cast<long long>(d.B) * d.Hkv * n_sub;
+    const long long min_sub = std::max<long long>(kDecMinSub, (n_sub + kDecMaxPieces - 3) / (kDecMaxPieces - 2));
+    return DecCut{static_cast<int>(min_sub), std::max(1ll, std::min(subs / min_sub, resident))};
+}
 
 // part: [2 x CTAs, group, D] fp32, part_ml: [2 x CTAs, group] fp32 pairs, done: [B, Hkv] int32
 size_t decode_ws_layout(const logo_dims& d, char* base, DecParams* p)
 {
-    const size_t rows = 2 * static_cast<size_t>(kDecCtasPerSm) * device_sm_count() * (d.Hq / d.Hkv);
+    const long long ctas = dec_cut(d, static_cast<long long>(kDecCtasPerSm) * device_sm_count()).ctas;
+    const size_t rows = 2 * static_cast<size_t>(ctas) * (d.Hq / d.Hkv);
     size_t off = round_up(rows * d.D * sizeof(float), 256);
     const size_t o_ml = off;
     off = round_up(off + rows * sizeof(float2), 256);
@@ -588,7 +604,7 @@ int check_decode(const logo_dims& d)
 }
 
 template <int D, bool RING>
-int launch_decode(DecParams& prm, cudaStream_t st)
+int launch_decode(DecParams& prm, const logo_dims& dims, cudaStream_t st)
 {
     static bool attr_done = false;  // benign race: setting the attribute twice is harmless
     if (!attr_done) {
@@ -613,8 +629,7 @@ int launch_decode(DecParams& prm, cudaStream_t st)
     const long long ctas = static_cast<long long>(std::min(per_sm, kDecCtasPerSm)) * device_sm_count();
     // Whole pairs when cutting them saves less than kDecSplitCost sub-tiles of
     // the longest run (with full caches; the merge and the counters' clearing
-    // cost that much), else equal runs: short enough to fill the GPU, at least
-    // kDecMinSub, and long enough for kDecMaxPieces pieces of a pair.
+    // cost that much), else equal runs.
     const long long whole_run = (pairs + ctas - 1) / ctas * n_sub;
     const long long cut_run = std::max<long long>(kDecMinSub, (pairs * n_sub + ctas - 1) / ctas);
     long long grid;
@@ -622,8 +637,9 @@ int launch_decode(DecParams& prm, cudaStream_t st)
         prm.done = nullptr;
         grid = std::min(pairs, ctas);
     } else {
-        prm.min_sub = static_cast<int>(std::max<long long>(kDecMinSub, (n_sub + kDecMaxPieces - 3) / (kDecMaxPieces - 2)));
-        grid = std::max(1ll, std::min(pairs * n_sub / prm.min_sub, ctas));
+        const DecCut cut = dec_cut(dims, ctas);
+        prm.min_sub = cut.min_sub;
+        grid = cut.ctas;
         if (cudaMemsetAsync(prm.done, 0, static_cast<size_t>(pairs) * sizeof(int32_t), st) != cudaSuccess)
             return LOGO_ERR_CUDA;
     }
@@ -662,8 +678,8 @@ int run_decode(bool ring, const logo_bf16* q, const logo_bf16* k, const logo_bf1
     prm.window = window;
     prm.scale_log2 = scale * kLog2e;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (dims.D == 128) return ring ? launch_decode<128, true>(prm, st) : launch_decode<128, false>(prm, st);
-    return ring ? launch_decode<64, true>(prm, st) : launch_decode<64, false>(prm, st);
+    if (dims.D == 128) return ring ? launch_decode<128, true>(prm, dims, st) : launch_decode<128, false>(prm, dims, st);
+    return ring ? launch_decode<64, true>(prm, dims, st) : launch_decode<64, false>(prm, dims, st);
 }
 
 }  // namespace
