@@ -52,6 +52,7 @@ constexpr int kDecRowsPerWarp = kDecRows / 4;
 constexpr int kDecMaxGroup = 16;  // query heads per KV head (the mma tile's 16 rows)
 constexpr int kDecMinSub = 2;     // sub-tiles of a CTA's run at least
 constexpr int kDecSplitCost = 4;  // what cutting pairs into pieces has to save, in sub-tiles
+constexpr int kDecMaxWholeDense = 24, kDecMaxWholeRing = 32;  // sub-tiles of a pair left whole at most
 constexpr int kDecStages = 3;     // TMA ring depth
 
 struct DecParams {
@@ -629,11 +630,18 @@ int launch_decode(DecParams& prm, const logo_dims& dims, cudaStream_t st)
     const long long ctas = static_cast<long long>(std::min(per_sm, kDecCtasPerSm)) * device_sm_count();
     // Whole pairs when cutting them saves less than kDecSplitCost sub-tiles of
     // the longest run (with full caches; the merge and the counters' clearing
-    // cost that much), else equal runs.
+    // cost that much), else equal runs.  What is selected and how long the
+    // sequences are is not known here, so a pair of more than kMaxWhole sub-tiles
+    // is always cut: one CTA takes 0.7 us for a sub-tile and may be the only one
+    // with work.  38 sequences of 16K rows and 8 KV heads (a pair a CTA) whole and
+    // cut: 4 selected 192 and 50 us, all 375 and 378; of 2K rows: 2 selected 30
+    // and 12, all 51 and 55; a ring of 4K slots, one sequence long 60 and 17, all
+    // 94 and 99.
+    constexpr int kMaxWhole = RING ? kDecMaxWholeRing : kDecMaxWholeDense;
     const long long whole_run = (pairs + ctas - 1) / ctas * n_sub;
     const long long cut_run = std::max<long long>(kDecMinSub, (pairs * n_sub + ctas - 1) / ctas);
     long long grid;
-    if (whole_run <= cut_run + kDecSplitCost) {
+    if (n_sub <= kMaxWhole && whole_run <= cut_run + kDecSplitCost) {
         prm.done = nullptr;
         grid = std::min(pairs, ctas);
     } else {
