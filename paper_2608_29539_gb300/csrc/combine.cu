@@ -770,13 +770,14 @@ __global__ void __launch_bounds__(MAXT) combine_gained_bwd_kernel(
         const bool sel = rt.row >= 0;
         const float pt = rt.p, wl = sel ? 1.0f - pt : 1.0f;
         const Vec8 g = unpack8(*reinterpret_cast<const uint4*>(slot));
-        float dp = 0.f;
+        float dp = 0.f, r_l, xl;  // the local branch's 1 / rms, and this lane's part of x dy / wl
         {  // dy = dO wl; dx = r gain dy - x r^3 mean(x gain dy); d gain = dy x r
             const Vec8 x = unpack8(*reinterpret_cast<const uint4*>(slot + nthr));
             const Vec8 gy = mul8(g, kInRegs ? gl_r : slot_load(sh_gain, nthr, 0, threadIdx.x));
             const float ss = lane_sum<VPR>(sumsq8(x));
-            const float xd = lane_sum<VPR>(dot8(x, gy));
-            const float r = rsqrtf(ss * (1.0f / D) + eps);
+            xl = dot8(x, gy);
+            const float xd = lane_sum<VPR>(xl);
+            const float r = r_l = rsqrtf(ss * (1.0f / D) + eps);
             if (live) store_bf16x8(dO_l + off, axpby8(gy, r * wl, &x, -(r * r * r * (xd * wl) * (1.0f / D))));
             if (DGAIN && kInRegs) fma8(sum_l, g, x, live ? wl * r : 0.f);
             if (DGAIN && !kInRegs && live) {
@@ -784,13 +785,12 @@ __global__ void __launch_bounds__(MAXT) combine_gained_bwd_kernel(
                 fma8(a, g, x, wl * r);
                 slot_store(sh_sum, nthr, 0, threadIdx.x, a);
             }
-            dp = -r * xd;  // sum over d of dO o~L: the head's sum
         }
         if (sel) {
             const Vec8 x = unpack8(*reinterpret_cast<const uint4*>(slot + 2 * nthr));
             const Vec8 gy = mul8(g, kInRegs ? gg_r : slot_load(sh_gain, nthr, 1, threadIdx.x));
             const float ss = lane_sum<VPR>(sumsq8(x));
-            const float xd = lane_sum<VPR>(dot8(x, gy));
+            const float xg = dot8(x, gy), xd = lane_sum<VPR>(xg);
             const float r = rsqrtf(ss * (1.0f / D) + eps);
             if (live)
                 store_bf16x8(dc_v + static_cast<int64_t>(rt.row) * (nvec * 8),
@@ -801,8 +801,12 @@ __global__ void __launch_bounds__(MAXT) combine_gained_bwd_kernel(
                 fma8(a, g, x, pt * r);
                 slot_store(sh_sum, nthr, 1, threadIdx.x, a);
             }
-            // dp_t = z_t sum over heads and d of dO (o~G - o~L): one lane a head
-            dp = lane_sum<32>(me.active && me.j0 == 0 ? dp + r * xd : 0.f);
+            // dp_t = z_t sum over heads and d of dO (o~G - o~L), the difference taken
+            // of each lane's eight elements: the branches' outputs may nearly agree,
+            // and the difference of their heads' sums then had 1.8 times the error
+            // (five times where they are equal; these products are rounded alike, not
+            // one of them by an FMA, so that equal branches give zero)
+            dp = lane_sum<32>(__fsub_rn(__fmul_rn(r, xg), __fmul_rn(r_l, xl)));
         }
         if ((threadIdx.x & 31) == 0) sh_dp[buf][k][warp] = sel ? dp : 0.f;
         if (++k == kGroup || tb + step >= ntok) {  // (two buffers: one barrier a group is enough)
