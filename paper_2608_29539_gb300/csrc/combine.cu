@@ -779,7 +779,7 @@ __global__ void __launch_bounds__(MAXT) combine_gained_bwd_kernel(
             const float xd = lane_sum<VPR>(xl);
             const float r = r_l = rsqrtf(ss * (1.0f / D) + eps);
             if (live) store_bf16x8(dO_l + off, axpby8(gy, r * wl, &x, -(r * r * r * (xd * wl) * (1.0f / D))));
-            if (DGAIN && kInRegs) fma8(sum_l, g, x, live ? wl * r : 0.f);
+            if (DGAIN && kInRegs && live) fma8(sum_l, g, x, wl * r);  // (a slot past the end may hold infinities)
             if (DGAIN && !kInRegs && live) {
                 Vec8 a = slot_load(sh_sum, nthr, 0, threadIdx.x);
                 fma8(a, g, x, wl * r);
@@ -795,7 +795,7 @@ __global__ void __launch_bounds__(MAXT) combine_gained_bwd_kernel(
             if (live)
                 store_bf16x8(dc_v + static_cast<int64_t>(rt.row) * (nvec * 8),
                              axpby8(gy, r * pt, &x, -(r * r * r * (xd * pt) * (1.0f / D))));
-            if (DGAIN && kInRegs) fma8(sum_g, g, x, live ? pt * r : 0.f);
+            if (DGAIN && kInRegs && live) fma8(sum_g, g, x, pt * r);
             if (DGAIN && !kInRegs && live) {
                 Vec8 a = slot_load(sh_sum, nthr, 1, threadIdx.x);
                 fma8(a, g, x, pt * r);
