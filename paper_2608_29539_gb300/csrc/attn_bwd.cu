@@ -69,7 +69,7 @@ struct BwdParams {
     const int32_t* cu_q;
     const int32_t* first_row;  // global: [B, nblk] first packed row of sequence b whose position reaches block j
     logo_bf16* dq_fill;        // global: dense dQ [B, T, Hq, D] whose unselected rows this kernel zeroes
-    int B, T, Hq, Hkv, window, cap, nblk, q_tiles;
+    int B, T, Hq, Hkv, window, cap, nblk;
     float scale, scale_log2;
 };
 
@@ -1418,7 +1418,6 @@ extern "C" int logo_local_attn_bwd(const logo_bf16* q, const logo_bf16* k, const
     prm.window = window > dims.T ? dims.T : window;
     prm.cap = rows;
     prm.nblk = (dims.T + kBN - 1) / kBN;
-    prm.q_tiles = (dims.T + kBM - 1) / kBM;
     prm.scale = scale;
     prm.scale_log2 = scale * kLog2e;
     rc = dims.D == 128 ? launch_bwd<128, false>(prm, st) : launch_bwd<64, false>(prm, st);
@@ -1488,7 +1487,6 @@ extern "C" int logo_global_sparse_attn_bwd(const logo_bf16* q, const logo_bf16* 
     prm.window = kNoWindow;
     prm.cap = cap;
     prm.nblk = (dims.T + kBN - 1) / kBN;
-    prm.q_tiles = 0;
     prm.scale = scale;
     prm.scale_log2 = scale * kLog2e;
     rc = dims.D == 128 ? launch_bwd<128, true>(prm, st) : launch_bwd<64, true>(prm, st);

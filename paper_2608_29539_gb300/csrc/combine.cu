@@ -275,13 +275,12 @@ __global__ void __launch_bounds__(kThreads, fwd_min_blocks<GPT, G, UNIT>()) comb
 
 // Register bound of a backward variant: with unit gains one two-vector group
 // per thread is held to 4 blocks per SM (3 with the gain sums in shared
-// memory), one one-vector group to 5; one-vector groups with the gain sums,
-// or with gains read, up to two per thread, are held to 3.
+// memory), one one-vector group to 5, with the gain sums up to two of them to 3.
 template <int GPT, int G, bool DGAIN, bool UNIT>
 __host__ __device__ constexpr int bwd_min_blocks()
 {
     return G == 2 ? (GPT == 1 ? (DGAIN ? 3 : 4) : 1)
-                  : ((DGAIN || !UNIT) && GPT <= 2 ? 3 : (UNIT && GPT == 1 ? 5 : 1));
+                  : (DGAIN && GPT <= 2 ? 3 : (UNIT && GPT == 1 ? 5 : 1));
 }
 
 // part (DGAIN): [gridDim.x][2][H*D] float32 per-block sums of the local and
@@ -294,7 +293,7 @@ __global__ void __launch_bounds__(kThreads, bwd_min_blocks<GPT, G, DGAIN, UNIT>(
     const float* __restrict__ gain_l, const float* __restrict__ gain_g, float eps, logo_bf16* __restrict__ dO_l,
     logo_bf16* __restrict__ dO_c, float* __restrict__ dgate_p, float* __restrict__ part, int64_t ntok, int H, int D)
 {
-    static_assert(G == 1 || (G == 2 && UNIT), "two-vector groups only with unit gains");
+    static_assert(UNIT || (G == 1 && !DGAIN), "two-vector groups and gain sums only with unit gains");
     __shared__ float sh_dp[2][kThreads / 32];
     const int vpr = D / 8, gpr = vpr / G;
     const int nvec = H * vpr, ngrp = nvec / G;
@@ -399,12 +398,6 @@ __global__ void __launch_bounds__(kThreads, bwd_min_blocks<GPT, G, DGAIN, UNIT>(
 #pragma unroll
             for (int i = 0; i < 8; ++i) dxl.v[i] = r_l * gl.v[i] * g[0].v[i] * wl - xl[0].v[i] * cl;
             if (active) store_bf16x8(dO_l + (bt * nvec + v0) * 8, dxl);
-            if constexpr (DGAIN) {  // d gain_l = dy * x r
-                Vec8 c;
-#pragma unroll
-                for (int i = 0; i < 8; ++i) c.v[i] = g[0].v[i] * wl * xl[0].v[i] * r_l;
-                if (active) acc_add8(sh_acc, nvec, 0, u, c);
-            }
             if (sel) {
                 const Vec8 xg = unpack8(rg[k][0]);
                 const Vec8 gg = load_gain(gain_g, h, D, j0);
@@ -425,12 +418,6 @@ __global__ void __launch_bounds__(kThreads, bwd_min_blocks<GPT, G, DGAIN, UNIT>(
                     dp_acc += g[0].v[i] * (xg.v[i] * r_g * gg.v[i] - xl[0].v[i] * r_l * gl.v[i]);
                 }
                 if (active) store_bf16x8(dO_c + (row * nvec + v0) * 8, dxg);
-                if constexpr (DGAIN) {
-                    Vec8 c;
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) c.v[i] = g[0].v[i] * pt * xg.v[i] * r_g;
-                    if (active) acc_add8(sh_acc, nvec, 1, u, c);
-                }
             }
         }
         if constexpr (UNIT) {
@@ -507,17 +494,6 @@ struct GainCfg {
     static constexpr bool kInRegs = MAXT <= 512;
     static constexpr int kRingBwd = kInRegs ? 4 : 2;
 };
-
-__device__ __forceinline__ void copy16_async(uint32_t dst, const void* src)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
-}
-__device__ __forceinline__ void copies_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void copies_wait()  // all but the newest N groups have landed
-{
-    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
 
 struct Routing {
     int row;  // packed row, -1: not selected (or no such token)
@@ -652,10 +628,10 @@ __global__ void __launch_bounds__(MAXT, MAXT == 512 ? 2 : 1) combine_gained_fwd_
     auto issue = [&]() {
         const Routing nx = ahead.get(z, row_of, gate_p, t_issue, step, ntok);
         if (me.active && t_issue < ntok) {
-            copy16_async(dst, o_l + off_issue);
-            if (nx.row >= 0) copy16_async(dst + nthr * 16, oc_v + static_cast<int64_t>(nx.row) * (nvec * 8));
+            cp_async16(dst, o_l + off_issue);
+            if (nx.row >= 0) cp_async16(dst + nthr * 16, oc_v + static_cast<int64_t>(nx.row) * (nvec * 8));
         }
-        copies_commit();
+        cp_async_commit();
         if ((threadIdx.x & 31) == 0) *rt_issue = nx;
         t_issue += step;
         off_issue += step_el;
@@ -671,7 +647,7 @@ __global__ void __launch_bounds__(MAXT, MAXT == 512 ? 2 : 1) combine_gained_fwd_
     for (; t < ntok; t += step, off += step_el) {
         __syncwarp();  // every lane has read the routing slot that is written next
         issue();
-        copies_wait<S - 1>();
+        cp_async_wait<S - 1>();
         __syncwarp();
         const Routing rt = sh_rt[st][warp];
         const Vec8 x = unpack8(*reinterpret_cast<const uint4*>(slot));
@@ -693,7 +669,7 @@ __global__ void __launch_bounds__(MAXT, MAXT == 512 ? 2 : 1) combine_gained_fwd_
         st = wrap ? 0 : st;
         slot = wrap ? sh_dyn + threadIdx.x : slot + 2 * nthr;
     }
-    copies_wait<0>();
+    cp_async_wait<0>();
 }
 
 // part (DGAIN): [gridDim.x][2][H*D] float32 per-block sums of the local and
@@ -742,11 +718,11 @@ __global__ void __launch_bounds__(MAXT) combine_gained_bwd_kernel(
     auto issue = [&]() {
         const Routing nx = ahead.get(z, row_of, gate_p, t_issue, step, ntok);
         if (me.active && t_issue < ntok) {
-            copy16_async(dst, dO + off_issue);
-            copy16_async(dst + nthr * 16, o_l + off_issue);
-            if (nx.row >= 0) copy16_async(dst + nthr * 32, oc_v + static_cast<int64_t>(nx.row) * (nvec * 8));
+            cp_async16(dst, dO + off_issue);
+            cp_async16(dst + nthr * 16, o_l + off_issue);
+            if (nx.row >= 0) cp_async16(dst + nthr * 32, oc_v + static_cast<int64_t>(nx.row) * (nvec * 8));
         }
-        copies_commit();
+        cp_async_commit();
         if ((threadIdx.x & 31) == 0) *rt_issue = nx;
         t_issue += step;
         off_issue += step_el;
@@ -763,7 +739,7 @@ __global__ void __launch_bounds__(MAXT) combine_gained_bwd_kernel(
     for (int64_t tb = static_cast<int64_t>(blockIdx.x) * rows; tb < ntok; tb += step, t += step, off += step_el) {
         __syncwarp();  // every lane has read the routing slot that is written next
         issue();
-        copies_wait<S - 1>();
+        cp_async_wait<S - 1>();
         __syncwarp();
         const Routing rt = sh_rt[st][warp];
         const bool live = me.active && t < ntok;
@@ -826,7 +802,7 @@ __global__ void __launch_bounds__(MAXT) combine_gained_bwd_kernel(
         st = wrap ? 0 : st;
         slot = wrap ? sh_dyn + threadIdx.x : slot + 3 * nthr;
     }
-    copies_wait<0>();
+    cp_async_wait<0>();
     if (DGAIN) {
         // the block's rows of threads in order, then its partial row
         if (kInRegs) {

@@ -48,14 +48,6 @@ __device__ __forceinline__ int64_t row_token(const RowSet& R, int r)
     return static_cast<int64_t>(b) * R.T + R.pos[r];
 }
 
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_one() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
-
 // out[h][e] = sum over c of part[h][c][e], e < per_head (a multiple of 4).
 // Thread (x, g) of a block adds chunks g, g + 4, .. of four columns, then the
 // four sums are added in order: a fixed order, and every load in flight.  `out`
@@ -315,12 +307,12 @@ __global__ void __launch_bounds__(32 * (kLpProducers<GATHER> + 5), 1) lp_tc_fwd_
                 }
                 cp_async_commit();
                 if (k > 0) {  // tile k-1 has landed while tile k was issued
-                    cp_async_wait_one();
+                    cp_async_wait<1>();
                     fence_proxy_async_smem();
                     mbar_arrive(smem_u32(&bar_u_full[st ^ 1]));
                 }
             }
-            cp_async_wait_all();
+            cp_async_wait<0>();
             if (ok && k > 0) {
                 fence_proxy_async_smem();
                 mbar_arrive(smem_u32(&bar_u_full[(k - 1) & 1]));
@@ -603,12 +595,12 @@ __global__ void __launch_bounds__(kLpBwdThreads, 1) lp_tc_bwd_kernel(const __gri
                 }
                 cp_async_commit();
                 if (k > 0) {  // tile k-1 has landed while tile k was issued
-                    cp_async_wait_one();
+                    cp_async_wait<1>();
                     fence_proxy_async_smem();
                     mbar_arrive(smem_u32(&bar_in_full[st ^ 1]));
                 }
             }
-            cp_async_wait_all();
+            cp_async_wait<0>();
             if (ok && k > 0) {
                 fence_proxy_async_smem();
                 mbar_arrive(smem_u32(&bar_in_full[(k - 1) & 1]));
