@@ -186,8 +186,9 @@ LOGO_API float logo_pmask_initial_threshold(float gamma, long long pmask_steps);
  *   Cache rows the step does not see (past seq_len, outside the window) may
  *   hold anything.  dims: B, T = R or L, Hq, Hkv (Hq / Hkv <= 16), D in
  *   {64, 128}; window >= 1 (local); scale as elsewhere (0 = 1/sqrt(D)).
- *   Workspace: logo_decode_workspace_size(dims) bytes (per-chunk fp32
- *   partials), one workspace per call in flight. */
+ *   Workspace: logo_decode_workspace_size(dims) bytes (fp32 partials of the
+ *   pieces that a cache is cut into, and a counter per cache and KV head), one
+ *   workspace per call in flight. */
 LOGO_API size_t logo_decode_workspace_size(logo_dims dims);
 LOGO_API int logo_decode_local_attn(const logo_bf16* q, const logo_bf16* k_ring, const logo_bf16* v_ring,
                 const int32_t* seq_len, logo_bf16* o, logo_dims dims, int window, float scale, void* workspace,
@@ -326,7 +327,7 @@ LOGO_API int logo_gate_bwd(const logo_bf16* x, const float* w_g, const float* ga
  *   logo_select): Q, of which the global branch reads those rows alone.
  * In : u_l [B,T,H,D] bf16 with H = dims.Hq, the head count of this tensor (Hq
  *      for Q, Hkv for K and V; dims.Hkv is not read); D 64 or 128; H*D <= 8192.
- *      LP runs on the tensor cores (warp-level MMA), SO elementwise.
+ *      LP runs on the tensor cores (tcgen05), SO elementwise.
  * Out: u_g [B,T,H,D] bf16: the listed rows written, other rows untouched.
  * Errors: LOGO_ERR_INVALID_ARG for a missing or doubled form or pointer;
  *      LOGO_ERR_UNSUPPORTED for D, H*D or 16-byte alignment. */

@@ -160,12 +160,15 @@ __device__ __forceinline__ void zero_unselected_dq(const BwdParams& p, int D, in
 //                atomics into the dQ accumulator (one 128-byte row segment per
 //                warp instruction); dK/dV epilogue at the end of each item
 //   warp 14      global branch: zero rows of the dense dQ for unselected tokens
-// Shared memory's bandwidth bounds it: a tile (2270 clocks in steady state) has
-// the MMAs read 192 KB (an N = 64 product reads its whole 4 KB A step: 48 clocks
-// by itself, 64 for N = 128), the copies write 32, dS^T 16, the statistics 16,
-// and the reductions 32 on their way through L1, 2300 clocks at 128 bytes each;
-// the data banks are busy 94% of the kernel's time.  Tiles of 128 rows move a
-// sixth less, but leave no TMEM for anything to overlap (5250 clocks and more).
+// Shared memory's bandwidth bounds it where items are long.  In a tile the MMAs
+// read 192 KB (an N = 64 product reads its whole 4 KB A step: 48 clocks by itself,
+// 64 for N = 128), the copies write 32, dS^T 16, the statistics 16, and the
+// reductions move 32 through L1: 2300 clocks at 128 bytes each, beside barriers
+// and the items' K, V, dK and dV.  16K, window 1024: 2590 clocks of the kernel's
+// time a tile, of which ncu counts 2570 as data-bank cycles (99%; the global call
+// at 16K 100%).  At 4K, with 9 (local) and 4.5 (global) tiles an item, they are
+// busy 83% and 72%: the item switches.  Tiles of 128 rows move a sixth less, but
+// leave no TMEM for anything to overlap (5250 clocks and more).
 struct Bwd2Cfg {
     static constexpr int D = 128;
     static constexpr int kBQ = 64;                 // queries per tile

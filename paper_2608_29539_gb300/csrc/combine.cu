@@ -480,8 +480,9 @@ __global__ void __launch_bounds__(kThreads, bwd_min_blocks<GPT, G, DGAIN, UNIT>(
 // the first version of this layout ran 200 and 280 instructions a vector and
 // was bound by issue.  Before, a thread had one token's loads in flight,
 // fetched the gains from L1 for every token and kept the sums in shared
-// memory.  16K, 32 heads, d 128, 1/8 selected: forward 68 -> 48 us (6.3 TB/s,
-// 93% of HBM), backward with gain gradients 128 -> 80 us (5.4 TB/s).
+// memory.  16K, 32 heads, d 128, 1/8 selected (kernel times by ncu): forward 70 ->
+// 46 us (287 MB, 6.2 TB/s, 91% of the copy rate), backward with gain gradients
+// 124 -> 78 us (436 MB, 5.6 TB/s, 82%).
 template <int MAXT>
 struct GainCfg {
     // The forward runs two blocks of 512 threads an SM at 64 registers, its

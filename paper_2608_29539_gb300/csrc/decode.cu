@@ -15,7 +15,7 @@
 // differ in length and pairs seldom divide by the CTAs (chunks of 1024 rows
 // handed out one by one: 4 of 32 sequences of 8K to 16K rows selected 58 us,
 // now 49; all 32 selected 360 us, now 252, 6.5 TB/s).  Where that saves little
-// (many pairs of equal length, as the rings are) a CTA takes whole pairs.
+// (many short pairs of equal length, as the rings are) a CTA takes whole pairs.
 // A CTA (4 warps) walks its run through a 3-stage TMA ring (128-byte
 // swizzle), a stage refilled once all four warps have released it, and
 // serves every query head of the KV head's group from each: S = q.K^T and
@@ -285,7 +285,7 @@ __global__ void __launch_bounds__(kDecThreads, 2) decode_attn_kernel(const __gri
     // inside the sub-tile loop waits for another warp: S = q.K^T lands in mma
     // fragments, P = 2^(S - m) goes from those straight into the A fragments
     // of O += P.V (a pair of 8-column S tiles is one 16-deep A fragment), and
-    // the four warps' results are combined once per item.
+    // the four warps' results are combined once per piece.
     constexpr int NT = D / 8;
     int consumed = 0;
     for (; cur.s < cur.s1 && ok; dec_next_piece<RING>(p, n_rows, cur)) {

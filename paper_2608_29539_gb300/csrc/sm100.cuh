@@ -420,7 +420,7 @@ __device__ __forceinline__ void umma_commit(uint32_t bar)
 
 // ------------------------------------------------------- warp-level MMA
 // Warp-level bf16 products (mma.sync m16n8k16, fp32 accumulate) for the small
-// contractions (decode rows, per-head transforms), operands fetched from
+// contractions (the decode step's rows), operands fetched from
 // shared memory by ldmatrix.
 __device__ __forceinline__ void ldsm_x4(uint32_t addr, uint32_t& r0, uint32_t& r1, uint32_t& r2, uint32_t& r3)
 {
