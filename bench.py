@@ -180,12 +180,12 @@ def gpu_launches_per_step(w):
     """The launches of a step as they are issued: the global forward's gather
     and schedule share one, its merge has none in sequences too short to be
     split (fewer than 32 blocks of 128 keys), and threshold selection takes
-    one for up to 128K tokens of the batch."""
+    one for up to 32K tokens of the batch, three beyond."""
     n = launches_per_step(w) - 1
     if -(-w.T // 128) < 32:
         n -= 1
-    if w.mode != "ratio" and w.B * w.T <= 131072:
-        n -= LAUNCHES_PER_STEP["select"] - 1
+    if w.mode != "ratio":
+        n -= LAUNCHES_PER_STEP["select"] - (1 if w.B * w.T <= 32768 else 3)
     return n
 
 
@@ -411,7 +411,7 @@ def routing_bench(layer, x, w, dev):
         L.logo_budget_update(rl_bufs[4], w.B, w.T, w.ratio, 2.0 ** -11, b_dev, f_out=f_dev)
 
     # each step reads the threshold the previous one wrote: 50 steps in one graph
-    return {"us_per_step": graph_ms(routing_step, 50) * 1e3, "launches_per_step": 2 if w.B * w.T <= 131072 else 4,
+    return {"us_per_step": graph_ms(routing_step, 50) * 1e3, "launches_per_step": 2 if w.B * w.T <= 32768 else 4,
             "note": "logo_select_device_threshold + logo_budget_update, no host sync; device time per step "
                     "(50 steps captured as one CUDA graph)"}
 

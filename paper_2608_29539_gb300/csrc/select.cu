@@ -12,7 +12,7 @@
 //                        cu_q[] and the total N.
 //   write_kernel         per chunk: block-wide prefix sums (warp ballots) turn
 //                        the decisions into z, pos and row_of, in ascending t.
-// Threshold mode on up to 128K tokens of the batch takes one launch instead:
+// Threshold mode on up to 32K tokens of the batch takes one launch instead:
 //   select_threshold_kernel  one block, or one 8-CTA cluster, over all of them.
 // Ratio mode with 4K < T <= 128K takes one launch too:
 //   select_ratio_cluster_kernel  one 8-CTA cluster per sequence; the CTAs share
@@ -784,9 +784,15 @@ cudaError_t launch_threshold(const float* p, const logo_dims& d, float b_th, con
                               row_of, n_sel);
 }
 
-// Threshold mode: one launch up to 128K tokens, else counts, scan, write.  Up
+// Threshold mode: one launch up to 32K tokens, else counts, scan, write.  Up
 // to 4K tokens one block is enough (four loads a thread); above, the cluster's
-// eight SMs share the loads and stores.
+// eight SMs share the loads and stores.  Past four tokens a thread their strided
+// loads and byte stores take longer than the launches saved: 64K tokens of one
+// sequence 24.5 us with 16 a thread, 6.6 in three launches over all SMs; 32K 5.6
+// and 6.3.  Many short sequences (more than kManyChunks chunks, which the one scan
+// block takes 256 at a time in ~1.3 us) stay with the one launch up to 128K.
+constexpr int64_t kManyChunks = 2048;
+
 int select_threshold(const float* p, const logo_dims& d, float b_th, const float* b_th_dev, uint8_t* z, int32_t* pos,
                      int32_t* cu_q, int32_t* row_of, int32_t* n_sel, const SelectWs& ws, cudaStream_t st)
 {
@@ -796,7 +802,8 @@ int select_threshold(const float* p, const logo_dims& d, float b_th, const float
     else if (n <= 4 * 1024) e = launch_threshold<1, 4>(p, d, b_th, b_th_dev, z, pos, cu_q, row_of, n_sel, st);
     else if (n <= 16 * 1024) e = launch_threshold<8, 2>(p, d, b_th, b_th_dev, z, pos, cu_q, row_of, n_sel, st);
     else if (n <= 32 * 1024) e = launch_threshold<8, 4>(p, d, b_th, b_th_dev, z, pos, cu_q, row_of, n_sel, st);
-    else if (n <= 128 * 1024) e = launch_threshold<8, 16>(p, d, b_th, b_th_dev, z, pos, cu_q, row_of, n_sel, st);
+    else if (n <= 128 * 1024 && d.B * static_cast<int64_t>((d.T + kChunk - 1) / kChunk) > kManyChunks)
+        e = launch_threshold<8, 16>(p, d, b_th, b_th_dev, z, pos, cu_q, row_of, n_sel, st);
     else {
         const int nchunk = (d.T + kChunk - 1) / kChunk;
         const dim3 grid(nchunk, d.B);
