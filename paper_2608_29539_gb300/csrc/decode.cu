@@ -373,7 +373,10 @@ __global__ void __launch_bounds__(kDecThreads, 2) decode_attn_kernel(const __gri
             // wherever the run was cut.  (Against the running max itself that holds
             // only where the max is set, so the error grew with the run: relative L2
             // against 64 bits over nine sizes from 1 x 868 to 32 x 16K tokens,
-            // local 0.00204 and global 0.00202, now 0.00197 and 0.00193.)
+            // local 0.00204 and global 0.00202, now 0.00197 and 0.00193.)  A sub-tile
+            // whose max lies 64 octaves below has nothing to keep exact, and with
+            // scores of 2^24 and more below the sum would be off by octaves: the
+            // reference stays.
             float alpha[2], m_use[2];
 #pragma unroll
             for (int r = 0; r < 2; ++r) {
@@ -381,7 +384,7 @@ __global__ void __launch_bounds__(kDecThreads, 2) decode_attn_kernel(const __gri
                 mx[r] = fmaxf(mx[r], __shfl_xor_sync(0xffffffffu, mx[r], 2));
                 m_run[r] = fmaxf(m_run[r], mx[r]);
                 const float old = m_ref[r];
-                if (mx[r] != -INFINITY) m_ref[r] = mx[r] + rintf(m_run[r] - mx[r]);
+                if (mx[r] - m_run[r] > -64.f) m_ref[r] = mx[r] + rintf(m_run[r] - mx[r]);
                 m_use[r] = m_ref[r] == -INFINITY ? 0.f : m_ref[r];
                 alpha[r] = ex2_approx(old - m_use[r]);  // 0 while nothing was seen
             }
