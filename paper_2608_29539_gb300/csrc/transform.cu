@@ -799,6 +799,16 @@ int so_bwd_blocks(const logo_dims& d)
     return static_cast<int>(rows < cap ? rows : cap);
 }
 
+// Every row: no row depends on where its sequence begins, so the batch is taken as
+// one sequence and a 128-row tile goes on across the ends (a tile a sequence at
+// least: 600 sequences of 10 rows, 16 heads of 64, forward and backward
+// 25.8 -> 6.6 and 47.5 -> 12.8 us).
+void every_row(logo_dims* d)
+{
+    d->T *= d->B;
+    d->B = 1;
+}
+
 int check_transform(const logo_dims& d, const void* u, const void* out)
 {
     if (d.B < 1 || d.T < 1 || d.Hq < 1) return LOGO_ERR_INVALID_ARG;
@@ -827,6 +837,7 @@ extern "C" int logo_branch_transform(const logo_bf16* u_l, const logo_bf16* a_lp
     if (!a_lp && (!s_so || !b_so)) return LOGO_ERR_INVALID_ARG;
     if (pos && (!cu_q || !n_sel_total)) return LOGO_ERR_INVALID_ARG;
     if (a_lp && !aligned16(a_lp)) return LOGO_ERR_UNSUPPORTED;
+    if (!pos) every_row(&dims);
     const RowSet R{pos, cu_q, n_sel_total, dims.B, dims.T};
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (a_lp && !pos) {
@@ -870,6 +881,7 @@ extern "C" int logo_branch_transform_bwd(const logo_bf16* u_l, const logo_bf16* 
     if (!aligned16(du_g) || (a_lp && !aligned16(a_lp))) return LOGO_ERR_UNSUPPORTED;
     if (!workspace || workspace_bytes < logo_branch_transform_bwd_workspace_size(dims)) return LOGO_ERR_WORKSPACE;
     if (a_lp && !aligned16(workspace)) return LOGO_ERR_WORKSPACE;  // the partial dA go there as float4
+    if (!pos) every_row(&dims);
     const RowSet R{pos, cu_q, n_sel_total, dims.B, dims.T};
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     float* part = static_cast<float*>(workspace);
