@@ -51,7 +51,7 @@ constexpr int kDecRows = 64;      // cache rows per sub-tile, 16 per warp
 constexpr int kDecRowsPerWarp = kDecRows / 4;
 constexpr int kDecMaxGroup = 16;  // query heads per KV head (the mma tile's 16 rows)
 constexpr int kDecMinSub = 2;     // sub-tiles of a CTA's run at least
-constexpr int kDecSplitCost = 4;  // what cutting pairs into pieces has to save, in sub-tiles
+constexpr int kDecSplitCost = 8;  // what cutting pairs into pieces has to save, in sub-tiles
 constexpr int kDecMaxWholeDense = 24, kDecMaxWholeRing = 32;  // sub-tiles of a pair left whole at most
 constexpr int kDecStages = 3;     // TMA ring depth
 
@@ -131,7 +131,11 @@ struct DecPiece {
 };
 
 // The next piece: of the next pair in order, or (whole pairs) of the pair a
-// grid further on.
+// grid further on: of all that the call could have while each gets a CTA of its
+// own or all are selected, else among those of the packed rows.  (Dealt out over
+// all the sequences, a few CTAs had two of the pairs of 14 selected of 49 x 192
+// rows, 8 KV heads of 128, and most had none: 10.4 us, now 7.0.  Finding a row's
+// sequence costs 0.5 us.)
 template <bool RING>
 __device__ __forceinline__ void dec_next_piece(const DecParams& p, int n_rows, DecPiece& c)
 {
@@ -141,9 +145,11 @@ __device__ __forceinline__ void dec_next_piece(const DecParams& p, int n_rows, D
         c.subs = 0;
         while (c.subs == 0) {
             c.pair += gridDim.x;
-            if (c.pair >= p.B * p.Hkv) return;
-            c.b = c.pair / p.Hkv;
-            c.kvh = c.pair - c.b * p.Hkv;
+            const bool direct = RING || p.B * p.Hkv <= static_cast<int>(gridDim.x) || n_rows == p.B;
+            if (c.pair >= (direct ? p.B : min(n_rows, p.cu_q[p.B])) * p.Hkv) return;
+            const int r = c.pair / p.Hkv;
+            c.b = direct ? r : seq_of_row(p.cu_q, p.B, r);
+            c.kvh = c.pair - r * p.Hkv;
             c.subs = dec_subs<RING>(p, n_rows, c.b, &c.len);
         }
         c.s1 = c.subs;
@@ -632,8 +638,11 @@ int launch_decode(DecParams& prm, const logo_dims& dims, cudaStream_t st)
     const long long n_sub = (prm.R + kDecRows - 1) / kDecRows, pairs = static_cast<long long>(prm.B) * prm.Hkv;
     const long long ctas = static_cast<long long>(std::min(per_sm, kDecCtasPerSm)) * device_sm_count();
     // Whole pairs when cutting them saves less than kDecSplitCost sub-tiles of
-    // the longest run (with full caches; the merge and the counters' clearing
-    // cost that much), else equal runs.  What is selected and how long the
+    // the longest run (with full caches), else equal runs: finding the runs, the
+    // counters' clearing and the merge cost about that many.  A call in runs of two
+    // sub-tiles takes 12 to 16 us (28 x 448 rows, one head of 64), whole pairs of
+    // seven 7.5; 90 x 768 rows, 8 heads of 128, whole and cut 50.4 and 53.6 with
+    // all selected, 15.2 and 21.3 with 23.  What is selected and how long the
     // sequences are is not known here, so a pair of more than kMaxWhole sub-tiles
     // is always cut: one CTA takes 0.7 us for a sub-tile and may be the only one
     // with work.  38 sequences of 16K rows and 8 KV heads (a pair a CTA) whole and
