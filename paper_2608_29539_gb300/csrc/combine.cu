@@ -927,9 +927,12 @@ int64_t gains_blocks(const logo_dims& d)
         with_gained_bwd<true>(d, [&](auto kernel, int slots) { return gain_launch(kernel, d, slots).grid; });
     int64_t unit = 0;
     const int gu = group_vectors(d, true), gpt = groups_per_thread(d, gu);
-    if (gu == 1) {
+    if (gu == 1 && gpt == 1) {
         gains_smem_ok(combine_bwd_kernel<1, 1, true, true>);
         unit = wave_blocks(combine_bwd_kernel<1, 1, true, true>, ntok, smem);
+    } else if (gu == 1) {
+        gains_smem_ok(combine_bwd_kernel<2, 1, true, true>);
+        unit = wave_blocks(combine_bwd_kernel<2, 1, true, true>, ntok, smem);
     } else if (gpt == 1) {
         gains_smem_ok(combine_bwd_kernel<1, 2, true, true>);
         unit = wave_blocks(combine_bwd_kernel<1, 2, true, true>, ntok, smem);
@@ -1044,7 +1047,8 @@ int combine_bwd_common(const logo_bf16* dO, const logo_bf16* o_l, const logo_bf1
                                                                    eps, dO_l, dO_c, dgate_p, part, ntok, dims.Hq,    \
                                                                    dims.D)
     if (gains && unit) {
-        if (g == 1) { LOGO_COMBINE_BWD(1, 1, true, true); }
+        if (g == 1 && gpt == 1) { LOGO_COMBINE_BWD(1, 1, true, true); }
+        else if (g == 1) { LOGO_COMBINE_BWD(2, 1, true, true); }  // more than kThreads vectors a token
         else if (gpt == 1) { LOGO_COMBINE_BWD(1, 2, true, true); }
         else { LOGO_COMBINE_BWD(2, 2, true, true); }
     } else if (!unit && dims.Hq * (dims.D / 8) <= kMaxVecGains) {
